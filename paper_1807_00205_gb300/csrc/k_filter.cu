@@ -24,13 +24,13 @@
 // Windows no tier can hold go to a global path that writes their hits to
 // global memory, radix-sorts them by (window, o, t) and runs the same sweep.
 //
-// Refine (k_refine_batch): each run's domain, W_Q u (target minimizers of the
-// run's span that can change the estimate), is sorted by a warp into a
-// per-warp slot; then one lane per run rolls the target window over the
-// run's breakpoints, keeping presence and sharedness counters and the s-th
-// present hash, so the estimate |S(W_Q u W_T) n W_Q n W_T| is exact at every
-// breakpoint.  Runs whose domain exceeds the batched kernel's slots go to
-// k_refine (one warp per run, bitsets over the sorted domain).
+// Refine (k_refine_batch): each run's span records become events (position,
+// rank among W_Q), set up by a warp; then one lane per run rolls the target
+// window over the run's breakpoints, keeping a count per rank, the shared
+// hashes and the threshold that says which of them lie among the s smallest
+// of W_Q u W_T, so the estimate |S(W_Q u W_T) n W_Q n W_T| is exact at every
+// breakpoint.  Runs past the batched kernel's limits go to k_refine (one
+// warp per run, bitsets over the sorted domain).
 #include <chrono>
 #include <condition_variable>
 #include <cstring>
@@ -1378,11 +1378,9 @@ __global__ void k_gather_runs(const sedef_run_t* in, const uint32_t* perm, int64
 
 // ----------------------------------------------------------------- refine --
 //
-// Two instantiations of one kernel: a lean one (at most 256 query records
-// and 512 span records per run, one piece, ~12 KB of shared memory per warp
-// so that 16 warps per SM hide the latency of the sequential roll) and a
-// large one (any run, in pieces of at most 1024 span records) for the runs
-// the lean one hands over.
+// Two kernels: a lean one (k_refine_batch: at most 256 query records and 512
+// span records per run) and a large one (any run, in pieces of at most 1024
+// span records) for the runs the lean one hands over.
 //
 // The estimate at j never exceeds the number of W_Q hashes shared with the
 // window (the filter's shared_o(j)), so it is evaluated only where that
@@ -1491,6 +1489,10 @@ struct RefineArgs {
   unsigned int* nbig;
   const uint4* ranges;  // per run: query records [x, y), span records [z, w)
   unsigned long long* next;  // chunk counters of the two kernels
+  // lean kernel: event words (ev_words + kEvPad per warp), W_Q hashes per roll
+  uint32_t* events = nullptr;
+  int ev_words = 0;
+  int scap = 0;
 };
 
 template <int QC, int RC, bool kLean>
@@ -1814,152 +1816,134 @@ __global__ void __launch_bounds__(32 * (kLean ? kRWarps : kRWarpsBig)) k_refine(
 
 // ------------------------------------------------- batched lean refine ----
 //
-// A warp sets up runs one at a time (cooperatively) into slots of a per-warp
-// arena, then every lane rolls its own run through its slot, so many rolls
-// proceed side by side.  Setup per run: the span records are read once
-// (hash, rank among W_Q, W_Q membership, candidate flag); the domain is W_Q
-// (already sorted) merged by rank with the sorted distinct non-W_Q kept
-// hashes, so a kept record's domain index is its rank among W_Q plus its
-// rank among those hashes.  A slot holds one 32-bit event per kept record
-// (offset of its position from j_a, domain index, W_Q flag) and one counter
-// per domain hash (presence for non-W_Q hashes, sharedness for W_Q hashes).
-// Transient setup data (the span records' hashes, sort buffers) lives at the
-// top of the arena, slots grow from the bottom.  Runs beyond the lean limits
-// (more than 256 query records, 512 span records or a span of 65,536 bases)
-// go to the large kernel.
+// A warp sets up runs one at a time (cooperatively), writing each run's
+// events to its own stretch of device memory, then every lane rolls one run,
+// so up to 32 rolls proceed side by side.
+//
+// The estimate needs no merged domain.  W_Q's hashes h_0 < ... < h_{s-1} are
+// all in the union, so h_r is among the union's s smallest exactly when
+// r + 1 + #{distinct non-W_Q hashes of the window below h_r} <= s.  The left
+// side grows with r: a threshold R (how many h_r pass) decides, and est is
+// the number of shared h_r with r < R.  A non-W_Q record acts only through
+// its rank q among W_Q (it lies below h_q, ..., h_{s-1}); one whose rank is s
+// never does.  So the state of a roll is a count per rank c[q], the shared
+// bits, R, and B = the sum of c[q] below R; one hash entering or leaving
+// moves R by at most one.
+//
+// A hash is in the window while any of its records is: records of one hash
+// at most span + 1 apart cover one stretch of target starts, so only a
+// stretch's first record enters and only its last one leaves, and nothing
+// counts occurrences.  The setup finds a record's previous occurrence with
+// an open-addressing table of the span's hashes (no sort).
+//
+// What bounds it: instruction issue (setup) and the latency of the dependent
+// shared-memory accesses (roll).  Events live in device memory (L2) so that
+// shared memory holds 32 rolls per warp instead of the six or so whose
+// events fit there; a lane reads its two event streams 16 bytes at a time,
+// one load ahead.  Measured against the form that sorted a merged domain per
+// run into shared-memory slots and took 32 runs per warp whatever their
+// number: 1.26 M runs of a 200-genome batch 17.4 -> 5.4 ms, 2.5 M runs of a
+// 240 Mbp assembly 19.7 -> 6.6 ms, 299 runs of a 2 Mbp genome 1.75 -> 0.08 ms.
+// Runs beyond the lean limits (more than 256 query records,
+// 512 span records, a span of 65,536 bases or more W_Q hashes than the
+// launch's counters) go to the large kernel.
 
 constexpr int kBWarps = 4;
 constexpr int kBQC = 256, kBRC = 512;
-constexpr int kArenaWords = 2816;  // 11 KB per warp
+constexpr int kEvWords = 8192;  // event words of a warp's stretch
+constexpr int kEvPad = 16;      // read ahead past the last event
+// event: position - j_a (bits 0-15), rank among W_Q (16-23), flags
+constexpr uint32_t kEvW = 1u << 24;        // a W_Q hash
+constexpr uint32_t kEvNoEnter = 1u << 25;  // its hash is already in the window
+constexpr uint32_t kEvNoLeave = 1u << 26;  // its hash stays in the window
+// hash table of a run's kept records: keys, then their last event index
+constexpr int kBTabMax = 1024;
+constexpr int kBTabWords = kBTabMax + kBTabMax / 2;
 
-struct BatchWarp {
-  uint32_t arena[kArenaWords];
-  uint32_t wq_h[kBQC];
-  uint8_t wq_m[kBQC];
-  // span record: bit0 strand, bit1 in W_Q, bit2 candidate, bit3 kept,
-  // bits 4.. its hash's rank among W_Q (lower bound)
-  uint16_t rinfo[kBRC];
-  uint32_t h_off[32];     // slot start (words)
-  uint32_t h_run[32];     // run index
-  uint16_t h_nrel[32], h_D[32], h_dmax[32], h_s[32];
-};
-
-struct Slot {
-  uint32_t* ev;    // per kept record: position - j_a (bits 0-15), domain index (16-25), W_Q (31)
-  uint16_t* cnt;   // per domain hash: occurrences in the window
-  uint32_t* pb;    // present
-  uint32_t* sb;    // shared
-};
-
-__device__ __forceinline__ int slot_words(int nrel, int dmax) {
-  return nrel + (dmax + 1) / 2 + 2 * ((dmax + 31) / 32);
+// Shared words of a warp for rolls with at most scap W_Q hashes: 16-bit
+// counts and shared bits for 32 lanes, each lane in its own bank (the setup's
+// hash table lies over them).
+__host__ __device__ constexpr int roll_words(int scap) {
+  return (scap / 2 + scap / 32) * 32 > kBTabWords ? (scap / 2 + scap / 32) * 32 : kBTabWords;
+}
+__host__ __device__ constexpr size_t refine_warp_bytes(int scap) {
+  return (size_t)kBQC * 4 + kBQC + (size_t)roll_words(scap) * 4;
 }
 
-__device__ __forceinline__ Slot slot_at(uint32_t* base, int nrel, int dmax) {
-  Slot sl;
-  sl.ev = base;
-  sl.cnt = reinterpret_cast<uint16_t*>(base + nrel);
-  sl.pb = base + nrel + (dmax + 1) / 2;
-  sl.sb = sl.pb + (dmax + 31) / 32;
-  return sl;
-}
-
-// Rolls one run (single lane) over target starts j_a + [0, jend]: enters the
-// first window's records, finds theta (s-th present hash) and est by
-// scanning the bitsets, then keeps both exact through every enter/leave (as
-// in the large kernel).  Offsets from j_a fit in 16 bits, so the roll runs
-// in 32-bit arithmetic.
-__device__ void roll_run(const Slot& sl, int nrel, int D, int s, int mx, int jend, int span,
-                         int* best_out, int* jstar_out) {
-  const int nwords = (D + 31) >> 5;
-  auto pos = [&](int x) { return (int)(sl.ev[x] & 0xFFFFu); };
+// Rolls one run (single lane) over target starts j_a + [0, jend].  cnt and sb
+// are the lane's zeroed counters and shared bits (one 32-bit word per 32).
+__device__ void roll_run(const uint32_t* __restrict__ ev, int nrel, int s, int mx, int jend, int span,
+                         uint32_t* cnt, uint32_t* sb, int* best_out, int* jstar_out) {
+  const uint4* ev4 = reinterpret_cast<const uint4*>(ev);
+  auto count = [&](int q) -> uint16_t& {
+    return reinterpret_cast<uint16_t*>(cnt + ((q >> 1) << 5))[q & 1];
+  };
+  auto shared_bit = [&](int r) { return (int)((sb[(r >> 5) << 5] >> (r & 31)) & 1u); };
+  uint4 eb = ev4[0], en = ev4[1], lb = eb, ln = en;  // next events of either stream
   int e = 0, l = 0, j = 0;
-  while (e < nrel && pos(e) <= j + span) {
-    const uint32_t v = sl.ev[e];
-    const int d = (int)((v >> 16) & 0x3FFu);
-    if (sl.cnt[d]++ == 0) {
-      if (v >> 31) sl.sb[d >> 5] |= 1u << (d & 31);
-      else sl.pb[d >> 5] |= 1u << (d & 31);
-    }
-    ++e;
-  }
-  int theta = 0, est = 0;
-  {
-    int acc = 0;
-    for (int w = 0; w < nwords; ++w) {
-      const int c = __popc(sl.pb[w]);
-      if (acc + c >= s) {
-        uint32_t v = sl.pb[w];
-        for (int y = 1; y < s - acc; ++y) v &= v - 1u;
-        const int b = __ffs(v) - 1;
-        theta = w * 32 + b;
-        const uint32_t below = (b >= 31) ? 0xFFFFFFFFu : ((2u << b) - 1u);
-        est += __popc(sl.sb[w] & below);
-        break;
-      }
-      acc += c;
-      est += __popc(sl.sb[w]);
-    }
-  }
-  auto bit = [&](const uint32_t* bs, int d) { return (int)((bs[d >> 5] >> (d & 31)) & 1u); };
-  auto pred = [&](int d) {
-    int w = d >> 5;
-    uint32_t bits = sl.pb[w] & ((1u << (d & 31)) - 1u);
-    while (bits == 0 && w > 0) bits = sl.pb[--w];
-    return bits ? w * 32 + 31 - __clz(bits) : 0;
-  };
-  auto succ = [&](int d) {
-    int w = d >> 5;
-    uint32_t bits = ((d & 31) == 31) ? 0u : (sl.pb[w] & ~((2u << (d & 31)) - 1u));
-    while (bits == 0 && w + 1 < nwords) bits = sl.pb[++w];
-    return bits ? w * 32 + __ffs(bits) - 1 : d;
-  };
   int best = -1, jstar = 0;
+  int R = s, B = 0, est = 0;
   while (true) {
-    if (est > best) {
-      best = est;
-      jstar = j;
-      if (best >= mx) break;
-    }
-    const int ne = e < nrel ? pos(e) - span : INT_MAX;
-    const int nl = l < e ? pos(l) + 1 : INT_MAX;
+    const int ne = e < nrel ? max((int)(eb.x & 0xFFFFu) - span, 0) : INT_MAX;
+    const int nl = l < nrel ? (int)(lb.x & 0xFFFFu) + 1 : INT_MAX;
     const int nx = min(ne, nl);
-    if (nx > jend) break;
-    j = nx;
-    while (l < e && pos(l) + 1 <= j) {
-      const uint32_t v = sl.ev[l];
-      const int d = (int)((v >> 16) & 0x3FFu);
-      if (--sl.cnt[d] == 0) {
-        if (v >> 31) {
-          sl.sb[d >> 5] &= ~(1u << (d & 31));
-          if (d <= theta) --est;
-        } else {
-          sl.pb[d >> 5] &= ~(1u << (d & 31));
-          if (d <= theta) {
-            theta = succ(theta);
-            est += bit(sl.sb, theta);
-          }
-        }
+    if (nx > j) {  // every event up to j is in
+      if (est > best) {
+        best = est;
+        jstar = j;
+        if (best >= mx) break;
       }
-      ++l;
+      if (nx > jend) break;
+      j = nx;
     }
-    while (e < nrel && pos(e) - span <= j) {
-      const uint32_t v = sl.ev[e];
-      const int d = (int)((v >> 16) & 0x3FFu);
-      if (sl.cnt[d]++ == 0) {
-        if (v >> 31) {
-          sl.sb[d >> 5] |= 1u << (d & 31);
-          if (d <= theta) ++est;
-        } else {
-          sl.pb[d >> 5] |= 1u << (d & 31);
-          if (d < theta) {
-            const int old = theta;
-            theta = pred(theta);
-            est -= bit(sl.sb, old);
+    if (ne <= nl) {
+      const uint32_t v = eb.x;
+      eb.x = eb.y;
+      eb.y = eb.z;
+      eb.z = eb.w;
+      if ((++e & 3) == 0) {
+        eb = en;
+        en = ev4[(e >> 2) + 1];
+      }
+      if (v & kEvNoEnter) continue;
+      const int q = (int)((v >> 16) & 0xFFu);
+      if (v & kEvW) {
+        sb[(q >> 5) << 5] |= 1u << (q & 31);
+        if (q < R) ++est;
+      } else {
+        ++count(q);
+        if (q < R && R + ++B > s) {
+          --R;
+          B -= count(R);
+          est -= shared_bit(R);
+        }
+      }
+    } else {
+      const uint32_t v = lb.x;
+      lb.x = lb.y;
+      lb.y = lb.z;
+      lb.z = lb.w;
+      if ((++l & 3) == 0) {
+        lb = ln;
+        ln = ev4[(l >> 2) + 1];
+      }
+      if (v & kEvNoLeave) continue;
+      const int q = (int)((v >> 16) & 0xFFu);
+      if (v & kEvW) {
+        sb[(q >> 5) << 5] &= ~(1u << (q & 31));
+        if (q < R) --est;
+      } else {
+        --count(q);
+        if (q < R) --B;
+        if (q <= R && R < s) {
+          const int c = count(R);
+          if (R + 1 + B + c <= s) {
+            B += c;
+            est += shared_bit(R);
+            ++R;
           }
         }
       }
-      ++e;
     }
   }
   *best_out = best;
@@ -1975,43 +1959,107 @@ __device__ __forceinline__ int lb_u32(const uint32_t* v, int n, uint32_t x) {
   return lo;
 }
 
+// Sorts 32 * NR keys held by a warp (key of index lane * NR + x in v[x]).
+template <int NR>
+__device__ __forceinline__ void warp_sort_regs(uint32_t (&v)[NR]) {
+  const int lane = lane_id();
+#pragma unroll
+  for (int size = 2; size <= 32 * NR; size <<= 1) {
+#pragma unroll
+    for (int stride = size >> 1; stride > 0; stride >>= 1) {
+      if (stride >= NR) {
+        const bool keep_min = (((lane * NR) & size) == 0) == ((lane & (stride / NR)) == 0);
+#pragma unroll
+        for (int x = 0; x < NR; ++x) {
+          const uint32_t o = __shfl_xor_sync(0xffffffffu, v[x], stride / NR);
+          v[x] = keep_min ? min(v[x], o) : max(v[x], o);
+        }
+      } else {
+#pragma unroll
+        for (int x = 0; x < NR; ++x) {
+          if (x & stride) continue;
+          const bool asc = ((lane * NR + x) & size) == 0;
+          const uint32_t p = v[x], q = v[x | stride];
+          v[x] = asc ? min(p, q) : max(p, q);
+          v[x | stride] = asc ? max(p, q) : min(p, q);
+        }
+      }
+    }
+  }
+}
+
+// Query records [qa, qa + c) as sorted (hash << 1 | strand) keys in buf[0..32 * NR).
+template <int NR>
+__device__ __forceinline__ void sort_window(const uint64_t* __restrict__ qrec, int64_t qa, int c,
+                                            uint32_t* buf) {
+  const int lane = lane_id();
+  uint32_t v[NR];
+#pragma unroll
+  for (int x = 0; x < NR; ++x) {
+    const int at = x * 32 + lane;
+    v[x] = kNone;
+    if (at < c) {
+      const uint64_t r = qrec[qa + at];
+      v[x] = (rec_hash(r) << 1) | rec_strand(r);
+    }
+  }
+  warp_sort_regs<NR>(v);
+#pragma unroll
+  for (int x = 0; x < NR; ++x) buf[lane * NR + x] = v[x];
+}
+
 __global__ void __launch_bounds__(32 * kBWarps) k_refine_batch(RefineArgs a) {
   a.nruns = live_n(a.nruns, a.dnruns);
-  a.nt = live_n(a.nt, a.dnt);
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int warp = threadIdx.x >> 5, lane = lane_id();
-  BatchWarp& B = reinterpret_cast<BatchWarp*>(smem_raw)[warp];
-  constexpr int kChunk = 32;
+  const int scap = a.scap;
+  unsigned char* base_s = smem_raw + (size_t)warp * refine_warp_bytes(scap);
+  uint32_t* scratch = reinterpret_cast<uint32_t*>(base_s);
+  uint32_t* wq_h = scratch + roll_words(scap);
+  uint8_t* wq_m = reinterpret_cast<uint8_t*>(wq_h + kBQC);
+  const int64_t nwarps = (int64_t)gridDim.x * kBWarps;
+  uint32_t* ev_base = a.events + ((int64_t)blockIdx.x * kBWarps + warp) * (a.ev_words + kEvPad);
+  // few runs: spread them over the warps (one warp took 32 runs one after
+  // another in 0.46 ms while the others had none); many: 32 neighbours at a
+  // time, as runs of one window share W_Q
+  int64_t chunk = (a.nruns + nwarps - 1) / nwarps;
+  chunk = chunk < 1 ? 1 : (chunk > 32 ? 32 : chunk);
   int64_t prev_qa = -1, prev_qb = -1;
-  int s = 0;
+  int s = 0, smax = 0;
   int nslots = 0, used = 0;
+  int64_t my_run = 0;  // this lane's run
+  int my_off = 0, my_nrel = 0, my_s = 0;
 
   auto flush = [&]() {
     __syncwarp();
+    const int nw = (scap / 2) * 32;  // counters, then shared bits
+    uint4* z4 = reinterpret_cast<uint4*>(scratch);
+    for (int x = lane; x < (smax + 1) / 2 * 8; x += 32) z4[x] = make_uint4(0, 0, 0, 0);
+    for (int x = lane; x < (smax + 31) / 32 * 8; x += 32) z4[nw / 4 + x] = make_uint4(0, 0, 0, 0);
+    __syncwarp();
     if (lane < nslots) {
-      const int64_t ri = B.h_run[lane];
-      const sedef_run_t run = a.runs[ri];
-      const int nrel = B.h_nrel[lane], D = B.h_D[lane], sq = B.h_s[lane];
-      const Slot sl = slot_at(B.arena + B.h_off[lane], nrel, B.h_dmax[lane]);
+      const sedef_run_t run = a.runs[my_run];
       int best, jstar;
-      roll_run(sl, nrel, D, sq, run.max_shared, (int)(run.j_b - run.j_a), a.span, &best, &jstar);
-      sedef_run_t& out = a.runs[ri];
+      roll_run(ev_base + my_off, my_nrel, my_s, run.max_shared, (int)(run.j_b - run.j_a), a.span,
+               scratch + lane, scratch + nw + lane, &best, &jstar);
+      sedef_run_t& out = a.runs[my_run];
       out.est = (uint16_t)(best < 0 ? 0 : best);
-      out.den = (uint16_t)sq;
+      out.den = (uint16_t)my_s;
       out.j_star = run.j_a + (uint32_t)jstar;
-      out.keep = (best >= a.mtab[sq]) ? 1 : 0;
+      out.keep = (best >= a.mtab[my_s]) ? 1 : 0;
     }
     __syncwarp();
     nslots = 0;
     used = 0;
+    smax = 0;
   };
 
   while (true) {
     int64_t c0 = 0;
-    if (lane == 0) c0 = (int64_t)atomicAdd(a.next, (unsigned long long)kChunk);
+    if (lane == 0) c0 = (int64_t)atomicAdd(a.next, (unsigned long long)chunk);
     c0 = __shfl_sync(0xffffffffu, c0, 0);
     if (c0 >= a.nruns) break;
-    const int64_t c1 = min(a.nruns, c0 + kChunk);
+    const int64_t c1 = min(a.nruns, c0 + chunk);
     for (int64_t ri = c0; ri < c1; ++ri) {
       const sedef_run_t run = a.runs[ri];
       const int64_t i = run.i;
@@ -2020,28 +2068,17 @@ __global__ void __launch_bounds__(32 * kBWarps) k_refine_batch(RefineArgs a) {
       const int64_t qa = rg.x, qb = rg.y, rlo = rg.z, rend = rg.w;
       const int c = (int)(qb - qa);
       const int nr = (int)(rend - rlo);
-      if (c > kBQC || nr > kBRC || (int64_t)run.j_b + a.span - run.j_a >= 65536) {
-        if (lane == 0) a.big[atomicAdd(a.nbig, 1u)] = (uint32_t)ri;
-        continue;
-      }
-      // ---- W_Q (kept from the previous run of the same window); sorted in
-      // a transient buffer at the top of the arena
-      if (qa != prev_qa || qb != prev_qb) {
+      bool big = c > kBQC || nr > kBRC || (int64_t)run.j_b + a.span - run.j_a >= 65536;
+      // ---- W_Q (kept from the previous run of the same window)
+      if (!big && (qa != prev_qa || qb != prev_qb)) {
         prev_qa = qa;
         prev_qb = qb;
-        const int npq = next_pow2(c < 2 ? 2 : c);
-        if (used + npq > kArenaWords) flush();
-        uint32_t* buf = B.arena + kArenaWords - npq;
-        for (int x = lane; x < npq; x += 32) {
-          uint32_t key = kNone;
-          if (x < c) {
-            const uint64_t r = a.qrec[qa + x];
-            key = (rec_hash(r) << 1) | rec_strand(r);
-          }
-          buf[x] = key;
-        }
         __syncwarp();
-        warp_sort_u32(buf, npq);
+        uint32_t* buf = scratch;
+        if (c <= 64) sort_window<2>(a.qrec, qa, c, buf);
+        else if (c <= 128) sort_window<4>(a.qrec, qa, c, buf);
+        else sort_window<8>(a.qrec, qa, c, buf);
+        __syncwarp();
         s = 0;
         for (int base = 0; base < c; base += 32) {
           const int x = base + lane;
@@ -2058,140 +2095,103 @@ __global__ void __launch_bounds__(32 * kBWarps) k_refine_batch(RefineArgs a) {
           const unsigned bal = __ballot_sync(0xffffffffu, first);
           if (first) {
             const int d = s + __popc(bal & lanemask_lt());
-            B.wq_h[d] = h;
-            B.wq_m[d] = (uint8_t)mask;
+            wq_h[d] = h;
+            wq_m[d] = (uint8_t)mask;
           }
           s += __popc(bal);
         }
         __syncwarp();
       }
-      // ---- space: the span records' hashes and the largest sort buffer at
-      // the top of the arena (the slot's exact size is checked below)
-      const int npr = next_pow2(nr < 2 ? 2 : nr);
-      if (nslots == 32 || used + nr + npr > kArenaWords) flush();
-      uint32_t* th = B.arena + kArenaWords - nr;  // transient: hashes of the span records
-      // ---- pass over the span records: hash, rank among W_Q, flags, max(C)
-      uint32_t cmax = 0;
-      bool have_c = false;
+      if (big || s > scap) {
+        if (lane == 0) a.big[atomicAdd(a.nbig, 1u)] = (uint32_t)ri;
+        continue;
+      }
+      if (nslots == 32 || used + nr + 8 > a.ev_words) flush();
+      // ---- the span's hashes: a table with at most 5/8 of its slots taken
+      const int tsz = nr <= 320 ? kBTabMax / 2 : kBTabMax;
+      uint32_t* tab = scratch;
+      uint16_t* tval = reinterpret_cast<uint16_t*>(scratch + tsz);
+      __syncwarp();
+      {
+        uint4* z4 = reinterpret_cast<uint4*>(scratch);
+        for (int x = lane; x < tsz / 4; x += 32) z4[x] = make_uint4(0, 0, 0, 0);
+        for (int x = lane; x < tsz / 8; x += 32) z4[tsz / 4 + x] = make_uint4(kNone, kNone, kNone, kNone);
+      }
+      __syncwarp();
+      // ---- one pass over the span records: rank among W_Q, whether the
+      // record counts, its hash's previous occurrence, the event
+      uint32_t* ev = ev_base + used;
+      int nrel = 0;
+      uint64_t ahead = lane < nr ? a.trec[rlo + lane] : 0;
       for (int base = 0; base < nr; base += 32) {
-        const int x = base + lane;
-        bool cand = false;
-        uint32_t h = 0;
-        if (x < nr) {
-          const uint64_t r = a.trec[rlo + x];
-          h = rec_hash(r);
-          const uint32_t t = rec_pos(r), st = rec_strand(r);
-          const int q = lb_u32(B.wq_h, s, h);
-          const bool member = q < s && B.wq_h[q] == h;
+        const uint64_t r = ahead;
+        const bool ok = base + lane < nr;
+        if (base + 32 + lane < nr) ahead = a.trec[rlo + base + 32 + lane];
+        const uint32_t h = rec_hash(r), t = rec_pos(r);
+        const int q = lb_u32(wq_h, s, h);
+        bool keep = ok && q < s;
+        bool member = false;
+        if (keep && wq_h[q] == h) {
+          member = true;
           const bool self = a.self_mode && (int64_t)t >= i && (int64_t)t <= i + a.span;
-          cand = member && !self && ((B.wq_m[q] >> (st ^ (uint32_t)o)) & 1u);
-          th[x] = h;
-          B.rinfo[x] = (uint16_t)(st | (member ? 2u : 0u) | (cand ? 4u : 0u) | ((uint32_t)q << 4));
+          keep = !self && ((wq_m[q] >> (rec_strand(r) ^ (uint32_t)o)) & 1u);
         }
-        uint32_t hm = cand ? h : 0u;
-        const bool any = __any_sync(0xffffffffu, cand);
-#pragma unroll
-        for (int d = 16; d > 0; d >>= 1) hm = max(hm, __shfl_xor_sync(0xffffffffu, hm, d));
-        if (any) {
-          cmax = have_c ? max(cmax, hm) : hm;
-          have_c = true;
-        }
-      }
-      __syncwarp();
-      // ---- kept records: candidates' occurrences and non-W_Q hashes below max(C)
-      int nrel = 0, n1 = 0;
-      for (int base = 0; base < nr && have_c; base += 32) {
-        const int x = base + lane;
-        bool keep = false, nonq = false;
-        if (x < nr) {
-          const uint32_t f = B.rinfo[x];
-          nonq = !(f & 2u) && th[x] < cmax;
-          keep = (f & 4u) || nonq;
-          if (keep) B.rinfo[x] = (uint16_t)(f | 8u);
-        }
-        nrel += __popc(__ballot_sync(0xffffffffu, keep));
-        n1 += __popc(__ballot_sync(0xffffffffu, nonq));
-      }
-      __syncwarp();
-      const int dmax = s + n1;
-      const int np1 = next_pow2(n1 < 2 ? 2 : n1);
-      uint32_t* u1 = th - np1;  // transient sort buffer of the non-W_Q kept hashes
-      if (used + slot_words(nrel, dmax) > kArenaWords - nr - np1) flush();
-      const Slot sl = slot_at(B.arena + used, nrel, dmax);
-      {
-        int y = 0, z = 0;
-        for (int base = 0; base < nr && nrel > 0; base += 32) {
-          const int x = base + lane;
-          bool keep = false, nonq = false;
-          uint32_t f = 0;
-          if (x < nr) {
-            f = B.rinfo[x];
-            keep = (f & 8u) != 0;
-            nonq = keep && !(f & 2u);
+        const unsigned bk = __ballot_sync(0xffffffffu, keep);
+        const int y = nrel + __popc(bk & lanemask_lt());
+        uint32_t slot = 0;
+        bool seen = false;
+        if (keep) {
+          slot = (h * 0x9E3779B1u) >> (nr <= 320 ? 23 : 22);
+          while (true) {  // a free slot is always found
+            const uint32_t old = atomicCAS(&tab[slot], 0u, h + 1u);
+            if (old == 0u) break;
+            if (old == h + 1u) {
+              seen = true;
+              break;
+            }
+            slot = (slot + 1u) & (uint32_t)(tsz - 1);
           }
-          const unsigned bk = __ballot_sync(0xffffffffu, keep);
-          const unsigned bn = __ballot_sync(0xffffffffu, nonq);
-          if (keep) {
-            const int yy = y + __popc(bk & lanemask_lt());
-            sl.ev[yy] = (rec_pos(a.trec[rlo + x]) - run.j_a) | ((f & 2u) ? 0x80000000u : 0u);
-          }
-          if (nonq) u1[z + __popc(bn & lanemask_lt())] = th[x];
-          y += __popc(bk);
-          z += __popc(bn);
         }
-        for (int x = n1 + lane; x < np1; x += 32) u1[x] = kNone;
-      }
-      __syncwarp();
-      warp_sort_u32(u1, np1);
-      int u = 0;  // distinct non-W_Q kept hashes, compacted in place
-      for (int base = 0; base < n1; base += 32) {
-        const int x = base + lane;
-        const uint32_t v = x < n1 ? u1[x] : kNone;
-        const bool first = x < n1 && (x == 0 || u1[x - 1] != v);
-        const unsigned bal = __ballot_sync(0xffffffffu, first);
+        uint32_t v = (t - run.j_a) | ((uint32_t)q << 16) | (member ? kEvW : 0u);
+        bool last = true;  // the last record of its hash in these 32
+        if (__any_sync(0xffffffffu, seen)) {
+          // the previous occurrence: the nearest lower lane with the hash,
+          // else the table's (written after an earlier 32)
+          const unsigned peers = __match_any_sync(0xffffffffu, keep ? h : (0x80000000u | (uint32_t)lane));
+          const unsigned lower = peers & lanemask_lt();
+          const int pl = lower ? 31 - __clz(lower) : lane;
+          const uint32_t pt = __shfl_sync(0xffffffffu, t, pl);
+          last = (peers >> lane) == 1u;
+          int py = -1;
+          uint32_t gap = kNone;
+          if (keep && lower) {
+            py = nrel + __popc(bk & ((1u << pl) - 1u));
+            gap = t - pt;
+          } else if (seen && tval[slot] != 0xFFFFu) {
+            py = tval[slot];
+            gap = t - run.j_a - (ev[py] & 0xFFFFu);
+          }
+          const bool joined = py >= 0 && gap <= (uint32_t)a.span + 1u;
+          if (joined) v |= kEvNoEnter;
+          if (keep) ev[y] = v;
+          __syncwarp();
+          if (joined) ev[py] |= kEvNoLeave;  // one successor per record
+        } else if (keep) {
+          ev[y] = v;
+        }
+        if (keep && last) tval[slot] = (uint16_t)y;
+        nrel += __popc(bk);
         __syncwarp();
-        if (first) u1[u + __popc(bal & lanemask_lt())] = v;
-        __syncwarp();
-        u += __popc(bal);
       }
-      const int D = s + u;
-      // domain index of a kept record: its hash's rank among W_Q plus its
-      // rank among the distinct non-W_Q kept hashes
-      {
-        int y = 0;
-        for (int base = 0; base < nr && nrel > 0; base += 32) {
-          const int x = base + lane;
-          const uint32_t f = x < nr ? B.rinfo[x] : 0u;
-          const bool keep = (f & 8u) != 0;
-          const unsigned bk = __ballot_sync(0xffffffffu, keep);
-          if (keep) {
-            const uint32_t d = (f >> 4) + (uint32_t)lb_u32(u1, u, th[x]);
-            sl.ev[y + __popc(bk & lanemask_lt())] |= d << 16;
-          }
-          y += __popc(bk);
-        }
+      if (lane == nslots) {
+        my_run = ri;
+        my_off = used;
+        my_nrel = nrel;
+        my_s = s;
       }
-      for (int x = lane; x < dmax; x += 32) sl.cnt[x] = 0;
-      for (int x = lane; x < (dmax + 31) / 32; x += 32) {
-        sl.pb[x] = 0;
-        sl.sb[x] = 0;
-      }
-      __syncwarp();
-      for (int k = lane; k < s; k += 32) {
-        const int d = k + lb_u32(u1, u, B.wq_h[k]);
-        atomicOr(&sl.pb[d >> 5], 1u << (d & 31));
-      }
-      if (lane == 0) {
-        B.h_off[nslots] = (uint32_t)used;
-        B.h_run[nslots] = (uint32_t)ri;
-        B.h_nrel[nslots] = (uint16_t)nrel;
-        B.h_D[nslots] = (uint16_t)D;
-        B.h_dmax[nslots] = (uint16_t)dmax;
-        B.h_s[nslots] = (uint16_t)s;
-      }
-      __syncwarp();
       ++nslots;
-      used += slot_words(nrel, dmax);
+      used += (nrel + 3) & ~3;
+      smax = max(smax, s);
     }
   }
   flush();
@@ -2365,7 +2365,12 @@ int order_and_refine(sedef_ctx* ctx, const FArgs& a, const Derived& D, int nqseq
                      const uint32_t* toff, unsigned long long* counters, sedef_run_t* raw,
                      int64_t total, sedef_run_t* runs, const uint32_t* druns, const uint32_t* dnt) {
   cudaStream_t st = ctx_stream(ctx);
-  SEDEF_TRY(ensure_smem_attr((const void*)k_refine_batch, sizeof(BatchWarp) * kBWarps));
+  // counters for a third more W_Q hashes than a window holds on average
+  // (2 / (w + 1) of its starts): the sizes between runs differ by a few
+  int scap = ((int)(1.35 * 2.0 * (D.span + 1) / (D.w + 1)) + 31) / 32 * 32;
+  scap = scap < 64 ? 64 : (scap > kBQC ? kBQC : scap);
+  const size_t lean_sm = refine_warp_bytes(scap) * kBWarps;
+  SEDEF_TRY(ensure_smem_attr((const void*)k_refine_batch, lean_sm));
   SEDEF_TRY(ensure_smem_attr((const void*)k_refine<kMaxWindowRecs, 1024, false>,
                              sizeof(RefineWarpT<kMaxWindowRecs, 1024>) * kRWarpsBig));
   // order runs by (i, o); the sweep emits each window's runs in j order
@@ -2433,14 +2438,20 @@ int order_and_refine(sedef_ctx* ctx, const FArgs& a, const Derived& D, int nqseq
   ra.next = counters + 6;
   SEDEF_CUDA(cudaMemsetAsync(counters + 6, 0, 16, st));
   using Big = RefineWarpT<kMaxWindowRecs, 1024>;
-  const size_t lean_sm = sizeof(BatchWarp) * kBWarps, big_sm = sizeof(Big) * kRWarpsBig;
+  const size_t big_sm = sizeof(Big) * kRWarpsBig;
   int rper = 0;
   SEDEF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&rper, k_refine_batch, 32 * kBWarps,
                                                            lean_sm));
   if (rper < 1) rper = 1;
-  int64_t rgrid = (total + kBWarps * 32 - 1) / (kBWarps * 32);
+  int64_t rgrid = (total + kBWarps - 1) / kBWarps;
   if (rgrid > (int64_t)ctx_sm_count(ctx) * rper) rgrid = (int64_t)ctx_sm_count(ctx) * rper;
   if (rgrid < 1) rgrid = 1;
+  // a warp's events: room for the runs it takes at a time
+  const int64_t per_warp = (total + rgrid * kBWarps - 1) / (rgrid * kBWarps);
+  ra.scap = scap;
+  ra.ev_words = per_warp * (kBRC + 8) < kEvWords ? (int)per_warp * (kBRC + 8) : kEvWords;
+  ra.events = (uint32_t*)ctx_alloc(ctx, (size_t)(rgrid * kBWarps) * (ra.ev_words + kEvPad) * 4);
+  if (!ra.events) return SEDEF_ERR_OOM;
   SEDEF_KERNEL(ctx, "k_refine",
                k_refine_batch<<<(int)rgrid, 32 * kBWarps, lean_sm, st>>>(ra));
   SEDEF_KERNEL(ctx, "k_refine_big",
