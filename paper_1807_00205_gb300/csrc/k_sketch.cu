@@ -4,19 +4,22 @@
 // thread and one mask/N word per lane pair (warp shuffle), so every global
 // access is coalesced.  HBM-bound: 1 B read + 0.5 B written per base.
 //
-// sketch: one CTA per tile of 2048 consecutive windows.  The packed words,
-// mask and N bits of the tile (plus halo) are staged in shared memory; every
-// thread computes the canonical k-mer hashes of 8-9 positions from two 32-bit
-// words (forward code by bit reversal, reverse complement by complementing),
-// then the rightmost minimum of its 9 windows with a van Herk / Gil-Werman
-// split (suffix minima, a shared middle, prefix minima), and keeps a window's
-// argmin when it differs from the previous window's (winnowing argmins are
+// sketch: a warp takes a stretch of 512 positions, 16 consecutive ones per
+// lane, all in registers.  A lane reads two packed words and two 16-bit
+// pieces of the mask and N bits; forward codes and reverse complements are
+// funnel shifts of the words and of their reversal, eligibility of its 16
+// k-mers a few shifts of the bit-vectors.  Window minima come from doubling
+// (minima over 1, 2, 4, ... positions, then one combination of two
+// overlapping ones), reading the lanes above by shuffles; a window's argmin
+// is kept when it differs from the previous window's (winnowing argmins are
 // non-decreasing, so this emits each selected position once, in order).  The
-// window keys are (hash, reversed slot): 32 bits when the hash has at most 24
-// bits and a thread's windows span at most 128 slots, else 64.  The eager
-// pass writes its records in the same pass, finding each tile's offset by a
-// decoupled look-back over the tiles taken before it; the planned (graph)
-// pass and the allocation-free call count, scan and write instead.
+// window keys are (hash, reversed offset from the lane's first position), so
+// that equal hashes go to the rightmost: 32 bits when the hash has at most
+// 24 bits and a window at most 112 positions, else 64.  Eight warps share a
+// CTA tile; the eager pass writes its records in the same pass, finding each
+// tile's offset by a decoupled look-back over the tiles taken before it; the
+// planned (graph) pass and the allocation-free call count, scan and write
+// instead.
 #include <cstring>
 
 #include "common.cuh"
@@ -34,6 +37,19 @@ __device__ __forceinline__ void classify(uint32_t b, uint32_t& code, uint32_t& m
   isn = acgt ? 0u : 1u;
 }
 
+// Four bases at once: a code per byte, and which bytes are not ACGTacgt (a
+// non-zero byte in the result).  The code picks the letter it stands for,
+// and a byte is a base when it is that letter.
+__device__ __forceinline__ uint32_t codes4(uint32_t v, uint32_t& code) {
+  const uint32_t u = v | 0x20202020u;
+  code = ((u >> 1) ^ (u >> 2)) & 0x03030303u;  // a=0 c=1 g=2 t=3
+  const uint32_t pick = __byte_perm(code | (code >> 4), 0, 0x4420);  // a nibble per byte
+  return __byte_perm(0x74676361u, 0, pick) ^ u;
+}
+
+// A thread classifies its 16 bytes four at a time (one at a time, 17
+// instructions a base, was bound by their issue: 3.1 Gbp in 2.78 ms; now 1.00
+// ms, 4.65 TB/s read and written); 16 bytes with a letter other than ACGT among them go one at a time.
 template <bool kAligned>
 __global__ void __launch_bounds__(256) k_pack(const uint8_t* __restrict__ seq, int64_t n,
                                               uint32_t* __restrict__ packed,
@@ -50,13 +66,26 @@ __global__ void __launch_bounds__(256) k_pack(const uint8_t* __restrict__ seq, i
       if (kAligned && p0 + 16 <= n) {
         const uint4 q = __ldg(reinterpret_cast<const uint4*>(seq + p0));
         v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
+        uint32_t other = 0;
 #pragma unroll
-        for (int x = 0; x < 16; ++x) {
-          uint32_t code, ms, isn;
-          classify((v[x >> 2] >> (8 * (x & 3))) & 0xFFu, code, ms, isn);
-          word |= code << (2 * x);
-          m16 |= ms << x;
-          n16 |= isn << x;
+        for (int x = 0; x < 4; ++x) {
+          uint32_t code;
+          other |= codes4(v[x], code);
+          // the multiplications bring the bytes' 2-bit codes and case bits
+          // together in the top byte (no two partial products meet)
+          word |= ((code * 0x01041040u) >> 24) << (8 * x);
+          m16 |= ((((v[x] >> 5) & 0x01010101u) * 0x01020408u) >> 24) << (4 * x);
+        }
+        if (other) {
+          word = m16 = 0;
+#pragma unroll
+          for (int x = 0; x < 16; ++x) {
+            uint32_t code, ms, isn;
+            classify((v[x >> 2] >> (8 * (x & 3))) & 0xFFu, code, ms, isn);
+            word |= code << (2 * x);
+            m16 |= ms << x;
+            n16 |= isn << x;
+          }
         }
       } else {
         for (int x = 0; x < 16; ++x) {
@@ -82,21 +111,24 @@ __global__ void __launch_bounds__(256) k_pack(const uint8_t* __restrict__ seq, i
 }
 
 constexpr int kSkThreads = 256;
-constexpr int kSkWPT = 8;                          // windows per thread
-constexpr int kSkTile = kSkThreads * kSkWPT;       // windows per CTA
+constexpr int kSkWarps = kSkThreads / 32;
+constexpr int kSkP = 16;                           // positions per lane
 constexpr int kSkMaxW = 256;
-constexpr int kSkHashes = kSkTile + kSkMaxW;       // hash slots (tile + halo)
-// Hash slot x lives at x + x/8: a thread's windows start kSkWPT = 8 slots
-// after its neighbour's, and the padding turns that stride into 9 words, so
-// the lanes of a warp read distinct banks.
-constexpr int kSkHashesP = kSkHashes + kSkHashes / 8 + 1;
-__device__ __forceinline__ int hslot(int x) { return x + (x >> 3); }
-constexpr int kSkWords16 = (kSkHashes + 16) / 16 + 4;
-constexpr int kSkWords32 = (kSkHashes + 16) / 32 + 4;
+// Lanes of a warp that own windows: not the first (it gives the window
+// before lane 1's first) and not the last ceil((w - 1) / 16), whose windows
+// would leave the warp's positions.
+__host__ __device__ constexpr int sk_lanes(int w) { return 31 - (w - 1 + kSkP - 1) / kSkP; }
+__host__ __device__ constexpr int sk_warp_windows(int w) { return sk_lanes(w) * kSkP; }
+// Stretches of one warp in a CTA tile.  Long inputs take four, for a quarter
+// of the look-backs; short ones one, for more CTAs.
+constexpr int kSkRep = 4;
+constexpr int64_t kSkRepBases = int64_t(32) << 20;
+__host__ __device__ constexpr int64_t sk_tile_windows(int w, int rep) {
+  return (int64_t)sk_warp_windows(w) * kSkWarps * rep;
+}
+constexpr int sk_rep(int64_t n) { return n >= kSkRepBases ? kSkRep : 1; }
+constexpr int kSkStage = 31 * kSkP * kSkRep;       // k-mers a warp can select
 
-// Canonical hash of the k-mer whose first base is bit-offset `sh` into the
-// 64-bit pair (lo, hi) of packed words.  Returns kInfHash for an ineligible
-// k-mer (N inside, too few unmasked bases, palindrome).
 __device__ __forceinline__ uint32_t bijective_hash(uint32_t x, int k, uint32_t M) {
   // A permutation of [0, 4^k): xor-shift-right and odd multipliers, all
   // modulo 2^(2k) (2k <= 30 bits, so 32-bit arithmetic is exact mod 2^(2k)).
@@ -118,6 +150,7 @@ struct SketchArgs {
   int64_t N;
   int k, w, min_unmasked;
   uint32_t kmask;
+  int rep;         // stretches of a warp per CTA tile
   int64_t ntiles;
 };
 
@@ -138,305 +171,338 @@ constexpr unsigned long long kLbAggregate = 1ull << 62, kLbPrefix = 2ull << 62;
 constexpr unsigned long long kLbValue = (1ull << 62) - 1;
 constexpr unsigned int kLbSpins = 1u << 20;  // polls of one predecessor before giving up
 
-__device__ __forceinline__ unsigned long long ld_acquire_gpu(const unsigned long long* p) {
+// A status word holds its flag and its value, and nothing else is read after
+// it, so its accesses need no ordering (an acquire load throws away the SM's
+// L1, a release store waits for the CTA's earlier writes).
+__device__ __forceinline__ unsigned long long ld_status(const unsigned long long* p) {
   unsigned long long v;
-  asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
   return v;
 }
 
-__device__ __forceinline__ void st_release_gpu(unsigned long long* p, unsigned long long v) {
-  asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+__device__ __forceinline__ void st_status(unsigned long long* p, unsigned long long v) {
+  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
 
 // Records before tile `tile`; warp 0 of the CTA calls it once per tile.  The
-// warp reads the status of the 32 tiles below its window at once: the
-// nearest one that has published its inclusive prefix ends the walk, and
-// the counts of the tiles above it are summed by the warp (a look-back one
-// tile at a time falls behind the tiles that are in flight).
+// warp reads the status of the 256 tiles below its window at once (eight
+// independent loads per lane: as many tiles are in flight, so a narrower
+// window walks several round trips to the nearest published prefix): the
+// nearest tile that has published its inclusive prefix ends the walk, and
+// the counts of the tiles above it are summed by the warp.
 __device__ long long look_back(const LookBack& lb, int64_t tile, int64_t ntiles,
                                unsigned long long count) {
+  constexpr int kWide = 8;
   const int lane = threadIdx.x & 31;
   long long before = 0;
   if (tile > 0) {
-    if (lane == 0) st_release_gpu(lb.status + tile, kLbAggregate | count);
+    if (lane == 0) st_status(lb.status + tile, kLbAggregate | count);
     int64_t j = tile - 1;  // the walk's top tile
     unsigned int spins = 0;
-    while (true) {
-      const int64_t at = j - lane;
-      // below tile 0 reads as a published prefix of zero
-      const unsigned long long v = at >= 0 ? ld_acquire_gpu(lb.status + at) : kLbPrefix;
-      const unsigned long long flag = v & ~kLbValue;
-      const unsigned prefix = __ballot_sync(0xffffffffu, flag == kLbPrefix);
-      const int p = prefix ? __ffs(prefix) - 1 : 31;  // lanes 0..p take part
-      const unsigned need = p == 31 ? 0xffffffffu : ((1u << (p + 1)) - 1u);
-      const unsigned waiting = __ballot_sync(0xffffffffu, flag == 0) & need;
-      if (waiting) {
-        if (++spins > kLbSpins) {
-          if (lane == 0) atomicExch(lb.err, 1);
+    bool done = false;
+    while (!done) {
+      unsigned long long v[kWide];
+#pragma unroll
+      for (int x = 0; x < kWide; ++x) {
+        const int64_t at = j - x * 32 - lane;
+        // below tile 0 reads as a published prefix of zero
+        v[x] = at >= 0 ? ld_status(lb.status + at) : kLbPrefix;
+      }
+#pragma unroll
+      for (int x = 0; x < kWide; ++x) {
+        const unsigned long long flag = v[x] & ~kLbValue;
+        const unsigned prefix = __ballot_sync(0xffffffffu, flag == kLbPrefix);
+        const int p = prefix ? __ffs(prefix) - 1 : 31;  // lanes 0..p take part
+        const unsigned need = p == 31 ? 0xffffffffu : ((1u << (p + 1)) - 1u);
+        if (__ballot_sync(0xffffffffu, flag == 0) & need) {
+          if (++spins > kLbSpins) {
+            if (lane == 0) atomicExch(lb.err, 1);
+            done = true;
+          }
+          break;  // read again from this window's top
+        }
+        spins = 0;
+        before += lane <= p ? (long long)(v[x] & kLbValue) : 0;
+        if (prefix) {
+          done = true;
           break;
         }
-        __nanosleep(64);
-        continue;
+        j -= 32;
       }
-      spins = 0;
-      long long part = lane <= p ? (long long)(v & kLbValue) : 0;
-#pragma unroll
-      for (int d = 16; d > 0; d >>= 1) part += __shfl_xor_sync(0xffffffffu, part, d);
-      before += part;
-      if (prefix) break;
-      j -= 32;
     }
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) before += __shfl_xor_sync(0xffffffffu, before, d);
   }
   if (lane == 0) {
-    st_release_gpu(lb.status + tile, kLbPrefix | ((unsigned long long)before + count));
+    st_status(lb.status + tile, kLbPrefix | ((unsigned long long)before + count));
     if (tile == ntiles - 1) *lb.total = (unsigned long long)before + count;
   }
   return before;
 }
 
-// Exclusive sum over the CTA.  Unlike block_exclusive_sum it ends without a
-// barrier: the next tile reaches s_tmp only after at least two more.
-__device__ __forceinline__ int tile_exclusive_sum(int v, int* tmp, int* total) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int inc = warp_inclusive_sum(v);
-  if (lane == 31) tmp[warp] = inc;
-  __syncthreads();
-  if (warp == 0) {
-    const int x = lane < kSkThreads / 32 ? tmp[lane] : 0;
-    const int xi = warp_inclusive_sum(x);
-    if (lane < kSkThreads / 32) tmp[lane] = xi - x;
-    if (lane == 31) tmp[32] = xi;
+// Window keys: a hash over the reversed offset of its position from the
+// lane's first one (so that the rightmost of equal hashes is the least); the
+// ineligible key lies above every hash.  A key read from the lane d lanes up
+// is rebased by subtracting 16 d.
+template <typename K>
+struct Key;
+template <>
+struct Key<uint32_t> {  // 24-bit hashes, offsets up to 127
+  static __device__ __forceinline__ uint32_t make(uint32_t h, int off) { return h * 128u + (127u - off); }
+  static __device__ __forceinline__ uint32_t none(int off) { return 0x80000000u + (127u - off); }
+  static __device__ __forceinline__ bool is_none(uint32_t v) { return (int)v < 0; }
+  static __device__ __forceinline__ int off(uint32_t v) { return 127 - (int)(v & 127u); }
+};
+template <>
+struct Key<uint64_t> {
+  static __device__ __forceinline__ uint64_t make(uint32_t h, int off) {
+    return ((uint64_t)h << 32) | (uint32_t)(0xFFFF - off);
   }
-  __syncthreads();
-  *total = tmp[32];
-  return tmp[warp] + inc - v;
+  static __device__ __forceinline__ uint64_t none(int off) { return make(kInfHash, off); }
+  static __device__ __forceinline__ bool is_none(uint64_t v) { return (uint32_t)(v >> 32) == kInfHash; }
+  static __device__ __forceinline__ int off(uint64_t v) { return 0xFFFF - (int)(uint32_t)v; }
+};
+
+// v[x] = the value D positions on (D < 16; the next lane's, rebased, past the end).
+template <int D, typename K>
+__device__ __forceinline__ void shift_positions(K (&v)[kSkP]) {
+  K next[D];
+#pragma unroll
+  for (int x = 0; x < D; ++x) next[x] = __shfl_down_sync(0xffffffffu, v[x], 1) - (K)kSkP;
+#pragma unroll
+  for (int x = 0; x < kSkP; ++x) v[x] = x + D < kSkP ? v[x + D] : next[x + D - kSkP];
 }
 
-// Window minima for the windows starting at local slot B + t, t in
-// [0, kSkWPT]: key[t] = min over slots [B + t, B + t + w) of kx(slot).
-template <typename K, typename KX>
-__device__ __forceinline__ void window_minima(int w, int B, KX kx, K (&key)[kSkWPT + 1]) {
-  const K inf = ~K(0);
-  if (w <= kSkWPT) {
+// v[x] = min(v[x], the value D positions on).
+template <int D, typename K>
+__device__ __forceinline__ void min_positions(K (&v)[kSkP]) {
+  K next[D];
 #pragma unroll
-    for (int t = 0; t <= kSkWPT; ++t) {
-      K m = inf;
-      for (int x = B + t; x < B + t + w; ++x) m = min(m, kx(x));
-      key[t] = m;
+  for (int x = 0; x < D; ++x) next[x] = __shfl_down_sync(0xffffffffu, v[x], 1) - (K)kSkP;
+#pragma unroll
+  for (int x = 0; x < kSkP; ++x) v[x] = min(v[x], x + D < kSkP ? v[x + D] : next[x + D - kSkP]);
+}
+
+// key[x]: minimum over the w positions from x on.
+template <typename K>
+__device__ __forceinline__ void window_minima(int w, K (&key)[kSkP]) {
+  int len = 1;
+  if (w >= 2) min_positions<1>(key), len = 2;
+  if (w >= 4) min_positions<2>(key), len = 4;
+  if (w >= 8) min_positions<4>(key), len = 8;
+  if (w >= 16) min_positions<8>(key), len = 16;
+  while (2 * len <= w) {  // whole lanes
+#pragma unroll
+    for (int x = 0; x < kSkP; ++x)
+      key[x] = min(key[x], (K)(__shfl_down_sync(0xffffffffu, key[x], len / kSkP) - (K)len));
+    len *= 2;
+  }
+  const int r = w - len;  // the rest: two overlapping minima
+  if (r > 0) {
+    K v[kSkP];
+#pragma unroll
+    for (int x = 0; x < kSkP; ++x) v[x] = key[x];
+    if (r & 1) shift_positions<1>(v);
+    if (r & 2) shift_positions<2>(v);
+    if (r & 4) shift_positions<4>(v);
+    if (r & 8) shift_positions<8>(v);
+    const int up = r / kSkP;
+    if (up > 0) {
+#pragma unroll
+      for (int x = 0; x < kSkP; ++x) v[x] = __shfl_down_sync(0xffffffffu, v[x], up) - (K)(up * kSkP);
     }
-  } else {
-    // suffix minima over [B+t, B+7], middle over [B+8, B+w-1], prefix
-    // minima over [B+w, B+w+t-1]
-    K suf[kSkWPT + 1];
-    suf[kSkWPT] = inf;
 #pragma unroll
-    for (int t = kSkWPT - 1; t >= 0; --t) suf[t] = min(suf[t + 1], kx(B + t));
-    K mid = inf;
-    for (int x = B + kSkWPT; x < B + w; ++x) mid = min(mid, kx(x));
-    K pre = inf;
-#pragma unroll
-    for (int t = 0; t <= kSkWPT; ++t) {
-      if (t > 0) pre = min(pre, kx(B + w + t - 1));
-      key[t] = min(min(suf[t], mid), pre);
-    }
+    for (int x = 0; x < kSkP; ++x) key[x] = min(key[x], v[x]);
   }
 }
 
-// kMode 0: count the records of each tile; 1: write them at the tile
-// offsets given; 2: one pass, offsets by look-back.  Four CTAs per SM (64
-// registers a thread): while one CTA's warp 0 walks back, the others compute.
-// kNarrow (2k <= 24 and w + kSkWPT <= 128): a window key is 32 bits, the
-// hash (ineligible as 2^24) over 7 bits of the slot's reversed offset from
-// the thread's first slot, so that equal hashes still go to the rightmost.
-template <int kMode, bool kNarrow>
-__global__ void __launch_bounds__(kSkThreads, 4) k_sketch(SketchArgs a, uint32_t* __restrict__ tile_count,
-                                                       const uint32_t* __restrict__ tile_offset,
-                                                       uint64_t* __restrict__ out, int64_t cap,
-                                                       LookBack lb) {
-  __shared__ uint32_t s_pk[kSkWords16];
-  __shared__ uint32_t s_mk[kSkWords32];
-  __shared__ uint32_t s_nb[kSkWords32];
-  __shared__ uint32_t s_h[kSkHashesP];
-  __shared__ uint8_t s_sg[kSkHashesP];
-  __shared__ int s_tmp[33];
+// The 2-bit groups of a word in reverse order.
+__device__ __forceinline__ uint32_t reverse_pairs(uint32_t v) {
+  v = __brev(v);
+  return ((v >> 1) & 0x55555555u) | ((v & 0x55555555u) << 1);
+}
+
+// kMode 0: count the records of each CTA tile; 1: write them at the tile
+// offsets given; 2: one pass, offsets by look-back.
+//
+// Bound by the integer pipes: little over one warp instruction per base at
+// k = 12, w = 16 (the form that hashed into shared memory and took van Herk
+// minima from it ran 8.1).  A lane holds as many positions as its registers
+// allow (16 keys and their shifted copies in 64 registers, four CTAs per SM);
+// the lanes without windows, two of 32 at w = 16, are the waste.  3.1 Gbp:
+// 33.7 -> 9.8 ms, 240 Mbp: 2.6 -> 0.78 ms.  Of that the look-back was most:
+// with a 32-tile window, one stretch per warp and the next ticket taken
+// before the walk the same kernel took 35.7 ms at 3.1 Gbp.
+template <int kMode, typename K>
+__global__ void __launch_bounds__(kSkThreads, sizeof(K) == 4 ? 4 : 2) k_sketch(SketchArgs a, uint32_t* __restrict__ tile_count,
+                                                          const uint32_t* __restrict__ tile_offset,
+                                                          uint64_t* __restrict__ out, int64_t cap,
+                                                          LookBack lb) {
+  // selected positions from the warp's first one, in order
+  __shared__ uint16_t s_stage[kMode == 0 ? 1 : kSkWarps][kMode == 0 ? 1 : kSkStage];
+  __shared__ int s_cnt[kSkWarps], s_off[kSkWarps];
   __shared__ long long s_tile, s_base;
-  __shared__ long long s_seg_lo, s_seg_hi;  // the sequence holding the tile's first position
-
   const int k = a.k, w = a.w;
-  const int tid = threadIdx.x;
-  for (int64_t it = blockIdx.x;; it += gridDim.x) {
-    int64_t tile = it;
-    if (kMode == 2) {
-      // every thread read the last tile's s_tile before the barriers of
-      // that tile's body, so tid 0 may overwrite it now
-      if (tid == 0) s_tile = (long long)atomicAdd(lb.ticket, 1u);
-      __syncthreads();
-      tile = s_tile;
+  const int lane = lane_id(), warp = threadIdx.x >> 5;
+  const int wlanes = sk_lanes(w), wwin = sk_warp_windows(w);
+  const uint32_t kmask = a.kmask;
+  const int64_t nw16 = (a.N + 15) >> 4;
+  const uint16_t* mask16 = reinterpret_cast<const uint16_t*>(a.mask);
+  const uint16_t* nbits16 = reinterpret_cast<const uint16_t*>(a.nbits);
+  int64_t seg_lo = 0, seg_hi = -1;  // the sequence that held the last stretch's first position
+  int64_t tile = blockIdx.x;
+  if (kMode == 2) {
+    if (threadIdx.x == 0) s_tile = (long long)atomicAdd(lb.ticket, 1u);
+    __syncthreads();
+    tile = s_tile;
+  }
+  while (tile < a.ntiles) {
+    const int64_t base0 = (tile * kSkWarps + warp) * (int64_t)(wwin * a.rep) - kSkP;
+    int n = 0;  // k-mers selected
+    for (int rep = 0; rep < a.rep; ++rep) {
+      const int64_t base = base0 + rep * wwin, first = base + kSkP;  // first: the first window
+      int cnt = 0;
+      uint32_t flags = 0;
+      K key[kSkP];
+      if (first < a.N) {
+        if (first < seg_lo || first >= seg_hi) {
+          const int s = seq_of(a.off, a.nseq, first);
+          seg_lo = a.off[s];
+          seg_hi = a.off[s + 1];
+        }
+        const int64_t p0 = base + lane * kSkP;
+        const int64_t wi = p0 >> 4;
+        const bool in0 = wi >= 0 && wi < nw16, in1 = wi + 1 < nw16;
+        const uint32_t w0 = in0 ? __ldg(a.packed + wi) : 0u;
+        const uint32_t w1 = in1 ? __ldg(a.packed + wi + 1) : 0u;
+        const uint32_t mk = (in0 ? (uint32_t)__ldg(mask16 + wi) : 0xFFFFu) |
+                            ((in1 ? (uint32_t)__ldg(mask16 + wi + 1) : 0xFFFFu) << 16);
+        const uint32_t nb = (in0 ? (uint32_t)__ldg(nbits16 + wi) : 0xFFFFu) |
+                            ((in1 ? (uint32_t)__ldg(nbits16 + wi + 1) : 0xFFFFu) << 16);
+        // bit x: the k-mer at p0 + x holds an N, or (min_unmasked = 1) only
+        // masked bases; the shifts reach bit 15 + 14 at most
+        uint32_t bad = nb, all = mk;
+        {
+          int len = 1;
+          for (; 2 * len <= k; len *= 2) {
+            bad |= bad >> len;
+            all &= all >> len;
+          }
+          bad |= bad >> (k - len);
+          all &= all >> (k - len);
+        }
+        if (a.min_unmasked == 1) {
+          bad |= all;
+        } else if (a.min_unmasked > 1) {
+          const uint32_t kb = (1u << k) - 1u;
+  #pragma unroll
+          for (int x = 0; x < kSkP; ++x)
+            if (k - __popc((mk >> x) & kb) < a.min_unmasked) bad |= 1u << x;
+        }
+        // windows that lie in one sequence; only lanes near a sequence's end
+        // look at their positions one by one
+        uint32_t ok = 0xFFFFu;
+        if (p0 < seg_lo || p0 + kSkP - 1 + w + k - 1 > seg_hi) {
+          ok = 0;
+          int64_t lo = seg_lo, hi = seg_hi;
+          for (int x = 0; x < kSkP; ++x) {
+            const int64_t p = p0 + x;
+            if (p < 0 || p >= a.N) {
+              bad |= 1u << x;
+              continue;
+            }
+            if (p < lo || p >= hi) {
+              const int s = seq_of(a.off, a.nseq, p);
+              lo = a.off[s];
+              hi = a.off[s + 1];
+            }
+            if (p + k > hi) bad |= 1u << x;
+            if (p + w + k - 1 <= hi) ok |= 1u << x;
+          }
+        }
+        const uint32_t r0 = reverse_pairs(w0), r1 = reverse_pairs(w1);
+  #pragma unroll
+        for (int x = 0; x < kSkP; ++x) {
+          // forward code: first base most significant; the reverse complement's
+          // is the complement with the first base least significant
+          const uint32_t f = __funnelshift_l(r1, r0, 2 * x) >> (32 - 2 * k);
+          const uint32_t rc = ~__funnelshift_r(w0, w1, 2 * x) & kmask;
+          const uint32_t h = bijective_hash(f < rc ? f : rc, k, kmask);
+          key[x] = ((bad >> x) & 1u) || f == rc ? Key<K>::none(x) : Key<K>::make(h, x);
+        }
+        window_minima(w, key);
+        // selected: an eligible minimum that is not the previous window's
+        const K before = __shfl_up_sync(0xffffffffu, key[kSkP - 1], 1) + (K)kSkP;
+        uint32_t valid = 0;
+  #pragma unroll
+        for (int x = 0; x < kSkP; ++x)
+          if (!Key<K>::is_none(key[x])) valid |= 1u << x;
+        valid &= ok;
+        uint32_t same = 0;
+  #pragma unroll
+        for (int x = 0; x < kSkP; ++x)
+          if (key[x] == (x ? key[x - 1] : before)) same |= 1u << x;
+        const uint32_t vb = __shfl_up_sync(0xffffffffu, valid >> (kSkP - 1), 1);
+        flags = valid & ~(same & ((valid << 1) | (vb & 1u)));
+        if (lane == 0 || lane > wlanes) flags = 0;
+        cnt = __popc(flags);
+      }
+      const int inc = warp_inclusive_sum(cnt);
+      if (kMode != 0) {
+        int at = n + inc - cnt;
+  #pragma unroll
+        for (int x = 0; x < kSkP; ++x) {
+          if ((flags >> x) & 1u) {
+            s_stage[warp][at] = (uint16_t)(rep * wwin + lane * kSkP + Key<K>::off(key[x]));
+            ++at;
+          }
+        }
+      }
+      n += __shfl_sync(0xffffffffu, inc, 31);
     }
-    if (tile >= a.ntiles) break;
-    const int64_t Q0 = tile * kSkTile;
-    const int64_t HB = Q0 - 1;                    // first hash position of the tile
-    const int nh = kSkTile + w;                   // hash positions [HB, HB + nh)
-    const int64_t b_lo = HB < 0 ? 0 : HB;
-    const int64_t wb16 = b_lo >> 4, wb32 = b_lo >> 5;
-    const int64_t nw16 = (a.N + 15) >> 4, nw32 = (a.N + 31) >> 5;
-    const int64_t last = HB + nh + k;             // one past the last base read
-    const int n16 = (int)(((last + 15) >> 4) - wb16 + 1);
-    const int n32 = (int)(((last + 31) >> 5) - wb32 + 1);
-    // no barrier here: the staging buffers were last read in the previous
-    // tile's hash stage, which a barrier ends
-    if (tid == 0) {
-      const int s = seq_of(a.off, a.nseq, b_lo);
-      s_seg_lo = a.off[s];
-      s_seg_hi = a.off[s + 1];
-    }
-    for (int x = tid; x < n16; x += kSkThreads) {
-      const int64_t g = wb16 + x;
-      s_pk[x] = g < nw16 ? __ldg(a.packed + g) : 0u;
-    }
-    for (int x = tid; x < n32; x += kSkThreads) {
-      const int64_t g = wb32 + x;
-      s_mk[x] = g < nw32 ? __ldg(a.mask + g) : 0xFFFFFFFFu;
-      s_nb[x] = g < nw32 ? __ldg(a.nbits + g) : 0xFFFFFFFFu;
+    if (lane == 0) s_cnt[warp] = n;
+    __syncthreads();
+    if (warp == 0) {
+      const int c = lane < kSkWarps ? s_cnt[lane] : 0;
+      const int ci = warp_inclusive_sum(c);
+      const int total = __shfl_sync(0xffffffffu, ci, 31);
+      if (lane < kSkWarps) s_off[lane] = ci - c;
+      if (kMode == 0) {
+        if (lane == 0) tile_count[tile] = (uint32_t)total;
+      } else if (kMode == 1) {
+        if (lane == 0) s_base = (long long)tile_offset[tile];
+      } else {
+        const long long before = look_back(lb, tile, a.ntiles, (unsigned long long)total);
+        // the next ticket only now: an earlier one would keep the tiles
+        // above it waiting through this look-back
+        if (lane == 0) {
+          s_base = before;
+          s_tile = (long long)atomicAdd(lb.ticket, 1u);
+        }
+      }
     }
     __syncthreads();
-
-    // ---- hashes of positions HB + x, x in [0, nh)
-    {
-      const int per = (nh + kSkThreads - 1) / kSkThreads;
-      const int x0 = tid * per;
-      int64_t segend = s_seg_hi, segstart = s_seg_lo;
-      // every k-mer of this thread inside the tile's first sequence: no
-      // per-position bounds checks
-      const int xe = min(x0 + per, nh);
-      const bool inside = HB + x0 >= segstart && HB + xe - 1 + k <= segend;
-      for (int r = 0; r < per; ++r) {
-        const int x = x0 + r;
-        if (x >= nh) break;
-        const int64_t p = HB + x;
-        uint32_t h = kInfHash, sg = 0;
-        if (inside || (p >= 0 && p + k <= a.N)) {
-          if (!inside && (p >= segend || p < segstart)) {
-            const int s = seq_of(a.off, a.nseq, p);
-            segstart = a.off[s];
-            segend = a.off[s + 1];
-          }
-          if (inside || p + k <= segend) {
-            const int64_t lp = p - (wb16 << 4);
-            const int wi = (int)(lp >> 4), sh = (int)(lp & 15) * 2;
-            const uint64_t pair = (uint64_t)s_pk[wi] | ((uint64_t)s_pk[wi + 1] << 32);
-            const uint32_t g = (uint32_t)(pair >> sh) & a.kmask;   // first base in the low bits
-            const int64_t lb = p - (wb32 << 5);
-            const int bi = (int)(lb >> 5), bs = (int)(lb & 31);
-            const uint64_t kb = (1ull << k) - 1;
-            const uint64_t nb = (((uint64_t)s_nb[bi] | ((uint64_t)s_nb[bi + 1] << 32)) >> bs) & kb;
-            const uint64_t mk = (((uint64_t)s_mk[bi] | ((uint64_t)s_mk[bi + 1] << 32)) >> bs) & kb;
-            // forward code: reverse the order of the k 2-bit groups
-            uint32_t f = __brev(g);
-            f = ((f >> 1) & 0x55555555u) | ((f & 0x55555555u) << 1);
-            f >>= (32 - 2 * k);
-            const uint32_t rc = g ^ a.kmask;  // complement each base, order reversed
-            const int unmasked = k - __popcll(mk);
-            if (nb == 0 && unmasked >= a.min_unmasked && f != rc) {
-              h = bijective_hash(f < rc ? f : rc, k, a.kmask);
-              sg = rc < f ? 1u : 0u;
-            }
-          }
-        }
-        s_h[hslot(x)] = h;
-        s_sg[hslot(x)] = (uint8_t)sg;
+    if (kMode != 0) {
+      const int64_t o = s_base + s_off[warp];
+      for (int x = lane; x < n; x += 32) {
+        // the selected k-mer's hash and strand, from its codes again
+        const int64_t p = base0 + s_stage[warp][x];
+        const int64_t wi = p >> 4;
+        const uint32_t w0 = __ldg(a.packed + wi), w1 = wi + 1 < nw16 ? __ldg(a.packed + wi + 1) : 0u;
+        const uint32_t g = __funnelshift_r(w0, w1, 2 * (int)(p & 15)) & kmask;
+        const uint32_t f = reverse_pairs(g) >> (32 - 2 * k);
+        const uint32_t rc = g ^ kmask;
+        const uint32_t h = bijective_hash(f < rc ? f : rc, k, kmask);
+        if (o + x < cap) out[o + x] = ((uint64_t)h << 33) | ((uint64_t)p << 1) | (uint64_t)(rc < f ? 1u : 0u);
       }
+      __syncwarp();
     }
-    __syncthreads();
-
-    // ---- windows q = HB + B + t, t in [0, 9): local hash range [B + t, B + t + w)
-    const int B = tid * kSkWPT;
-    uint32_t xs[kSkWPT + 1];  // slot of each window's minimizer
-    uint32_t inf = 0;         // bit t: window t's minimum is ineligible
-    if (kNarrow) {
-      uint32_t key[kSkWPT + 1];
-      auto kx = [&](int x) -> uint32_t {
-        return (min(s_h[hslot(x)], 1u << 24) << 7) | (uint32_t)(127 - (x - B));
-      };
-      window_minima(w, B, kx, key);
-#pragma unroll
-      for (int t = 0; t <= kSkWPT; ++t) {
-        xs[t] = (uint32_t)(B + 127) - (key[t] & 127u);
-        if ((key[t] >> 7) >= (1u << 24)) inf |= 1u << t;
-      }
-    } else {
-      uint64_t key[kSkWPT + 1];
-      auto kx = [&](int x) -> uint64_t {
-        return ((uint64_t)s_h[hslot(x)] << 32) | (uint64_t)(0xFFFFFFFFu - (uint32_t)x);
-      };
-      window_minima(w, B, kx, key);
-#pragma unroll
-      for (int t = 0; t <= kSkWPT; ++t) {
-        xs[t] = 0xFFFFFFFFu - (uint32_t)key[t];
-        if ((uint32_t)(key[t] >> 32) == kInfHash) inf |= 1u << t;
-      }
-    }
-    // validity and selection flags for windows t = 1..8
-    uint32_t flags = 0;
-    {
-      int64_t segend = s_seg_hi, segstart = s_seg_lo;
-      // all nine windows inside the tile's first sequence
-      const bool inside = HB + B >= segstart && HB + B + kSkWPT + w + k - 1 <= segend;
-      bool prev_ok = false;
-      uint32_t prev_arg = 0;
-#pragma unroll
-      for (int t = 0; t <= kSkWPT; ++t) {
-        const int64_t q = HB + B + t;
-        bool ok;
-        if (inside) {
-          ok = !((inf >> t) & 1u);
-        } else {
-          ok = false;
-          if (q >= 0 && q + w + k - 1 <= a.N) {
-            if (q >= segend || q < segstart) {
-              const int s = seq_of(a.off, a.nseq, q);
-              segstart = a.off[s];
-              segend = a.off[s + 1];
-            }
-            ok = (q + w + k - 1 <= segend) && !((inf >> t) & 1u);
-          }
-        }
-        const uint32_t arg = xs[t];
-        if (t > 0 && ok && !(prev_ok && prev_arg == arg)) flags |= 1u << t;
-        prev_ok = ok;
-        prev_arg = arg;
-      }
-    }
-    const int cnt = __popc(flags);
-    int total;
-    const int excl = tile_exclusive_sum(cnt, s_tmp, &total);
-    if (kMode == 0) {
-      if (tid == 0) tile_count[tile] = (uint32_t)total;
-    } else {
-      if (kMode == 2) {
-        if (tid < 32) {
-          const long long before = look_back(lb, tile, a.ntiles, (unsigned long long)total);
-          if (tid == 0) s_base = before;
-        }
-        __syncthreads();
-      }
-      int64_t o = (kMode == 2 ? (int64_t)s_base : (int64_t)tile_offset[tile]) + excl;
-#pragma unroll
-      for (int t = 1; t <= kSkWPT; ++t) {
-        if (flags >> t & 1u) {
-          const uint32_t x = xs[t];
-          const uint64_t pos = (uint64_t)(HB + x);
-          if (o < cap)
-            out[o] = ((uint64_t)s_h[hslot((int)x)] << 33) | (pos << 1) | (uint64_t)s_sg[hslot((int)x)];
-          ++o;
-        }
-      }
-    }
+    tile = kMode == 2 ? s_tile : tile + gridDim.x;
   }
 }
 
-// The 32-bit window keys hold a hash of 2k bits and a 7-bit slot offset.
-bool narrow_keys(const Derived& D) { return 2 * D.k <= 24 && D.w + kSkWPT <= 128; }
+// The 32-bit window keys hold a hash of 2k bits and a 7-bit offset.
+bool narrow_keys(const Derived& D) { return 2 * D.k <= 24 && D.w <= 112; }
 
 }  // namespace
 
@@ -473,7 +539,8 @@ int run_sketch(sedef_ctx* ctx, const uint32_t* packed, const uint32_t* mask, con
   a.min_unmasked = D.min_unmasked;
   a.kmask = D.kmask;
   const int64_t nwin = N;  // window starts q in [0, N)
-  a.ntiles = (nwin + kSkTile - 1) / kSkTile;
+  a.rep = sk_rep(N);
+  a.ntiles = (nwin + sk_tile_windows(D.w, a.rep) - 1) / sk_tile_windows(D.w, a.rep);
   int64_t* d_off = (int64_t*)ctx_alloc(ctx, (size_t)(nseq + 1) * 8);
   if (!d_off) return SEDEF_ERR_OOM;
   if (pl) {
@@ -506,10 +573,10 @@ int run_sketch(sedef_ctx* ctx, const uint32_t* packed, const uint32_t* mask, con
     SEDEF_CUDA(cudaMemsetAsync(status, 0, (size_t)(a.ntiles + 4) * 8, st));
     if (narrow)
       SEDEF_KERNEL(ctx, "k_sketch",
-                   k_sketch<2, true><<<(int)grid, kSkThreads, 0, st>>>(a, nullptr, nullptr, rec, cap, lb));
+                   k_sketch<2, uint32_t><<<(int)grid, kSkThreads, 0, st>>>(a, nullptr, nullptr, rec, cap, lb));
     else
       SEDEF_KERNEL(ctx, "k_sketch",
-                   k_sketch<2, false><<<(int)grid, kSkThreads, 0, st>>>(a, nullptr, nullptr, rec, cap, lb));
+                   k_sketch<2, uint64_t><<<(int)grid, kSkThreads, 0, st>>>(a, nullptr, nullptr, rec, cap, lb));
     unsigned long long* h = (unsigned long long*)ctx_host(ctx, 16);
     if (!h) return SEDEF_ERR_OOM;
     SEDEF_CUDA(cudaMemcpyAsync(h, status + 1, 16, cudaMemcpyDeviceToHost, st));
@@ -527,20 +594,20 @@ int run_sketch(sedef_ctx* ctx, const uint32_t* packed, const uint32_t* mask, con
   if (!cnt || !toff) return SEDEF_ERR_OOM;
   if (narrow)
     SEDEF_KERNEL(ctx, "k_sketch_count",
-                 k_sketch<0, true><<<(int)grid, kSkThreads, 0, st>>>(a, cnt, nullptr, nullptr, 0, LookBack{}));
+                 k_sketch<0, uint32_t><<<(int)grid, kSkThreads, 0, st>>>(a, cnt, nullptr, nullptr, 0, LookBack{}));
   else
     SEDEF_KERNEL(ctx, "k_sketch_count",
-                 k_sketch<0, false><<<(int)grid, kSkThreads, 0, st>>>(a, cnt, nullptr, nullptr, 0, LookBack{}));
+                 k_sketch<0, uint64_t><<<(int)grid, kSkThreads, 0, st>>>(a, cnt, nullptr, nullptr, 0, LookBack{}));
   SEDEF_TRY(scan_exclusive_u32(ctx, cnt, toff, a.ntiles, toff + a.ntiles));
   pl->n_rec = toff + a.ntiles;
   SEDEF_TRY(plan_check(ctx, pl, toff + a.ntiles, cap, 0));
   *nrec = cap;
   if (narrow)
     SEDEF_KERNEL(ctx, "k_sketch_write",
-                 k_sketch<1, true><<<(int)grid, kSkThreads, 0, st>>>(a, nullptr, toff, rec, cap, LookBack{}));
+                 k_sketch<1, uint32_t><<<(int)grid, kSkThreads, 0, st>>>(a, nullptr, toff, rec, cap, LookBack{}));
   else
     SEDEF_KERNEL(ctx, "k_sketch_write",
-                 k_sketch<1, false><<<(int)grid, kSkThreads, 0, st>>>(a, nullptr, toff, rec, cap, LookBack{}));
+                 k_sketch<1, uint64_t><<<(int)grid, kSkThreads, 0, st>>>(a, nullptr, toff, rec, cap, LookBack{}));
   return SEDEF_OK;
 }
 
@@ -560,7 +627,12 @@ namespace {
 
 constexpr int64_t kNoallocMaxBases = int64_t(256) << 20;  // 268,435,456 bases
 constexpr int kNoallocMaxSeqs = 4096;
-constexpr int64_t kNoallocMaxTiles = (kNoallocMaxBases + kSkTile - 1) / kSkTile;
+// the widest window has the fewest windows per tile; inputs just below the
+// long ones have the most tiles of one stretch
+constexpr int64_t kNoallocMaxTiles =
+    (kNoallocMaxBases + sk_tile_windows(kSkMaxW, kSkRep) - 1) / sk_tile_windows(kSkMaxW, kSkRep);
+static_assert(kNoallocMaxTiles >= (kSkRepBases + sk_tile_windows(kSkMaxW, 1) - 1) / sk_tile_windows(kSkMaxW, 1),
+              "the shorter inputs' tiles must fit too");
 constexpr size_t kNoallocCountBytes = (size_t)(kNoallocMaxTiles + 1) * 4;
 constexpr size_t kNoallocBytes = 2 * kNoallocCountBytes + (size_t)(kNoallocMaxSeqs + 1) * 8;
 
@@ -569,7 +641,7 @@ constexpr size_t kNoallocBytes = 2 * kNoallocCountBytes + (size_t)(kNoallocMaxSe
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoallocBytes];
 
 
-// Exclusive scan of n counts by one block (n is at most 131,073 here).
+// Exclusive scan of n counts by one block (n is at most 34,953 here).
 __global__ void __launch_bounds__(1024) k_scan_one_block(const uint32_t* __restrict__ in,
                                                          uint32_t* __restrict__ out, int64_t n) {
   __shared__ int tmp[33];
@@ -641,14 +713,15 @@ extern "C" int sedef_sketch_noalloc(const uint32_t* d_packed, const uint32_t* d_
   a.w = D.w;
   a.min_unmasked = D.min_unmasked;
   a.kmask = D.kmask;
-  a.ntiles = (N + kSkTile - 1) / kSkTile;
+  a.rep = sk_rep(N);
+  a.ntiles = (N + sk_tile_windows(D.w, a.rep) - 1) / sk_tile_windows(D.w, a.rep);
   int sms = 0;
   SEDEF_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   int64_t grid = a.ntiles < (int64_t)sms * 8 ? a.ntiles : (int64_t)sms * 8;
   if (narrow_keys(D))
-    k_sketch<0, true><<<(int)grid, kSkThreads, 0, st>>>(a, cnt, nullptr, nullptr, 0, LookBack{});
+    k_sketch<0, uint32_t><<<(int)grid, kSkThreads, 0, st>>>(a, cnt, nullptr, nullptr, 0, LookBack{});
   else
-    k_sketch<0, false><<<(int)grid, kSkThreads, 0, st>>>(a, cnt, nullptr, nullptr, 0, LookBack{});
+    k_sketch<0, uint64_t><<<(int)grid, kSkThreads, 0, st>>>(a, cnt, nullptr, nullptr, 0, LookBack{});
   count_launch();
   SEDEF_LAUNCHED("k_sketch_count");
   k_scan_one_block<<<1, 1024, 0, st>>>(cnt, toff, a.ntiles);
@@ -660,9 +733,9 @@ extern "C" int sedef_sketch_noalloc(const uint32_t* d_packed, const uint32_t* d_
   *h_nrec = total;
   if ((int64_t)total > rec_cap) return fail(SEDEF_ERR_CAPACITY, "record buffer too small");
   if (narrow_keys(D))
-    k_sketch<1, true><<<(int)grid, kSkThreads, 0, st>>>(a, nullptr, toff, d_rec, rec_cap, LookBack{});
+    k_sketch<1, uint32_t><<<(int)grid, kSkThreads, 0, st>>>(a, nullptr, toff, d_rec, rec_cap, LookBack{});
   else
-    k_sketch<1, false><<<(int)grid, kSkThreads, 0, st>>>(a, nullptr, toff, d_rec, rec_cap, LookBack{});
+    k_sketch<1, uint64_t><<<(int)grid, kSkThreads, 0, st>>>(a, nullptr, toff, d_rec, rec_cap, LookBack{});
   count_launch();
   SEDEF_LAUNCHED("k_sketch_write");
   SEDEF_CUDA(cudaStreamSynchronize(st));

@@ -64,3 +64,59 @@ def test_refine_recurring_hashes(ctx, pd):
     runs, n = ctx.sedef_filter(rec, g.offsets, rec, srt, off, g.offsets, p)
     assert n > 20
     assert_rows_equal(run_rows(runs), want, "runs")
+
+
+def sketch_rows(ctx, g, d):
+    p = binding.params_from_dict(d)
+    torch = need_gpu()
+    packed, mask, nbits = ctx.sedef_pack(to_dev(g.seq))
+    rec = ctx.sedef_sketch(packed, mask, nbits, g.offsets, p)
+    static = torch.zeros(g.length + 1, dtype=torch.int64, device="cuda:0")
+    n = binding.sedef_sketch_noalloc(packed, mask, nbits, g.offsets, p, static,
+                                     torch.cuda.current_stream())
+    assert n == rec.numel() and torch.equal(static[:n], rec)  # count and write = one pass
+    return rec_rows(rec)
+
+
+# around a lane's 16 positions, whole lanes, the 32-bit keys' limit (112) and the widest
+@pytest.mark.parametrize("w", [1, 2, 3, 7, 8, 9, 15, 16, 17, 31, 33, 50, 63, 64, 97, 111, 112, 113,
+                               128, 200, 255, 256])
+@pytest.mark.parametrize("k", [2, 8, 12, 13, 15])
+def test_sketch_window_lengths(ctx, k, w):
+    rng = np.random.default_rng(w * 16 + k)
+    lengths = [k + w - 2, k + w - 1, k + w, 5, 0, 1, 700, 481, 3841, 9000]
+    parts = [synth.random_bases(rng, n) for n in lengths]
+    parts[-1][2000:2600] = ord("A")  # equal and palindromic k-mers
+    parts[-1][3000:3400] = np.frombuffer(b"ACGT" * 100, dtype=np.uint8)
+    g = synth.genome_from_parts(parts)
+    s = g.seq
+    low = rng.random(len(s)) < 0.4
+    s[low] |= 32
+    s[rng.integers(0, len(s), 12)] = ord("N")
+    for least in (0, 1, 4):
+        d = oracle.params(k=k, w=w, min_unmasked=least)
+        assert_rows_equal(sketch_rows(ctx, g, d), oracle.sketch(g.seq, g.offsets, d),
+                          f"k {k} w {w} min_unmasked {least}")
+
+
+@pytest.mark.parametrize("n", [479, 480, 481, 3839, 3840, 3841, 15 * 16 * 8 * 40 + 7])
+def test_sketch_tile_ends(ctx, n):
+    """Window counts around a warp's and a CTA's tile, sequences that end inside one."""
+    rng = np.random.default_rng(n)
+    for cut in (0, 1, 16, n // 2):
+        parts = [synth.random_bases(rng, cut), synth.random_bases(rng, n - cut)]
+        g = synth.genome_from_parts(parts)
+        d = oracle.params()
+        assert_rows_equal(sketch_rows(ctx, g, d), oracle.sketch(g.seq, g.offsets, d), f"{n} {cut}")
+
+
+def test_pack_every_byte(ctx):
+    """Every byte value in every place of a thread's 16, alone among bases."""
+    seq = np.frombuffer(b"ACGTacgt" * 2, dtype=np.uint8)
+    rows = np.tile(seq, (256 * 16, 1))
+    for b in range(256):
+        for x in range(16):
+            rows[b * 16 + x, x] = b
+    flat = np.ascontiguousarray(rows.ravel())
+    for got, want in zip(ctx.sedef_pack(to_dev(flat)), oracle.pack(flat)):
+        assert np.array_equal(got.cpu().numpy().view(np.uint32)[:len(want)], want)
