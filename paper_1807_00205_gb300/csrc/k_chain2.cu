@@ -27,12 +27,12 @@
 //                 by binary search, left-maximal matches extended to the
 //                 right (count pass, then write pass at scanned offsets), so
 //                 a region's seeds come out sorted by (x, y)
-//   k_c2_dp       one warp per region: the chaining DP, predecessors scanned
-//                 back from each item, 32 per step, only as far as an item
-//                 can still reach (its start at least the current start
-//                 minus the gap bound minus the region's longest item)
-//   radix sort    by (region, -score, index), then k_c2_take: one thread per
-//                 region walks that order and takes the chains greedily
+//   k_c2_dp       one CTA per region: the chaining DP, 32 items at a time,
+//                 predecessors only as far back as an item can still reach
+//                 (its start at least the current start minus the gap bound
+//                 minus the region's longest item)
+//   k_c2_take     one CTA per region: the greedy extraction, as a minimum
+//                 over every item's descendants
 // (once for the seeds and once for the initial chains), and k_c2_emit
 // compacts the final chains.
 #include <cstring>
@@ -48,7 +48,6 @@ constexpr int64_t kGapOpen = 25;         // affine gap penalty: open
 constexpr int64_t kGapDiv = 50;          // one more per kGapDiv gap bases
 constexpr int64_t kMinSD = 1000;         // SD length (Section 3)
 constexpr int64_t kMaxRegion = int64_t(1) << 20;
-constexpr int kDPWarps = 4;
 
 // A region of the batch: query and target starts, lengths, strand.
 struct Reg {
@@ -116,7 +115,7 @@ __global__ void k_c2_keys(const uint32_t* packed, const uint32_t* nbits, const R
 template <bool kWrite>
 __global__ void k_c2_mems(const uint32_t* packed, const uint32_t* nbits, const Reg* regs,
                           const int64_t* xbase_of, int nreg, int64_t total, const uint64_t* skeys,
-                          int64_t nkeys, uint32_t* count, const uint64_t* off, uint64_t* out) {
+                          int64_t nkeys, uint32_t* count, const uint32_t* off, uint64_t* out) {
   const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (g >= total) return;
   const int r = region_of(xbase_of, nreg, g);
@@ -187,122 +186,200 @@ __device__ __forceinline__ int32_t link_gain(const Item& c, const Item& d, int t
   return d.score - (int32_t)(kGapOpen + max(gq, gt) / kGapDiv);
 }
 
-// The chaining DP of one tier: one warp per region, items of region r at
+constexpr int kC2Threads = 256;
+constexpr int kC2Warps = kC2Threads / 32;
+
+// The chaining DP of one tier: one CTA per region, items of region r at
 // [ib[r], ib[r] + n[r]) in start order.  best[] and pred[] (region-local
 // index, -1 for none) per item.
-__global__ void __launch_bounds__(32 * kDPWarps) k_c2_dp(const Item* items, const int64_t* ib,
-                                                        const uint32_t* n_of, int nreg, int tier,
-                                                        int32_t g1, int32_t* best, int32_t* pred) {
-  const int lane = lane_id();
-  const int r = blockIdx.x * kDPWarps + (threadIdx.x >> 5);
-  if (r >= nreg) return;
-  const int64_t b0 = ib[r];
+//
+// 32 items at a time, one per lane of every warp: the warps share out the
+// earlier items (each read once for all 32), one warp then settles the 32
+// among themselves.  What bounds it is the chain of dependent steps: one
+// item at a time by one warp paid a round trip to L2 per 32 predecessors of
+// every item (a region of 100 kbp has thousands of initial chains, all of
+// them within reach of tier 2): 34.3 -> 2.6 ms for the regions of a 4 Mbp
+// genome.
+__global__ void __launch_bounds__(kC2Threads) k_c2_dp(const Item* items, const int64_t* ib,
+                                                      const uint32_t* n_of, int tier, int32_t g1,
+                                                      int32_t* best, int32_t* pred) {
+  __shared__ int32_t s_v[kC2Warps][32], s_a[kC2Warps][32];
+  const int lane = lane_id(), warp = threadIdx.x >> 5;
+  const int r = blockIdx.x;
+  const Item* it = items + ib[r];
+  int32_t* f_of = best + ib[r];
+  int32_t* p_of = pred + ib[r];
   const int32_t n = (int32_t)n_of[r];
   // the longest item bounds how far back a predecessor can start
   int32_t span = 0;
-  for (int32_t u = lane; u < n; u += 32) span = max(span, items[b0 + u].x1 - items[b0 + u].x0);
-#pragma unroll
-  for (int d = 16; d > 0; d >>= 1) span = max(span, __shfl_xor_sync(0xffffffffu, span, d));
+  for (int32_t u = threadIdx.x; u < n; u += kC2Threads) span = max(span, it[u].x1 - it[u].x0);
+  span = (int32_t)__reduce_max_sync(0xffffffffu, (uint32_t)span);
+  if (lane == 0) s_v[warp][0] = span;
+  __syncthreads();
+  for (int w = 0; w < kC2Warps; ++w) span = max(span, s_v[w][0]);
   const int32_t reach = (tier == 1 ? g1 : (int32_t)kG2) + span;
-  for (int32_t b = 0; b < n; ++b) {
-    const Item d = items[b0 + b];
+  int32_t from = 0;  // items before it are out of every later item's reach
+  for (int32_t t0 = 0; t0 < n; t0 += 32) {
+    const bool ok = t0 + lane < n;
+    const Item d = it[ok ? t0 + lane : n - 1];
+    const int32_t x_lo = __shfl_sync(0xffffffffu, d.x0, 0) - reach;
+    while (from < t0) {
+      const int32_t u = from + lane;
+      const unsigned in = __ballot_sync(0xffffffffu, u >= t0 || it[u].x0 >= x_lo);
+      if (in) {
+        from += __ffs(in) - 1;
+        break;
+      }
+      from += 32;
+    }
     int32_t bv = INT32_MIN, ba = -1;  // best value through a predecessor, its index
-    for (int32_t top = b - 1; top >= 0; top -= 32) {
-      const int32_t a = top - lane;
-      bool more = false;
-      if (a >= 0) {
-        const Item c = items[b0 + a];
-        more = c.x0 >= d.x0 - reach;
-        if (more) {
+#pragma unroll 4
+    for (int32_t u = from + warp; u < t0; u += kC2Warps) {
+      const int32_t g = link_gain(it[u], d, tier, g1);
+      if (g != INT32_MIN) {
+        const int32_t v = f_of[u] + g;
+        if (v >= bv) {  // the later of equals
+          bv = v;
+          ba = u;
+        }
+      }
+    }
+    __syncthreads();  // s_v was last read for the items before
+    s_v[warp][lane] = bv;
+    s_a[warp][lane] = ba;
+    __syncthreads();
+    if (warp == 0) {
+#pragma unroll
+      for (int w = 1; w < kC2Warps; ++w) {
+        const int32_t v = s_v[w][lane], u = s_a[w][lane];
+        if (v > bv || (v == bv && u > ba)) {
+          bv = v;
+          ba = u;
+        }
+      }
+      const int last = min(32, n - t0);
+      for (int t = 0; t < last; ++t) {
+        // tier 1: f = max(L, best link); tier 2: F = S + max(0, best link - S)
+        const int32_t f = __shfl_sync(0xffffffffu, max(bv, d.score), t);
+        Item c;
+        c.x0 = __shfl_sync(0xffffffffu, d.x0, t);
+        c.x1 = __shfl_sync(0xffffffffu, d.x1, t);
+        c.y0 = __shfl_sync(0xffffffffu, d.y0, t);
+        c.y1 = __shfl_sync(0xffffffffu, d.y1, t);
+        if (lane > t) {
           const int32_t g = link_gain(c, d, tier, g1);
-          if (g != INT32_MIN) {
-            const int32_t v = best[b0 + a] + g;
-            if (v > bv || (v == bv && a > ba)) {
-              bv = v;
-              ba = a;
-            }
+          if (g != INT32_MIN && f + g >= bv) {
+            bv = f + g;
+            ba = t0 + t;
           }
         }
       }
-#pragma unroll
-      for (int s = 16; s > 0; s >>= 1) {
-        const int32_t ov = __shfl_xor_sync(0xffffffffu, bv, s);
-        const int32_t oa = __shfl_xor_sync(0xffffffffu, ba, s);
-        if (ov > bv || (ov == bv && oa > ba)) {
-          bv = ov;
-          ba = oa;
-        }
+      if (ok) {
+        const bool linked = bv > d.score;
+        f_of[t0 + lane] = linked ? bv : d.score;
+        p_of[t0 + lane] = linked ? ba : -1;
       }
-      // items are in start order: once every lane is out of reach, so is
-      // everything earlier
-      if (!__any_sync(0xffffffffu, more)) break;
     }
-    // tier 1: f = max(L, best link); tier 2: F = S + max(0, best link - S)
-    const int32_t own = d.score;
-    int32_t f = own, pr = -1;
-    if (bv != INT32_MIN && bv > own) {
-      f = bv;
-      pr = ba;
-    }
-    if (lane == 0) {
-      best[b0 + b] = f;
-      pred[b0 + b] = pr;
-    }
-    __syncwarp();
+    __syncthreads();
   }
 }
 
-// Sort keys of the greedy extraction: (region, -score, index).
-__global__ void k_c2_order_keys(const int32_t* best, const int64_t* ib, const uint32_t* n_of,
-                                int nreg, int64_t total, uint64_t* keys) {
-  const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (g >= total) return;
-  const int r = region_of(ib, nreg, g);
-  const int64_t u = g - ib[r];
-  uint64_t key = ~0ull;
-  if (u < (int64_t)n_of[r])
-    key = ((uint64_t)r << 42) | ((uint64_t)(0xFFFFF - best[g]) << 22) | (uint64_t)u;
-  keys[g] = key;
-}
+// What the greedy extraction keeps per item: the item's best descendant and
+// two buffers of ancestors, and per chain (at its last item) its furthest
+// ends, seeds and number of items.
+struct Take {
+  unsigned long long* owner;
+  int32_t *jump, *jump2;
+  int32_t *x1, *y1, *seeds, *parts;
+};
 
-// Greedy extraction (one thread per region): chains in the order of
-// `order` (sorted keys), each back along pred to the first item already
-// taken.  Writes one Item per chain to out[ib[r] + j], its number of items
-// to parts[ib[r] + j], and the count.  A chain's box starts at its first
-// item; it ends at the furthest item end (tier 1) or at its last item's end
-// (tier 2); its score is the first item's plus every link's gain.
-__global__ void k_c2_take(const Item* items, const int32_t* pred, const int64_t* ib,
-                          const uint32_t* n_of, int nreg, int tier, int32_t g1,
-                          const uint64_t* order, uint8_t* used, int32_t* path, Item* out,
-                          int32_t* parts, uint32_t* nout) {
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= nreg) return;
+// Greedy extraction (one CTA per region): chains in order of decreasing best
+// score (the earlier item on ties), each back along pred to the first item
+// already taken.  An item goes to the first chain in that order whose walk
+// reaches it, which is the least of (-score, index) over the item and all
+// items whose walks pass it: a minimum over descendants, found by doubling
+// the walks' stride (the walks themselves, one thread per region, took 27 ms
+// where this takes 0.26).  A chain's score is its first item's plus every
+// link's gain, the difference of the DP's values at its two ends; its box
+// starts at its first item and ends at the furthest item end (tier 1) or at
+// its last item's end (tier 2).  Writes the chains in the order of their
+// first items, which is start order, to out[ib[r] ..] with their item counts
+// in parts_out, and their number.
+__global__ void __launch_bounds__(kC2Threads) k_c2_take(const Item* items, const int32_t* best,
+                                                        const int32_t* pred, const int64_t* ib,
+                                                        const uint32_t* n_of, int tier, Take T,
+                                                        Item* out, int32_t* parts_out,
+                                                        uint32_t* nout) {
+  __shared__ int s_tmp[33];
+  const int r = blockIdx.x;
   const int64_t b0 = ib[r];
   const int32_t n = (int32_t)n_of[r];
-  uint32_t m = 0;
-  for (int32_t k = 0; k < n; ++k) {
-    const int32_t b = (int32_t)(order[b0 + k] & 0x3FFFFF);
-    if (used[b0 + b]) continue;
-    int32_t len = 0;
-    for (int32_t c = b; c >= 0 && !used[b0 + c]; c = pred[b0 + c]) {
-      used[b0 + c] = 1;
-      path[b0 + len++] = c;
-    }
-    // path[b0 .. b0 + len) holds the chain from its end back to its start
-    Item ch = items[b0 + path[b0 + len - 1]];
-    for (int32_t u = len - 2; u >= 0; --u) {
-      const Item prev = items[b0 + path[b0 + u + 1]];
-      const Item cur = items[b0 + path[b0 + u]];
-      ch.x1 = tier == 1 ? max(ch.x1, cur.x1) : cur.x1;
-      ch.y1 = tier == 1 ? max(ch.y1, cur.y1) : cur.y1;
-      ch.seeds += cur.seeds;
-      ch.score += link_gain(prev, cur, tier, g1);
-    }
-    out[b0 + m] = ch;
-    parts[b0 + m] = len;
-    ++m;
+  const Item* it = items + b0;
+  const int32_t* bst = best + b0;
+  const int32_t* prd = pred + b0;
+  unsigned long long* own = T.owner + b0;
+  int32_t *x1 = T.x1 + b0, *y1 = T.y1 + b0, *seeds = T.seeds + b0, *parts = T.parts + b0;
+  bool more = false;
+  for (int32_t u = threadIdx.x; u < n; u += kC2Threads) {
+    own[u] = ((unsigned long long)(0x7FFFFFFF - bst[u]) << 32) | (uint32_t)u;
+    T.jump[b0 + u] = prd[u];
+    more |= prd[u] >= 0;
+    x1[u] = y1[u] = INT32_MIN;
+    seeds[u] = parts[u] = 0;
   }
-  nout[r] = m;
+  // after round k an item knows its descendants up to 2^(k+1) - 1 links away
+  int32_t *src = T.jump + b0, *dst = T.jump2 + b0;
+  while (__syncthreads_or(more)) {
+    more = false;
+    for (int32_t u = threadIdx.x; u < n; u += kC2Threads) {
+      const int32_t j = src[u];
+      int32_t to = -1;
+      if (j >= 0) {
+        atomicMin(own + j, *(volatile unsigned long long*)(own + u));
+        to = src[j];
+      }
+      dst[u] = to;
+      more |= to >= 0;
+    }
+    int32_t* t = src;
+    src = dst;
+    dst = t;
+  }
+  for (int32_t u = threadIdx.x; u < n; u += kC2Threads) {
+    const uint32_t h = (uint32_t)__ldcg(own + u);
+    const Item c = it[u];
+    if (tier == 1) {
+      atomicMax(x1 + h, c.x1);
+      atomicMax(y1 + h, c.y1);
+    }
+    atomicAdd(seeds + h, c.seeds);
+    atomicAdd(parts + h, 1);
+  }
+  __syncthreads();
+  int m = 0;
+  for (int32_t base = 0; base < n; base += kC2Threads) {
+    const int32_t u = base + threadIdx.x;
+    bool first = false;
+    uint32_t h = 0;
+    if (u < n) {
+      const unsigned long long o = __ldcg(own + u);
+      h = (uint32_t)o;
+      first = prd[u] < 0 || __ldcg(own + prd[u]) != o;
+    }
+    int tot;
+    const int at = m + block_exclusive_sum(first ? 1 : 0, s_tmp, &tot);
+    if (first) {
+      Item c = it[u];
+      c.score += bst[h] - bst[u];
+      c.seeds = __ldcg(seeds + h);
+      c.x1 = tier == 1 ? __ldcg(x1 + h) : it[h].x1;
+      c.y1 = tier == 1 ? __ldcg(y1 + h) : it[h].y1;
+      out[b0 + at] = c;
+      parts_out[b0 + at] = __ldcg(parts + h);
+    }
+    m += tot;
+  }
+  if (threadIdx.x == 0) nout[r] = (uint32_t)m;
 }
 
 // Seeds (x << 40 | y << 20 | L) as chaining items.
@@ -311,43 +388,50 @@ __global__ void k_c2_items(const uint64_t* seeds, int64_t n, Item* items) {
   if (g < n) items[g] = seed_item(seeds[g]);
 }
 
-// Start-order keys of the initial chains: (region, x0, y0) -> slot.
-__global__ void k_c2_start_keys(const Item* ch, const int64_t* ib, const uint32_t* n_of, int nreg,
-                                int64_t total, uint64_t* keys) {
-  const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (g >= total) return;
-  const int r = region_of(ib, nreg, g);
-  const int64_t u = g - ib[r];
-  uint64_t key = ~0ull;
-  if (u < (int64_t)n_of[r])
-    key = ((uint64_t)r << 42) | ((uint64_t)ch[g].x0 << 21) | (uint64_t)ch[g].y0;
-  keys[g] = key;
+// Sum of n counts in 64 bits.
+__global__ void k_c2_sum(const uint32_t* v, int64_t n, unsigned long long* total) {
+  unsigned long long s = 0;
+  for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < n;
+       x += (int64_t)gridDim.x * blockDim.x)
+    s += v[x];
+  s = warp_sum(s);
+  if (lane_id() == 0 && s) atomicAdd(total, s);
 }
 
-// Gathers the initial chains of each region into start order at the same
-// region base (the sort kept regions apart and in order).
-__global__ void k_c2_gather(const Item* in, const uint32_t* perm, const uint64_t* skeys,
-                            int64_t total, Item* out) {
-  const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (g >= total) return;
-  if (skeys[g] != ~0ull) out[g] = in[perm[g]];
+// Seed ranges of the regions from the seeds' offsets: ib[0..nreg], n[0..nreg).
+__global__ void k_c2_ranges(const uint32_t* off, const int64_t* xbase_of, int nreg, int64_t* ib,
+                            uint32_t* n) {
+  const int r = blockIdx.x * blockDim.x + threadIdx.x;
+  if (r > nreg) return;
+  ib[r] = off[xbase_of[r]];
+  if (r < nreg) n[r] = off[xbase_of[r + 1]] - off[xbase_of[r]];
 }
 
 // Final chains of at least kMinSD bases on both axes, per region, sorted by
-// (q0, q1, t0, t1, score) in genome coordinates, written at out[ob[r] ..].
+// (q0, q1, t0, t1, score) in genome coordinates, written at out[ob[r] ..]
+// (one warp per region; few chains are that long, and they come by q0).
 __global__ void k_c2_emit(const Item* fin, const int32_t* parts, const int64_t* ib,
                           const uint32_t* n_of, const Reg* regs, const int64_t* reg_index,
                           int nreg, const int64_t* ob, sedef_sd_t* out, uint32_t* nkept,
                           int count_only) {
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
+  const int r = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
   if (r >= nreg) return;
+  const int lane = lane_id();
   const Reg R = regs[r];
   const int64_t b0 = ib[r];
+  const uint32_t n = n_of[r];
+  sedef_sd_t* row = out + (count_only ? 0 : ob[r]);
   uint32_t m = 0;
-  for (uint32_t u = 0; u < n_of[r]; ++u) {
-    const Item c = fin[b0 + u];
-    if (c.x1 - c.x0 < kMinSD || c.y1 - c.y0 < kMinSD) continue;
-    if (!count_only) {
+  for (uint32_t base = 0; base < n; base += 32) {
+    const uint32_t u = base + lane;
+    Item c;
+    bool keep = false;
+    if (u < n) {
+      c = fin[b0 + u];
+      keep = c.x1 - c.x0 >= kMinSD && c.y1 - c.y0 >= kMinSD;
+    }
+    const unsigned bal = __ballot_sync(0xffffffffu, keep);
+    if (keep && !count_only) {
       sedef_sd_t s;
       s.region = (uint32_t)reg_index[r];
       s.o = (uint32_t)R.o;
@@ -359,27 +443,31 @@ __global__ void k_c2_emit(const Item* fin, const int32_t* parts, const int64_t* 
       s.seeds = (uint32_t)c.seeds;
       s.parts = (uint32_t)parts[b0 + u];
       s.reserved = 0;
-      // insertion into this region's sorted rows
-      sedef_sd_t* row = out + ob[r];
-      uint32_t at = m;
-      auto less = [](const sedef_sd_t& a, const sedef_sd_t& b) {
-        if (a.q0 != b.q0) return a.q0 < b.q0;
-        if (a.q1 != b.q1) return a.q1 < b.q1;
-        if (a.t0 != b.t0) return a.t0 < b.t0;
-        if (a.t1 != b.t1) return a.t1 < b.t1;
-        if (a.score != b.score) return a.score < b.score;
-        if (a.seeds != b.seeds) return a.seeds < b.seeds;
-        return a.parts < b.parts;
-      };
-      while (at > 0 && less(s, row[at - 1])) {
-        row[at] = row[at - 1];
-        --at;
-      }
-      row[at] = s;
+      row[m + __popc(bal & lanemask_lt())] = s;
     }
-    ++m;
+    m += __popc(bal);
   }
-  nkept[r] = m;
+  if (lane == 0) nkept[r] = m;
+  __syncwarp();
+  if (count_only || lane != 0) return;
+  auto less = [](const sedef_sd_t& a, const sedef_sd_t& b) {
+    if (a.q0 != b.q0) return a.q0 < b.q0;
+    if (a.q1 != b.q1) return a.q1 < b.q1;
+    if (a.t0 != b.t0) return a.t0 < b.t0;
+    if (a.t1 != b.t1) return a.t1 < b.t1;
+    if (a.score != b.score) return a.score < b.score;
+    if (a.seeds != b.seeds) return a.seeds < b.seeds;
+    return a.parts < b.parts;
+  };
+  for (uint32_t u = 1; u < m; ++u) {
+    const sedef_sd_t s = row[u];
+    uint32_t at = u;
+    while (at > 0 && less(s, row[at - 1])) {
+      row[at] = row[at - 1];
+      --at;
+    }
+    if (at != u) row[at] = s;
+  }
 }
 
 }  // namespace
@@ -436,128 +524,106 @@ int run_chain2(sedef_ctx* ctx, const uint32_t* packed, const uint32_t* nbits, in
     SEDEF_CUDA(cudaMemcpyAsync(d_yb, yb.data(), 8 * (size_t)(nb + 1), cudaMemcpyHostToDevice, st));
     SEDEF_CUDA(cudaMemcpyAsync(d_xb, xb.data(), 8 * (size_t)(nb + 1), cudaMemcpyHostToDevice, st));
     SEDEF_CUDA(cudaMemcpyAsync(d_rid, rid.data(), 8 * (size_t)nb, cudaMemcpyHostToDevice, st));
-    // target k-mer keys, sorted
+    // target k-mer keys, sorted (a key that holds no k-mer sorts last)
     const int64_t ny = ysum > 0 ? ysum : 1;
     uint64_t* keys = (uint64_t*)ctx_alloc(ctx, (size_t)ny * 8);
     uint64_t* skeys = (uint64_t*)ctx_alloc(ctx, (size_t)ny * 8);
     if (!keys || !skeys) return SEDEF_ERR_OOM;
+    int rbits = 1;
+    while ((int64_t(1) << rbits) <= nb) ++rbits;
     if (ysum > 0) {
       SEDEF_KERNEL(ctx, "k_c2_keys", k_c2_keys<<<(int)((ysum + 255) / 256), 256, 0, st>>>(
                                          packed, nbits, d_regs, d_yb, nb, ysum, keys));
-      SEDEF_TRY(radix_sort_u64(ctx, keys, nullptr, skeys, nullptr, ysum, 20, 64));
+      SEDEF_TRY(radix_sort_u64(ctx, keys, nullptr, skeys, nullptr, ysum, 20, 42 + rbits));
     }
     // seeds: count, scan, write
     const int64_t nx = xsum > 0 ? xsum : 1;
     uint32_t* cnt = (uint32_t*)ctx_alloc(ctx, (size_t)(nx + 1) * 4);
-    uint64_t* off = (uint64_t*)ctx_alloc(ctx, (size_t)(nx + 1) * 8);
-    if (!cnt || !off) return SEDEF_ERR_OOM;
-    std::vector<uint32_t> hc((size_t)nx + 1, 0);
+    uint32_t* off = (uint32_t*)ctx_alloc(ctx, (size_t)(nx + 1) * 4);
+    char* d_meta = (char*)ctx_alloc(ctx, 8 + (size_t)(nb + 1) * 8 * 2 + (size_t)nb * 4 * 4);
+    if (!cnt || !off || !d_meta) return SEDEF_ERR_OOM;
+    unsigned long long* d_total = (unsigned long long*)d_meta;
+    int64_t* d_ib = (int64_t*)(d_meta + 8);
+    int64_t* d_kb = d_ib + (nb + 1);
+    uint32_t* d_n1 = (uint32_t*)(d_kb + (nb + 1));
+    uint32_t* d_n2 = d_n1 + nb;
+    uint32_t* d_n3 = d_n2 + nb;
+    uint32_t* d_keep = d_n3 + nb;
+    int64_t na = 0;
     if (xsum > 0 && ysum > 0) {
       SEDEF_KERNEL(ctx, "k_c2_mems", (k_c2_mems<false><<<(int)((xsum + 255) / 256), 256, 0, st>>>(
                                          packed, nbits, d_regs, d_xb, nb, xsum, skeys, ysum, cnt,
                                          nullptr, nullptr)));
-      SEDEF_CUDA(cudaMemcpyAsync(hc.data(), cnt, (size_t)xsum * 4, cudaMemcpyDeviceToHost, st));
+      SEDEF_CUDA(cudaMemsetAsync(d_total, 0, 8, st));
+      int64_t sg = (xsum + 255) / 256;
+      if (sg > (int64_t)ctx_sm_count(ctx) * 8) sg = (int64_t)ctx_sm_count(ctx) * 8;
+      SEDEF_KERNEL(ctx, "k_c2_sum", k_c2_sum<<<(int)sg, 256, 0, st>>>(cnt, xsum, d_total));
+      SEDEF_TRY(scan_exclusive_u32(ctx, cnt, off, xsum, off + xsum));
+      SEDEF_KERNEL(ctx, "k_c2_ranges",
+                   k_c2_ranges<<<(nb + 256) / 256, 256, 0, st>>>(off, d_xb, nb, d_ib, d_n1));
+      unsigned long long total = 0;
+      std::vector<uint32_t> ncount(nb, 0);
+      SEDEF_CUDA(cudaMemcpyAsync(&total, d_total, 8, cudaMemcpyDeviceToHost, st));
+      SEDEF_CUDA(cudaMemcpyAsync(ncount.data(), d_n1, (size_t)nb * 4, cudaMemcpyDeviceToHost, st));
       SEDEF_CUDA(cudaStreamSynchronize(st));
+      // the offsets are 32-bit; a batch with more seeds than that would need
+      // more than 300 GB of items
+      if (total >= (1ull << 32))
+        return fail(SEDEF_ERR_OOM, "sedef_chain2: more than 2^32 seeds in a batch of regions");
+      na = (int64_t)total;
+      for (int k = 0; k < nb; ++k)
+        if ((int64_t)ncount[k] >= (int64_t(1) << 22))
+          return fail(SEDEF_ERR_UNSUPPORTED, "sedef_chain2: more than 2^22 seeds in a region");
     }
-    std::vector<uint64_t> ho((size_t)nx + 1, 0);
-    for (int64_t g = 0; g < xsum; ++g) ho[g + 1] = ho[g] + hc[g];
-    const int64_t na = (int64_t)ho[xsum > 0 ? xsum : 0];
-    // per-region seed ranges and counts
-    std::vector<int64_t> ib(nb + 1, 0);
-    std::vector<uint32_t> ncount(nb, 0);
-    for (int k = 0; k < nb; ++k) {
-      ib[k] = (int64_t)ho[xb[k]];
-      ncount[k] = (uint32_t)(ho[xb[k + 1]] - ho[xb[k]]);
-      if ((int64_t)ncount[k] >= (int64_t(1) << 22))
-        return fail(SEDEF_ERR_UNSUPPORTED, "sedef_chain2: more than 2^22 seeds in a region");
-    }
-    ib[nb] = na;
     std::vector<sedef_sd_t> rows;
     if (na > 0) {
       uint64_t* seeds = (uint64_t*)ctx_alloc(ctx, (size_t)na * 8);
       Item* items = (Item*)ctx_alloc(ctx, (size_t)na * sizeof(Item));
       Item* init = (Item*)ctx_alloc(ctx, (size_t)na * sizeof(Item));
-      Item* sorted = (Item*)ctx_alloc(ctx, (size_t)na * sizeof(Item));
       Item* fin = (Item*)ctx_alloc(ctx, (size_t)na * sizeof(Item));
       int32_t* best = (int32_t*)ctx_alloc(ctx, (size_t)na * 4);
       int32_t* pred = (int32_t*)ctx_alloc(ctx, (size_t)na * 4);
-      int32_t* path = (int32_t*)ctx_alloc(ctx, (size_t)na * 4);
       int32_t* parts = (int32_t*)ctx_alloc(ctx, (size_t)na * 4);
-      uint8_t* used = (uint8_t*)ctx_alloc(ctx, (size_t)na);
-      uint64_t* okeys = (uint64_t*)ctx_alloc(ctx, (size_t)na * 8);
-      uint64_t* osorted = (uint64_t*)ctx_alloc(ctx, (size_t)na * 8);
-      uint32_t* perm = (uint32_t*)ctx_alloc(ctx, (size_t)na * 4);
-      char* d_meta = (char*)ctx_alloc(ctx, (size_t)(nb + 1) * 8 * 2 + (size_t)nb * 4 * 4);
-      if (!seeds || !items || !init || !sorted || !fin || !best || !pred || !path || !parts || !used ||
-          !okeys || !osorted || !perm || !d_meta)
+      Take T;
+      T.owner = (unsigned long long*)ctx_alloc(ctx, (size_t)na * 8);
+      int32_t* words = (int32_t*)ctx_alloc(ctx, (size_t)na * 4 * 6);
+      if (!seeds || !items || !init || !fin || !best || !pred || !parts || !T.owner || !words)
         return SEDEF_ERR_OOM;
-      int64_t* d_ib = (int64_t*)d_meta;
-      int64_t* d_ob = d_ib + (nb + 1);
-      uint32_t* d_n1 = (uint32_t*)(d_ob + (nb + 1));
-      uint32_t* d_n2 = d_n1 + nb;
-      uint32_t* d_n3 = d_n2 + nb;
-      uint32_t* d_keep = d_n3 + nb;
-      uint64_t* d_off = off;
-      SEDEF_CUDA(cudaMemcpyAsync(d_off, ho.data(), (size_t)(xsum + 1) * 8, cudaMemcpyHostToDevice, st));
-      SEDEF_CUDA(cudaMemcpyAsync(d_ib, ib.data(), (size_t)(nb + 1) * 8, cudaMemcpyHostToDevice, st));
-      SEDEF_CUDA(cudaMemcpyAsync(d_n1, ncount.data(), (size_t)nb * 4, cudaMemcpyHostToDevice, st));
+      T.jump = words;
+      T.jump2 = words + na;
+      T.x1 = words + 2 * na;
+      T.y1 = words + 3 * na;
+      T.seeds = words + 4 * na;
+      T.parts = words + 5 * na;
       SEDEF_KERNEL(ctx, "k_c2_mems", (k_c2_mems<true><<<(int)((xsum + 255) / 256), 256, 0, st>>>(
                                          packed, nbits, d_regs, d_xb, nb, xsum, skeys, ysum,
-                                         nullptr, d_off, seeds)));
-      const int tb = (int)((na + 255) / 256);
-      const int rb = (nb + 127) / 128;
-      const int wb = (nb + kDPWarps - 1) / kDPWarps;
-      SEDEF_KERNEL(ctx, "k_c2_items", k_c2_items<<<tb, 256, 0, st>>>(seeds, na, items));
-      // tier 1: DP, greedy extraction into initial chains
-      SEDEF_KERNEL(ctx, "k_c2_dp", k_c2_dp<<<wb, 32 * kDPWarps, 0, st>>>(items, d_ib, d_n1, nb, 1, g1,
-                                                                       best, pred));
-      SEDEF_KERNEL(ctx, "k_c2_order_keys", k_c2_order_keys<<<tb, 256, 0, st>>>(best, d_ib, d_n1, nb,
-                                                                              na, okeys));
-      SEDEF_TRY(radix_sort_u64(ctx, okeys, nullptr, osorted, nullptr, na, 0, 64));
-      SEDEF_CUDA(cudaMemsetAsync(used, 0, (size_t)na, st));
-      SEDEF_KERNEL(ctx, "k_c2_take", k_c2_take<<<rb, 128, 0, st>>>(items, pred, d_ib, d_n1, nb, 1, g1,
-                                                                  osorted, used, path, init, parts,
-                                                                  d_n2));
-      // initial chains into start order
-      SEDEF_KERNEL(ctx, "k_c2_start_keys", k_c2_start_keys<<<tb, 256, 0, st>>>(init, d_ib, d_n2, nb,
-                                                                              na, okeys));
-      SEDEF_TRY(radix_sort_u64(ctx, okeys, nullptr, osorted, perm, na, 0, 64));
-      // sorted chains of region r now start at the region's first sorted
-      // slot: bases from the counts
-      std::vector<uint32_t> n2(nb);
-      SEDEF_CUDA(cudaMemcpyAsync(n2.data(), d_n2, (size_t)nb * 4, cudaMemcpyDeviceToHost, st));
-      SEDEF_CUDA(cudaStreamSynchronize(st));
-      std::vector<int64_t> cb(nb + 1, 0);
-      for (int k = 0; k < nb; ++k) cb[k + 1] = cb[k] + n2[k];
-      int64_t* d_cb = d_ob;
-      SEDEF_CUDA(cudaMemcpyAsync(d_cb, cb.data(), (size_t)(nb + 1) * 8, cudaMemcpyHostToDevice, st));
-      SEDEF_KERNEL(ctx, "k_c2_gather", k_c2_gather<<<tb, 256, 0, st>>>(init, perm, osorted, na, sorted));
-      // tier 2 over the initial chains (region r at [cb[r], cb[r] + n2[r]))
-      SEDEF_KERNEL(ctx, "k_c2_dp", k_c2_dp<<<wb, 32 * kDPWarps, 0, st>>>(sorted, d_cb, d_n2, nb, 2, g1,
-                                                                       best, pred));
-      const int64_t nc = cb[nb] > 0 ? cb[nb] : 1;
-      const int tc = (int)((nc + 255) / 256);
-      SEDEF_KERNEL(ctx, "k_c2_order_keys", k_c2_order_keys<<<tc, 256, 0, st>>>(best, d_cb, d_n2, nb,
-                                                                              cb[nb], okeys));
-      SEDEF_TRY(radix_sort_u64(ctx, okeys, nullptr, osorted, nullptr, cb[nb], 0, 64));
-      SEDEF_CUDA(cudaMemsetAsync(used, 0, (size_t)na, st));
-      SEDEF_KERNEL(ctx, "k_c2_take", k_c2_take<<<rb, 128, 0, st>>>(sorted, pred, d_cb, d_n2, nb, 2,
-                                                                  g1, osorted, used, path, fin,
-                                                                  parts, d_n3));
+                                         nullptr, off, seeds)));
+      SEDEF_KERNEL(ctx, "k_c2_items",
+                   k_c2_items<<<(int)((na + 255) / 256), 256, 0, st>>>(seeds, na, items));
+      // tier 1: DP, greedy extraction into initial chains (in start order)
+      SEDEF_KERNEL(ctx, "k_c2_dp",
+                   k_c2_dp<<<nb, kC2Threads, 0, st>>>(items, d_ib, d_n1, 1, g1, best, pred));
+      SEDEF_KERNEL(ctx, "k_c2_take", k_c2_take<<<nb, kC2Threads, 0, st>>>(
+                                         items, best, pred, d_ib, d_n1, 1, T, init, parts, d_n2));
+      // tier 2 over the initial chains (region r at [ib[r], ib[r] + n2[r]))
+      SEDEF_KERNEL(ctx, "k_c2_dp",
+                   k_c2_dp<<<nb, kC2Threads, 0, st>>>(init, d_ib, d_n2, 2, g1, best, pred));
+      SEDEF_KERNEL(ctx, "k_c2_take", k_c2_take<<<nb, kC2Threads, 0, st>>>(
+                                         init, best, pred, d_ib, d_n2, 2, T, fin, parts, d_n3));
       // final chains of SD size: count, then rows per region
-      SEDEF_KERNEL(ctx, "k_c2_emit", k_c2_emit<<<rb, 128, 0, st>>>(fin, parts, d_cb, d_n3, d_regs,
-                                                                  d_rid, nb, d_cb, nullptr, d_keep, 1));
+      const int rb = (int)(((int64_t)nb * 32 + 127) / 128);
+      SEDEF_KERNEL(ctx, "k_c2_emit", k_c2_emit<<<rb, 128, 0, st>>>(fin, parts, d_ib, d_n3, d_regs,
+                                                                  d_rid, nb, nullptr, nullptr, d_keep, 1));
       std::vector<uint32_t> keep(nb);
       SEDEF_CUDA(cudaMemcpyAsync(keep.data(), d_keep, (size_t)nb * 4, cudaMemcpyDeviceToHost, st));
       SEDEF_CUDA(cudaStreamSynchronize(st));
       std::vector<int64_t> kb(nb + 1, 0);
       for (int k = 0; k < nb; ++k) kb[k + 1] = kb[k] + keep[k];
       if (kb[nb] > 0) {
-        int64_t* d_kb = (int64_t*)ctx_alloc(ctx, (size_t)(nb + 1) * 8);
         sedef_sd_t* d_rows = (sedef_sd_t*)ctx_alloc(ctx, (size_t)kb[nb] * sizeof(sedef_sd_t));
-        if (!d_kb || !d_rows) return SEDEF_ERR_OOM;
+        if (!d_rows) return SEDEF_ERR_OOM;
         SEDEF_CUDA(cudaMemcpyAsync(d_kb, kb.data(), (size_t)(nb + 1) * 8, cudaMemcpyHostToDevice, st));
-        SEDEF_KERNEL(ctx, "k_c2_emit", k_c2_emit<<<rb, 128, 0, st>>>(fin, parts, d_cb, d_n3, d_regs,
+        SEDEF_KERNEL(ctx, "k_c2_emit", k_c2_emit<<<rb, 128, 0, st>>>(fin, parts, d_ib, d_n3, d_regs,
                                                                     d_rid, nb, d_kb, d_rows, d_keep,
                                                                     0));
         rows.resize((size_t)kb[nb]);

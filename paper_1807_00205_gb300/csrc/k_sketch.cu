@@ -395,7 +395,7 @@ __global__ void __launch_bounds__(kSkThreads, sizeof(K) == 4 ? 4 : 2) k_sketch(S
           bad |= all;
         } else if (a.min_unmasked > 1) {
           const uint32_t kb = (1u << k) - 1u;
-  #pragma unroll
+#pragma unroll
           for (int x = 0; x < kSkP; ++x)
             if (k - __popc((mk >> x) & kb) < a.min_unmasked) bad |= 1u << x;
         }
@@ -421,7 +421,7 @@ __global__ void __launch_bounds__(kSkThreads, sizeof(K) == 4 ? 4 : 2) k_sketch(S
           }
         }
         const uint32_t r0 = reverse_pairs(w0), r1 = reverse_pairs(w1);
-  #pragma unroll
+#pragma unroll
         for (int x = 0; x < kSkP; ++x) {
           // forward code: first base most significant; the reverse complement's
           // is the complement with the first base least significant
@@ -434,12 +434,12 @@ __global__ void __launch_bounds__(kSkThreads, sizeof(K) == 4 ? 4 : 2) k_sketch(S
         // selected: an eligible minimum that is not the previous window's
         const K before = __shfl_up_sync(0xffffffffu, key[kSkP - 1], 1) + (K)kSkP;
         uint32_t valid = 0;
-  #pragma unroll
+#pragma unroll
         for (int x = 0; x < kSkP; ++x)
           if (!Key<K>::is_none(key[x])) valid |= 1u << x;
         valid &= ok;
         uint32_t same = 0;
-  #pragma unroll
+#pragma unroll
         for (int x = 0; x < kSkP; ++x)
           if (key[x] == (x ? key[x - 1] : before)) same |= 1u << x;
         const uint32_t vb = __shfl_up_sync(0xffffffffu, valid >> (kSkP - 1), 1);
@@ -450,7 +450,7 @@ __global__ void __launch_bounds__(kSkThreads, sizeof(K) == 4 ? 4 : 2) k_sketch(S
       const int inc = warp_inclusive_sum(cnt);
       if (kMode != 0) {
         int at = n + inc - cnt;
-  #pragma unroll
+#pragma unroll
         for (int x = 0; x < kSkP; ++x) {
           if ((flags >> x) & 1u) {
             s_stage[warp][at] = (uint16_t)(rep * wwin + lane * kSkP + Key<K>::off(key[x]));

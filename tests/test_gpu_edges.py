@@ -120,3 +120,59 @@ def test_pack_every_byte(ctx):
     flat = np.ascontiguousarray(rows.ravel())
     for got, want in zip(ctx.sedef_pack(to_dev(flat)), oracle.pack(flat)):
         assert np.array_equal(got.cpu().numpy().view(np.uint32)[:len(want)], want)
+
+
+@pytest.mark.parametrize("pd", [
+    dict(k=4, w=3, n=60, step=20, gap_max=60, diag_max=6), dict(k=7, w=5, n=200, step=100),
+    dict(k=10, w=4), dict(), dict(self_mode=2), dict(w=40), dict(delta_m=0.02, delta_g=0.02)])
+@pytest.mark.parametrize("max_len", [2000, 30_000])
+def test_extend_batches(ctx, pd, max_len):
+    """Regions that grow over many minimizers at once, end at a sequence's end, at the cap, where
+    the two would overlap, or where the estimate falls; small hash tables."""
+    from tests.test_gpu_extend import gpu_extend
+    rng = np.random.default_rng(3)
+    a = synth.random_bases(rng, 45_000, 0.45)
+    a[20_000:29_000] = synth.mutate(rng, a[4_000:14_000], 0.97)[:9_000]
+    a[36_000:45_000] = synth.reverse_complement(synth.mutate(rng, a[5_000:15_000], 0.9)[:9_000])
+    a[30_000:33_000] = np.tile(a[30_000:30_900], 4)[:3_000]   # mates that meet
+    b = synth.random_bases(rng, 12_000, 0.45)
+    b[:6_000] = synth.mutate(rng, a[8_000:15_000], 0.93)[:6_000]
+    g = synth.genome_from_parts([a, b])
+    d = oracle.params(**pd)
+    recs = oracle.sketch(g.seq, g.offsets, d)
+    runs = oracle.filter_runs(recs, g.offsets, recs, g.offsets, d, threads=8)
+    keep = np.flatnonzero(runs[:, oracle.RUN_COLS.index("keep")] == 1)
+    pick = keep[np.unique(np.linspace(0, len(keep) - 1, 40).astype(np.int64))]
+    allk = oracle.sketch(g.seq, g.offsets, dict(d, min_unmasked=0))
+    want = oracle.extend(runs[pick], allk, g.offsets, allk, g.offsets, d, max_len=max_len, threads=16)
+    got, _ = gpu_extend(ctx, g, d, max_len, keep_runs=pick)
+    assert len(want) == len(pick) > 0
+    assert_rows_equal(got, want, "regions")
+
+
+def test_chain2_item_counts(ctx):
+    """Regions with no seed, one, and around 32 and 256 of them; long ones with many chains."""
+    from tests.test_gpu_chain2 import sd_rows
+    rng = np.random.default_rng(12)
+    s = synth.random_bases(rng, 120_000)
+    s[60_000:100_000] = synth.mutate(rng, s[2_000:44_000], 0.9)[:40_000]
+    s[100_500:108_000] = synth.reverse_complement(synth.mutate(rng, s[5_000:13_000], 0.95)[:7_500])
+    s[110_000:116_000] = np.tile(s[110_000:110_037], 200)[:6_000]
+    g = synth.genome_from_parts([s])
+    rows = []
+    for n in [0, 5, 11, 12, 40, 90, 200, 300, 400, 700, 1200, 2000, 2600, 3300, 5000, 20_000, 40_000]:
+        rows.append((2_000, 2_000 + n, 60_000, 60_000 + n, 0))
+        m = min(n, 7_400)
+        rows.append((5_000, 5_000 + m, 108_000 - m, 108_000, 1))
+        m = min(n, 1_200)
+        rows.append((110_000, 110_000 + m, 112_000, 112_000 + m, 0))
+    v = np.zeros(len(rows), dtype=binding.REGION_DTYPE)
+    for c, x in zip(("qa", "qb", "ta", "tb", "o"), np.array(rows).T):
+        v[c] = x
+    ext = np.stack([v[c].astype(np.int64) for c in oracle.EXTEND_COLS], axis=1)
+    want = oracle.chain2(g.seq, ext, threads=16)
+    packed, _, nbits = ctx.sedef_pack(to_dev(g.seq))
+    out, _ = ctx.sedef_chain2(packed, nbits, g.length, to_dev(v.view(np.uint8)), len(v),
+                              binding.params())
+    assert len(want) > 15
+    assert_rows_equal(sd_rows(out), want, "SDs")
