@@ -352,7 +352,7 @@ __host__ __device__ __forceinline__ void posting_window(const uint64_t* idx, con
 
 __global__ void k_sample_pos(const uint64_t* __restrict__ idx, int64_t nt, const uint32_t* dnt,
                              uint32_t* __restrict__ samp) {
-  const int64_t n = dnt ? (int64_t)*dnt : nt;
+  const int64_t n = live_n(nt, dnt);
   const int64_t ns = (n + kSampleStride - 1) >> kSampleShift;
   for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < ns;
        k += (int64_t)gridDim.x * blockDim.x)
@@ -365,7 +365,7 @@ __global__ void k_sample_pos(const uint64_t* __restrict__ idx, int64_t nt, const
 // dependent loads.  Records are sorted by position, so neighbouring threads
 // share a genome and often a hash.
 __global__ void k_qpost(FArgs a, int64_t nq, const uint32_t* dnq, uint2* out) {
-  const int64_t n = dnq ? (int64_t)*dnq : nq;
+  const int64_t n = live_n(nq, dnq);
   for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < n;
        x += (int64_t)gridDim.x * blockDim.x) {
     const uint64_t r = a.qrec[x];

@@ -176,3 +176,24 @@ def test_chain2_item_counts(ctx):
                               binding.params())
     assert len(want) > 15
     assert_rows_equal(sd_rows(out), want, "SDs")
+
+
+@pytest.mark.parametrize("mode", [1, 2])
+def test_graph_record_overflow(ctx, mode):
+    """A captured pass whose record capacity is far too small: every kernel keeps to the records
+    that were written, the totals come back, and a graph rebuilt with them gives the eager pass."""
+    g = synth.small_case(17, lengths=(90_000, 40_000), n_sd=6, sd_lo=2000, sd_hi=8000, mask_frac=0.2)
+    p = binding.params(self_mode=mode)
+    d = to_dev(g.seq)
+    eager = ctx.selfsearch(d, g.offsets, p)
+    caps = {k: 1 << 20 for k in binding.CAP_NAMES}
+    caps["records"] = 3
+    gr = binding.Graph(ctx, d, g.offsets, p, caps)
+    gr.launch()
+    with pytest.raises(binding.SedefError) as e:
+        gr.wait()
+    assert e.value.status == binding.SEDEF_ERR_CAPACITY
+    assert gr.need["records"] == eager["rec"].numel()
+    gr.close()
+    out = ctx.selfsearch_graph(d, g.offsets, p, caps={k: 1 for k in binding.CAP_NAMES}).outputs()
+    assert np.array_equal(run_rows(out["runs"]), run_rows(eager["runs"]))
