@@ -61,15 +61,17 @@ struct FArgs {
   const uint32_t* win_qa;  // first query record of the window
   const uint32_t* win_qb;  // one past the last
   const int32_t* win_seq;  // query sequence of the window
-  // per query record: its hash's posting range narrowed to the record's own
-  // genome (batch self-search), or (kNone, 0) when the list passes max_occ;
-  // nullptr when the tiers look postings up themselves
+  // per query record of a self-search: its hash's posting range from after
+  // its own entry on (after_own), narrowed to the record's own genome in a
+  // batch, or (kNone, 0) when the list passes max_occ; nullptr when the tiers
+  // look postings up themselves
   const uint2* qpost;
   const uint32_t* tsamp;  // positions of every kSampleStride-th index entry, or nullptr
   int64_t nwin;
   int ntseq, nqseq;
   int64_t ttotal;  // target total length
   int k, n, span, max_occ, self_mode, overlap;
+  int after_own;   // qpost holds only the entries after a record's own one
   sedef_run_t* runs;
   unsigned long long* nruns;
   int64_t run_cap;
@@ -78,6 +80,18 @@ struct FArgs {
   unsigned int* next_window;
   unsigned long long* stats;  // [0] hits enumerated, [1] hits collected (fast path)
 };
+
+// A self-search has no use for a hit at t when no valid target start is at or
+// before it (starts lie at i + n - overlap or later), or when t lies in the
+// query window's own span.  Half of all hits, the mates before the window,
+// go this way.
+__device__ __forceinline__ uint32_t first_useful(const FArgs& a, int64_t i) {
+  const int64_t lo = a.self_mode ? i + a.n - a.overlap : 0;
+  return lo < 0 ? 0u : (uint32_t)min(lo, (int64_t)0xFFFFFFFF);
+}
+__device__ __forceinline__ bool useless_hit(const FArgs& a, uint32_t t, uint32_t i, uint32_t lo) {
+  return a.self_mode && (t < lo || t - i <= (uint32_t)a.span);
+}
 
 // ----------------------------------------------------------- run emission --
 
@@ -359,11 +373,11 @@ __global__ void k_sample_pos(const uint64_t* __restrict__ idx, int64_t nt, const
     samp[k] = rec_pos(idx[k << kSampleShift]);
 }
 
-// Posting range of every query record of a batch self-search, resolved once
-// per record rather than once per window that holds it (a record lies in
-// n / step windows), by threads that each follow one record's chain of
-// dependent loads.  Records are sorted by position, so neighbouring threads
-// share a genome and often a hash.
+// Posting range of every query record of a self-search, resolved once per
+// record rather than once per window that holds it (a record lies in n / step
+// windows), by threads that each follow one record's chain of dependent
+// loads.  Records are sorted by position, so neighbouring threads share a
+// genome and often a hash.
 __global__ void k_qpost(FArgs a, int64_t nq, const uint32_t* dnq, uint2* out) {
   const int64_t n = live_n(nq, dnq);
   for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < n;
@@ -375,8 +389,13 @@ __global__ void k_qpost(FArgs a, int64_t nq, const uint32_t* dnq, uint2* out) {
       out[x] = make_uint2(kNone, 0u);
       continue;
     }
-    const int sq = seq_of(a.qseq, a.nqseq, (int64_t)rec_pos(r));
-    posting_window(a.tsorted, a.tsamp, &st, &len, a.tseq[sq], a.tseq[sq + 1]);
+    int64_t lo = a.after_own ? (int64_t)rec_pos(r) + 1 : 0, hi = INT64_MAX;
+    if (a.self_mode == 2) {
+      const int sq = seq_of(a.qseq, a.nqseq, (int64_t)rec_pos(r));
+      lo = max(lo, a.tseq[sq]);
+      hi = a.tseq[sq + 1];
+    }
+    posting_window(a.tsorted, a.tsamp, &st, &len, lo, hi);
     out[x] = make_uint2(st, len);
   }
 }
@@ -423,13 +442,13 @@ __device__ int build_wq(const FArgs& a, QBuild q, int c, int64_t seq_lo = 0, int
   return s_count;
 }
 
-// Posting ranges in index order (eager batch self-search).  The query
-// records of a self-search are the index's own records, and the entries of
-// the index with one hash in one genome form a run that is the narrowed
-// posting range of each of its records.  So the ranges come from one walk
-// over the index: a warp reads 32 consecutive entries, splits them into runs
-// by (hash, genome), and searches only for the ends of the runs that leave
-// its 32 entries.  Each range goes to its record, found by the rank of the
+// Posting ranges in index order (eager self-search).  The query records of a
+// self-search are the index's own records, and the entries of the index with
+// one hash (in a batch: one hash in one genome) form a run whose entries
+// after e are the posting range of e's record.  So the ranges come from one
+// walk over the index: a warp reads 32 consecutive entries, splits them into
+// runs, and in a batch searches only for the ends of the run that leaves its
+// 32 entries.  Each range goes to its record, found by the rank of the
 // record's position among all record positions: a bitmap of the positions
 // with the count of set bits before each 32-bit word.
 struct RankWord {
@@ -478,38 +497,45 @@ __global__ void k_qpost_index(FArgs a, int64_t n, const RankWord* __restrict__ r
                               uint2* __restrict__ out) {
   const int lane = lane_id();
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  const bool batch = a.self_mode == 2;
   for (int64_t e0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) & ~(int64_t)31; e0 < n;
        e0 += stride) {
     const int64_t e = e0 + lane;
     const int L = (int)(n - 1 - e0 < 31 ? n - 1 - e0 : 31);  // last lane with an entry
     const bool ok = lane <= L;
-    uint32_t h = 0xFFFFFFFFu, p = 0;
-    int g = -1;
+    uint32_t h = 0xFFFFFFFFu, p = 0, lo = 0, hi = 0;
     if (ok) {
       const uint64_t r = a.tsorted[e];
       h = rec_hash(r);
       p = rec_pos(r);
-      g = seq_of(a.tseq, a.ntseq, (int64_t)p);
+      hi = a.toff[h + 1];
+      if (a.max_occ > 0 || !a.after_own) lo = a.toff[h];
     }
-    const uint32_t ph = __shfl_up_sync(0xffffffffu, h, 1), nh = __shfl_down_sync(0xffffffffu, h, 1);
-    const int pg = __shfl_up_sync(0xffffffffu, g, 1), ng = __shfl_down_sync(0xffffffffu, g, 1);
-    const bool st = ok && (lane == 0 || ph != h || pg != g);
-    const bool en = ok && (lane == L || nh != h || ng != g);
-    const unsigned sb = __ballot_sync(0xffffffffu, st), eb = __ballot_sync(0xffffffffu, en);
-    const int fl = 31 - __clz(sb & ((2u << lane) - 1u));  // first lane of my run
-    const int ll = __ffs(eb & ~((1u << lane) - 1u)) - 1;  // last lane of my run
-    // the run holding the first entry may start before it, the run holding
-    // the last one may end after it
-    uint32_t s0 = 0, eL = 0;
-    if (lane == 0) s0 = pos_lower_bound(a.tsorted, a.toff[h], (uint32_t)e0, a.tseq[g]);
-    if (lane == L) eL = pos_gallop_forward(a.tsorted, (uint32_t)e + 1, a.toff[h + 1], a.tseq[g + 1]);
-    s0 = __shfl_sync(0xffffffffu, s0, 0);
-    eL = __shfl_sync(0xffffffffu, eL, L);
+    // the run of e: from its first entry (lo) to past its last (hi)
+    uint32_t rs = lo, re = hi;
+    if (batch) {
+      const int g = ok ? seq_of(a.tseq, a.ntseq, (int64_t)p) : -1;
+      const uint32_t ph = __shfl_up_sync(0xffffffffu, h, 1), nh = __shfl_down_sync(0xffffffffu, h, 1);
+      const int pg = __shfl_up_sync(0xffffffffu, g, 1), ng = __shfl_down_sync(0xffffffffu, g, 1);
+      const bool st = ok && (lane == 0 || ph != h || pg != g);
+      const bool en = ok && (lane == L || nh != h || ng != g);
+      const unsigned sb = __ballot_sync(0xffffffffu, st), eb = __ballot_sync(0xffffffffu, en);
+      const int fl = 31 - __clz(sb & ((2u << lane) - 1u));  // first lane of my run
+      const int ll = __ffs(eb & ~((1u << lane) - 1u)) - 1;  // last lane of my run
+      // the run holding the first entry may start before it, the run holding
+      // the last one may end after it
+      uint32_t s0 = 0, eL = 0;
+      if (lane == 0 && !a.after_own) s0 = pos_lower_bound(a.tsorted, lo, (uint32_t)e0, a.tseq[g]);
+      if (lane == L) eL = pos_gallop_forward(a.tsorted, (uint32_t)e + 1, hi, a.tseq[g + 1]);
+      s0 = __shfl_sync(0xffffffffu, s0, 0);
+      eL = __shfl_sync(0xffffffffu, eL, L);
+      rs = fl == 0 ? s0 : (uint32_t)(e0 + fl);
+      re = ll == L ? eL : (uint32_t)(e0 + ll + 1);
+    }
     if (ok) {
-      const uint32_t rs = fl == 0 ? s0 : (uint32_t)(e0 + fl);
-      const uint32_t re = ll == L ? eL : (uint32_t)(e0 + ll + 1);
+      if (a.after_own) rs = (uint32_t)e + 1;
       uint2 v = make_uint2(rs, re - rs);
-      if (a.max_occ > 0 && (int)(a.toff[h + 1] - a.toff[h]) > a.max_occ) v = make_uint2(kNone, 0u);
+      if (a.max_occ > 0 && (int)(hi - lo) > a.max_occ) v = make_uint2(kNone, 0u);
       const RankWord q = rw[p >> 5];
       out[q.before + __popc(q.bits & ((1u << (p & 31)) - 1u))] = v;
     }
@@ -565,6 +591,7 @@ __device__ __forceinline__ uint32_t slot_count(const uint32_t* slots, uint32_t s
 // kept hash with a compatible relative strand (self positions skipped).
 template <typename Smem, typename F>
 __device__ __forceinline__ void for_hits(const FArgs& a, const Smem& S, int64_t i, int H, F f) {
+  const uint32_t tlo = first_useful(a, i);
   for (int e = threadIdx.x; e < H; e += blockDim.x) {
     int lo = 0, hi = S.s;  // list with pre[l] <= e < pre[l+1]
     while (hi - lo > 1) {
@@ -573,7 +600,7 @@ __device__ __forceinline__ void for_hits(const FArgs& a, const Smem& S, int64_t 
     }
     const uint64_t r = __ldg(a.tsorted + S.pst[lo] + (uint32_t)(e - (int)S.pre[lo]));
     const uint32_t t = rec_pos(r), st = rec_strand(r);
-    if (a.self_mode && (int64_t)t >= i && (int64_t)t <= i + a.span) continue;
+    if (useless_hit(a, t, (uint32_t)i, tlo)) continue;
     const uint32_t qm = S.dm[lo];
     if ((qm >> st) & 1u) f(t, (uint32_t)lo, 0u);
     if ((qm >> (st ^ 1u)) & 1u) f(t, (uint32_t)lo, 1u);
@@ -783,341 +810,548 @@ __global__ void __launch_bounds__(TPB) k_filter_fast(FArgs a, TierIO io) {
 
 // ------------------------------------------------------------- warp tier --
 //
-// Small windows (at most 128 query records, 4,096 hits, 256 collected hits
-// and 64 dense groups) take the same steps as k_filter_fast with one warp
-// per window and no block barriers: W_Q by insertion into a hash table (no
-// sort), hits found 32 at a time by a shuffle search over the posting prefix
-// sums, (bin, o) counters as the prefilter (a window with no adjacent bin
-// pair reaching m stops there), collected hits sorted per strand, dense
-// groups found by the warp and swept exactly by lane 0.  Windows past any
-// limit go to the next tier.
+// Small windows (at most kWH posting entries and 256 collected hits) by one
+// warp each, no block barriers:
+//   1. every posting of every query record is counted into 8-bit (bin, o)
+//      counters, without building W_Q first: a hash that occurs twice in the
+//      window only counts too much.  The number of distinct hashes is bounded
+//      from below by the bits they set in a 2,048-bit map, and with it m.
+//      When no two adjacent bins reach that m the window is done: most
+//      windows end here;
+//   2. the others build W_Q in a hash table (exact s and m; the table's slot
+//      is a hash's id) and collect the hits of the bins whose pair can pass;
+//   3. the collected hits are sorted by (o, t) in registers, and the runs of
+//      each strand come from its events: the hits of one hash at most span + 1
+//      apart keep it in the target window over one stretch of starts, so only
+//      a stretch's first hit enters and only its last one leaves.  The shared
+//      count after an event is the number of enters up to it less the number
+//      of leaves, found by rank (a binary search) for all events at once;
+//      a run starts where it first reaches m and ends where it falls below.
+// Windows past a limit go to the next tier.
+//
+// Bound by instruction issue and, as a window's path is long and the warps
+// of an SM are all at different places of it, by the instruction cache: sorts
+// unrolled in place, or four chunks of postings in flight, made it slower
+// (13.5 -> 18.8 ms on the batch below), and a separate small kernel for step
+// 1 gained 5% there and lost 16% on an assembly.  The form that built W_Q for
+// every window, looked at the hits before the window too, searched the
+// posting lists per hit and swept groups with one lane took about 4,600
+// instructions a window: 4.7 M windows of a 200-genome batch 21.7 -> 8.2 ms
+// (tier 1 over the windows handed on 3.9 -> 0.5 ms), a 240 Mbp assembly 10.8
+// -> 3.5 ms.
 
-constexpr int kWQ = 128;        // query records
-static_assert(kWQ <= 128, "a lane holds at most four of a window's query records");
-constexpr int kWSlots = 1024;   // (bin, o) 16-bit counters (512 bins)
+constexpr int kWSlots = 4096;   // 8-bit (bin, o) counters
 constexpr int kWL = 256;        // collected hits
-constexpr int kWG = 64;         // dense groups
-constexpr int kWH = 4096;       // enumerated hits
-constexpr int kWWarps = 8;
-constexpr int kWTab = 2 * kWL;   // W_Q hash-table slots (u32, over the hit buffer)
-static_assert(kWTab >= 2 * kWQ && kWTab <= kWSlots / 2, "the W_Q table and its masks must fit");
+constexpr int kWH = 2048;       // posting entries (a counter per two of them)
+constexpr int kWWarps = 4;
 
-struct WarpSmem {
-  uint32_t qkey[kWQ];
-  uint32_t pst[kWQ];
-  uint32_t plen[kWQ];
-  uint32_t pre[kWQ + 1];
-  uint8_t dm[kWQ];
-  uint32_t slots[kWSlots / 2];
-  unsigned long long hits[kWL];
-  uint32_t glo[kWG];
-  uint32_t ghi[kWG];
-  uint16_t cnt[kWQ];
-  int nhit;
+// QC: query records a window may have.
+template <int QC>
+struct WarpSmemT {
+  uint32_t table[kWSlots / 4];   // counters; then a strand's events
+  uint2 lists[QC];               // posting lists; then per-hash and per-run places
+  unsigned long long hits[kWL];  // W_Q's hash table; then the collected hits
+  uint32_t starts[kWH / 32];     // map of hashes; then bit e: a list starts at hit e
+  uint32_t strands[2 * QC / 16]; // W_Q's strands, two bits per table slot
+};
+static_assert(kWH / 32 == 64, "the map of hashes lies over the list starts");
+
+// Sorts n 64-bit keys in shared memory (n <= 32 * NR) through registers.
+// The stages are loops and not unrolled: the kernel around it is bound by its
+// instruction cache when they are.
+template <int NR>
+__device__ __noinline__ void warp_sort_hits(unsigned long long* v, int n) {
+  const int lane = lane_id();
+  unsigned long long r[NR];
+#pragma unroll
+  for (int x = 0; x < NR; ++x) {
+    const int at = x * 32 + lane;
+    r[x] = at < n ? v[at] : ~0ull;
+  }
+#pragma unroll 1
+  for (int size = 2; size <= 32 * NR; size <<= 1) {
+#pragma unroll 1
+    for (int stride = size >> 1; stride >= NR; stride >>= 1) {
+      const bool keep_min = (((lane * NR) & size) == 0) == ((lane & (stride / NR)) == 0);
+#pragma unroll
+      for (int x = 0; x < NR; ++x) {
+        const unsigned long long o = __shfl_xor_sync(0xffffffffu, r[x], stride / NR);
+        if ((o < r[x]) == keep_min) r[x] = o;
+      }
+    }
+#pragma unroll
+    for (int stride = NR / 2; stride > 0; stride >>= 1) {
+      if (stride >= size) continue;
+#pragma unroll
+      for (int x = 0; x < NR; ++x) {
+        if (x & stride) continue;
+        const bool asc = ((lane * NR + x) & size) == 0;
+        const unsigned long long p = r[x], q = r[x | stride];
+        if ((p > q) == asc) {
+          r[x] = q;
+          r[x | stride] = p;
+        }
+      }
+    }
+  }
+  __syncwarp();
+#pragma unroll
+  for (int x = 0; x < NR; ++x) v[lane * NR + x] = r[x];
+  __syncwarp();
+}
+
+// First place in v[0..n) whose value is >= x.
+__device__ __forceinline__ int lb_u32(const uint32_t* v, int n, uint32_t x) {
+  int lo = 0, hi = n;
+  while (lo < hi) {
+    const int mid = (lo + hi) >> 1;
+    if (v[mid] < x) lo = mid + 1; else hi = mid;
+  }
+  return lo;
+}
+
+// hits: o << 63 | t << 20 | hid, with these flags once a strand's stretches are known
+constexpr unsigned long long kHitNoEnter = 1ull << 52, kHitNoLeave = 1ull << 53;
+__device__ __forceinline__ uint32_t hit_pos(unsigned long long h) { return (uint32_t)(h >> 20); }
+
+// Where a strand's events go (shared memory of one warp).
+struct EventMem {
+  uint32_t* enter;   // sorted target positions; a window [j, j + span] holds them from j + span on
+  uint32_t* leave;   // first j + span past the stretch
+  uint16_t* val;     // shared count at each enter
+  uint32_t* end;     // per run: its last j + span
+  uint16_t* first;   // per run: the enter that starts it
+  uint16_t* last;    // per hash id: its last hit
+  int nlast;         // hash ids
 };
 
-template <typename T>
-__device__ void warp_sort(T* v, int n) {  // n a power of two
+// The runs of one strand from its n collected hits, sorted by t (n <= 256).
+// The whole warp calls.
+__device__ __noinline__ void strand_runs(const FArgs& a, const WinInfo& w, unsigned long long* hits, int n,
+                            const EventMem& M) {
   const int lane = lane_id();
-  for (int size = 2; size <= n; size <<= 1)
-    for (int stride = size >> 1; stride > 0; stride >>= 1) {
-      for (int t = lane; t < (n >> 1); t += 32) {
-        const int lo = ((t & ~(stride - 1)) << 1) | (t & (stride - 1));
-        const int hi = lo + stride;
-        const bool asc = (lo & size) == 0;
-        const T x = v[lo], y = v[hi];
-        if ((x > y) == asc) {
-          v[lo] = y;
-          v[hi] = x;
+  const uint32_t span = (uint32_t)a.span;
+  for (int x = lane; x < M.nlast / 2; x += 32) reinterpret_cast<uint32_t*>(M.last)[x] = 0xFFFFFFFFu;
+  __syncwarp();
+  // stretches: a hit joined to the previous one of its hash does not enter,
+  // and that one does not leave
+  for (int base = 0; base < n; base += 32) {
+    const int x = base + lane;
+    const bool ok = x < n;
+    const unsigned long long h = ok ? hits[x] : 0ull;
+    const uint32_t t = hit_pos(h), id = (uint32_t)h & 0xFFFFFu;
+    const unsigned peers = __match_any_sync(0xffffffffu, ok ? id : (0x80000000u | (uint32_t)lane));
+    const unsigned lower = peers & lanemask_lt();
+    int p = -1;
+    if (ok) {
+      if (lower) p = base + 31 - __clz(lower);
+      else if (M.last[id] != 0xFFFFu) p = M.last[id];
+    }
+    const bool joined = p >= 0 && t - hit_pos(hits[p]) <= span + 1u;
+    __syncwarp();
+    if (joined) {
+      atomicOr(reinterpret_cast<unsigned int*>(hits + x) + 1, (unsigned int)(kHitNoEnter >> 32));
+      atomicOr(reinterpret_cast<unsigned int*>(hits + p) + 1, (unsigned int)(kHitNoLeave >> 32));
+    }
+    if (ok && (peers >> lane) == 1u) M.last[id] = (uint16_t)x;
+    __syncwarp();
+  }
+  int ne = 0, nl = 0;
+  for (int base = 0; base < n; base += 32) {
+    const int x = base + lane;
+    const unsigned long long h = x < n ? hits[x] : (kHitNoEnter | kHitNoLeave);
+    const uint32_t t = hit_pos(h);
+    const unsigned be = __ballot_sync(0xffffffffu, !(h & kHitNoEnter));
+    const unsigned bl = __ballot_sync(0xffffffffu, !(h & kHitNoLeave));
+    if (!(h & kHitNoEnter)) M.enter[ne + __popc(be & lanemask_lt())] = t;
+    // t + 1 + span, short of wrapping (no window starts that far)
+    if (!(h & kHitNoLeave))
+      M.leave[nl + __popc(bl & lanemask_lt())] = t < 0xFFFFFFFFu - span - 1u ? t + span + 1u : 0xFFFFFFFFu;
+    ne += __popc(be);
+    nl += __popc(bl);
+  }
+  __syncwarp();
+  const int m = w.m;
+  int nr = 0, nend = 0;
+  for (int base = 0; base < ne; base += 32) {
+    const int x = base + lane;
+    bool start = false;
+    if (x < ne) {
+      const uint32_t j = M.enter[x];
+      const int before = lb_u32(M.leave, nl, j);             // leaves before j
+      const int upto = before + (before < nl && M.leave[before] == j ? 1 : 0);
+      const int v = x + 1 - upto;
+      M.val[x] = (uint16_t)v;
+      start = v >= m && x - before < m;
+    }
+    const unsigned b = __ballot_sync(0xffffffffu, start);
+    if (start) M.first[nr + __popc(b & lanemask_lt())] = (uint16_t)x;
+    nr += __popc(b);
+  }
+  if (nr == 0) return;
+  for (int base = 0; base < nl; base += 32) {
+    const int x = base + lane;
+    bool stop = false;
+    uint32_t j = 0;
+    if (x < nl) {
+      j = M.leave[x];
+      const int before = lb_u32(M.enter, ne, j);
+      const int upto = before + (before < ne && M.enter[before] == j ? 1 : 0);
+      stop = upto - (x + 1) < m && before - x >= m;
+    }
+    const unsigned b = __ballot_sync(0xffffffffu, stop);
+    if (stop) M.end[nend + __popc(b & lanemask_lt())] = j - 1u;
+    nend += __popc(b);
+  }
+  __syncwarp();
+  // every run starts and ends once, in order; split it by target sequence
+  // and the validity rules.  Many runs: one per lane; few: the warp takes
+  // them in turn and shares their enters out.
+  const bool by_lane = nr >= 8;
+  for (int r = by_lane ? lane : 0; r < nr; r += by_lane ? 32 : 1) {
+    const int64_t lo = (int64_t)M.enter[M.first[r]] - span, hi = (int64_t)M.end[r] - span;
+    int64_t x = lo < 0 ? 0 : lo;
+    for (int u = seq_of(a.tseq, a.ntseq, x); u < a.ntseq && x <= hi; ++u) {
+      const int64_t st = a.tseq[u], en = a.tseq[u + 1];
+      bool ok = true;
+      int64_t from = st;
+      if (a.self_mode) {
+        if (u < w.qseq) ok = false;
+        else if (u == w.qseq) from = max(from, w.i + a.n - a.overlap);
+        else if (a.self_mode == 2) ok = false;  // independent genomes
+      }
+      const int64_t vlo = max(x, from), vhi = min(hi, en - a.n);
+      x = en;
+      if (!ok || vlo > vhi) continue;
+      // the largest count on [vlo, vhi]: at vlo, or at an enter after it
+      const uint32_t j0 = (uint32_t)(vlo + span), j1 = (uint32_t)(vhi + span);
+      int e = lb_u32(M.enter, ne, j0);
+      e += e < ne && M.enter[e] == j0 ? 1 : 0;
+      int l = lb_u32(M.leave, nl, j0);
+      l += l < nl && M.leave[l] == j0 ? 1 : 0;
+      uint32_t best = 0;  // count, then the earliest
+      for (int y = by_lane ? e : e + lane; y < ne && M.enter[y] <= j1; y += by_lane ? 1 : 32)
+        best = max(best, ((uint32_t)M.val[y] << 16) | (uint32_t)(0xFFFF - y));
+      if (!by_lane) best = __reduce_max_sync(0xffffffffu, best);
+      RunState run;
+      run.open = true;
+      run.ja = vlo;
+      run.jb = vhi;
+      run.mx = e - l;
+      run.jmx = vlo;
+      if ((int)(best >> 16) > run.mx) {
+        run.mx = (int)(best >> 16);
+        run.jmx = (int64_t)M.enter[0xFFFF - (best & 0xFFFFu)] - span;
+      }
+      if (by_lane || lane == 0) emit_run(a, w, run);
+    }
+  }
+}
+
+// posting_window by value (out of line, see warp_sort_hits).
+__device__ __noinline__ uint2 posting_window_of(const uint64_t* idx, const uint32_t* samp, uint32_t st,
+                                                uint32_t len, int64_t lo, int64_t hi) {
+  posting_window(idx, samp, &st, &len, lo, hi);
+  return make_uint2(st, len);
+}
+
+template <int QC>
+__global__ void __launch_bounds__(32 * kWWarps, QC == 128 ? 7 : 5) k_filter_warp(FArgs a, TierIO io,
+                                                                                int per_grab) {
+  constexpr int NC = QC / 32;    // records per lane
+  constexpr int TS = 2 * QC;     // W_Q table slots
+  static_assert(TS * 4 <= kWL * 8, "W_Q's table lies over the hits");
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int warp = threadIdx.x >> 5, lane = lane_id();
+  WarpSmemT<QC>& S = reinterpret_cast<WarpSmemT<QC>*>(smem_raw)[warp];
+  const uint32_t lt = lanemask_lt();
+  const int64_t count = io.in_list ? (int64_t)*io.in_count : a.nwin;
+  unsigned long long n_hits = 0, n_collected = 0;
+  while (true) {
+    // several windows at a time: they share query records, and the work
+    // counter is one word for the whole grid
+    int64_t k0 = 0;
+    if (lane == 0) k0 = (int64_t)atomicAdd(io.next, (unsigned int)per_grab);
+    k0 = __shfl_sync(0xffffffffu, k0, 0);
+    if (k0 >= count) break;
+    const int nk = (int)min((int64_t)per_grab, count - k0);
+    uint32_t l_w = 0, l_i = 0, l_qa = 0, l_qb = 0;
+    if (lane < nk) {
+      l_w = io.in_list ? io.in_list[k0 + lane] : (uint32_t)(k0 + lane);
+      l_i = a.win_i[l_w];
+      l_qa = a.win_qa[l_w];
+      l_qb = a.win_qb[l_w];
+    }
+    for (int kk = 0; kk < nk; ++kk) {
+      const uint32_t wdx = __shfl_sync(0xffffffffu, l_w, kk), i = __shfl_sync(0xffffffffu, l_i, kk);
+      const uint32_t qa = __shfl_sync(0xffffffffu, l_qa, kk);
+      const int c = (int)(__shfl_sync(0xffffffffu, l_qb, kk) - qa);
+      if (c == 0) continue;
+      auto hand_over = [&](bool wide) {
+        if (lane != 0) return;
+        if (wide && io.wide_list) io.wide_list[atomicAdd(io.wide_count, 1u)] = wdx;
+        else io.out_list[atomicAdd(io.out_count, 1u)] = wdx;
+      };
+      if (c > QC) {
+        hand_over(false);
+        continue;
+      }
+      __syncwarp();  // the previous window's shared memory is free
+      S.starts[lane] = 0u;
+      S.starts[lane + 32] = 0u;
+      __syncwarp();
+      // ---- the records: hash and strand, posting range
+      uint32_t key[NC], st[NC], len[NC];
+      unsigned kept = 0;
+#pragma unroll
+      for (int ch = 0; ch < NC; ++ch) {
+        const int x = ch * 32 + lane;
+        key[ch] = st[ch] = len[ch] = 0;
+        if (x < c) {
+          const uint64_t r = __ldg(a.qrec + qa + x);
+          const uint32_t h = rec_hash(r);
+          key[ch] = (h << 1) | rec_strand(r);
+          if (a.qpost) {
+            const uint2 pp = __ldg(a.qpost + qa + x);
+            st[ch] = pp.x;
+            len[ch] = pp.y;
+            if (pp.x != kNone) kept |= 1u << ch;
+          } else {
+            st[ch] = a.toff[h];
+            len[ch] = a.toff[h + 1] - st[ch];
+            if (!(a.max_occ > 0 && (int)len[ch] > a.max_occ)) {
+              kept |= 1u << ch;
+              if (a.self_mode == 2) {
+                const int sq = a.win_seq[wdx];
+                const uint2 pw = posting_window_of(a.tsorted, a.tsamp, st[ch], len[ch], a.tseq[sq], a.tseq[sq + 1]);
+                st[ch] = pw.x;
+                len[ch] = pw.y;
+              }
+            }
+          }
+          if ((kept >> ch) & 1u) {
+            const uint32_t g = (h * 0x9E3779B1u) >> 21;
+            atomicOr(&S.starts[g >> 5], 1u << (g & 31));
+          } else {
+            len[ch] = 0;
+          }
         }
       }
       __syncwarp();
-    }
-}
-
-__device__ __forceinline__ uint32_t wslot_of(uint32_t t, uint32_t o) {
-  return (((t >> kBinShift) << 1) | o) & (kWSlots - 1);
-}
-
-__global__ void __launch_bounds__(32 * kWWarps) k_filter_warp(FArgs a, TierIO io) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int warp = threadIdx.x >> 5, lane = lane_id();
-  WarpSmem& S = reinterpret_cast<WarpSmem*>(smem_raw)[warp];
-  for (int x = lane; x < kWQ; x += 32) S.cnt[x] = 0;
-  const int64_t count = io.in_list ? (int64_t)*io.in_count : a.nwin;
-  auto hand_over = [&](int64_t wdx) {
-    if (lane == 0) io.out_list[atomicAdd(io.out_count, 1u)] = (uint32_t)wdx;
-  };
-  while (true) {
-    int64_t k = 0;
-    if (lane == 0) k = (int64_t)atomicAdd(io.next, 1u);
-    k = __shfl_sync(0xffffffffu, k, 0);
-    if (k >= count) break;
-    const int64_t wdx = io.in_list ? (int64_t)io.in_list[k] : k;
-    const int64_t i = a.win_i[wdx];
-    const uint32_t qa = a.win_qa[wdx], qb = a.win_qb[wdx];
-    const int c = (int)(qb - qa);
-    if (c == 0) continue;
-    if (c > kWQ) {
-      hand_over(wdx);
-      continue;
-    }
-    // W_Q: the window's distinct hashes, by insertion into an open-addressing
-    // table (key hash + 1, linear probing from the hash's low bits) laid
-    // over the hit buffer, with each hash's strand mask beside it in the
-    // counter table (both are rebuilt later for the hits).  The order of W_Q
-    // plays no part in the counts, so no sort is needed.  A record that
-    // inserts its hash first owns it.
-    uint32_t* tab = reinterpret_cast<uint32_t*>(S.hits);
-    uint32_t* tmask = S.slots;
-    for (int x = lane; x < kWTab; x += 32) {
-      tab[x] = 0u;
-      tmask[x] = 0u;
-    }
-    __syncwarp();
-    const bool packed = a.qpost != nullptr;
-    uint32_t own_slot[kWQ / 32], own_h[kWQ / 32];
-    unsigned owner = 0;
+      const int s_least = (int)__reduce_add_sync(0xffffffffu, __popc(S.starts[lane]) + __popc(S.starts[lane + 32]));
+      if (s_least == 0) continue;  // every hash passes max_occ
+      // ---- posting lists with an entry, one after another
+      uint32_t H = 0;
+      uint32_t at[NC];
 #pragma unroll
-    for (int ch = 0; ch < kWQ / 32; ++ch) {
-      const int x = ch * 32 + lane;
-      own_slot[ch] = 0;
-      own_h[ch] = 0;
-      if (x < c) {
-        const uint64_t r = __ldg(a.qrec + qa + x);
-        const uint32_t h = rec_hash(r);
-        uint32_t slot = h & (kWTab - 1);
-        while (true) {  // at most kWQ keys in kWTab slots: a free slot is always found
-          const uint32_t old = atomicCAS(&tab[slot], 0u, h + 1u);
-          if (old == 0u) {
-            owner |= 1u << ch;
-            break;
-          }
-          if (old == h + 1u) break;
-          slot = (slot + 1u) & (kWTab - 1);
-        }
-        atomicOr(&tmask[slot], 1u << rec_strand(r));
-        own_slot[ch] = slot;
-        own_h[ch] = h;
+      for (int ch = 0; ch < NC; ++ch) {
+        at[ch] = 0;
+        if (ch * 32 >= c) break;
+        const uint32_t v = min(len[ch], 1u << 20);  // no sum can wrap
+        const uint32_t inc = warp_inclusive_sum(v);
+        at[ch] = H + inc - v;
+        H += __shfl_sync(0xffffffffu, inc, 31);
       }
-    }
-    int64_t seq_lo = 0, seq_hi = 0;
-    if (a.self_mode == 2) {
-      const int sq = a.win_seq[wdx];
-      seq_lo = a.tseq[sq];
-      seq_hi = a.tseq[sq + 1];
-    }
-    __syncwarp();
-    int s = 0;
-#pragma unroll
-    for (int ch = 0; ch < kWQ / 32; ++ch) {
-      if (ch * 32 >= c) break;
-      const int x = ch * 32 + lane;
-      bool keep = false;
-      uint32_t st = 0, len = 0, mask = 0;
-      if ((owner >> ch) & 1u) {
-        const uint32_t h = own_h[ch];
-        mask = tmask[own_slot[ch]];
-        if (packed) {
-          const uint2 pp = a.qpost[qa + x];
-          st = pp.x;
-          len = pp.y;
-          keep = pp.x != kNone;
-        } else {
-          st = a.toff[h];
-          len = a.toff[h + 1] - st;
-          keep = !(a.max_occ > 0 && (int)len > a.max_occ);
-          if (keep && a.self_mode == 2) posting_window(a.tsorted, a.tsamp, &st, &len, seq_lo, seq_hi);
-        }
-      }
-      const unsigned km = __ballot_sync(0xffffffffu, keep);
-      if (keep) {
-        const int d = s + __popc(km & lanemask_lt());
-        S.pst[d] = st;
-        S.plen[d] = len;
-        S.dm[d] = (uint8_t)mask;
-      }
-      s += __popc(km);
-    }
-    __syncwarp();
-    if (s == 0) continue;
-    // prefix sums of the posting lengths
-    uint32_t run = 0;
-    for (int base = 0; base < s; base += 32) {
-      const int x = base + lane;
-      const uint32_t v = x < s ? S.plen[x] : 0u;
-      const uint32_t inc = warp_inclusive_sum(v);
-      if (x < s) S.pre[x] = run + inc - v;
-      run += __shfl_sync(0xffffffffu, inc, 31);
-    }
-    if (lane == 0) S.pre[s] = run;
-    const uint32_t H = run;
-    if (H == 0) continue;
-    if (H > (uint32_t)kWH) {
-      hand_over(wdx);
-      continue;
-    }
-    const int m = a.mtab[s];
-    for (int x = lane; x < kWSlots / 2; x += 32) S.slots[x] = 0;
-    if (lane == 0) S.nhit = 0;
-    __syncwarp();
-    // Hits in chunks of 32 consecutive ones.  The list holding hit e is the
-    // last x with pre[x] <= e: for the chunk at base it is cur (the list
-    // holding the previous chunk's last hit) plus the number of lists after
-    // cur that start at or before e, found by a 5-step search over the next
-    // 32 lists' starts (pre is nondecreasing) instead of a search per hit.
-    auto each_hit = [&](auto f) {
-      int cur = 0;
-      for (int base = 0; base < (int)H; base += 32) {
-        const int e = base + lane;
-        int lo = cur;
-        for (int from = cur + 1;; from += 32) {
-          const int x = from + lane;
-          const int d = x < s ? (int)S.pre[x] - base : INT_MAX;
-          int n = 0;  // lists among from .. from + 30 starting at or before e
-#pragma unroll
-          for (int step = 16; step > 0; step >>= 1) {
-            const int v = __shfl_sync(0xffffffffu, d, n + step - 1);
-            if (v <= lane) n += step;
-          }
-          const int d31 = __shfl_sync(0xffffffffu, d, 31);
-          if (d31 <= lane) n = 32;
-          if (n > 0) lo = from + n - 1;
-          if (d31 > 31) break;  // no list past these starts inside the chunk
-        }
-        cur = __shfl_sync(0xffffffffu, lo, 31);
-        if (e >= (int)H) continue;
-        const uint64_t r = __ldg(a.tsorted + S.pst[lo] + (uint32_t)(e - (int)S.pre[lo]));
-        const uint32_t t = rec_pos(r), st = rec_strand(r);
-        if (a.self_mode && (int64_t)t >= i && (int64_t)t <= i + a.span) continue;
-        const uint32_t qm = S.dm[lo];
-        if ((qm >> st) & 1u) f(t, (uint32_t)lo, 0u);
-        if ((qm >> (st ^ 1u)) & 1u) f(t, (uint32_t)lo, 1u);
-      }
-    };
-    each_hit([&](uint32_t t, uint32_t, uint32_t o) {
-      const uint32_t sl = wslot_of(t, o);
-      atomicAdd(&S.slots[sl >> 1], 1u << ((sl & 1) * 16));
-    });
-    __syncwarp();
-    // A hit is collected only when its bin's counter and a neighbouring
-    // bin's (same strand) sum to m or more.  Word x of the table holds bin x
-    // (both strands), so when no two cyclically adjacent words reach m on
-    // either strand, nothing would be collected: the window ends here.
-    {
-      bool pass = false;
-      for (int x = lane; x < kWSlots / 2; x += 32) {
-        const uint32_t c = S.slots[x], d = S.slots[(x + 1) & (kWSlots / 2 - 1)];
-        pass |= (c & 0xFFFFu) + (d & 0xFFFFu) >= (uint32_t)m || (c >> 16) + (d >> 16) >= (uint32_t)m;
-      }
-      if (!__any_sync(0xffffffffu, pass)) {
-        if (io.stats && lane == 0) atomicAdd(a.stats + 0, (unsigned long long)H);
+      if (H == 0) continue;
+      if (H > io.hlim || H > (uint32_t)kWH) {
+        hand_over(true);
         continue;
       }
-    }
-    each_hit([&](uint32_t t, uint32_t hid, uint32_t o) {
-      const uint32_t b = t >> kBinShift;
-      const uint32_t c0 = slot_count(S.slots, wslot_of(t, o));
-      const uint32_t cn = slot_count(S.slots, (((b + 1) << 1) | o) & (kWSlots - 1));
-      bool need = c0 + cn >= (uint32_t)m;
-      if (!need && b > 0) {
-        const uint32_t cp = slot_count(S.slots, (((b - 1) << 1) | o) & (kWSlots - 1));
-        need = cp + c0 >= (uint32_t)m;
+      __syncwarp();
+      S.starts[lane] = 0u;
+      S.starts[lane + 32] = 0u;
+      uint32_t nslots = 512;
+      while (nslots < 4u * H && nslots < (uint32_t)kWSlots) nslots <<= 1;
+      const uint32_t smask = nslots - 1;
+      for (int x = lane; x < (int)nslots / 16; x += 32)
+        reinterpret_cast<uint4*>(S.table)[x] = make_uint4(0, 0, 0, 0);
+      __syncwarp();
+      int nlist = 0;
+      uint32_t lid[NC];
+#pragma unroll
+      for (int ch = 0; ch < NC; ++ch) {
+        lid[ch] = 0;
+        if (ch * 32 >= c) break;
+        const unsigned some = __ballot_sync(0xffffffffu, len[ch] > 0);
+        if (len[ch] > 0) {
+          lid[ch] = nlist + __popc(some & lt);
+          S.lists[lid[ch]] = make_uint2(st[ch] - at[ch], key[ch] & 1u);
+          atomicOr(&S.starts[at[ch] >> 5], 1u << (at[ch] & 31));
+        }
+        nlist += __popc(some);
       }
-      if (need) {
-        const int at = atomicAdd(&S.nhit, 1);
-        if (at < kWL)
-          S.hits[at] = ((unsigned long long)o << 63) | ((unsigned long long)t << 20) | hid;
+      __syncwarp();
+      // hit e lies in the last list that starts at or before it; f is called
+      // by every lane (on: the lane has a hit that a target window can use)
+      const uint32_t tlo = first_useful(a, i);
+      auto each_hit = [&](auto f) {
+        int lists_before = -1;
+        for (uint32_t base = 0; base < H; base += 32) {
+          const unsigned sb = S.starts[base >> 5];
+          const int li = lists_before + __popc(sb & (lt | (1u << lane)));
+          lists_before += __popc(sb);
+          bool on = base + lane < H;
+          uint32_t t = 0, o = 0, y = 0;
+          if (on) {
+            const uint2 list = S.lists[li];
+            const uint64_t r = __ldg(a.tsorted + (list.x + base + lane));
+            t = rec_pos(r);
+            y = list.y;
+            o = (y ^ rec_strand(r)) & 1u;
+            on = !useless_hit(a, t, i, tlo);
+          }
+          f(on, t, o, y);
+        }
+      };
+      uint32_t most = 0;  // the largest counter
+      each_hit([&](bool on, uint32_t t, uint32_t o, uint32_t) {
+        if (!on) return;
+        const uint32_t sl = slot_of(t, o, smask), sh = (sl & 3u) * 8u;
+        const uint32_t was = (atomicAdd(&S.table[sl >> 2], 1u << sh) >> sh) & 0xFFu;
+        most = max(most, was + 1u);
+      });
+      most = __reduce_max_sync(0xffffffffu, most);
+      if (most > 255u) {  // a counter ran into its neighbour
+        hand_over(false);
+        continue;
       }
-    });
-    __syncwarp();
-    const int L = S.nhit;
-    if (L > kWL) {
-      hand_over(wdx);
-      continue;
-    }
-    if (L < m) {
-      if (io.stats && lane == 0) {
-        atomicAdd(a.stats + 0, (unsigned long long)H);
-        atomicAdd(a.stats + 1, (unsigned long long)L);
+      __syncwarp();
+      {
+        const uint32_t m = (uint32_t)a.mtab[s_least];
+        bool pass = 2u * most >= m;
+        if (pass) {
+          // word x: bins 2x and 2x + 1, both strands; the bins wrap around
+          pass = false;
+          const int nw = (int)nslots / 4;
+          for (int x = lane; x < nw; x += 32) {
+            const uint32_t c0 = S.table[x], c1 = S.table[(x + 1) & (nw - 1)];
+            const uint32_t even = c0 & 0x00FF00FFu, odd = (c0 >> 8) & 0x00FF00FFu;  // strands 0, 1
+            const uint32_t enext = c1 & 0x00FF00FFu, onext = (c1 >> 8) & 0x00FF00FFu;
+            pass |= (even & 0xFFFFu) + (even >> 16) >= m || (odd & 0xFFFFu) + (odd >> 16) >= m ||
+                    (even >> 16) + (enext & 0xFFFFu) >= m || (odd >> 16) + (onext & 0xFFFFu) >= m;
+          }
+        }
+        if (!__any_sync(0xffffffffu, pass)) {
+          n_hits += H;
+          continue;
+        }
       }
-      continue;
-    }
-    const int nh = next_pow2(L < 2 ? 2 : L);
-    for (int x = L + lane; x < nh; x += 32) S.hits[x] = ~0ull;
-    __syncwarp();
-    warp_sort(S.hits, nh);
-    int split;
-    {
-      int lo2 = 0, hi2 = L;  // first hit with o = 1
-      while (lo2 < hi2) {
-        const int mid = (lo2 + hi2) >> 1;
-        if ((S.hits[mid] >> 63) == 0) lo2 = mid + 1; else hi2 = mid;
+      // ---- W_Q: a hash's id is its slot; a record whose hash and strand are
+      // in already adds nothing
+      uint32_t* tab = reinterpret_cast<uint32_t*>(S.hits);
+      for (int x = lane; x < TS / 4; x += 32) reinterpret_cast<uint4*>(tab)[x] = make_uint4(0, 0, 0, 0);
+      if (lane < TS / 16) S.strands[lane] = 0u;
+      __syncwarp();
+      int fresh = 0;
+#pragma unroll
+      for (int ch = 0; ch < NC; ++ch) {
+        if ((kept >> ch) & 1u) {
+          const uint32_t h = key[ch] >> 1;
+          uint32_t slot = (h * 0x9E3779B1u) >> (QC == 128 ? 24 : 23);
+          while (true) {  // at most QC keys in TS slots: a free slot is always found
+            const uint32_t old = atomicCAS(&tab[slot], 0u, h + 1u);
+            if (old == 0u) ++fresh;
+            if (old == 0u || old == h + 1u) break;
+            slot = (slot + 1u) & (uint32_t)(TS - 1);
+          }
+          const uint32_t bit = 1u << ((slot & 15) * 2 + (key[ch] & 1u));
+          const bool twice = (atomicOr(&S.strands[slot >> 4], bit) & bit) != 0u;
+          if (len[ch] > 0) S.lists[lid[ch]].y = (key[ch] & 1u) | (twice ? 2u : 0u) | (slot << 2);
+        }
       }
-      split = lo2;
-    }
-    int ng = 0, ng0 = 0;
-    for (int o = 0; o < 2; ++o) {
-      const unsigned long long* base = S.hits + (o ? split : 0);
-      const int64_t cnt = o ? L - split : split;
-      find_groups(
-          [&](int64_t x) {
-            const unsigned long long h = base[x];
-            return make_uint2((uint32_t)(h >> 20), (uint32_t)(h & 0xFFFFFu));
-          },
-          cnt, m, a.span, [&](int64_t lo, int64_t hi) {
-            if (lane == 0 && ng < kWG) {
-              S.glo[ng] = (uint32_t)(lo < 0 ? 0 : lo);
-              S.ghi[ng] = (uint32_t)hi;
-            }
-            ++ng;
-          });
-      if (o == 0) ng0 = ng;
-    }
-    __syncwarp();
-    if (ng > kWG) {
-      hand_over(wdx);
-      continue;
-    }
-    if (io.stats && lane == 0) {
-      atomicAdd(a.stats + 0, (unsigned long long)H);
-      atomicAdd(a.stats + 1, (unsigned long long)L);
-    }
-    if (lane == 0) {
+      const int s = (int)__reduce_add_sync(0xffffffffu, fresh);
+      const int m = a.mtab[s];
+      __syncwarp();
+      int L = 0;
+      each_hit([&](bool on, uint32_t t, uint32_t o, uint32_t y) {
+        bool need = false;
+        if (on && !(y & 2u)) {
+          const uint32_t b = t >> kBinShift;
+          auto cnt = [&](uint32_t bin) {
+            const uint32_t sl = ((bin << 1) | o) & smask;
+            return (S.table[sl >> 2] >> ((sl & 3u) * 8u)) & 0xFFu;
+          };
+          const uint32_t c0 = cnt(b);
+          need = c0 + cnt(b + 1) >= (uint32_t)m || (b > 0 && c0 + cnt(b - 1) >= (uint32_t)m);
+        }
+        const unsigned bn = __ballot_sync(0xffffffffu, need);
+        const int to = L + __popc(bn & lt);
+        if (need && to < kWL)
+          S.hits[to] = ((unsigned long long)o << 63) | ((unsigned long long)t << 20) | (y >> 2);
+        L += __popc(bn);
+      });
+      __syncwarp();
+      if (L > kWL) {
+        hand_over(false);
+        continue;
+      }
+      n_hits += H;
+      n_collected += L;
+      if (L < m) continue;
+      if (L <= 128) warp_sort_hits<4>(S.hits, L);
+      else warp_sort_hits<8>(S.hits, L);
+      int split = 0;  // first hit with o = 1
+      for (int base = 0; base < L; base += 32)
+        split += __popc(__ballot_sync(0xffffffffu, base + lane < L && (S.hits[base + lane] >> 63) == 0));
+      EventMem M;
+      M.enter = S.table;
+      M.leave = S.table + kWL;
+      M.end = S.table + 2 * kWL;
+      M.val = reinterpret_cast<uint16_t*>(S.table + 3 * kWL);
+      M.last = reinterpret_cast<uint16_t*>(S.lists);
+      M.nlast = TS;
+      M.first = M.last + TS;
+      static_assert(kWSlots / 4 >= 3 * kWL + kWL / 2 && sizeof(S.lists) >= (TS + kWL) * 2,
+                    "a strand's events lie over the counters and the lists");
       WinInfo w;
       w.i = i;
       w.qseq = a.win_seq[wdx];
       w.s = s;
       w.m = m;
-      for (int g = 0; g < ng; ++g) {
-        w.o = g < ng0 ? 0 : 1;
-        const unsigned long long* base = S.hits + (w.o ? split : 0);
-        const int64_t cnt = w.o ? L - split : split;
-        sweep_group(a, w,
-                    [&](int64_t x) {
-                      const unsigned long long h = base[x];
-                      return make_uint2((uint32_t)(h >> 20), (uint32_t)(h & 0xFFFFFu));
-                    },
-                    cnt, S.cnt, (int64_t)S.glo[g], (int64_t)S.ghi[g]);
+#pragma unroll 1
+      for (int o = 0; o < 2; ++o) {
+        const int n = o ? L - split : split;
+        if (n < m) continue;
+        w.o = o;
+        strand_runs(a, w, S.hits + (o ? split : 0), n, M);
+        __syncwarp();
       }
     }
-    __syncwarp();
+  }
+  if (io.stats && lane == 0) {
+    if (n_hits) atomicAdd(a.stats + 0, n_hits);
+    if (n_collected) atomicAdd(a.stats + 1, n_collected);
   }
 }
 
-int launch_warp_tier(sedef_ctx* ctx, const FArgs& a, const TierIO& io, int64_t max_windows,
-                     const char* name) {
-  const size_t sm = sizeof(WarpSmem) * kWWarps;
-  SEDEF_TRY(ensure_smem_attr((const void*)k_filter_warp, sm));
+template <int QC>
+int launch_warp_tier_as(sedef_ctx* ctx, const FArgs& a, const TierIO& io, int64_t max_windows,
+                        const char* name) {
+  const size_t sm = sizeof(WarpSmemT<QC>) * kWWarps;
+  SEDEF_TRY(ensure_smem_attr((const void*)k_filter_warp<QC>, sm));
   int per_sm = 0;
-  SEDEF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_filter_warp, 32 * kWWarps, sm));
+  SEDEF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_filter_warp<QC>, 32 * kWWarps, sm));
   if (per_sm < 1) per_sm = 1;
   int64_t grid = (int64_t)ctx_sm_count(ctx) * per_sm;
+  // a few windows: one per warp; many: eight at a time
+  int64_t grab = max_windows / (grid * kWWarps * 4);
+  grab = grab < 1 ? 1 : (grab > 8 ? 8 : grab);
   const int64_t need = (max_windows + kWWarps - 1) / kWWarps;
   if (grid > need) grid = need;
   if (grid < 1) grid = 1;
-  SEDEF_KERNEL(ctx, name, k_filter_warp<<<(int)grid, 32 * kWWarps, sm, ctx_stream(ctx)>>>(a, io));
+  SEDEF_KERNEL(ctx, name,
+               k_filter_warp<QC><<<(int)grid, 32 * kWWarps, sm, ctx_stream(ctx)>>>(a, io, (int)grab));
   return SEDEF_OK;
+}
+
+// w: winnowing window.  A query window holds 2 / (w + 1) of its starts as
+// records on average; the form for 256 records has five CTAs per SM where the
+// one for 128 has seven, so it is taken only where 128 would not do.
+int launch_warp_tier(sedef_ctx* ctx, const FArgs& a, const TierIO& io, int64_t max_windows, int w,
+                     const char* name) {
+  if (1.35 * 2.0 * (a.span + 1) / (w + 1) <= 128.0)
+    return launch_warp_tier_as<128>(ctx, a, io, max_windows, name);
+  return launch_warp_tier_as<256>(ctx, a, io, max_windows, name);
 }
 
 // ------------------------------------------------------------- slow path --
@@ -1162,13 +1396,14 @@ __device__ int slow_wq(const FArgs& a, SlowSmem& S, int64_t wdx) {
 // Hits of overflow window v: visits (t, hid, o) for every compatible posting.
 template <typename F>
 __device__ void slow_hits(const FArgs& a, const SlowSmem& S, int s, int64_t i, F f) {
+  const uint32_t tlo = first_useful(a, i);
   for (int l = 0; l < s; ++l) {
     const uint32_t st0 = S.pst[l], len = S.plen[l];
     const uint32_t qm = S.dm[l];
     for (uint32_t x = threadIdx.x; x < len; x += blockDim.x) {
       const uint64_t r = a.tsorted[st0 + x];
       const uint32_t t = rec_pos(r), st = rec_strand(r);
-      if (a.self_mode && (int64_t)t >= i && (int64_t)t <= i + a.span) continue;
+      if (useless_hit(a, t, (uint32_t)i, tlo)) continue;
       if ((qm >> st) & 1u) f(t, (uint32_t)l, 0u);
       if ((qm >> (st ^ 1u)) & 1u) f(t, (uint32_t)l, 1u);
     }
@@ -1501,7 +1736,6 @@ __global__ void __launch_bounds__(32 * (kLean ? kRWarps : kRWarpsBig)) k_refine(
   a.nt = live_n(a.nt, a.dnt);
   using RW = RefineWarpT<QC, RC>;
   constexpr int DC = RW::DC;
-  constexpr int NW = kLean ? kRWarps : kRWarpsBig;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int warp = threadIdx.x >> 5, lane = lane_id();
   RW& R = reinterpret_cast<RW*>(smem_raw)[warp];
@@ -1950,18 +2184,9 @@ __device__ void roll_run(const uint32_t* __restrict__ ev, int nrel, int s, int m
   *jstar_out = jstar;
 }
 
-__device__ __forceinline__ int lb_u32(const uint32_t* v, int n, uint32_t x) {
-  int lo = 0, hi = n;
-  while (lo < hi) {
-    const int mid = (lo + hi) >> 1;
-    if (v[mid] < x) lo = mid + 1; else hi = mid;
-  }
-  return lo;
-}
-
 // Sorts 32 * NR keys held by a warp (key of index lane * NR + x in v[x]).
-template <int NR>
-__device__ __forceinline__ void warp_sort_regs(uint32_t (&v)[NR]) {
+template <typename T, int NR>
+__device__ __forceinline__ void warp_sort_regs(T (&v)[NR]) {
   const int lane = lane_id();
 #pragma unroll
   for (int size = 2; size <= 32 * NR; size <<= 1) {
@@ -1971,7 +2196,7 @@ __device__ __forceinline__ void warp_sort_regs(uint32_t (&v)[NR]) {
         const bool keep_min = (((lane * NR) & size) == 0) == ((lane & (stride / NR)) == 0);
 #pragma unroll
         for (int x = 0; x < NR; ++x) {
-          const uint32_t o = __shfl_xor_sync(0xffffffffu, v[x], stride / NR);
+          const T o = __shfl_xor_sync(0xffffffffu, v[x], stride / NR);
           v[x] = keep_min ? min(v[x], o) : max(v[x], o);
         }
       } else {
@@ -1979,7 +2204,7 @@ __device__ __forceinline__ void warp_sort_regs(uint32_t (&v)[NR]) {
         for (int x = 0; x < NR; ++x) {
           if (x & stride) continue;
           const bool asc = ((lane * NR + x) & size) == 0;
-          const uint32_t p = v[x], q = v[x | stride];
+          const T p = v[x], q = v[x | stride];
           v[x] = asc ? min(p, q) : max(p, q);
           v[x | stride] = asc ? max(p, q) : min(p, q);
         }
@@ -1987,6 +2212,7 @@ __device__ __forceinline__ void warp_sort_regs(uint32_t (&v)[NR]) {
     }
   }
 }
+
 
 // Query records [qa, qa + c) as sorted (hash << 1 | strand) keys in buf[0..32 * NR).
 template <int NR>
@@ -2003,7 +2229,7 @@ __device__ __forceinline__ void sort_window(const uint64_t* __restrict__ qrec, i
       v[x] = (rec_hash(r) << 1) | rec_strand(r);
     }
   }
-  warp_sort_regs<NR>(v);
+  warp_sort_regs(v);
 #pragma unroll
   for (int x = 0; x < NR; ++x) buf[lane * NR + x] = v[x];
 }
@@ -2197,6 +2423,14 @@ __global__ void __launch_bounds__(32 * kBWarps) k_refine_batch(RefineArgs a) {
   flush();
 }
 
+// Every run to the large kernel.
+__global__ void k_refine_all(RefineArgs a) {
+  const int64_t n = live_n(a.nruns, a.dnruns);
+  const int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (x < n) a.big[x] = (uint32_t)x;
+  if (x == 0) *a.nbig = (unsigned int)n;
+}
+
 // Per-run record ranges for the refine: query records of the run's window
 // (from the window table) and target records of its span [j_a, j_b+n-k].
 __global__ void k_run_ranges(const sedef_run_t* runs, int64_t n, const int64_t* qseq, int nqseq,
@@ -2232,10 +2466,13 @@ int launch_fast(sedef_ctx* ctx, const FArgs& a, const TierIO& io_in, int64_t max
   static_assert(sizeof(FastSmemT<TPB, LCAP, GCAP, SLOTS>) <= 227 * 1024,
                 "a filter tier must fit one CTA's shared memory");
   SEDEF_TRY(ensure_smem_attr((const void*)k_filter_fast<TPB, LCAP, GCAP, SLOTS>, sm));
-  // a table of SLOTS counters keeps its aliasing low up to 2 * SLOTS hits;
-  // windows with more go on (to the wide tier when the caller names one)
+  // a table of 2,048 counters separates about as many hits: a window with
+  // more passes nearly all of them on to its sort, and is better off in the
+  // wide tier (a 100 Mbp chromosome's tiers took 17.6 ms with the line at
+  // twice as many hits and 10.2 ms with it here; half as many: the wide
+  // tier's fixed cost per window, a 240 Mbp assembly 57.0 -> 65.7 ms)
   TierIO io = io_in;
-  io.hlim = (uint32_t)(2 * SLOTS);
+  io.hlim = (uint32_t)(SLOTS == kSlots ? SLOTS : 2 * SLOTS);
   int per_sm = 0;
   SEDEF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm,
                                                            k_filter_fast<TPB, LCAP, GCAP, SLOTS>,
@@ -2275,7 +2512,7 @@ const FastLaunch kTierWideMid = launch_fast<512, 8192, 1024, kWideSlots>;
 using WideMidSmem = FastSmemT<512, 8192, 1024, kWideSlots>;
 static_assert(sizeof(FastSmemT<512, 8192, 2048, 2048>) <= kTierSmemFloor &&
                   sizeof(FastSmemT<512, 2048, 512, kWideSlots>) <= kTierSmemFloor &&
-                  sizeof(WarpSmem) * kWWarps <= kTierSmemFloor,
+                  sizeof(WarpSmemT<256>) * kWWarps <= kTierSmemFloor,
               "a tier that always runs needs more shared memory than a tier cap may be");
 // variant = (warp tier off) * 12 + t1 * kNumTier2 + t2
 constexpr int kNumShapes = kNumTier1 * kNumTier2;
@@ -2446,14 +2683,23 @@ int order_and_refine(sedef_ctx* ctx, const FArgs& a, const Derived& D, int nqseq
   int64_t rgrid = (total + kBWarps - 1) / kBWarps;
   if (rgrid > (int64_t)ctx_sm_count(ctx) * rper) rgrid = (int64_t)ctx_sm_count(ctx) * rper;
   if (rgrid < 1) rgrid = 1;
-  // a warp's events: room for the runs it takes at a time
-  const int64_t per_warp = (total + rgrid * kBWarps - 1) / (rgrid * kBWarps);
+  // a warp's events: room for the runs it takes at a time; under a cap on the
+  // context's scratch fewer warps, and where not even one CTA's fit the large
+  // kernel takes every run
   ra.scap = scap;
-  ra.ev_words = per_warp * (kBRC + 8) < kEvWords ? (int)per_warp * (kBRC + 8) : kEvWords;
-  ra.events = (uint32_t*)ctx_alloc(ctx, (size_t)(rgrid * kBWarps) * (ra.ev_words + kEvPad) * 4);
-  if (!ra.events) return SEDEF_ERR_OOM;
-  SEDEF_KERNEL(ctx, "k_refine",
-               k_refine_batch<<<(int)rgrid, 32 * kBWarps, lean_sm, st>>>(ra));
+  while (true) {
+    const int64_t per_warp = (total + rgrid * kBWarps - 1) / (rgrid * kBWarps);
+    ra.ev_words = per_warp * (kBRC + 8) < kEvWords ? (int)per_warp * (kBRC + 8) : kEvWords;
+    ra.events = (uint32_t*)ctx_alloc(ctx, (size_t)(rgrid * kBWarps) * (ra.ev_words + kEvPad) * 4);
+    if (ra.events || rgrid == 1) break;
+    rgrid /= 2;
+  }
+  if (ra.events) {
+    SEDEF_KERNEL(ctx, "k_refine",
+                 k_refine_batch<<<(int)rgrid, 32 * kBWarps, lean_sm, st>>>(ra));
+  } else {
+    SEDEF_KERNEL(ctx, "k_refine_all", k_refine_all<<<tb, 256, 0, st>>>(ra));
+  }
   SEDEF_KERNEL(ctx, "k_refine_big",
                k_refine<kMaxWindowRecs, 1024, false><<<ctx_sm_count(ctx), 32 * kRWarpsBig, big_sm,
                                                        st>>>(ra));
@@ -2567,14 +2813,16 @@ int run_filter(sedef_ctx* ctx, const uint64_t* qrec, int64_t nq, const int64_t* 
     SEDEF_KERNEL(ctx, "k_sample_pos", k_sample_pos<<<(int)g, 256, 0, st>>>(tsorted, nt, dnt, samp));
     a.tsamp = samp;
   }
-  if (D.self_mode == 2 && 2 * D.k <= 24) {
-    // batch self-search: every query record's posting range in its own
-    // genome, once (the warp tier reads them by record offset).  An eager
-    // pass walks the index (the query records are its records, with the
-    // same sequence offsets); a planned pass, whose counts live on the
-    // device, searches per record.
+  a.after_own = D.overlap <= D.n ? 1 : 0;
+  if (D.self_mode == 2 || (D.self_mode == 1 && a.after_own)) {
+    // self-search: every query record's useful posting range, once (the warp
+    // tier reads them by record offset).  An eager pass walks the index (the
+    // query records are its records, with the same sequence offsets); a
+    // planned pass, whose counts live on the device, searches per record.
+    // With target starts at i + n - overlap or later and overlap <= n, only
+    // the entries after the record's own one can be hits.
+    const std::vector<char> used_before = ctx_pool_snapshot(ctx);
     uint2* qp = (uint2*)ctx_alloc(ctx, (size_t)nq * sizeof(uint2));
-    if (!qp) return SEDEF_ERR_OOM;
     const int64_t nw = (a.ttotal + 31) >> 5;
     const bool walk = !pl && nqseq == ntseq &&
                       std::memcmp(h_qoff, h_toff, (size_t)(ntseq + 1) * sizeof(int64_t)) == 0;
@@ -2582,22 +2830,28 @@ int run_filter(sedef_ctx* ctx, const uint64_t* qrec, int64_t nq, const int64_t* 
     uint32_t* pcnt = walk ? (uint32_t*)ctx_alloc(ctx, (size_t)(nw + 1) * 4) : nullptr;
     uint32_t* pbef = walk ? (uint32_t*)ctx_alloc(ctx, (size_t)(nw + 1) * 4) : nullptr;
     RankWord* rw = walk ? (RankWord*)ctx_alloc(ctx, (size_t)(nw + 1) * sizeof(RankWord)) : nullptr;
-    if (walk && (!pbits || !pcnt || !pbef || !rw)) return SEDEF_ERR_OOM;
-    int64_t g = (nq + 255) / 256;
-    if (g > (int64_t)ctx_sm_count(ctx) * 16) g = (int64_t)ctx_sm_count(ctx) * 16;
-    if (g < 1) g = 1;
-    if (!walk) {
-      SEDEF_KERNEL(ctx, "k_qpost", k_qpost<<<(int)g, 256, 0, st>>>(a, nq, dnq, qp));
+    if (!qp || (walk && (!pbits || !pcnt || !pbef || !rw))) {
+      // no room under the context's cap: the tiers look postings up themselves
+      if (D.self_mode == 2) return SEDEF_ERR_OOM;
+      ctx_pool_restore(ctx, used_before);
+      qp = nullptr;
     } else {
-      int64_t gw = (nw + 255) / 256;
-      if (gw > (int64_t)ctx_sm_count(ctx) * 16) gw = (int64_t)ctx_sm_count(ctx) * 16;
-      if (gw < 1) gw = 1;
-      SEDEF_CUDA(cudaMemsetAsync(pbits, 0, (size_t)(nw + 1) * 4, st));
-      SEDEF_KERNEL(ctx, "k_pos_bits", k_pos_bits<<<(int)g, 256, 0, st>>>(qrec, nq, pbits));
-      SEDEF_KERNEL(ctx, "k_pos_popc", k_pos_popc<<<(int)gw, 256, 0, st>>>(pbits, nw, pcnt));
-      SEDEF_TRY(scan_exclusive_u32(ctx, pcnt, pbef, nw, pbef + nw));
-      SEDEF_KERNEL(ctx, "k_rank_words", k_rank_words<<<(int)gw, 256, 0, st>>>(pbits, pbef, nw, rw));
-      SEDEF_KERNEL(ctx, "k_qpost", k_qpost_index<<<(int)g, 256, 0, st>>>(a, nt, rw, qp));
+      int64_t g = (nq + 255) / 256;
+      if (g > (int64_t)ctx_sm_count(ctx) * 16) g = (int64_t)ctx_sm_count(ctx) * 16;
+      if (g < 1) g = 1;
+      if (!walk) {
+        SEDEF_KERNEL(ctx, "k_qpost", k_qpost<<<(int)g, 256, 0, st>>>(a, nq, dnq, qp));
+      } else {
+        int64_t gw = (nw + 255) / 256;
+        if (gw > (int64_t)ctx_sm_count(ctx) * 16) gw = (int64_t)ctx_sm_count(ctx) * 16;
+        if (gw < 1) gw = 1;
+        SEDEF_CUDA(cudaMemsetAsync(pbits, 0, (size_t)(nw + 1) * 4, st));
+        SEDEF_KERNEL(ctx, "k_pos_bits", k_pos_bits<<<(int)g, 256, 0, st>>>(qrec, nq, pbits));
+        SEDEF_KERNEL(ctx, "k_pos_popc", k_pos_popc<<<(int)gw, 256, 0, st>>>(pbits, nw, pcnt));
+        SEDEF_TRY(scan_exclusive_u32(ctx, pcnt, pbef, nw, pbef + nw));
+        SEDEF_KERNEL(ctx, "k_rank_words", k_rank_words<<<(int)gw, 256, 0, st>>>(pbits, pbef, nw, rw));
+        SEDEF_KERNEL(ctx, "k_qpost", k_qpost_index<<<(int)g, 256, 0, st>>>(a, nt, rw, qp));
+      }
     }
     a.qpost = qp;
   }
@@ -2630,9 +2884,11 @@ int run_filter(sedef_ctx* ctx, const uint64_t* qrec, int64_t nq, const int64_t* 
       float best_rep = 1e30f;
       for (int rep = 0; rep < 3; ++rep) {  // the first repetition warms up
         SEDEF_CUDA(cudaMemsetAsync(counters, 0, 80, st));
-        SEDEF_CUDA(cudaMemsetAsync(counters + 12, 0, 48, st));
+        SEDEF_CUDA(cudaMemsetAsync(counters + 12, 0, 64, st));
         TierIO io0{d_sample, (const unsigned int*)(counters + 10), ovl0,
                    (unsigned int*)(counters + 12), (unsigned int*)(counters + 13), 0};
+        io0.wide_list = ovlw;
+        io0.wide_count = (unsigned int*)(counters + 14);
         TierIO io{warp_tier ? ovl0 : d_sample,
                   (const unsigned int*)(counters + (warp_tier ? 12 : 10)), ovl1,
                   (unsigned int*)(counters + 9), (unsigned int*)(counters + 2), 0};
@@ -2647,7 +2903,7 @@ int run_filter(sedef_ctx* ctx, const uint64_t* qrec, int64_t nq, const int64_t* 
         TierIO iow2{ovlw2, (const unsigned int*)(counters + 16), ovl,
                     (unsigned int*)(counters + 1), (unsigned int*)(counters + 17), 0};
         SEDEF_CUDA(cudaEventRecord(e0, st));
-        if (warp_tier) SEDEF_TRY(launch_warp_tier(ctx, a, io0, ns, "k_filter_tune"));
+        if (warp_tier) SEDEF_TRY(launch_warp_tier(ctx, a, io0, ns, D.w, "k_filter_tune"));
         SEDEF_TRY(kTier1[sh / kNumTier2](ctx, a, io, ns, "k_filter_tune"));
         SEDEF_TRY(kTier2[sh % kNumTier2](ctx, a, io2, ns, "k_filter_tune"));
         SEDEF_TRY(kTierWide(ctx, a, iow, ns, "k_filter_tune"));
@@ -2682,7 +2938,9 @@ int run_filter(sedef_ctx* ctx, const uint64_t* qrec, int64_t nq, const int64_t* 
     if (warp_tier) {
       TierIO io0{nullptr, nullptr, ovl0, (unsigned int*)(counters + 12),
                  (unsigned int*)(counters + 13), 1};
-      SEDEF_TRY(launch_warp_tier(ctx, a, io0, nwin, "k_filter_warp"));
+      io0.wide_list = ovlw;
+      io0.wide_count = (unsigned int*)(counters + 14);
+      SEDEF_TRY(launch_warp_tier(ctx, a, io0, nwin, D.w, "k_filter_warp"));
     }
     TierIO io1{warp_tier ? ovl0 : nullptr,
                warp_tier ? (const unsigned int*)(counters + 12) : nullptr, ovl1,

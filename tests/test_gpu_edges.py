@@ -178,6 +178,76 @@ def test_chain2_item_counts(ctx):
     assert_rows_equal(sd_rows(out), want, "SDs")
 
 
+def crowded_genome(seed=9):
+    """Windows with few hits, around 2,048 of them (the warp tier's most), with a counter past
+    255 and with more than 256 collected: families of copies of one element, of many sizes."""
+    rng = np.random.default_rng(seed)
+    seq = synth.random_bases(rng, 260_000, 0.45)
+    at = 2_000
+    for copies in (2, 5, 12, 20, 24, 28, 40, 70):
+        unit = synth.random_bases(rng, 800, 0.45)
+        for _ in range(copies):
+            pc = synth.mutate(rng, unit, float(rng.uniform(0.9, 1.0)))
+            if rng.random() < 0.4:
+                pc = synth.reverse_complement(pc)
+            seq[at:at + len(pc)] = pc
+            at += len(pc) + int(rng.integers(0, 700))
+    seq[at:at + 4_000] = np.tile(synth.random_bases(rng, 25, 0.5), 160)
+    return synth.genome_from_parts([seq[:150_000], seq[150_000:]])
+
+
+@pytest.mark.parametrize("pd", [dict(), dict(w=11), dict(w=40), dict(k=9, w=20), dict(k=14),
+                                dict(delta_m=0.5, delta_g=0.5, w=60, step=700),
+                                dict(delta_m=0.9, delta_g=0.2, w=60, step=700), dict(max_occ=30)])
+@pytest.mark.parametrize("mode", [0, 1, 2])
+def test_filter_crowded_windows(ctx, pd, mode):
+    """Every self mode (target starts before the window too, when overlap > n), eager and captured."""
+    d = oracle.params(self_mode=mode, **pd)
+    g = crowded_genome()
+    recs = oracle.sketch(g.seq, g.offsets, d)
+    want = oracle.filter_runs(recs, g.offsets, recs, g.offsets, d, threads=16)
+    assert len(want) > 100
+    p = binding.params_from_dict(d)
+    seq = to_dev(g.seq)
+    rec = ctx.sedef_sketch(*ctx.sedef_pack(seq), g.offsets, p)
+    srt, off = ctx.sedef_index(rec, p)
+    runs, _ = ctx.sedef_filter(rec, g.offsets, rec, srt, off, g.offsets, p)
+    assert_rows_equal(run_rows(runs), want, "runs")
+    if mode and not pd.get("delta_m"):
+        out = ctx.selfsearch_graph(seq, g.offsets, p).outputs()
+        assert_rows_equal(run_rows(out["runs"]), want, "captured runs")
+
+
+def test_filter_under_scratch_caps(ctx):
+    """With too little scratch for the record posting ranges the tiers look postings up themselves,
+    with less the refine runs fewer warps and then its large kernel alone: the same runs down to
+    the cap where the call is refused."""
+    g = crowded_genome()
+    p = binding.params()
+    c = binding.Context(0)
+    rec = c.sedef_sketch(*c.sedef_pack(to_dev(g.seq)), g.offsets, p)
+    srt, off = c.sedef_index(rec, p)
+    want, n = c.sedef_filter(rec, g.offsets, rec, srt, off, g.offsets, p)
+    want, refused = want.cpu(), 0
+    caps = np.geomspace(64 << 20, 32 << 10, 100).astype(np.int64)
+    c.sedef_trace_enable(True)
+    names = set()
+    for nbytes in caps:
+        c.sedef_set_scratch_limit(0)
+        c.sedef_set_scratch_limit(int(nbytes))
+        try:
+            runs, m = c.sedef_filter(rec, g.offsets, rec, srt, off, g.offsets, p, cap=n + 1)
+        except binding.SedefError as e:
+            assert e.status == -2
+            refused += 1
+            continue
+        names |= set(c.sedef_trace_report(reset=True))
+        assert m == n and bool((runs.cpu() == want).all())
+    assert 0 < refused < len(caps)
+    assert any(x.endswith("k_refine_all") for x in names), names
+    c.close()
+
+
 @pytest.mark.parametrize("mode", [1, 2])
 def test_graph_record_overflow(ctx, mode):
     """A captured pass whose record capacity is far too small: every kernel keeps to the records
