@@ -561,11 +561,11 @@ int sedef_graph_destroy(sedef_graph* g);
  * poll runs on another; submit and poll are not reentrant.  finish may run
  * on several threads at once for different slots: up to five calls work at
  * the same time, each on its own stream, and further calls wait for one of
- * them to return.  The kernel keeps a window with more than 4,096 hits for
- * finish, which runs the wide shared-memory tier over such windows.
+ * them to return.  The kernel leaves a window with more than 16,384 posting
+ * entries to finish, which runs the broader tier over such windows.
  * sedef_server_destroy stops the kernel and frees the server.
  * The persistent kernel asks for the largest L1 / shared-memory split and
- * keeps 62 KB of shared memory on every SM while it runs; a kernel of
+ * keeps 30 KB of shared memory on every SM while it runs; a kernel of
  * another stream that needs more than what is left waits for it to leave.
  * sedef_server_smem_left gives that bound (bytes per CTA); finish keeps its
  * own filter tiers within it, and a context that runs beside the server

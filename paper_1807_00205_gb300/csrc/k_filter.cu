@@ -1,28 +1,29 @@
 // a4-a6: candidate lookup, sliding count of shared minimizers against m(s),
 // and the winnowed MinHash refine (Sections 2.2 and 3.1).
 //
-// Shared-memory tiers (one CTA per query window, persistent CTAs):
-//   1. the window's query minimizers are sorted by hash in shared memory and
-//      deduplicated into W_Q (s hashes, each with its strand set);
-//   2. every posting of every hash of W_Q is a hit (t, hid, o).  Hits are
-//      counted into direct-mapped 16-bit counters keyed by (t >> 10, o):
-//      a target window [j, j+n-k] lies inside bins j>>10 and (j>>10)+1, so a
-//      j can only pass when those two counters sum to m or more (aliasing
-//      only adds false candidates).  The table has the smallest power of two
-//      >= 4 H slots (H = the window's hits), at least 2,048 and at most the
-//      tier's size, so the prefilter stays selective when posting lists are
-//      long (a large target);
-//   3. hits whose bin pair can pass are collected and sorted by (o, t); the
-//      exact sweep (one thread, per-hash counters) runs only over j ranges
-//      where m consecutive hits fit in n-k bases.  Any j whose true count
-//      reaches m has all of its hits collected, and a count computed from a
-//      subset never exceeds the true one, so the runs are exact.
-// The tiers differ only in their shared-memory budget: an optional warp tier
-// (one warp per small window), tier 1 (autotuned shape), tier 2 (more
-// collected hits) and the wide tier (32,768 counters) for windows with more
-// than 4,096 hits, which tiers 1 and 2 hand over before enumerating them.
-// Windows no tier can hold go to a global path that writes their hits to
-// global memory, radix-sorts them by (window, o, t) and runs the same sweep.
+// Every tier takes the same steps for a query window:
+//   1. every posting of the window's query minimizers is a hit (t, hash, o).
+//      Hits are counted into direct-mapped counters keyed by (t >> 10, o): a
+//      target window [j, j+n-k] lies inside bins j>>10 and (j>>10)+1, so a j
+//      can only pass when those two counters sum to m or more (aliasing and
+//      hits counted twice only add false candidates).  The table has the
+//      smallest power of two >= 4 H slots (H = the window's posting entries)
+//      up to the tier's size, so the prefilter stays selective when posting
+//      lists are long (a large target);
+//   2. W_Q: the distinct hashes (s of them, each with its strand set) and m;
+//   3. hits whose bin pair can pass are collected and sorted by (o, t), and
+//      the runs found exactly from them.  Any j whose true count reaches m
+//      has all of its hits collected, and a count computed from a subset
+//      never exceeds the true one, so the runs are exact.
+// Tiers, by what a window needs: the warp tier (a warp per window), the
+// narrow and the broad CTA tier (k_filter_cta), the second wide tier
+// (16,384 collected hits).  Windows none of them can hold go to a global path
+// that writes their hits to global memory, radix-sorts them by (window, o, t)
+// and sweeps their dense groups.  The autotuner may leave the warp tier out
+// for tiers 1 and 2, CTAs of chosen shapes over windows of up to 2,048
+// entries (launch_fast; the second wide tier is one of these): W_Q sorted in
+// shared memory, 16-bit counters, and one thread that sweeps each dense group
+// (m consecutive hits within n-k bases) with per-hash counters.
 //
 // Refine (k_refine_batch): each run's span records become events (position,
 // rank among W_Q), set up by a warp; then one lane per run rolls the target
@@ -221,26 +222,19 @@ __device__ void sweep_group(const FArgs& a, const WinInfo& w, Get get, int64_t L
   emit_run(a, w, r);
 }
 
-__device__ __forceinline__ int64_t warp_excl_max(int64_t v) {
-  const int lane = lane_id();
-  int64_t inc = v;
-#pragma unroll
-  for (int d = 1; d < 32; d <<= 1) {
-    const int64_t o = __shfl_up_sync(0xffffffffu, inc, d);
-    if (lane >= d && o > inc) inc = o;
-  }
-  const int64_t ex = __shfl_up_sync(0xffffffffu, inc, 1);
-  return lane == 0 ? INT64_MIN : ex;
-}
-
 // Dense groups of one strand's t-sorted hits (warp-cooperative; every lane
 // calls).  Hit x is dense when the m hits from x on fit in n-k bases; every
 // j whose count reaches m lies in [t(x+m-1) - (n-k), t(x)] for some dense x.
-// Overlapping or touching such ranges form a group; emit(Jlo, Jhi) is called
-// by every lane, once per group, in increasing order.
+// Overlapping or touching such ranges form a group.  emit(mine, Jlo, Jhi) is
+// called by every lane, for the groups of the lanes with `mine`, in
+// increasing order (a lane that starts a group closes the one before it, so
+// up to 32 groups go out at once: one after another, a window whose every hit
+// is a group took 0.5 us for each of its thousands, 1.46 -> 0.12 ms for the
+// global path of a 950 kbp region against a 3.1 Gbp index).
 template <typename Get, typename Emit>
 __device__ void find_groups(Get get, int64_t L, int m, int span, Emit emit) {
   const int lane = lane_id();
+  const unsigned lt = lanemask_lt();
   int64_t carry_hi = INT64_MIN;  // largest jhi of the dense hits seen so far
   int64_t cur_lo = 0;
   bool open = false;
@@ -256,28 +250,21 @@ __device__ void find_groups(Get get, int64_t L, int m, int span, Emit emit) {
         jhi = ta;
       }
     }
-    int64_t before = warp_excl_max(dense ? jhi : INT64_MIN);
-    if (carry_hi > before) before = carry_hi;
+    const unsigned dm = __ballot_sync(0xffffffffu, dense);
+    // the hits are sorted, so the nearest dense one before has the largest jhi
+    const int64_t near = __shfl_sync(0xffffffffu, jhi, dm & lt ? 31 - __clz(dm & lt) : lane);
+    const int64_t before = dm & lt ? near : carry_hi;
     const bool start = dense && (before == INT64_MIN || jlo > before + 1);
-    unsigned starts = __ballot_sync(0xffffffffu, start);
-    while (starts) {
-      const int ls = __ffs(starts) - 1;
-      starts &= starts - 1;
-      const int64_t b_ls = __shfl_sync(0xffffffffu, before, ls);
-      const int64_t lo_ls = __shfl_sync(0xffffffffu, jlo, ls);
-      if (open) emit(cur_lo, b_ls);
-      cur_lo = lo_ls;
+    const unsigned starts = __ballot_sync(0xffffffffu, start);
+    const int64_t lo_near = __shfl_sync(0xffffffffu, jlo, starts & lt ? 31 - __clz(starts & lt) : lane);
+    emit(start && (open || (starts & lt)), starts & lt ? lo_near : cur_lo, before);
+    if (starts) {
+      cur_lo = __shfl_sync(0xffffffffu, jlo, 31 - __clz(starts));
       open = true;
     }
-    int64_t mx = dense ? jhi : INT64_MIN;
-#pragma unroll
-    for (int d = 16; d > 0; d >>= 1) {
-      const int64_t o = __shfl_xor_sync(0xffffffffu, mx, d);
-      if (o > mx) mx = o;
-    }
-    if (mx > carry_hi) carry_hi = mx;
+    if (dm) carry_hi = __shfl_sync(0xffffffffu, jhi, 31 - __clz(dm));
   }
-  if (open) emit(cur_lo, carry_hi);
+  emit(open && lane == 0, cur_lo, carry_hi);
 }
 
 // ------------------------------------------------------ block bitonic sort --
@@ -741,12 +728,14 @@ __device__ void fast_window(const FArgs& a, const TierIO& io,
             const unsigned long long h = base[x];
             return make_uint2((uint32_t)(h >> 20), (uint32_t)(h & 0xFFFFFu));
           },
-          cnt, m, a.span, [&](int64_t lo, int64_t hi) {
-            if (threadIdx.x == 0 && ng < kGCap) {
-              S.glo[ng] = (uint32_t)(lo < 0 ? 0 : lo);
-              S.ghi[ng] = (uint32_t)hi;
+          cnt, m, a.span, [&](bool mine, int64_t lo, int64_t hi) {
+            const unsigned b = __ballot_sync(0xffffffffu, mine);
+            const int g = ng + __popc(b & lanemask_lt());
+            if (mine && g < kGCap) {
+              S.glo[g] = (uint32_t)(lo < 0 ? 0 : lo);
+              S.ghi[g] = (uint32_t)hi;
             }
-            ++ng;
+            ng += __popc(b);
           });
       if (o == 0 && threadIdx.x == 0) S.ng0 = ng;
     }
@@ -840,21 +829,29 @@ __global__ void __launch_bounds__(TPB) k_filter_fast(FArgs a, TierIO io) {
 // (tier 1 over the windows handed on 3.9 -> 0.5 ms), a 240 Mbp assembly 10.8
 // -> 3.5 ms.
 
-constexpr int kWSlots = 4096;   // 8-bit (bin, o) counters
-constexpr int kWL = 256;        // collected hits
-constexpr int kWH = 2048;       // posting entries (a counter per two of them)
 constexpr int kWWarps = 4;
 
-// QC: query records a window may have.
-template <int QC>
-struct WarpSmemT {
-  uint32_t table[kWSlots / 4];   // counters; then a strand's events
-  uint2 lists[QC];               // posting lists; then per-hash and per-run places
-  unsigned long long hits[kWL];  // W_Q's hash table; then the collected hits
-  uint32_t starts[kWH / 32];     // map of hashes; then bit e: a list starts at hit e
-  uint32_t strands[2 * QC / 16]; // W_Q's strands, two bits per table slot
+// QC: query records, SLOTS: 8-bit (bin, o) counters, WL: collected hits, WH:
+// posting entries, MINB: CTAs per SM.
+template <int QC_, int SLOTS_, int WL_, int WH_, int MINB_>
+struct WindowShape {
+  static constexpr int QC = QC_, SLOTS = SLOTS_, WL = WL_, WH = WH_, MINB = MINB_;
+  static constexpr int TS = 2 * QC;  // W_Q table slots
+  static_assert(WH / 32 >= 64, "the map of hashes lies over the list starts");
+  static_assert(TS * 4 <= WL * 8, "W_Q's table lies over the hits");
+  static_assert(WL * 16 <= SLOTS, "the strands' events lie over the counters");
 };
-static_assert(kWH / 32 == 64, "the map of hashes lies over the list starts");
+using WarpSparse = WindowShape<128, 4096, 256, 2048, 7>;
+using WarpDense = WindowShape<256, 4096, 256, 2048, 5>;
+
+template <typename W>
+struct WindowSmemT {
+  uint32_t table[W::SLOTS / 4];       // counters; then the strands' events
+  uint2 lists[W::QC];                 // posting lists; then per-hash places
+  unsigned long long hits[W::WL];     // W_Q's hash table; then the collected hits
+  uint32_t starts[W::WH / 32];        // map of hashes; then bit e: a list starts at hit e
+  uint32_t strands[W::TS / 16];       // W_Q's strands, two bits per table slot
+};
 
 // Sorts n 64-bit keys in shared memory (n <= 32 * NR) through registers.
 // The stages are loops and not unrolled: the kernel around it is bound by its
@@ -925,7 +922,31 @@ struct EventMem {
   int nlast;         // hash ids
 };
 
-// The runs of one strand from its n collected hits, sorted by t (n <= 256).
+// The places for a strand of n hits: 16 n bytes at `words`, nlast entries at `last`.
+__device__ __forceinline__ EventMem event_mem(uint32_t* words, int n, uint16_t* last, int nlast) {
+  EventMem M;
+  M.enter = words;
+  M.leave = words + n;
+  M.end = words + 2 * n;
+  M.val = reinterpret_cast<uint16_t*>(words + 3 * n);
+  M.first = M.val + n;
+  M.last = last;
+  M.nlast = nlast;
+  return M;
+}
+
+// Whether two adjacent bins that begin in word x of the counter table reach m
+// on a strand: the word holds bins 2x and 2x + 1, both strands; the bins wrap
+// around after nw words.
+__device__ __forceinline__ bool word_passes(const uint32_t* table, int x, int nw, uint32_t m) {
+  const uint32_t c0 = table[x], c1 = table[(x + 1) & (nw - 1)];
+  const uint32_t s0 = c0 & 0x00FF00FFu, s1 = (c0 >> 8) & 0x00FF00FFu;  // strands 0 and 1
+  const uint32_t n0 = c1 & 0x00FF00FFu, n1 = (c1 >> 8) & 0x00FF00FFu;
+  return (s0 & 0xFFFFu) + (s0 >> 16) >= m || (s1 & 0xFFFFu) + (s1 >> 16) >= m ||
+         (s0 >> 16) + (n0 & 0xFFFFu) >= m || (s1 >> 16) + (n1 & 0xFFFFu) >= m;
+}
+
+// The runs of one strand from its n collected hits, sorted by t.
 // The whole warp calls.
 __device__ __noinline__ void strand_runs(const FArgs& a, const WinInfo& w, unsigned long long* hits, int n,
                             const EventMem& M) {
@@ -1055,15 +1076,14 @@ __device__ __noinline__ uint2 posting_window_of(const uint64_t* idx, const uint3
   return make_uint2(st, len);
 }
 
-template <int QC>
-__global__ void __launch_bounds__(32 * kWWarps, QC == 128 ? 7 : 5) k_filter_warp(FArgs a, TierIO io,
-                                                                                int per_grab) {
+template <typename W>
+__global__ void __launch_bounds__(32 * kWWarps, W::MINB) k_filter_warp(FArgs a, TierIO io,
+                                                                     int per_grab) {
+  constexpr int QC = W::QC, TS = W::TS, kWL = W::WL, kWH = W::WH, kWSlots = W::SLOTS;
   constexpr int NC = QC / 32;    // records per lane
-  constexpr int TS = 2 * QC;     // W_Q table slots
-  static_assert(TS * 4 <= kWL * 8, "W_Q's table lies over the hits");
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int warp = threadIdx.x >> 5, lane = lane_id();
-  WarpSmemT<QC>& S = reinterpret_cast<WarpSmemT<QC>*>(smem_raw)[warp];
+  WindowSmemT<W>& S = reinterpret_cast<WindowSmemT<W>*>(smem_raw)[warp];
   const uint32_t lt = lanemask_lt();
   const int64_t count = io.in_list ? (int64_t)*io.in_count : a.nwin;
   unsigned long long n_hits = 0, n_collected = 0;
@@ -1220,16 +1240,9 @@ __global__ void __launch_bounds__(32 * kWWarps, QC == 128 ? 7 : 5) k_filter_warp
         const uint32_t m = (uint32_t)a.mtab[s_least];
         bool pass = 2u * most >= m;
         if (pass) {
-          // word x: bins 2x and 2x + 1, both strands; the bins wrap around
           pass = false;
           const int nw = (int)nslots / 4;
-          for (int x = lane; x < nw; x += 32) {
-            const uint32_t c0 = S.table[x], c1 = S.table[(x + 1) & (nw - 1)];
-            const uint32_t even = c0 & 0x00FF00FFu, odd = (c0 >> 8) & 0x00FF00FFu;  // strands 0, 1
-            const uint32_t enext = c1 & 0x00FF00FFu, onext = (c1 >> 8) & 0x00FF00FFu;
-            pass |= (even & 0xFFFFu) + (even >> 16) >= m || (odd & 0xFFFFu) + (odd >> 16) >= m ||
-                    (even >> 16) + (enext & 0xFFFFu) >= m || (odd >> 16) + (onext & 0xFFFFu) >= m;
-          }
+          for (int x = lane; x < nw; x += 32) pass |= word_passes(S.table, x, nw, m);
         }
         if (!__any_sync(0xffffffffu, pass)) {
           n_hits += H;
@@ -1293,16 +1306,7 @@ __global__ void __launch_bounds__(32 * kWWarps, QC == 128 ? 7 : 5) k_filter_warp
       int split = 0;  // first hit with o = 1
       for (int base = 0; base < L; base += 32)
         split += __popc(__ballot_sync(0xffffffffu, base + lane < L && (S.hits[base + lane] >> 63) == 0));
-      EventMem M;
-      M.enter = S.table;
-      M.leave = S.table + kWL;
-      M.end = S.table + 2 * kWL;
-      M.val = reinterpret_cast<uint16_t*>(S.table + 3 * kWL);
-      M.last = reinterpret_cast<uint16_t*>(S.lists);
-      M.nlast = TS;
-      M.first = M.last + TS;
-      static_assert(kWSlots / 4 >= 3 * kWL + kWL / 2 && sizeof(S.lists) >= (TS + kWL) * 2,
-                    "a strand's events lie over the counters and the lists");
+      const EventMem M = event_mem(S.table, L, reinterpret_cast<uint16_t*>(S.lists), TS);
       WinInfo w;
       w.i = i;
       w.qseq = a.win_seq[wdx];
@@ -1324,13 +1328,13 @@ __global__ void __launch_bounds__(32 * kWWarps, QC == 128 ? 7 : 5) k_filter_warp
   }
 }
 
-template <int QC>
+template <typename W>
 int launch_warp_tier_as(sedef_ctx* ctx, const FArgs& a, const TierIO& io, int64_t max_windows,
                         const char* name) {
-  const size_t sm = sizeof(WarpSmemT<QC>) * kWWarps;
-  SEDEF_TRY(ensure_smem_attr((const void*)k_filter_warp<QC>, sm));
+  const size_t sm = sizeof(WindowSmemT<W>) * kWWarps;
+  SEDEF_TRY(ensure_smem_attr((const void*)k_filter_warp<W>, sm));
   int per_sm = 0;
-  SEDEF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_filter_warp<QC>, 32 * kWWarps, sm));
+  SEDEF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_filter_warp<W>, 32 * kWWarps, sm));
   if (per_sm < 1) per_sm = 1;
   int64_t grid = (int64_t)ctx_sm_count(ctx) * per_sm;
   // a few windows: one per warp; many: eight at a time
@@ -1340,18 +1344,312 @@ int launch_warp_tier_as(sedef_ctx* ctx, const FArgs& a, const TierIO& io, int64_
   if (grid > need) grid = need;
   if (grid < 1) grid = 1;
   SEDEF_KERNEL(ctx, name,
-               k_filter_warp<QC><<<(int)grid, 32 * kWWarps, sm, ctx_stream(ctx)>>>(a, io, (int)grab));
+               k_filter_warp<W><<<(int)grid, 32 * kWWarps, sm, ctx_stream(ctx)>>>(a, io, (int)grab));
   return SEDEF_OK;
 }
 
 // w: winnowing window.  A query window holds 2 / (w + 1) of its starts as
-// records on average; the form for 256 records has five CTAs per SM where the
-// one for 128 has seven, so it is taken only where 128 would not do.
+// records on average; the shape for 256 records has five CTAs per SM where
+// the one for 128 has seven, so it is taken only where 128 would not do.
 int launch_warp_tier(sedef_ctx* ctx, const FArgs& a, const TierIO& io, int64_t max_windows, int w,
                      const char* name) {
   if (1.35 * 2.0 * (a.span + 1) / (w + 1) <= 128.0)
-    return launch_warp_tier_as<128>(ctx, a, io, max_windows, name);
-  return launch_warp_tier_as<256>(ctx, a, io, max_windows, name);
+    return launch_warp_tier_as<WarpSparse>(ctx, a, io, max_windows, name);
+  return launch_warp_tier_as<WarpDense>(ctx, a, io, max_windows, name);
+}
+
+// -------------------------------------------------------------- CTA tier --
+//
+// The warp tier's steps with one CTA per window, for windows with more
+// records, posting entries or collected hits than a warp keeps.  A record
+// per thread; the warps share out the posting chunks (a contiguous stretch
+// each, four chunks in flight); the collected hits are sorted by a warp (up
+// to 256) or the CTA; two warps take a strand each.
+//
+// Bound by the latency of the posting reads and, for windows of a few
+// thousand entries, by its barriers.  It replaced a form that sorted the
+// records for W_Q (28 barriers), searched the posting lists for each hit
+// with one read per thread in flight, cleared 64 KB of 16-bit counters and
+// swept groups one by one: 46 k windows of 7,700 entries against a 3.1 Gbp
+// index 8.3 -> 4.6 ms, a 240 Mbp assembly's 9.0 -> 4.8 ms.  One warp per such
+// window with eight chunks in flight took 5.5 + 2.4 ms on the former, and
+// 0.32 ms where 38 windows are all there is (0.09 this way).
+
+constexpr int kCThreads = 256, kCWarps = kCThreads / 32;
+// Up to 16,384 posting entries and 1,024 collected hits; up to 65,536 and 2,048.
+using CtaNarrow = WindowShape<kCThreads, 16384, 1024, 16384, 4>;
+using CtaBroad = WindowShape<kCThreads, 32768, 2048, 65536, 3>;
+
+template <typename W>
+struct CtaSmemT : WindowSmemT<W> {
+  uint32_t map[64];
+  uint32_t sum[kCWarps], lists_of[kCWarps];
+  uint32_t most;
+  int nhit;
+  int64_t win;
+};
+
+// One query window by the whole CTA; a window the shape cannot hold goes to
+// io.out_list, or for its posting entries to io.wide_list.  The caller
+// synchronizes the CTA before and after.  Query-side data is read past L1: a
+// serving slot's buffers are refilled while the kernel runs.
+template <typename W>
+__device__ void cta_window(const FArgs& a, const TierIO& io, CtaSmemT<W>& S, int64_t wdx) {
+  const int tid = threadIdx.x, lane = lane_id(), warp = tid >> 5;
+  const uint32_t lt = lanemask_lt();
+  const uint32_t i = __ldcg(a.win_i + wdx), qa = __ldcg(a.win_qa + wdx);
+  const int c = (int)(__ldcg(a.win_qb + wdx) - qa);
+  if (c == 0) return;
+  auto hand_over = [&](bool wide) {
+    if (tid != 0) return;
+    if (wide && io.wide_list) io.wide_list[atomicAdd(io.wide_count, 1u)] = (uint32_t)wdx;
+    else io.out_list[atomicAdd(io.out_count, 1u)] = (uint32_t)wdx;
+  };
+  if (c > W::QC) return hand_over(false);
+  if (tid < 64) S.map[tid] = 0u;
+  if (tid < W::TS / 16) S.strands[tid] = 0u;
+  if (tid == 0) {
+    S.most = 0;
+    S.nhit = 0;
+  }
+  __syncthreads();
+  // ---- this thread's record: hash and strand, posting range
+  uint32_t key = 0, st = 0, len = 0;
+  bool kept = false;
+  if (tid < c) {
+    const uint64_t r = __ldcg(a.qrec + qa + tid);
+    const uint32_t h = rec_hash(r);
+    key = (h << 1) | rec_strand(r);
+    if (a.qpost) {
+      const uint2 pp = __ldcg(a.qpost + qa + tid);
+      st = pp.x;
+      len = pp.y;
+      kept = pp.x != kNone;
+    } else {
+      st = a.toff[h];
+      len = a.toff[h + 1] - st;
+      kept = !(a.max_occ > 0 && (int)len > a.max_occ);
+      if (kept && a.self_mode == 2) {
+        const int sq = __ldcg(a.win_seq + wdx);
+        posting_window(a.tsorted, a.tsamp, &st, &len, a.tseq[sq], a.tseq[sq + 1]);
+      }
+    }
+    if (kept) {
+      const uint32_t g = (h * 0x9E3779B1u) >> 21;
+      atomicOr(&S.map[g >> 5], 1u << (g & 31));
+    } else {
+      len = 0;
+    }
+  }
+  // ---- posting lists with an entry, one after another
+  const uint32_t v = min(len, 1u << 20);  // no sum can wrap
+  const uint32_t inc = warp_inclusive_sum(v);
+  const unsigned some = __ballot_sync(0xffffffffu, len > 0);
+  if (lane == 31) S.sum[warp] = inc;
+  if (lane == 0) S.lists_of[warp] = __popc(some);
+  __syncthreads();
+  uint32_t at = inc - v, lid = __popc(some & lt), H = 0;
+#pragma unroll
+  for (int x = 0; x < kCWarps; ++x) {
+    const uint32_t y = S.sum[x];
+    if (x < warp) {
+      at += y;
+      lid += S.lists_of[x];
+    }
+    H += y;
+  }
+  const int s_least = (int)__reduce_add_sync(0xffffffffu, __popc(S.map[lane]) + __popc(S.map[lane + 32]));
+  if (s_least == 0 || H == 0) return;
+  if (H > io.hlim || H > (uint32_t)W::WH) return hand_over(true);
+  const int nchunk = (int)(H + 31) >> 5;
+  uint32_t nslots = 1024;
+  while (nslots < 4u * H && nslots < (uint32_t)W::SLOTS) nslots <<= 1;
+  const uint32_t smask = nslots - 1;
+  for (int x = tid; x < nchunk; x += kCThreads) S.starts[x] = 0u;
+  for (int x = tid; x < (int)nslots / 16; x += kCThreads)
+    reinterpret_cast<uint4*>(S.table)[x] = make_uint4(0, 0, 0, 0);
+  __syncthreads();
+  if (len > 0) {
+    S.lists[lid] = make_uint2(st - at, key & 1u);
+    atomicOr(&S.starts[at >> 5], 1u << (at & 31));
+  }
+  __syncthreads();
+  // this warp's chunks of 32 hits, and the lists that start before them
+  const int per = (nchunk + kCWarps - 1) / kCWarps;
+  const int c0 = min(warp * per, nchunk), c1 = min(c0 + per, nchunk);
+  int first_list = 0;
+  for (int x = lane; x < c0; x += 32) first_list += __popc(S.starts[x]);
+  first_list = (int)__reduce_add_sync(0xffffffffu, first_list) - 1;
+  const uint32_t tlo = first_useful(a, i);
+  auto each_hit = [&](auto f) {
+    constexpr int kAhead = 4;  // chunks in flight
+    int lists_before = first_list;
+    for (int ch = c0; ch < c1; ch += kAhead) {
+      uint64_t r[kAhead];
+      uint32_t y[kAhead];
+#pragma unroll
+      for (int q = 0; q < kAhead; ++q) {
+        const uint32_t e = (uint32_t)(ch + q) * 32 + lane;
+        r[q] = 0;
+        y[q] = 0;
+        if (ch + q < c1) {
+          const unsigned sb = S.starts[ch + q];
+          const int li = lists_before + __popc(sb & (lt | (1u << lane)));
+          lists_before += __popc(sb);
+          if (e < H) {
+            const uint2 list = S.lists[li];
+            y[q] = list.y;
+            r[q] = __ldg(a.tsorted + (list.x + e));
+          }
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < kAhead; ++q) {
+        if (ch + q >= c1) break;
+        const uint32_t t = rec_pos(r[q]);
+        const bool on = (uint32_t)(ch + q) * 32 + lane < H && !useless_hit(a, t, i, tlo);
+        f(on, t, (y[q] ^ rec_strand(r[q])) & 1u, y[q]);
+      }
+    }
+  };
+  {
+    uint32_t most = 0;
+    each_hit([&](bool on, uint32_t t, uint32_t o, uint32_t) {
+      if (!on) return;
+      const uint32_t sl = slot_of(t, o, smask), sh = (sl & 3u) * 8u;
+      most = max(most, ((atomicAdd(&S.table[sl >> 2], 1u << sh) >> sh) & 0xFFu) + 1u);
+    });
+    most = __reduce_max_sync(0xffffffffu, most);
+    if (lane == 0) atomicMax(&S.most, most);
+  }
+  __syncthreads();
+  const uint32_t most = S.most;
+  if (most > 255u) return hand_over(false);  // a counter ran into its neighbour
+  {
+    const uint32_t m = (uint32_t)a.mtab[s_least];
+    bool pass = false;
+    if (2u * most >= m) {
+      const int nw = (int)nslots / 4;
+      for (int x = tid; x < nw; x += kCThreads) pass |= word_passes(S.table, x, nw, m);
+    }
+    if (!__syncthreads_or(pass)) {
+      if (io.stats && tid == 0) atomicAdd(a.stats + 0, (unsigned long long)H);
+      return;
+    }
+  }
+  // ---- W_Q: a hash's id is its slot; a record whose hash and strand are in
+  // already adds nothing
+  uint32_t* tab = reinterpret_cast<uint32_t*>(S.hits);
+  for (int x = tid; x < W::TS / 4; x += kCThreads) reinterpret_cast<uint4*>(tab)[x] = make_uint4(0, 0, 0, 0);
+  __syncthreads();
+  bool fresh = false;
+  if (kept) {
+    const uint32_t h = key >> 1;
+    static_assert(W::TS == 512, "nine bits of the hash pick a slot");
+    uint32_t slot = (h * 0x9E3779B1u) >> 23;
+    while (true) {  // at most QC keys in TS slots: a free slot is always found
+      const uint32_t old = atomicCAS(&tab[slot], 0u, h + 1u);
+      fresh = old == 0u;
+      if (fresh || old == h + 1u) break;
+      slot = (slot + 1u) & (uint32_t)(W::TS - 1);
+    }
+    const uint32_t bit = 1u << ((slot & 15) * 2 + (key & 1u));
+    const bool twice = (atomicOr(&S.strands[slot >> 4], bit) & bit) != 0u;
+    if (len > 0) S.lists[lid].y = (key & 1u) | (twice ? 2u : 0u) | (slot << 2);
+  }
+  const int s = __syncthreads_count(fresh);
+  const int m = a.mtab[s];
+  each_hit([&](bool on, uint32_t t, uint32_t o, uint32_t y) {
+    bool need = false;
+    if (on && !(y & 2u)) {
+      const uint32_t b = t >> kBinShift;
+      auto cnt = [&](uint32_t bin) {
+        const uint32_t sl = ((bin << 1) | o) & smask;
+        return (S.table[sl >> 2] >> ((sl & 3u) * 8u)) & 0xFFu;
+      };
+      const uint32_t n0 = cnt(b);
+      need = n0 + cnt(b + 1) >= (uint32_t)m || (b > 0 && n0 + cnt(b - 1) >= (uint32_t)m);
+    }
+    const unsigned bn = __ballot_sync(0xffffffffu, need);
+    if (bn) {
+      int to = 0;
+      if (lane == 0) to = atomicAdd(&S.nhit, __popc(bn));
+      to = __shfl_sync(0xffffffffu, to, 0) + __popc(bn & lt);
+      if (need && to < W::WL)
+        S.hits[to] = ((unsigned long long)o << 63) | ((unsigned long long)t << 20) | (y >> 2);
+    }
+  });
+  __syncthreads();
+  const int L = S.nhit;
+  if (L > W::WL) return hand_over(false);
+  if (io.stats && tid == 0) {
+    atomicAdd(a.stats + 0, (unsigned long long)H);
+    atomicAdd(a.stats + 1, (unsigned long long)L);
+  }
+  if (L < m) return;
+  if (L <= 256) {
+    if (warp == 0) {
+      if (L <= 128) warp_sort_hits<4>(S.hits, L);
+      else warp_sort_hits<8>(S.hits, L);
+    }
+  } else {
+    const int np = next_pow2(L);
+    for (int x = L + tid; x < np; x += kCThreads) S.hits[x] = ~0ull;
+    __syncthreads();
+    block_sort(S.hits, np);
+  }
+  __syncthreads();
+  if (warp >= 2) return;
+  int split = 0;  // first hit with o = 1
+  for (int base = 0; base < L; base += 32)
+    split += __popc(__ballot_sync(0xffffffffu, base + lane < L && (S.hits[base + lane] >> 63) == 0));
+  const int n = warp ? L - split : split;
+  if (n < m) return;
+  WinInfo w;
+  w.i = i;
+  w.qseq = __ldcg(a.win_seq + wdx);
+  w.s = s;
+  w.m = m;
+  w.o = warp;
+  static_assert(W::TS * 4 <= W::QC * 8, "both strands' per-hash places lie over the lists");
+  strand_runs(a, w, S.hits + (warp ? split : 0), n,
+              event_mem(S.table + (warp ? 4 * split : 0), n,
+                        reinterpret_cast<uint16_t*>(S.lists) + warp * W::TS, W::TS));
+}
+
+template <typename W>
+__global__ void __launch_bounds__(kCThreads, W::MINB) k_filter_cta(FArgs a, TierIO io) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  CtaSmemT<W>& S = *reinterpret_cast<CtaSmemT<W>*>(smem_raw);
+  const int64_t count = (int64_t)*io.in_count;
+  unsigned int next = 0;
+  if (threadIdx.x == 0) next = atomicAdd(io.next, 1u);
+  while (true) {
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      S.win = (int64_t)next < count ? (int64_t)io.in_list[next] : -1;
+      if (S.win >= 0) next = atomicAdd(io.next, 1u);  // waited for after this window
+    }
+    __syncthreads();
+    if (S.win < 0) break;
+    cta_window(a, io, S, S.win);
+  }
+}
+
+template <typename W>
+int launch_cta_tier(sedef_ctx* ctx, const FArgs& a, const TierIO& io, int64_t max_windows,
+                    const char* name) {
+  const size_t sm = sizeof(CtaSmemT<W>);
+  static_assert(sizeof(CtaSmemT<W>) <= kTierSmemFloor, "the CTA tiers always run");
+  SEDEF_TRY(ensure_smem_attr((const void*)k_filter_cta<W>, sm));
+  int per_sm = 0;
+  SEDEF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_filter_cta<W>, kCThreads, sm));
+  if (per_sm < 1) per_sm = 1;
+  int64_t grid = (int64_t)ctx_sm_count(ctx) * per_sm;
+  if (grid > max_windows) grid = max_windows;
+  if (grid < 1) grid = 1;
+  SEDEF_KERNEL(ctx, name, k_filter_cta<W><<<(int)grid, kCThreads, sm, ctx_stream(ctx)>>>(a, io));
+  return SEDEF_OK;
 }
 
 // ------------------------------------------------------------- slow path --
@@ -1496,17 +1794,19 @@ __global__ void k_slow_groups(FArgs a, int64_t v0, int64_t v1, const unsigned lo
     for (int o = 0; o < 2; ++o) {
       const int64_t b = o ? split : lo, e = o ? hi : split;
       find_groups([&](int64_t x) { return make_uint2((uint32_t)keys[b + x], 0u); }, e - b, m,
-                  a.span, [&](int64_t jlo, int64_t jhi) {
-                    if (lane_id() == 0) {
-                      const unsigned long long at = atomicAdd(ntask, 1ull);
-                      if ((int64_t)at < task_cap) {
-                        SlowTask t;
-                        t.v = (uint32_t)v;
-                        t.o = (uint32_t)o;
-                        t.jlo = jlo < 0 ? 0 : jlo;
-                        t.jhi = jhi;
-                        tasks[at] = t;
-                      }
+                  a.span, [&](bool mine, int64_t jlo, int64_t jhi) {
+                    const unsigned bm = __ballot_sync(0xffffffffu, mine);
+                    if (bm == 0) return;
+                    unsigned long long at = 0;
+                    if (lane_id() == 0) at = atomicAdd(ntask, (unsigned long long)__popc(bm));
+                    at = __shfl_sync(0xffffffffu, at, 0) + __popc(bm & lanemask_lt());
+                    if (mine && (int64_t)at < task_cap) {
+                      SlowTask t;
+                      t.v = (uint32_t)v;
+                      t.o = (uint32_t)o;
+                      t.jlo = jlo < 0 ? 0 : jlo;
+                      t.jhi = jhi;
+                      tasks[at] = t;
                     }
                   });
     }
@@ -2497,13 +2797,10 @@ constexpr int kNumTier1 = 4;
 const FastLaunch kTier2[] = {launch_fast<256, 8192, 2048>, launch_fast<256, 4096, 1024>,
                              launch_fast<512, 8192, 2048>};
 constexpr int kNumTier2 = 3;
-// Wide tiers: windows with more hits than a 2,048-slot table can separate
-// (long posting lists of a large target), before the global path.  32,768
-// (bin, o) slots keep the prefilter selective up to 65,535 hits; the second
-// wide tier holds 16,384 collected hits for windows in regions with many
-// homologous copies.
+// Second wide tier: windows with more collected hits than the CTA tiers keep
+// (regions with many homologous copies), before the global path.  32,768
+// (bin, o) slots and 16,384 collected hits.
 constexpr int kWideSlots = 32768;
-const FastLaunch kTierWide = launch_fast<512, 2048, 512, kWideSlots>;
 const FastLaunch kTierWide2 = launch_fast<512, 16384, 1024, kWideSlots>;
 // The second wide tier in the form that fits beside the serving kernel
 // (8,192 collected hits instead of 16,384), for a context whose tier cap
@@ -2511,8 +2808,7 @@ const FastLaunch kTierWide2 = launch_fast<512, 16384, 1024, kWideSlots>;
 const FastLaunch kTierWideMid = launch_fast<512, 8192, 1024, kWideSlots>;
 using WideMidSmem = FastSmemT<512, 8192, 1024, kWideSlots>;
 static_assert(sizeof(FastSmemT<512, 8192, 2048, 2048>) <= kTierSmemFloor &&
-                  sizeof(FastSmemT<512, 2048, 512, kWideSlots>) <= kTierSmemFloor &&
-                  sizeof(WarpSmemT<256>) * kWWarps <= kTierSmemFloor,
+                  sizeof(WindowSmemT<WarpDense>) * kWWarps <= kTierSmemFloor,
               "a tier that always runs needs more shared memory than a tier cap may be");
 // variant = (warp tier off) * 12 + t1 * kNumTier2 + t2
 constexpr int kNumShapes = kNumTier1 * kNumTier2;
@@ -2755,16 +3051,16 @@ int run_filter(sedef_ctx* ctx, const uint64_t* qrec, int64_t nq, const int64_t* 
   int32_t* wseq = (int32_t*)ctx_alloc(ctx, (size_t)nwin * 4);
   uint32_t* ovl = (uint32_t*)ctx_alloc(ctx, (size_t)nwin * 4);
   uint32_t* ovl1 = (uint32_t*)ctx_alloc(ctx, (size_t)nwin * 4);
-  uint32_t* ovl0 = (uint32_t*)ctx_alloc(ctx, (size_t)nwin * 4);
   uint32_t* ovlw = (uint32_t*)ctx_alloc(ctx, (size_t)nwin * 4);
   uint32_t* ovlw2 = (uint32_t*)ctx_alloc(ctx, (size_t)nwin * 4);
-  if (!ovl0 || !ovlw || !ovlw2) return SEDEF_ERR_OOM;
+  uint32_t* ovlx = (uint32_t*)ctx_alloc(ctx, (size_t)nwin * 4);
+  if (!ovlw || !ovlw2 || !ovlx) return SEDEF_ERR_OOM;
   // [0] runs, [1] windows for the global path, [2] tier-1 work, [3] large
   // refine runs, [4] hits, [5] collected hits, [6]/[7] task and refine work,
   // [8] tier-2 work, [9] windows tier 1 handed to tier 2, [10] sample size,
   // [11] global-path hits (planned pass), [12]/[13] warp-tier hand-overs and
-  // work, [14] windows for the wide tier, [15] wide-tier work, [16]/[17] the
-  // same for the second wide tier
+  // work, [14] windows for the broad CTA tier, [15] its work, [16]/[17] the
+  // same for the second wide tier, [18]/[19] for the narrow CTA tier
   unsigned long long* counters = (unsigned long long*)ctx_alloc(ctx, 256);
   sedef_run_t* raw = (sedef_run_t*)ctx_alloc(ctx, (size_t)(cap > 0 ? cap : 1) * sizeof(sedef_run_t));
   if (!wi || !wqa || !wqb || !wseq || !ovl || !ovl1 || !counters || !raw) return SEDEF_ERR_OOM;
@@ -2885,28 +3181,29 @@ int run_filter(sedef_ctx* ctx, const uint64_t* qrec, int64_t nq, const int64_t* 
       for (int rep = 0; rep < 3; ++rep) {  // the first repetition warms up
         SEDEF_CUDA(cudaMemsetAsync(counters, 0, 80, st));
         SEDEF_CUDA(cudaMemsetAsync(counters + 12, 0, 64, st));
-        TierIO io0{d_sample, (const unsigned int*)(counters + 10), ovl0,
-                   (unsigned int*)(counters + 12), (unsigned int*)(counters + 13), 0};
-        io0.wide_list = ovlw;
-        io0.wide_count = (unsigned int*)(counters + 14);
-        TierIO io{warp_tier ? ovl0 : d_sample,
-                  (const unsigned int*)(counters + (warp_tier ? 12 : 10)), ovl1,
+        TierIO io0{d_sample, (const unsigned int*)(counters + 10), ovlx,
+                   (unsigned int*)(counters + 18), (unsigned int*)(counters + 13), 0};
+        TierIO io{d_sample, (const unsigned int*)(counters + 10), ovl1,
                   (unsigned int*)(counters + 9), (unsigned int*)(counters + 2), 0};
-        io.wide_list = ovlw;
-        io.wide_count = (unsigned int*)(counters + 14);
-        TierIO io2{ovl1, (const unsigned int*)(counters + 9), ovlw, (unsigned int*)(counters + 14),
+        io.wide_list = ovlx;
+        io.wide_count = (unsigned int*)(counters + 18);
+        TierIO io2{ovl1, (const unsigned int*)(counters + 9), ovlx, (unsigned int*)(counters + 18),
                    (unsigned int*)(counters + 8), 0};
-        io2.wide_list = ovlw;
-        io2.wide_count = (unsigned int*)(counters + 14);
+        TierIO iox{ovlx, (const unsigned int*)(counters + 18), ovlw, (unsigned int*)(counters + 14),
+                   (unsigned int*)(counters + 19), 0};
         TierIO iow{ovlw, (const unsigned int*)(counters + 14), ovlw2,
                    (unsigned int*)(counters + 16), (unsigned int*)(counters + 15), 0};
         TierIO iow2{ovlw2, (const unsigned int*)(counters + 16), ovl,
                     (unsigned int*)(counters + 1), (unsigned int*)(counters + 17), 0};
         SEDEF_CUDA(cudaEventRecord(e0, st));
-        if (warp_tier) SEDEF_TRY(launch_warp_tier(ctx, a, io0, ns, D.w, "k_filter_tune"));
-        SEDEF_TRY(kTier1[sh / kNumTier2](ctx, a, io, ns, "k_filter_tune"));
-        SEDEF_TRY(kTier2[sh % kNumTier2](ctx, a, io2, ns, "k_filter_tune"));
-        SEDEF_TRY(kTierWide(ctx, a, iow, ns, "k_filter_tune"));
+        if (warp_tier) {
+          SEDEF_TRY(launch_warp_tier(ctx, a, io0, ns, D.w, "k_filter_tune"));
+        } else {
+          SEDEF_TRY(kTier1[sh / kNumTier2](ctx, a, io, ns, "k_filter_tune"));
+          SEDEF_TRY(kTier2[sh % kNumTier2](ctx, a, io2, ns, "k_filter_tune"));
+        }
+        SEDEF_TRY(launch_cta_tier<CtaNarrow>(ctx, a, iox, ns, "k_filter_tune"));
+        SEDEF_TRY(launch_cta_tier<CtaBroad>(ctx, a, iow, ns, "k_filter_tune"));
         SEDEF_TRY(kTierWide2(ctx, a, iow2, ns, "k_filter_tune"));
         SEDEF_CUDA(cudaEventRecord(e1, st));
         SEDEF_CUDA(cudaEventSynchronize(e1));
@@ -2926,33 +3223,32 @@ int run_filter(sedef_ctx* ctx, const uint64_t* qrec, int64_t nq, const int64_t* 
     return SEDEF_OK;
   }
   {
-    // the warp tier over all windows (unless the autotuned variant leaves it
-    // out), tier 1 (autotuned shape) over what it could not hold, tier 2
-    // (4,096-8,192 hits in shared memory) after that, the wide tier over the
-    // windows with many hits (from tiers 1 and 2) and over what tier 2 could
-    // not hold, the global path last
+    // the warp tier over all windows, or where the variant leaves it out tier
+    // 1 (autotuned shape) over all windows and tier 2 (4,096-8,192 hits in
+    // shared memory) over what it could not hold; the CTA tiers over the
+    // windows those hand on, the second wide tier after that, the global path
+    // last
     int v = ctx_filter_variant(ctx);
     if (v < 0 || v >= kNumVariants) v = 0;
     const int sh = v % kNumShapes;
     const bool warp_tier = v < kNumShapes;
     if (warp_tier) {
-      TierIO io0{nullptr, nullptr, ovl0, (unsigned int*)(counters + 12),
+      TierIO io0{nullptr, nullptr, ovlx, (unsigned int*)(counters + 18),
                  (unsigned int*)(counters + 13), 1};
-      io0.wide_list = ovlw;
-      io0.wide_count = (unsigned int*)(counters + 14);
       SEDEF_TRY(launch_warp_tier(ctx, a, io0, nwin, D.w, "k_filter_warp"));
+    } else {
+      TierIO io1{nullptr, nullptr, ovl1, (unsigned int*)(counters + 9),
+                 (unsigned int*)(counters + 2), 1};
+      io1.wide_list = ovlx;
+      io1.wide_count = (unsigned int*)(counters + 18);
+      SEDEF_TRY(kTier1[sh / kNumTier2](ctx, a, io1, nwin, "k_filter_fast"));
+      TierIO io2{ovl1, (const unsigned int*)(counters + 9), ovlx, (unsigned int*)(counters + 18),
+                 (unsigned int*)(counters + 8), 1};
+      SEDEF_TRY(kTier2[sh % kNumTier2](ctx, a, io2, nwin, "k_filter_mid"));
     }
-    TierIO io1{warp_tier ? ovl0 : nullptr,
-               warp_tier ? (const unsigned int*)(counters + 12) : nullptr, ovl1,
-               (unsigned int*)(counters + 9), (unsigned int*)(counters + 2), 1};
-    io1.wide_list = ovlw;
-    io1.wide_count = (unsigned int*)(counters + 14);
-    SEDEF_TRY(kTier1[sh / kNumTier2](ctx, a, io1, nwin, "k_filter_fast"));
-    TierIO io2{ovl1, (const unsigned int*)(counters + 9), ovlw, (unsigned int*)(counters + 14),
-               (unsigned int*)(counters + 8), 1};
-    io2.wide_list = ovlw;
-    io2.wide_count = (unsigned int*)(counters + 14);
-    SEDEF_TRY(kTier2[sh % kNumTier2](ctx, a, io2, nwin, "k_filter_mid"));
+    TierIO iox{ovlx, (const unsigned int*)(counters + 18), ovlw, (unsigned int*)(counters + 14),
+               (unsigned int*)(counters + 19), 1};
+    SEDEF_TRY(launch_cta_tier<CtaNarrow>(ctx, a, iox, nwin, "k_filter_cta"));
     // where the second wide tier's CTA would pass the context's cap, its
     // 8,192-hit form takes its place, or, where that would pass it too, the
     // wide tier hands its leftovers straight to the global path
@@ -2962,7 +3258,7 @@ int run_filter(sedef_ctx* ctx, const uint64_t* qrec, int64_t nq, const int64_t* 
     const bool second = wide2 || mid;
     TierIO iow{ovlw, (const unsigned int*)(counters + 14), second ? ovlw2 : ovl,
                (unsigned int*)(counters + (second ? 16 : 1)), (unsigned int*)(counters + 15), 1};
-    SEDEF_TRY(kTierWide(ctx, a, iow, nwin, "k_filter_wide"));
+    SEDEF_TRY(launch_cta_tier<CtaBroad>(ctx, a, iow, nwin, "k_filter_wide"));
     TierIO iow2{ovlw2, (const unsigned int*)(counters + 16), ovl, (unsigned int*)(counters + 1),
                 (unsigned int*)(counters + 17), 1};
     if (wide2) SEDEF_TRY(kTierWide2(ctx, a, iow2, nwin, "k_filter_wide2"));
@@ -3085,17 +3381,16 @@ namespace sedef {
 namespace {
 
 constexpr int kServeMaxSlots = 64;
-// One CTA per SM of 256 threads (16 K registers) and ~62 KB of shared
+// One CTA per SM of 256 threads (16 K registers) and ~30 KB of shared
 // memory: the rest of every SM stays free for the admission and finishing
 // kernels (the radix sort's scatter alone takes ~39 K registers per CTA),
 // which would otherwise wait for the persistent kernel to leave.
-constexpr int kServeTPB = 256, kServeLCap = 2048, kServeGCap = 512, kServeSlots = 16384;
-using ServeSmem = FastSmemT<kServeTPB, kServeLCap, kServeGCap, kServeSlots>;
-// Windows with more hits than this go to the slot's wide list before their
-// hits are enumerated; the finishing call runs the wide tier (512 threads,
-// 32,768 counters) over them as an ordinary launch beside k_serve, as the
-// first tier of a whole-genome pass hands them on.
-constexpr uint32_t kServeHlim = 2 * kSlots;
+constexpr int kServeTPB = kCThreads;
+using ServeSmem = CtaSmemT<CtaNarrow>;
+// Windows with more posting entries than the shape keeps go to the slot's
+// wide list before they are read; the finishing call runs the broad CTA tier
+// over them as an ordinary launch beside k_serve, as the narrow one of a
+// whole-genome pass hands them on.
 // Finishing calls that may run at once (each on its own stream and context).
 constexpr int kServeFinishers = 5;
 
@@ -3117,7 +3412,7 @@ struct ServeCtl {
 struct SlotDev {
   FArgs a;              // the slot's query, windows and outputs
   unsigned int* done;   // windows finished (reset at admission)
-  uint32_t* wide_list;  // windows with more hits than k_serve keeps (for the wide tier)
+  uint32_t* wide_list;  // windows with more hits than k_serve keeps (for the broad CTA tier)
   unsigned int* wide_count;
   uint32_t* mid_list;   // windows k_serve could not hold (for the 8,192-hit tier)
   unsigned int* mid_count;
@@ -3149,7 +3444,6 @@ __global__ void __launch_bounds__(kServeTPB) k_serve(ServeArgs sv) {
   ServeSmem& S = *reinterpret_cast<ServeSmem*>(smem_raw);
   __shared__ long long s_item;
   __shared__ unsigned int s_slot, s_window;
-  for (int x = threadIdx.x; x < kQCap * (kServeTPB / 32); x += blockDim.x) (&S.cnt[0][0])[x] = 0;
   while (true) {
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -3195,10 +3489,9 @@ __global__ void __launch_bounds__(kServeTPB) k_serve(ServeArgs sv) {
     io.out_count = sd.mid_count;
     io.next = nullptr;
     io.stats = 1;
-    io.hlim = kServeHlim;
     io.wide_list = sd.wide_list;
     io.wide_count = sd.wide_count;
-    fast_window<kServeTPB, kServeLCap, kServeGCap, kServeSlots>(sd.a, io, S, (int64_t)s_window);
+    cta_window(sd.a, io, S, (int64_t)s_window);
     __syncthreads();
     if (threadIdx.x == 0) {
       __threadfence();  // this window's runs and hand-overs before its count
@@ -3464,7 +3757,7 @@ int sedef_server_create(sedef_ctx* ctx, const uint64_t* d_trec, const uint64_t* 
   // An SM splits its unified L1 / shared memory when a CTA arrives on an
   // idle SM and keeps the split while any CTA stays.  The persistent kernel
   // stays, so it asks for the largest shared-memory split: the other
-  // streams' kernels then find 228 - 63 KB per SM (the large refine kernel
+  // streams' kernels then find 228 - 30 KB per SM (the large refine kernel
   // takes 125 KB) instead of waiting for the persistent kernel to leave.
   if (cudaFuncSetAttribute(k_serve, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)sizeof(ServeSmem)) != cudaSuccess ||
@@ -3706,14 +3999,14 @@ int sedef_server_finish(sedef_server* srv, int32_t slot, sedef_cand_t* h_cands, 
   int64_t nc = 0;
   if (L.nwin > 0) {
     {
-      // the windows k_serve handed on for their many hits: the wide tier,
+      // the windows k_serve handed on for their many hits: the broad tier,
       // as an ordinary launch beside k_serve; what it cannot hold, and what
       // k_serve could not hold, goes through the 8,192-hit wide tier, and
       // what that cannot hold joins the slot's overflow list
       StageScope stage(c, "filter");
       TierIO iow{L.wl, (const unsigned int*)(L.counters + 14), L.ml,
                  (unsigned int*)(L.counters + 16), (unsigned int*)(L.counters + 15), 1};
-      int wst = kTierWide(c, L.a, iow, L.nwin, "k_filter_wide");
+      int wst = launch_cta_tier<CtaBroad>(c, L.a, iow, L.nwin, "k_filter_wide");
       TierIO iom{L.ml, (const unsigned int*)(L.counters + 16), L.ov,
                  (unsigned int*)(L.counters + 1), (unsigned int*)(L.counters + 17), 1};
       if (wst == SEDEF_OK) wst = kTierWideMid(c, L.a, iom, L.nwin, "k_filter_widemid");

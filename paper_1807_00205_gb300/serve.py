@@ -8,10 +8,10 @@ library's server (sedef_server_*).  A persistent filter kernel drains a work
 queue of query windows; an admission thread moves waiting requests into free
 request slots as slots free up (the slots are sized once, from free device
 memory), so a request that arrives while others are on the GPU joins the
-running kernel at once.  The kernel keeps the windows with at most 4,096
-hits and hands the heavier ones on; a completion thread polls for requests
+running kernel at once.  The kernel keeps the windows with at most 16,384
+posting entries and hands the heavier ones on; a completion thread polls for requests
 whose windows are done and passes each to one of five finishing threads,
-which run the rest on their own streams (the wide tier over the handed-on
+which run the rest on their own streams (the broad tier over the handed-on
 windows, the global path, refine, chaining, merging) while the kernel keeps
 filtering the others.
 
