@@ -137,6 +137,20 @@ __device__ __forceinline__ int block_exclusive_sum(int v, int* tmp, int* total) 
   return r;
 }
 
+// Status words of a decoupled look-back: a word holds its flag and its value,
+// and nothing else is read after it, so its accesses need no ordering (an
+// acquire load throws away the SM's L1, a release store waits for the CTA's
+// earlier writes).
+__device__ __forceinline__ unsigned long long ld_relaxed_gpu(const unsigned long long* p) {
+  unsigned long long v;
+  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+  return v;
+}
+
+__device__ __forceinline__ void st_relaxed_gpu(unsigned long long* p, unsigned long long v) {
+  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+
 // First index in [lo, hi) of a sorted uint64 array whose value is >= key
 // under the projection proj.
 template <typename F>
@@ -291,6 +305,12 @@ void* host_buf(sedef_ctx* ctx, Planned* pl, size_t bytes);
 int plan_check(sedef_ctx* ctx, Planned* pl, const uint32_t* d_count, int64_t cap, int which);
 int plan_check64(sedef_ctx* ctx, Planned* pl, const unsigned long long* d_count, int64_t cap,
                  int which);
+// Bits that hold every value below n.
+inline int bits_below(int64_t n) {
+  int b = 1;
+  while (b < 63 && (int64_t(1) << b) < n) ++b;
+  return b;
+}
 // m(s) for s in [0, smax] from the parameters' tau (Section 3.1).
 void mtable(const sedef_params* p, int32_t* m, int smax, double* tau_out);
 int launch_pack(sedef_ctx* ctx, const uint8_t* seq, int64_t n, uint32_t* packed, uint32_t* mask,
@@ -356,6 +376,11 @@ int64_t ctx_scratch_limit(sedef_ctx* ctx);  // sedef_set_scratch_limit's cap (-1
 void ctx_pool_restore(sedef_ctx* ctx, const std::vector<char>& used_before);
 void* ctx_host(sedef_ctx* ctx, size_t bytes);  // pinned host scratch
 int ctx_device(sedef_ctx* ctx);
+// The word (device view) that a kernel sets when one of its bounded waits
+// gives up, and the check that reports it (SEDEF_ERR_TIMEOUT) once the
+// context's stream has been synchronized.
+int* ctx_wait_flag(sedef_ctx* ctx);
+int ctx_check_waits(sedef_ctx* ctx);
 int ctx_sm_count(sedef_ctx* ctx);
 void ctx_set_stats(sedef_ctx* ctx, const int64_t* v, int n);  // last sedef_filter call
 void ctx_set_anchor_total(sedef_ctx* ctx, int64_t a);         // last sedef_chain call

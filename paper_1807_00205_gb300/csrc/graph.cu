@@ -194,6 +194,7 @@ int sedef_graph_wait(sedef_graph* g, int64_t* h_need) {
   if (!g) return fail(SEDEF_ERR_INVALID, "sedef_graph_wait: no graph");
   SEDEF_CUDA(cudaSetDevice(ctx_device(g->ctx)));
   SEDEF_CUDA(cudaStreamSynchronize(g->last ? g->last : g->stream));
+  SEDEF_TRY(ctx_check_waits(g->ctx));
   uint32_t flags = 0;
   std::memcpy(&flags, g->h_block, 4);
   unsigned long long need[8];

@@ -392,10 +392,10 @@ __global__ void k_root_flags(const int32_t* parent, int64_t n, uint32_t* flag, c
   if (x < n) flag[x] = (x < live_n(n, dn) && parent[x] == (int32_t)x) ? 1u : 0u;
 }
 
-// Candidate keys: primary (q0 << 32 | t0); the tie order (o, q1, t1) is
-// applied by k_fix_ties after the primary sort.
-__global__ void k_cand_emit(MergeArgs a, const Agg* agg, const uint32_t* pos, sedef_cand_t* tmp,
-                            uint64_t* key, int64_t ccap) {
+// Candidate keys: primary (q0, t0), tbits hold every target position; the tie
+// order (o, q1, t1) is applied by k_cand_final after the primary sort.
+__global__ void k_cand_emit(MergeArgs a, const Agg* agg, const uint32_t* pos, int tbits,
+                            sedef_cand_t* tmp, uint64_t* key, int64_t ccap) {
   a.n = live_n(a.n, a.dn);
   const int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (x >= a.n || a.parent[x] != (int32_t)x || (int64_t)pos[x] >= ccap) return;
@@ -413,7 +413,7 @@ __global__ void k_cand_emit(MergeArgs a, const Agg* agg, const uint32_t* pos, se
   d.nchains = g.count;
   d.reserved = 0;
   tmp[pos[x]] = d;
-  key[pos[x]] = ((uint64_t)g.q0 << 32) | g.t0;
+  key[pos[x]] = ((uint64_t)g.q0 << tbits) | g.t0;
 }
 
 __device__ __forceinline__ bool cand_less(const sedef_cand_t& x, const sedef_cand_t& y) {
@@ -466,9 +466,11 @@ __global__ void k_cand_final(const sedef_cand_t* tmp, const uint32_t* perm, cons
   }
 }
 
-__global__ void k_chain_keys(const sedef_chain_t* c, int64_t n, uint64_t* key, const uint32_t* dn) {
+// (o, q0); qbits hold every query position.
+__global__ void k_chain_keys(const sedef_chain_t* c, int64_t n, int qbits, uint64_t* key,
+                             const uint32_t* dn) {
   const int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (x < live_n(n, dn)) key[x] = ((uint64_t)c[x].o << 32) | c[x].q0;
+  if (x < live_n(n, dn)) key[x] = ((uint64_t)c[x].o << qbits) | c[x].q0;
 }
 
 int grid_of(int64_t n, int b) { return (int)((n + b - 1) / b); }
@@ -629,8 +631,10 @@ int run_merge(sedef_ctx* ctx, const sedef_chain_t* chains, int64_t n, const int6
   uint32_t* pos = (uint32_t*)ctx_alloc(ctx, (size_t)(n + 1) * 4);
   if (!key || !skey || !perm || !parent || !agg || !flag || !pos) return SEDEF_ERR_OOM;
   const int g = grid_of(n, 256);
-  SEDEF_KERNEL(ctx, "k_chain_keys", k_chain_keys<<<g, 256, 0, st>>>(chains, n, key, dn));
-  SEDEF_TRY(radix_sort_u64(ctx, key, nullptr, skey, perm, n, 0, 33, dn));
+  // sort keys of only as many bits as the positions have
+  const int qbits = bits_below(h_qoff[nqseq] + 1), tbits = bits_below(h_toff[ntseq] + 1);
+  SEDEF_KERNEL(ctx, "k_chain_keys", k_chain_keys<<<g, 256, 0, st>>>(chains, n, qbits, key, dn));
+  SEDEF_TRY(radix_sort_u64(ctx, key, nullptr, skey, perm, n, 0, qbits + 1, dn));
   MergeArgs a;
   a.ch = chains;
   a.n = n;
@@ -668,14 +672,14 @@ int run_merge(sedef_ctx* ctx, const sedef_chain_t* chains, int64_t n, const int6
   uint64_t* cskey = (uint64_t*)ctx_alloc(ctx, (size_t)nc * 8);
   uint32_t* cperm = (uint32_t*)ctx_alloc(ctx, (size_t)nc * 4);
   if (!tmp || !ckey || !cskey || !cperm) return SEDEF_ERR_OOM;
-  SEDEF_KERNEL(ctx, "k_cand_emit", k_cand_emit<<<g, 256, 0, st>>>(a, agg, pos, tmp, ckey, nc));
-  SEDEF_TRY(radix_sort_u64(ctx, ckey, nullptr, cskey, cperm, nc, 0, 64, dnc));
+  SEDEF_KERNEL(ctx, "k_cand_emit", k_cand_emit<<<g, 256, 0, st>>>(a, agg, pos, tbits, tmp, ckey, nc));
+  SEDEF_TRY(radix_sort_u64(ctx, ckey, nullptr, cskey, cperm, nc, 0, qbits + tbits, dnc));
   SEDEF_KERNEL(ctx, "k_cand_final",
                k_cand_final<<<grid_of(nc, 256), 256, 0, st>>>(tmp, cperm, cskey, nc, dq, dt, cands,
                                                               dnc));
   if (pl) return SEDEF_OK;
   SEDEF_CUDA(cudaStreamSynchronize(st));
-  return SEDEF_OK;
+  return ctx_check_waits(ctx);
 }
 
 }  // namespace sedef

@@ -1872,18 +1872,18 @@ __global__ void k_windows(const uint64_t* __restrict__ qrec, int64_t nq,
   wseq[w] = lo;
 }
 
-// Sort keys of the runs: (window index, o, j_a).  part 0: the whole key
-// when it fits 64 bits; part 1: j_a alone and part 2: (window, o), for a
-// two-pass stable sort otherwise.
+// Sort keys of the runs: (window index, o, j_a), tbits hold every j_a.  part
+// 0: the whole key when it fits 64 bits; part 1: j_a alone and part 2:
+// (window, o), for a two-pass stable sort otherwise.
 __global__ void k_run_keys(const sedef_run_t* runs, int64_t n, const int64_t* qseq, int nqseq,
-                           const int64_t* wbase, int step, int part, uint64_t* keys,
+                           const int64_t* wbase, int step, int part, int tbits, uint64_t* keys,
                            const uint32_t* dn) {
   const int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (x >= live_n(n, dn)) return;
   const sedef_run_t r = runs[x];
   const int sq = seq_of(qseq, nqseq, r.i);
   const uint64_t widx = (uint64_t)(wbase[sq] + ((int64_t)r.i - qseq[sq]) / step);
-  if (part == 0) keys[x] = (widx << 33) | ((uint64_t)r.o << 32) | r.j_a;
+  if (part == 0) keys[x] = (((widx << 1) | r.o) << tbits) | r.j_a;
   else if (part == 1) keys[x] = r.j_a;
   else keys[x] = (widx << 1) | r.o;
 }
@@ -2915,11 +2915,12 @@ int order_and_refine(sedef_ctx* ctx, const FArgs& a, const Derived& D, int nqseq
   const int tb = (int)((total + 255) / 256);
   int wb = 1;
   while ((int64_t(1) << wb) < nwin) ++wb;
-  if (33 + wb <= 64) {
+  const int tbits = bits_below(a.ttotal + 1);
+  if (tbits + 1 + wb <= 64) {
     SEDEF_KERNEL(ctx, "k_run_keys",
-                 k_run_keys<<<tb, 256, 0, st>>>(raw, total, a.qseq, nqseq, d_wbase, D.step, 0, keys,
-                                                druns));
-    SEDEF_TRY(radix_sort_u64(ctx, keys, nullptr, skeys, perm, total, 0, 33 + wb, druns));
+                 k_run_keys<<<tb, 256, 0, st>>>(raw, total, a.qseq, nqseq, d_wbase, D.step, 0, tbits,
+                                                keys, druns));
+    SEDEF_TRY(radix_sort_u64(ctx, keys, nullptr, skeys, perm, total, 0, tbits + 1 + wb, druns));
   } else {
     // stable two-pass order: by j_a, then by (window, o)
     uint32_t* perm1 = (uint32_t*)ctx_alloc(ctx, (size_t)total * 4);
@@ -2927,12 +2928,12 @@ int order_and_refine(sedef_ctx* ctx, const FArgs& a, const Derived& D, int nqseq
     uint64_t* k2 = (uint64_t*)ctx_alloc(ctx, (size_t)total * 8);
     if (!perm1 || !perm2 || !k2) return SEDEF_ERR_OOM;
     SEDEF_KERNEL(ctx, "k_run_keys",
-                 k_run_keys<<<tb, 256, 0, st>>>(raw, total, a.qseq, nqseq, d_wbase, D.step, 1, keys,
-                                                druns));
-    SEDEF_TRY(radix_sort_u64(ctx, keys, nullptr, skeys, perm1, total, 0, 32, druns));
+                 k_run_keys<<<tb, 256, 0, st>>>(raw, total, a.qseq, nqseq, d_wbase, D.step, 1, tbits,
+                                                keys, druns));
+    SEDEF_TRY(radix_sort_u64(ctx, keys, nullptr, skeys, perm1, total, 0, tbits, druns));
     SEDEF_KERNEL(ctx, "k_run_keys",
-                 k_run_keys<<<tb, 256, 0, st>>>(raw, total, a.qseq, nqseq, d_wbase, D.step, 2, keys,
-                                                druns));
+                 k_run_keys<<<tb, 256, 0, st>>>(raw, total, a.qseq, nqseq, d_wbase, D.step, 2, tbits,
+                                                keys, druns));
     SEDEF_KERNEL(ctx, "k_permute_u64",
                  k_permute_u64<<<tb, 256, 0, st>>>(keys, perm1, total, k2, druns));
     SEDEF_TRY(radix_sort_u64(ctx, k2, nullptr, skeys, perm2, total, 0, wb + 1, druns));
@@ -3349,8 +3350,7 @@ int run_filter(sedef_ctx* ctx, const uint64_t* qrec, int64_t nq, const int64_t* 
                               (int64_t)(h_cnt[3] & 0xFFFFFFFFull), slow_hits_total};
     ctx_set_stats(ctx, stats, 7);
   }
-  SEDEF_CUDA(cudaStreamSynchronize(st));
-  return SEDEF_OK;
+  return ctx_check_waits(ctx);
 }
 
 }  // namespace sedef

@@ -171,19 +171,6 @@ constexpr unsigned long long kLbAggregate = 1ull << 62, kLbPrefix = 2ull << 62;
 constexpr unsigned long long kLbValue = (1ull << 62) - 1;
 constexpr unsigned int kLbSpins = 1u << 20;  // polls of one predecessor before giving up
 
-// A status word holds its flag and its value, and nothing else is read after
-// it, so its accesses need no ordering (an acquire load throws away the SM's
-// L1, a release store waits for the CTA's earlier writes).
-__device__ __forceinline__ unsigned long long ld_status(const unsigned long long* p) {
-  unsigned long long v;
-  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-  return v;
-}
-
-__device__ __forceinline__ void st_status(unsigned long long* p, unsigned long long v) {
-  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
-}
-
 // Records before tile `tile`; warp 0 of the CTA calls it once per tile.  The
 // warp reads the status of the 256 tiles below its window at once (eight
 // independent loads per lane: as many tiles are in flight, so a narrower
@@ -196,7 +183,7 @@ __device__ long long look_back(const LookBack& lb, int64_t tile, int64_t ntiles,
   const int lane = threadIdx.x & 31;
   long long before = 0;
   if (tile > 0) {
-    if (lane == 0) st_status(lb.status + tile, kLbAggregate | count);
+    if (lane == 0) st_relaxed_gpu(lb.status + tile, kLbAggregate | count);
     int64_t j = tile - 1;  // the walk's top tile
     unsigned int spins = 0;
     bool done = false;
@@ -206,7 +193,7 @@ __device__ long long look_back(const LookBack& lb, int64_t tile, int64_t ntiles,
       for (int x = 0; x < kWide; ++x) {
         const int64_t at = j - x * 32 - lane;
         // below tile 0 reads as a published prefix of zero
-        v[x] = at >= 0 ? ld_status(lb.status + at) : kLbPrefix;
+        v[x] = at >= 0 ? ld_relaxed_gpu(lb.status + at) : kLbPrefix;
       }
 #pragma unroll
       for (int x = 0; x < kWide; ++x) {
@@ -234,7 +221,7 @@ __device__ long long look_back(const LookBack& lb, int64_t tile, int64_t ntiles,
     for (int d = 16; d > 0; d >>= 1) before += __shfl_xor_sync(0xffffffffu, before, d);
   }
   if (lane == 0) {
-    st_status(lb.status + tile, kLbPrefix | ((unsigned long long)before + count));
+    st_relaxed_gpu(lb.status + tile, kLbPrefix | ((unsigned long long)before + count));
     if (tile == ntiles - 1) *lb.total = (unsigned long long)before + count;
   }
   return before;

@@ -267,3 +267,22 @@ def test_graph_record_overflow(ctx, mode):
     gr.close()
     out = ctx.selfsearch_graph(d, g.offsets, p, caps={k: 1 for k in binding.CAP_NAMES}).outputs()
     assert np.array_equal(run_rows(out["runs"]), run_rows(eager["runs"]))
+
+
+@pytest.mark.parametrize("n", [1, 31, 257, 4095, 4096, 4097, 8192, 40_961, 1_300_003])
+@pytest.mark.parametrize("k", [2, 4, 8, 11, 13])
+def test_index_sort_sizes(ctx, n, k):
+    """The sort below, at and past one CTA's keys, over one to four passes, with digits that are
+    spread, skewed and all alike; equal hashes stay by position."""
+    torch = need_gpu()
+    rng = np.random.default_rng(n + k)
+    top = 4 ** k
+    for h in (rng.integers(0, top, n), (rng.random(n) ** 8 * top).astype(np.int64),
+              np.full(n, top - 1), np.sort(rng.integers(0, top, n))[::-1]):
+        rec = (h.astype(np.uint64) << np.uint64(33)) | (np.arange(n, dtype=np.uint64) * np.uint64(3) << np.uint64(1)) \
+            | rng.integers(0, 2, n).astype(np.uint64)
+        srt, off = ctx.sedef_index(to_dev(rec.view(np.int64)), binding.params(k=k))
+        want = rec[np.argsort(h, kind="stable")]
+        assert np.array_equal(srt.cpu().numpy().view(np.uint64), want)
+        cnt = np.concatenate([[0], np.cumsum(np.bincount(h, minlength=top))])
+        assert bool((off.cpu().to(torch.int64) == torch.from_numpy(cnt)).all())
