@@ -258,6 +258,24 @@ __host__ __device__ __forceinline__ uint32_t pos_gallop_forward(const uint64_t* 
   return hi;
 }
 
+// First index in [0, n) of position-sorted records whose position is >= key
+// (n when none), by a whole warp: 32 probes at a time, so a gigabase's
+// records take 6 dependent reads instead of 28.
+__device__ __forceinline__ int64_t warp_lower_pos(const uint64_t* rec, int64_t n, uint32_t key) {
+  int64_t lo = 0, hi = n;  // positions < key before lo, >= key from hi on
+  const int lane = lane_id();
+  while (hi > lo) {
+    const int64_t step = (hi - lo + 31) >> 5;
+    const int64_t at = lo + lane * step;
+    const uint32_t p = rec_pos(rec[at < hi ? at : lo]);
+    const int c = __popc(__ballot_sync(0xffffffffu, at < hi && p < key));  // the first c probes
+    const int64_t next = lo + c * step;
+    if (c > 0) lo += (c - 1) * step + 1;
+    if (next < hi) hi = next;
+  }
+  return lo;
+}
+
 // Index of the sequence containing global position pos (offsets has nseq+1
 // entries, offsets[0] = 0).
 __device__ __forceinline__ int seq_of(const int64_t* off, int nseq, int64_t pos) {

@@ -1,15 +1,18 @@
 // a7: chaining of each kept seed's minimizer anchors (Section 3.3) and the
 // merge of chains into SD candidates.
 //
-// Chain: one warp per kept run.  Anchors are enumerated straight from the
-// index: each query minimizer of the window searches its posting list for
-// the run's target span (an interpolated search, then a short gallop), so
-// anchors come out sorted by (p, t') without a sort (t' = t for o = 0; for
-// o = 1 the posting list is walked backwards).
-// The DP visits anchors in order; for anchor a the 32 lanes scan the
-// predecessors b (only those with p_b >= p_a - gap_max) and a warp max-reduce
-// over (f_b + 1, b) picks the predecessor with the larger count, then the
-// later index.
+// Chain: one warp per kept run finds its anchors, runs the DP over them in
+// shared memory and writes the chain (k_chain_seeds).  In a self-search the
+// target records by position are the query records, so the anchors are a join
+// of two contiguous stretches: the window's records go into a hash table and
+// the target span's records probe it.  Otherwise each query minimizer searches
+// its posting list for the target span (an interpolated search, then a short
+// gallop).  The anchors' order is (p, t') (t' = t for o = 0; for o = 1 the
+// target axis is reversed).  The DP settles 32 anchors at a time, one per
+// lane, from every earlier anchor within gap_max: the predecessor with the
+// larger count, then the later one.  Seeds past the shared-memory sizes take
+// three kernels instead (k_anchor_count, k_anchor_fill, k_chain_dp: anchors
+// in device memory, the DP an anchor at a time).
 //
 // Merge: chains sorted by (o, q0); every chain links to the following chains
 // whose query interval starts before its own ends; links are united with a
@@ -44,7 +47,10 @@ struct ChainArgs {
   const uint32_t* dnt = nullptr;
   int64_t acap = 0;
   uint32_t* flags = nullptr;
-  unsigned long long* atotal = nullptr;  // exact anchor total (planned pass)
+  unsigned long long* atotal = nullptr;  // exact anchor total
+  // seeds past k_chain_seeds' sizes: run indices and their number
+  uint32_t* big = nullptr;
+  uint32_t* nbig = nullptr;
 };
 
 // The chain DP is quadratic in a seed's anchors; a seed inside an unmasked
@@ -104,15 +110,241 @@ __device__ __forceinline__ void window_range(const ChainArgs& a, int64_t i, int6
   *qb = lower_bound_by(a.qrec, *qa, a.nq, (uint64_t)(i + a.span + 1), pos_of);
 }
 
-// Anchors per kept run (0 for runs that are not kept).
+// What k_chain_seeds keeps of a seed in shared memory.
+constexpr int kSeedWarps = 8;
+constexpr int kSeedQ = 256;            // query records
+constexpr int kSeedTab = 2 * kSeedQ;   // hash-table slots
+constexpr int kSeedA = 256;            // anchors
+constexpr int kSeedTBits = 22;         // target span below 2^22 bases
+struct alignas(16) SeedSmem {
+  uint32_t tab[kSeedTab];    // hash + 1 of a query record (equal ones each have a slot)
+  uint16_t info[kSeedTab];   // its offset in the window << 1 | strand
+  uint32_t anchor[kSeedA];   // (p - i) << kSeedTBits | t' - lowest t', sorted
+  uint16_t f[kSeedA];        // anchors of the best chain that ends here
+  uint16_t first[kSeedA];    // its first anchor
+  int n;
+};
+
+// Bound by the latency of its two record searches and, per seed, a thousand
+// or so instructions.  Count, fill and DP as kernels of their own searched
+// the records with one lane, the postings of every query record twice (in
+// memory the size of the index) and kept the DP's state in device memory:
+// 626 k seeds of a 200-genome batch 8.3 -> 2.6 ms, a 240 Mbp assembly's 3.5 ->
+// 1.2 ms.
+template <bool kJoin>
+__global__ void __launch_bounds__(32 * kSeedWarps) k_chain_seeds(ChainArgs a, sedef_chain_t* out) {
+  resolve(a);
+  __shared__ SeedSmem smem[kSeedWarps];
+  SeedSmem& S = smem[threadIdx.x >> 5];
+  const int lane = lane_id();
+  const unsigned lt = lanemask_lt();
+  unsigned long long anchors = 0;
+  const int64_t nw = (int64_t)gridDim.x * kSeedWarps;
+  for (int64_t r = (int64_t)blockIdx.x * kSeedWarps + (threadIdx.x >> 5); r < a.nruns; r += nw) {
+    const sedef_run_t run = a.runs[r];
+    if (!run.keep) {
+      if (lane == 0) out[r].score = 0;
+      continue;
+    }
+    const uint32_t i = run.i, tlo = run.j_a, thi = run.j_b + (uint32_t)a.span;
+    const uint32_t o = run.o;
+    const int64_t qa = warp_lower_pos(a.qrec, a.nq, i);
+    bool big = thi - tlo >= (1u << kSeedTBits);
+    int A = 0;
+    __syncwarp();
+    if (kJoin) {
+      // ---- the window's records into the table
+      for (int x = lane; x < kSeedTab / 4; x += 32)
+        reinterpret_cast<uint4*>(S.tab)[x] = make_uint4(0, 0, 0, 0);
+      if (lane == 0) S.n = 0;
+      const int64_t ta = warp_lower_pos(a.qrec, a.nq, tlo);
+      __syncwarp();
+      int c = 0;
+      for (int64_t x = qa; !big; x += 32) {
+        const uint64_t q = x + lane < a.nq ? a.qrec[x + lane] : 0ull;
+        const bool in = x + lane < a.nq && rec_pos(q) - i <= (uint32_t)a.span;
+        c += __popc(__ballot_sync(0xffffffffu, in));
+        if (c > kSeedQ) {
+          big = true;
+          break;
+        }
+        if (in) {
+          const uint32_t h = rec_hash(q);
+          if (!(a.max_occ > 0 && (int)(a.toff[h + 1] - a.toff[h]) > a.max_occ)) {
+            uint32_t slot = (h * 0x9E3779B1u) >> 23;
+            while (atomicCAS(&S.tab[slot], 0u, h + 1u) != 0u) slot = (slot + 1u) & (kSeedTab - 1);
+            S.info[slot] = (uint16_t)(((rec_pos(q) - i) << 1) | rec_strand(q));
+          }
+        }
+        if (!__all_sync(0xffffffffu, in)) break;
+      }
+      __syncwarp();
+      // ---- the target span's records probe it
+      for (int64_t x = ta; !big; x += 32) {
+        const uint64_t t = x + lane < a.nq ? a.qrec[x + lane] : 0ull;
+        const uint32_t p = rec_pos(t);
+        const bool in = x + lane < a.nq && p - tlo <= thi - tlo;
+        if (in && p - i > (uint32_t)a.span) {  // not in the window's own span
+          const uint32_t h = rec_hash(t);
+          for (uint32_t slot = (h * 0x9E3779B1u) >> 23; S.tab[slot] != 0u;
+               slot = (slot + 1u) & (kSeedTab - 1)) {
+            if (S.tab[slot] != h + 1u) continue;
+            const uint32_t q = S.info[slot];
+            if (((q ^ rec_strand(t)) & 1u) != o) continue;
+            const int at = atomicAdd(&S.n, 1);
+            if (at < kSeedA) S.anchor[at] = ((q >> 1) << kSeedTBits) | (o ? thi - p : p - tlo);
+          }
+        }
+        __syncwarp();
+        const int n = __shfl_sync(0xffffffffu, S.n, 0);  // the same answer for every lane
+        if (n > kSeedA || !__all_sync(0xffffffffu, in)) break;
+      }
+      __syncwarp();
+      A = S.n;
+      big |= A > kSeedA;
+      if (!big && A > 1) {
+        // order by (p, t')
+        int np = 2;
+        while (np < A) np <<= 1;
+        if (np <= 32) {
+          uint32_t v = lane < A ? S.anchor[lane] : 0xFFFFFFFFu;
+          for (int size = 2; size <= np; size <<= 1)
+            for (int stride = size >> 1; stride > 0; stride >>= 1) {
+              const uint32_t w = __shfl_xor_sync(0xffffffffu, v, stride);
+              v = ((lane & size) == 0) == ((lane & stride) == 0) ? min(v, w) : max(v, w);
+            }
+          if (lane < A) S.anchor[lane] = v;
+        } else {
+          for (int x = A + lane; x < np; x += 32) S.anchor[x] = 0xFFFFFFFFu;
+          __syncwarp();
+          for (int size = 2; size <= np; size <<= 1)
+            for (int stride = size >> 1; stride > 0; stride >>= 1) {
+              for (int t = lane; t < (np >> 1); t += 32) {
+                const int lo = ((t & ~(stride - 1)) << 1) | (t & (stride - 1)), hi = lo + stride;
+                const uint32_t v = S.anchor[lo], w = S.anchor[hi];
+                if ((v > w) == ((lo & size) == 0)) {
+                  S.anchor[lo] = w;
+                  S.anchor[hi] = v;
+                }
+              }
+              __syncwarp();
+            }
+        }
+        __syncwarp();
+      }
+    } else {
+      // ---- postings of the window's records inside the target span, in order
+      for (int64_t x = qa; !big; x += 32) {
+        const uint64_t q = x + lane < a.nq ? a.qrec[x + lane] : 0ull;
+        const bool in = x + lane < a.nq && rec_pos(q) - i <= (uint32_t)a.span;
+        uint32_t b0 = 0, b1 = 0;
+        int c = 0;
+        if (in) {
+          record_postings(a, run, q, &b0, &b1);
+          c = record_anchors(a, run, q, b0, b1, [](int, uint32_t, uint32_t) {});
+        }
+        const int inc = warp_inclusive_sum(min(c, kSeedA + 1));
+        const int to = A + inc - c;
+        A += __shfl_sync(0xffffffffu, inc, 31);
+        if (A > kSeedA) {
+          big = true;
+        } else if (c > 0) {
+          record_anchors(a, run, q, b0, b1, [&](int rank, uint32_t p, uint32_t t) {
+            S.anchor[to + rank] = ((p - i) << kSeedTBits) | (o ? thi - t : t - tlo);
+          });
+        }
+        if (!__all_sync(0xffffffffu, in)) break;
+      }
+      __syncwarp();
+    }
+    if (big) {
+      if (lane == 0) {
+        out[r].score = 0;
+        a.big[atomicAdd(a.nbig, 1u)] = (uint32_t)r;
+      }
+      continue;
+    }
+    anchors += A;
+    // ---- the DP, 32 anchors at a time
+    unsigned long long be = 0;  // best end: larger f, then the earlier anchor; f << 32 | ~index
+    for (int t0 = 0; t0 < A; t0 += 32) {
+      const int x = t0 + lane;
+      const uint32_t ax = x < A ? S.anchor[x] : 0u;
+      const int p = (int)(ax >> kSeedTBits), t = (int)(ax & ((1u << kSeedTBits) - 1u));
+      int bf = 0, bb = -1;  // best predecessor's count and index
+      auto look = [&](int pb, int tb, int f, int b) {
+        const int dp = p - pb, dt = t - tb, dd = dp - dt;
+        if (dp > 0 && dt > 0 && dp <= a.gap_max && dt <= a.gap_max && dd <= a.diag_max &&
+            -dd <= a.diag_max && f >= bf) {  // the later of equals
+          bf = f;
+          bb = b;
+        }
+      };
+      for (int b = 0; b < t0; ++b) {
+        const uint32_t v = S.anchor[b];
+        look((int)(v >> kSeedTBits), (int)(v & ((1u << kSeedTBits) - 1u)), S.f[b], b);
+      }
+      const int m = min(32, A - t0);
+      int my_first = bb >= 0 ? S.first[bb] : x;
+      for (int y = 0; y < m; ++y) {
+        const int fy = __shfl_sync(0xffffffffu, bf + 1, y), py = __shfl_sync(0xffffffffu, p, y);
+        const int ty = __shfl_sync(0xffffffffu, t, y), sy = __shfl_sync(0xffffffffu, my_first, y);
+        if (lane > y) {
+          const int before = bb;
+          look(py, ty, fy, t0 + y);
+          if (bb != before) my_first = sy;
+        }
+      }
+      if (x < A) {
+        S.f[x] = (uint16_t)(bf + 1);
+        S.first[x] = (uint16_t)my_first;
+        const unsigned long long v = ((unsigned long long)(bf + 1) << 32) | (0xFFFFFFFFu - (uint32_t)x);
+        if (v > be) be = v;
+      }
+      __syncwarp();
+    }
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) {
+      const unsigned long long v = __shfl_xor_sync(0xffffffffu, be, d);
+      if (v > be) be = v;
+    }
+    if (lane == 0) {
+      sedef_chain_t c;
+      c.i = i;
+      c.qseq = c.q0 = c.q1 = c.tseq = c.t0 = c.t1 = 0;
+      c.score = 0;
+      c.s = run.s;
+      c.o = o;
+      c.reserved = 0;
+      const int score = (int)(be >> 32);
+      if (A > 0 && score >= a.mtab[run.s]) {
+        // a chain advances on both axes: its ends are its box
+        const uint32_t end = 0xFFFFFFFFu - (uint32_t)be;
+        const uint32_t e1 = S.anchor[end], e0 = S.anchor[S.first[end]];
+        const uint32_t tm = (1u << kSeedTBits) - 1u;
+        c.q0 = i + (e0 >> kSeedTBits);
+        c.q1 = i + (e1 >> kSeedTBits) + (uint32_t)a.k;
+        c.t0 = o ? thi - (e1 & tm) : tlo + (e0 & tm);
+        c.t1 = (o ? thi - (e0 & tm) : tlo + (e1 & tm)) + (uint32_t)a.k;
+        c.qseq = (uint32_t)seq_of(a.qseq, a.nqseq, i);
+        c.tseq = (uint32_t)seq_of(a.tseq, a.ntseq, tlo);
+        c.score = (uint16_t)score;
+      }
+      out[r] = c;
+    }
+  }
+  if (lane == 0 && anchors) atomicAdd(a.atotal, anchors);
+}
+
+// Anchors of the seeds k_chain_seeds left (big[0..nbig)).
 __global__ void k_anchor_count(ChainArgs a, uint32_t* count) {
   resolve(a);
   const int lane = lane_id();
-  const int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  if (r >= a.nruns) return;
-  const sedef_run_t run = a.runs[r];
-  int total = 0;
-  if (run.keep) {
+  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < (int64_t)*a.nbig;
+       r += nw) {
+    const sedef_run_t run = a.runs[a.big[r]];
+    int total = 0;
     int64_t qa = 0, qb = 0;
     if (lane == 0) window_range(a, run.i, &qa, &qb);
     qa = __shfl_sync(0xffffffffu, qa, 0);
@@ -124,60 +356,59 @@ __global__ void k_anchor_count(ChainArgs a, uint32_t* count) {
       total += record_anchors(a, run, q, b0, b1, [](int, uint32_t, uint32_t) {});
     }
     total = warp_sum(total);
-  }
-  if (lane == 0) {
-    count[r] = (uint32_t)total;
-    if (a.atotal && total) atomicAdd(a.atotal, (unsigned long long)total);
+    if (lane == 0) {
+      count[r] = (uint32_t)total;
+      if (total) atomicAdd(a.atotal, (unsigned long long)total);
+    }
   }
 }
 
-// Writes anchors as (p << 32 | t') at the run's offset, in (p, t') order.
+// Writes anchors as (p << 32 | t') at the seed's offset, in (p, t') order.
 __global__ void k_anchor_fill(ChainArgs a, const uint32_t* aoff, uint64_t* anchors) {
   resolve(a);
   const int lane = lane_id();
-  const int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  if (r >= a.nruns) return;
-  const sedef_run_t run = a.runs[r];
-  if (!run.keep) return;
-  // 32-bit offsets: a range that wraps or ends past the capacity is skipped
-  if (aoff[r + 1] < aoff[r] || (int64_t)aoff[r + 1] > a.acap ||
-      aoff[r + 1] - aoff[r] > (uint32_t)kMaxChainAnchors)
-    return;
-  int64_t qa = 0, qb = 0;
-  if (lane == 0) window_range(a, run.i, &qa, &qb);
-  qa = __shfl_sync(0xffffffffu, qa, 0);
-  qb = __shfl_sync(0xffffffffu, qb, 0);
-  const uint32_t tref = run.j_b + (uint32_t)a.span;
-  uint32_t base = aoff[r];
-  for (int64_t x0 = qa; x0 < qb; x0 += 32) {
-    const int64_t x = x0 + lane;
-    int c = 0;
-    uint64_t q = 0;
-    uint32_t b0 = 0, b1 = 0;
-    if (x < qb) {
-      q = a.qrec[x];
-      record_postings(a, run, q, &b0, &b1);
-      c = record_anchors(a, run, q, b0, b1, [](int, uint32_t, uint32_t) {});
+  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < (int64_t)*a.nbig;
+       r += nw) {
+    const sedef_run_t run = a.runs[a.big[r]];
+    // 32-bit offsets: a range that wraps or ends past the capacity is skipped
+    if (aoff[r + 1] < aoff[r] || (int64_t)aoff[r + 1] > a.acap ||
+        aoff[r + 1] - aoff[r] > (uint32_t)kMaxChainAnchors)
+      continue;
+    int64_t qa = 0, qb = 0;
+    if (lane == 0) window_range(a, run.i, &qa, &qb);
+    qa = __shfl_sync(0xffffffffu, qa, 0);
+    qb = __shfl_sync(0xffffffffu, qb, 0);
+    const uint32_t tref = run.j_b + (uint32_t)a.span;
+    uint32_t base = aoff[r];
+    for (int64_t x0 = qa; x0 < qb; x0 += 32) {
+      const int64_t x = x0 + lane;
+      int c = 0;
+      uint64_t q = 0;
+      uint32_t b0 = 0, b1 = 0;
+      if (x < qb) {
+        q = a.qrec[x];
+        record_postings(a, run, q, &b0, &b1);
+        c = record_anchors(a, run, q, b0, b1, [](int, uint32_t, uint32_t) {});
+      }
+      const int inc = warp_inclusive_sum(c);
+      const uint32_t my = base + (uint32_t)(inc - c);
+      if (x < qb && c > 0)
+        record_anchors(a, run, q, b0, b1, [&](int rank, uint32_t p, uint32_t t) {
+          const uint32_t tp = run.o ? tref - t : t;
+          anchors[my + rank] = ((uint64_t)p << 32) | tp;
+        });
+      base += (uint32_t)__shfl_sync(0xffffffffu, inc, 31);
     }
-    const int inc = warp_inclusive_sum(c);
-    const uint32_t my = base + (uint32_t)(inc - c);
-    if (x < qb && c > 0)
-      record_anchors(a, run, q, b0, b1, [&](int rank, uint32_t p, uint32_t t) {
-        const uint32_t tp = run.o ? tref - t : t;
-        anchors[my + rank] = ((uint64_t)p << 32) | tp;
-      });
-    base += (uint32_t)__shfl_sync(0xffffffffu, inc, 31);
   }
 }
 
-// DP over each kept run's anchors; writes the run's chain (score 0 = none).
-__global__ void k_chain_dp(ChainArgs a, const uint32_t* aoff, const uint64_t* anchors, int32_t* f,
-                           int32_t* pred, sedef_chain_t* out) {
-  resolve(a);
+// DP over each of these seeds' anchors; writes the run's chain (score 0 =
+// none).
+__device__ void chain_one(const ChainArgs& a, int64_t r, const uint32_t* aoff, const uint64_t* anchors,
+                          int32_t* f, int32_t* pred, sedef_chain_t* out) {
   const int lane = lane_id();
-  const int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  if (r >= a.nruns) return;
-  const sedef_run_t run = a.runs[r];
+  const sedef_run_t run = a.runs[a.big[r]];
   sedef_chain_t c;
   c.i = run.i;
   c.o = run.o;
@@ -188,12 +419,12 @@ __global__ void k_chain_dp(ChainArgs a, const uint32_t* aoff, const uint64_t* an
   const bool wrapped = aoff[r + 1] < A0;
   const bool over = wrapped || (int64_t)aoff[r + 1] > a.acap;
   const bool big = !wrapped && A > (uint32_t)kMaxChainAnchors;
-  if (run.keep && (over || big) && a.flags && lane == 0)
+  if ((over || big) && a.flags && lane == 0)
     atomicOr(a.flags, (over ? (uint32_t)kOverAnchors : 0u) | (big ? (uint32_t)kAnchorLimit : 0u));
-  if (!run.keep || A == 0 || over || big) {
+  if (A == 0 || over || big) {
     if (lane == 0) {
       c.qseq = c.q0 = c.q1 = c.tseq = c.t0 = c.t1 = 0;
-      out[r] = c;
+      out[a.big[r]] = c;
     }
     return;
   }
@@ -263,7 +494,15 @@ __global__ void k_chain_dp(ChainArgs a, const uint32_t* aoff, const uint64_t* an
   c.t0 = t0;
   c.t1 = t1;
   c.score = (score >= a.mtab[run.s]) ? (uint16_t)score : 0;
-  out[r] = c;
+  out[a.big[r]] = c;
+}
+
+__global__ void k_chain_dp(ChainArgs a, const uint32_t* aoff, const uint64_t* anchors, int32_t* f,
+                           int32_t* pred, sedef_chain_t* out) {
+  resolve(a);
+  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < (int64_t)*a.nbig; r += nw)
+    chain_one(a, r, aoff, anchors, f, pred, out);
 }
 
 __global__ void k_max_u32(const uint32_t* v, int64_t n, uint32_t* out) {
@@ -534,58 +773,80 @@ int run_chain(sedef_ctx* ctx, const sedef_run_t* runs, int64_t nruns, const uint
   a.self_mode = D.self_mode;
   a.gap_max = D.gap_max;
   a.diag_max = D.diag_max;
-  unsigned long long* atotal = nullptr;
   if (pl) {
     a.dnruns = pl->n_runs;
     a.dnq = pl->n_rec;
     a.dnt = pl->n_rec;
     a.flags = pl->flags;
-    atotal = (unsigned long long*)ctx_alloc(ctx, 8);
-    if (!atotal) return SEDEF_ERR_OOM;
-    SEDEF_CUDA(cudaMemsetAsync(atotal, 0, 8, st));
-    a.atotal = atotal;
   }
-
+  // [0] anchors of every seed, [1] seeds for the device-memory path, [2] the
+  // most anchors one of them has
+  unsigned long long* sums = (unsigned long long*)ctx_alloc(ctx, 24);
   uint32_t* cnt = (uint32_t*)ctx_alloc(ctx, (size_t)(nruns + 1) * 4);
-  uint32_t* aoff = (uint32_t*)ctx_alloc(ctx, (size_t)(nruns + 1) * 4);
+  a.big = (uint32_t*)ctx_alloc(ctx, (size_t)nruns * 4);
   sedef_chain_t* tmp = (sedef_chain_t*)ctx_alloc(ctx, (size_t)nruns * sizeof(sedef_chain_t));
-  if (!cnt || !aoff || !tmp) return SEDEF_ERR_OOM;
-  const int wb = grid_of(nruns * 32, 256);
-  if (pl) SEDEF_CUDA(cudaMemsetAsync(cnt, 0, (size_t)(nruns + 1) * 4, st));
-  SEDEF_KERNEL(ctx, "k_anchor_count", k_anchor_count<<<wb, 256, 0, st>>>(a, cnt));
-  uint32_t* amax = (uint32_t*)ctx_alloc(ctx, 8);
-  if (!amax) return SEDEF_ERR_OOM;
-  SEDEF_CUDA(cudaMemsetAsync(amax, 0, 4, st));
-  SEDEF_KERNEL(ctx, "k_max_u32",
-               k_max_u32<<<grid_of(nruns < 65536 ? nruns : 65536, 256), 256, 0, st>>>(cnt, nruns, amax));
-  SEDEF_TRY(scan_exclusive_u32(ctx, cnt, aoff, nruns, aoff + nruns));
-  int64_t A;
-  if (pl) {
-    // anchors: planned capacity; seeds past it or over the limit are
-    // skipped and flagged by the DP
-    A = pl->anchors;
-    SEDEF_TRY(plan_check64(ctx, pl, atotal, A, 3));
-  } else {
-    uint32_t* h_tot = (uint32_t*)ctx_host(ctx, 8);
-    if (!h_tot) return SEDEF_ERR_OOM;
-    SEDEF_CUDA(cudaMemcpyAsync(h_tot, aoff + nruns, 4, cudaMemcpyDeviceToHost, st));
-    SEDEF_CUDA(cudaMemcpyAsync(h_tot + 1, amax, 4, cudaMemcpyDeviceToHost, st));
+  if (!sums || !cnt || !a.big || !tmp) return SEDEF_ERR_OOM;
+  SEDEF_CUDA(cudaMemsetAsync(sums, 0, 24, st));
+  a.atotal = sums;
+  a.nbig = (uint32_t*)(sums + 1);
+  uint32_t* amax = (uint32_t*)(sums + 2);
+  // a self-search's query records are its target records by position
+  const bool join = D.self_mode != 0 && nq == nt && nqseq == ntseq &&
+                    std::memcmp(h_qoff, h_toff, (size_t)(ntseq + 1) * sizeof(int64_t)) == 0;
+  const int64_t most = (int64_t)ctx_sm_count(ctx) * 5;
+  const int sg = (int)((nruns + kSeedWarps - 1) / kSeedWarps < most ? (nruns + kSeedWarps - 1) / kSeedWarps : most);
+  if (join)
+    SEDEF_KERNEL(ctx, "k_chain_seeds", k_chain_seeds<true><<<sg, 32 * kSeedWarps, 0, st>>>(a, tmp));
+  else
+    SEDEF_KERNEL(ctx, "k_chain_seeds", k_chain_seeds<false><<<sg, 32 * kSeedWarps, 0, st>>>(a, tmp));
+  int64_t nbig = nruns, A = 0;
+  unsigned long long* h_sums = nullptr;
+  if (!pl) {
+    h_sums = (unsigned long long*)ctx_host(ctx, 24);
+    if (!h_sums) return SEDEF_ERR_OOM;
+    SEDEF_CUDA(cudaMemcpyAsync(h_sums, sums, 24, cudaMemcpyDeviceToHost, st));
     SEDEF_CUDA(cudaStreamSynchronize(st));
-    A = *h_tot;
-    ctx_set_anchor_total(ctx, A);
-    // refuse instead of running for hours
-    if (h_tot[1] > (uint32_t)kMaxChainAnchors)
-      return fail(SEDEF_ERR_UNSUPPORTED,
-                  "sedef_chain: a seed has " + std::to_string(h_tot[1]) +
-                      " anchors (limit 65536); soft-mask low-complexity repeats or set max_occ");
+    nbig = (int64_t)(h_sums[1] & 0xFFFFFFFFull);
+    ctx_set_anchor_total(ctx, (int64_t)h_sums[0]);
   }
-  a.acap = A;
-  uint64_t* anchors = (uint64_t*)ctx_alloc(ctx, (size_t)(A ? A : 1) * 8);
-  int32_t* f = (int32_t*)ctx_alloc(ctx, (size_t)(A ? A : 1) * 4);
-  int32_t* pred = (int32_t*)ctx_alloc(ctx, (size_t)(A ? A : 1) * 4);
-  if (!anchors || !f || !pred) return SEDEF_ERR_OOM;
-  SEDEF_KERNEL(ctx, "k_anchor_fill", k_anchor_fill<<<wb, 256, 0, st>>>(a, aoff, anchors));
-  SEDEF_KERNEL(ctx, "k_chain_dp", k_chain_dp<<<wb, 256, 0, st>>>(a, aoff, anchors, f, pred, tmp));
+  if (nbig > 0) {
+    // the seeds past the shared-memory sizes (a planned pass does not know
+    // whether there are any)
+    uint32_t* aoff = (uint32_t*)ctx_alloc(ctx, (size_t)(nbig + 1) * 4);
+    if (!aoff) return SEDEF_ERR_OOM;
+    const int wb = grid_of(nbig * 32 < most * 256 ? nbig * 32 : most * 256, 256);
+    if (pl) SEDEF_CUDA(cudaMemsetAsync(cnt, 0, (size_t)(nbig + 1) * 4, st));
+    SEDEF_KERNEL(ctx, "k_anchor_count", k_anchor_count<<<wb, 256, 0, st>>>(a, cnt));
+    SEDEF_KERNEL(ctx, "k_max_u32",
+                 k_max_u32<<<grid_of(nbig < 65536 ? nbig : 65536, 256), 256, 0, st>>>(cnt, nbig, amax));
+    SEDEF_TRY(scan_exclusive_u32(ctx, cnt, aoff, nbig, aoff + nbig));
+    if (pl) {
+      // anchors: planned capacity; seeds past it or over the limit are
+      // skipped and flagged by the DP
+      A = pl->anchors;
+      SEDEF_TRY(plan_check64(ctx, pl, a.atotal, A, 3));
+    } else {
+      uint32_t* h_tot = (uint32_t*)h_sums;
+      SEDEF_CUDA(cudaMemcpyAsync(h_tot, aoff + nbig, 4, cudaMemcpyDeviceToHost, st));
+      SEDEF_CUDA(cudaMemcpyAsync(h_tot + 1, amax, 4, cudaMemcpyDeviceToHost, st));
+      SEDEF_CUDA(cudaMemcpyAsync(h_tot + 2, sums, 8, cudaMemcpyDeviceToHost, st));
+      SEDEF_CUDA(cudaStreamSynchronize(st));
+      A = h_tot[0];
+      ctx_set_anchor_total(ctx, (int64_t)(((uint64_t)h_tot[3] << 32) | h_tot[2]));
+      // refuse instead of running for hours
+      if (h_tot[1] > (uint32_t)kMaxChainAnchors)
+        return fail(SEDEF_ERR_UNSUPPORTED,
+                    "sedef_chain: a seed has " + std::to_string(h_tot[1]) +
+                        " anchors (limit 65536); soft-mask low-complexity repeats or set max_occ");
+    }
+    a.acap = A;
+    uint64_t* anchors = (uint64_t*)ctx_alloc(ctx, (size_t)(A ? A : 1) * 8);
+    int32_t* f = (int32_t*)ctx_alloc(ctx, (size_t)(A ? A : 1) * 4);
+    int32_t* pred = (int32_t*)ctx_alloc(ctx, (size_t)(A ? A : 1) * 4);
+    if (!anchors || !f || !pred) return SEDEF_ERR_OOM;
+    SEDEF_KERNEL(ctx, "k_anchor_fill", k_anchor_fill<<<wb, 256, 0, st>>>(a, aoff, anchors));
+    SEDEF_KERNEL(ctx, "k_chain_dp", k_chain_dp<<<wb, 256, 0, st>>>(a, aoff, anchors, f, pred, tmp));
+  }
   uint32_t* flag = cnt;  // reuse
   uint32_t* pos = (uint32_t*)ctx_alloc(ctx, (size_t)(nruns + 1) * 4);
   if (!pos) return SEDEF_ERR_OOM;

@@ -286,3 +286,27 @@ def test_index_sort_sizes(ctx, n, k):
         assert np.array_equal(srt.cpu().numpy().view(np.uint64), want)
         cnt = np.concatenate([[0], np.cumsum(np.bincount(h, minlength=top))])
         assert bool((off.cpu().to(torch.int64) == torch.from_numpy(cnt)).all())
+
+
+@pytest.mark.parametrize("pd", [dict(), dict(w=5), dict(w=2, n=400, step=200), dict(w=40), dict(k=9, w=8),
+                                dict(gap_max=60, diag_max=5), dict(max_occ=20), dict(min_unmasked=3)])
+@pytest.mark.parametrize("mode", [0, 1, 2])
+@pytest.mark.parametrize("which", ["tandem", "crowded"])
+def test_chain_anchor_counts(ctx, which, pd, mode):
+    """Seeds with a few anchors, around 32 and past the 256 that one warp keeps, with more than 256
+    query records, joined (self modes) and searched, on both strands."""
+    from tests.gpu_helpers import chain_rows
+    d = oracle.params(self_mode=mode, **pd)
+    g = tandem_genome(6) if which == "tandem" else crowded_genome(10)
+    recs = oracle.sketch(g.seq, g.offsets, d)
+    runs = oracle.filter_runs(recs, g.offsets, recs, g.offsets, d, threads=16)
+    runs = runs[::max(1, len(runs) // 400)]
+    want = oracle.chain(runs, recs, g.offsets, recs, g.offsets, d)
+    p = binding.params_from_dict(d)
+    rec = ctx.sedef_sketch(*ctx.sedef_pack(to_dev(g.seq)), g.offsets, p)
+    srt, tab = ctx.sedef_index(rec, p)
+    v = np.zeros(len(runs), dtype=binding.RUN_DTYPE)
+    for c in oracle.RUN_COLS:
+        v[c] = runs[:, oracle.RUN_COLS.index(c)]
+    chains, n = ctx.sedef_chain(to_dev(v.view(np.uint8)), len(v), rec, g.offsets, srt, tab, g.offsets, p)
+    assert_rows_equal(chain_rows(chains), want, "chains")
