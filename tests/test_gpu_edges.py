@@ -310,3 +310,30 @@ def test_chain_anchor_counts(ctx, which, pd, mode):
         v[c] = runs[:, oracle.RUN_COLS.index(c)]
     chains, n = ctx.sedef_chain(to_dev(v.view(np.uint8)), len(v), rec, g.offsets, srt, tab, g.offsets, p)
     assert_rows_equal(chain_rows(chains), want, "chains")
+
+
+def test_posting_ranges_parted(ctx):
+    """A batch with more records than the posting ranges are parted from (16 M): the candidates of
+    its genomes searched alone (fewer records each)."""
+    from paper_1807_00205_gb300 import batch
+    rng = np.random.default_rng(77)
+    parts = []
+    for n in (41_000_003, 17_000_001):
+        s = np.empty(n, dtype=np.uint8)
+        synth.random_bases_chunked(rng, s, 0.45)
+        for _ in range(60):
+            a, b = rng.integers(0, n - 9_000, 2)
+            c = synth.mutate(rng, s[a:a + 8_000], float(rng.uniform(0.85, 1.0)))
+            s[b:b + len(c)] = synth.reverse_complement(c)[:n - b] if rng.random() < 0.5 else c[:n - b]
+        parts.append(s)
+    g = synth.genome_from_parts(parts)
+    p = binding.params(w=5, self_mode=2)
+    both = to_dev(g.seq)
+    rec = ctx.sedef_sketch(*ctx.sedef_pack(both), g.offsets, p)
+    assert rec.numel() > 16 << 20
+    cands, n = ctx.sedef_selfsearch(both, g.offsets, p)
+    rows = batch.split_candidates(binding.struct_view(cands, binding.CAND_DTYPE), 2)
+    assert n > 100
+    for k, s in enumerate(parts):
+        alone, m = ctx.sedef_selfsearch(to_dev(s), [0, len(s)], binding.params(w=5))
+        assert np.array_equal(binding.struct_view(alone, binding.CAND_DTYPE), rows[k]), k
