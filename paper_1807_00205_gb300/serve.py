@@ -126,15 +126,17 @@ def search(ctx: "binding.Context", index: ResidentIndex, reqs: list, p: "binding
     """One pass for a batch of requests; fills each request's candidates."""
     import torch
     q = binding.params_from_struct(p, self_mode=0)
-    parts = [np.ascontiguousarray(r.seq, dtype=np.uint8) for r in reqs]
+    parts = [r.seq for r in reqs]
     offs = np.zeros(len(parts) + 1, dtype=np.int64)
     offs[1:] = np.cumsum([len(x) for x in parts])
     with torch.cuda.stream(ctx.stream):
-        if parts and offs[-1] >= len(parts) * SEPARATE_UPLOAD_BASES:
+        if (parts and offs[-1] >= len(parts) * SEPARATE_UPLOAD_BASES
+                and all(isinstance(x, np.ndarray) and x.dtype == np.uint8 and x.ndim == 1
+                        for x in parts)):
             d = torch.empty(int(offs[-1]), dtype=torch.uint8, device=ctx.device)
             for k, x in enumerate(parts):
                 if len(x):
-                    x = x if x.flags.writeable else x.copy()
+                    x = np.require(x, requirements="CW")
                     d[int(offs[k]):int(offs[k + 1])].copy_(torch.from_numpy(x))
         else:
             d = torch.from_numpy(np.concatenate(parts)).to(ctx.device, non_blocking=False)
