@@ -204,7 +204,8 @@ int sedef_set_scratch_limit(sedef_ctx* ctx, int64_t bytes);
  * this context may ask for (< 0: no cap, the default).  When the second
  * wide tier (16,384 collected hits, about 213 KB per CTA) is above the cap,
  * a form of it that holds 8,192 collected hits (about 150 KB) takes its
- * place, and when that is above the cap too the wide tier hands the windows
+ * place, and that of the deep CTA tier before it (12,288 hits, 203 KB; 8,192,
+ * 139 KB); when that is above the cap too the broad tier hands the windows
  * it cannot hold straight to the global path; the windows a smaller tier
  * cannot hold go to the global path, so the results do not change.  The
  * other tiers need at most 100 KB per CTA
@@ -565,7 +566,7 @@ int sedef_graph_destroy(sedef_graph* g);
  * entries to finish, which runs the broader tier over such windows.
  * sedef_server_destroy stops the kernel and frees the server.
  * The persistent kernel asks for the largest L1 / shared-memory split and
- * keeps 30 KB of shared memory on every SM while it runs; a kernel of
+ * keeps 53 KB of shared memory on every SM while it runs; a kernel of
  * another stream that needs more than what is left waits for it to leave.
  * sedef_server_smem_left gives that bound (bytes per CTA); finish keeps its
  * own filter tiers within it, and a context that runs beside the server

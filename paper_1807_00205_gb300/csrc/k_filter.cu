@@ -16,8 +16,8 @@
 //      has all of its hits collected, and a count computed from a subset
 //      never exceeds the true one, so the runs are exact.
 // Tiers, by what a window needs: the warp tier (a warp per window), the
-// narrow and the broad CTA tier (k_filter_cta), the second wide tier
-// (16,384 collected hits).  Windows none of them can hold go to a global path
+// narrow, the broad and the deep CTA tier (k_filter_cta: 2,048, 4,096 and
+// 12,288 collected hits), the second wide tier (16,384, counters of 16 bits).  Windows none of them can hold go to a global path
 // that writes their hits to global memory, radix-sorts them by (window, o, t)
 // and sweeps their dense groups.  The autotuner may leave the warp tier out
 // for tiers 1 and 2, CTAs of chosen shapes over windows of up to 2,048
@@ -1015,6 +1015,53 @@ __device__ __forceinline__ bool word_passes(const uint32_t* table, int x, int nw
          (s0 >> 16) + (n0 & 0xFFFFu) >= m || (s1 >> 16) + (n1 & 0xFFFFu) >= m;
 }
 
+// Emits the run of starts whose j + span are first..last of one strand (ne
+// enters with their counts, nl leaves), split by target sequence and the
+// validity rules.  by_lane: each lane has a run of its own; else the warp has
+// one run and shares its enters out.
+__device__ __forceinline__ void emit_valid(const FArgs& a, const WinInfo& w, const uint32_t* enter,
+                                           const uint16_t* val, int ne, const uint32_t* leave, int nl,
+                                           uint32_t first, uint32_t last, bool by_lane) {
+  const int lane = lane_id();
+  const uint32_t span = (uint32_t)a.span;
+  const int64_t lo = (int64_t)first - span, hi = (int64_t)last - span;
+  int64_t x = lo < 0 ? 0 : lo;
+  for (int u = seq_of(a.tseq, a.ntseq, x); u < a.ntseq && x <= hi; ++u) {
+    const int64_t st = a.tseq[u], en = a.tseq[u + 1];
+    bool ok = true;
+    int64_t from = st;
+    if (a.self_mode) {
+      if (u < w.qseq) ok = false;
+      else if (u == w.qseq) from = max(from, w.i + a.n - a.overlap);
+      else if (a.self_mode == 2) ok = false;  // independent genomes
+    }
+    const int64_t vlo = max(x, from), vhi = min(hi, en - a.n);
+    x = en;
+    if (!ok || vlo > vhi) continue;
+    // the largest count on [vlo, vhi]: at vlo, or at an enter after it
+    const uint32_t j0 = (uint32_t)(vlo + span), j1 = (uint32_t)(vhi + span);
+    int e = lb_u32(enter, ne, j0);
+    e += e < ne && enter[e] == j0 ? 1 : 0;
+    int l = lb_u32(leave, nl, j0);
+    l += l < nl && leave[l] == j0 ? 1 : 0;
+    uint32_t best = 0;  // count, then the earliest
+    for (int y = by_lane ? e : e + lane; y < ne && enter[y] <= j1; y += by_lane ? 1 : 32)
+      best = max(best, ((uint32_t)val[y] << 16) | (uint32_t)(0xFFFF - y));
+    if (!by_lane) best = __reduce_max_sync(0xffffffffu, best);
+    RunState run;
+    run.open = true;
+    run.ja = vlo;
+    run.jb = vhi;
+    run.mx = e - l;
+    run.jmx = vlo;
+    if ((int)(best >> 16) > run.mx) {
+      run.mx = (int)(best >> 16);
+      run.jmx = (int64_t)enter[0xFFFF - (best & 0xFFFFu)] - span;
+    }
+    if (by_lane || lane == 0) emit_run(a, w, run);
+  }
+}
+
 // The runs of one strand from its n collected hits, sorted by t.
 // The whole warp calls.
 __device__ __noinline__ void strand_runs(const FArgs& a, const WinInfo& w, unsigned long long* hits, int n,
@@ -1094,48 +1141,11 @@ __device__ __noinline__ void strand_runs(const FArgs& a, const WinInfo& w, unsig
     nend += __popc(b);
   }
   __syncwarp();
-  // every run starts and ends once, in order; split it by target sequence
-  // and the validity rules.  Many runs: one per lane; few: the warp takes
-  // them in turn and shares their enters out.
+  // every run starts and ends once, in order.  Many runs: one per lane; few:
+  // the warp takes them in turn and shares their enters out.
   const bool by_lane = nr >= 8;
-  for (int r = by_lane ? lane : 0; r < nr; r += by_lane ? 32 : 1) {
-    const int64_t lo = (int64_t)M.enter[M.first[r]] - span, hi = (int64_t)M.end[r] - span;
-    int64_t x = lo < 0 ? 0 : lo;
-    for (int u = seq_of(a.tseq, a.ntseq, x); u < a.ntseq && x <= hi; ++u) {
-      const int64_t st = a.tseq[u], en = a.tseq[u + 1];
-      bool ok = true;
-      int64_t from = st;
-      if (a.self_mode) {
-        if (u < w.qseq) ok = false;
-        else if (u == w.qseq) from = max(from, w.i + a.n - a.overlap);
-        else if (a.self_mode == 2) ok = false;  // independent genomes
-      }
-      const int64_t vlo = max(x, from), vhi = min(hi, en - a.n);
-      x = en;
-      if (!ok || vlo > vhi) continue;
-      // the largest count on [vlo, vhi]: at vlo, or at an enter after it
-      const uint32_t j0 = (uint32_t)(vlo + span), j1 = (uint32_t)(vhi + span);
-      int e = lb_u32(M.enter, ne, j0);
-      e += e < ne && M.enter[e] == j0 ? 1 : 0;
-      int l = lb_u32(M.leave, nl, j0);
-      l += l < nl && M.leave[l] == j0 ? 1 : 0;
-      uint32_t best = 0;  // count, then the earliest
-      for (int y = by_lane ? e : e + lane; y < ne && M.enter[y] <= j1; y += by_lane ? 1 : 32)
-        best = max(best, ((uint32_t)M.val[y] << 16) | (uint32_t)(0xFFFF - y));
-      if (!by_lane) best = __reduce_max_sync(0xffffffffu, best);
-      RunState run;
-      run.open = true;
-      run.ja = vlo;
-      run.jb = vhi;
-      run.mx = e - l;
-      run.jmx = vlo;
-      if ((int)(best >> 16) > run.mx) {
-        run.mx = (int)(best >> 16);
-        run.jmx = (int64_t)M.enter[0xFFFF - (best & 0xFFFFu)] - span;
-      }
-      if (by_lane || lane == 0) emit_run(a, w, run);
-    }
-  }
+  for (int r = by_lane ? lane : 0; r < nr; r += by_lane ? 32 : 1)
+    emit_valid(a, w, M.enter, M.val, ne, M.leave, nl, M.enter[M.first[r]], M.end[r], by_lane);
 }
 
 // posting_window by value (out of line, see warp_sort_hits).
@@ -1429,34 +1439,325 @@ int launch_warp_tier(sedef_ctx* ctx, const FArgs& a, const TierIO& io, int64_t m
 
 // -------------------------------------------------------------- CTA tier --
 //
-// The warp tier's steps with one CTA per window, for windows with more
-// records, posting entries or collected hits than a warp keeps.  A record
-// per thread; the warps share out the posting chunks (a contiguous stretch
-// each, four chunks in flight); the collected hits are sorted by a warp (up
-// to 256) or the CTA; two warps take a strand each.
+// A CTA per window, for windows with more records, posting entries or
+// collected hits than a warp keeps:
+//   1. W_Q in a hash table, a record per thread (a hash's id is its slot);
+//   2. the posting chunks, a contiguous stretch for each warp and four chunks
+//      in flight, counted into 8-bit (bin, o) counters; each hit's counter is
+//      kept (16 bits);
+//   3. the counters become a bit each: reaches m with a neighbour.  The sum of
+//      all counters tells whether one ran over;
+//   4. the kept counters are looked up in those bits and the records of the
+//      few that are set are read again;
+//   5. those hits are sorted by chunks in registers, merged by rank;
+//   6. the runs come from the strands' events as in the warp tier, with every
+//      step shared out to all warps.
 //
-// Bound by the latency of the posting reads and, for windows of a few
-// thousand entries, by its barriers.  It replaced a form that sorted the
-// records for W_Q (28 barriers), searched the posting lists for each hit
-// with one read per thread in flight, cleared 64 KB of 16-bit counters and
-// swept groups one by one: 46 k windows of 7,700 entries against a 3.1 Gbp
-// index 8.3 -> 4.6 ms, a 240 Mbp assembly's 9.0 -> 4.8 ms.  One warp per such
-// window with eight chunks in flight took 5.5 + 2.4 ms on the former, and
-// 0.32 ms where 38 windows are all there is (0.09 this way).
+// Bound by instruction issue (about half of the slots) and by latency: some
+// 4,000 cycles until a window's posting ranges are known, then steps that a
+// barrier ends.  A window of 10 k entries and 800 collected hits against a
+// 3.1 Gbp index takes 86 k cycles with four CTAs on an SM: postings 25 k,
+// second look 18 k, sort 14 k, runs 20 k.  46 k windows against that index
+// took 8.3 ms in a form that sorted the records (28 barriers), searched the
+// lists for each hit and swept groups one by one; 3.1 with this one's first
+// form, which read every posting twice (without keeping the counters: the
+// narrow shape 2.5 ms instead of 2.3), sorted with a barrier per stage and
+// left the runs of a strand to one warp; 2.3 now.  A 240 Mbp assembly's 79 k:
+// 3.5 -> 2.4 ms, and the windows that go on to the broad and the deep shape,
+// with twice the room for hits in the same memory, 2.0 -> 0.45 ms.  Six or
+// eight chunks in flight gave the same.
 
-constexpr int kCThreads = 256, kCWarps = kCThreads / 32;
-// Up to 16,384 posting entries and 1,024 collected hits; up to 65,536 and 2,048.
-using CtaNarrow = WindowShape<kCThreads, 16384, 1024, 16384, 4>;
-using CtaBroad = WindowShape<kCThreads, 32768, 2048, 65536, 3>;
+// SLOTS: 8-bit (bin, o) counters, WL: collected hits, WH: posting entries,
+// WC: posting entries whose counter is kept for the second look, TPB:
+// threads, MINB: CTAs per SM.
+template <int SLOTS_, int WL_, int WH_, int WC_, int TPB_, int MINB_>
+struct CtaShape {
+  static constexpr int QC = 256;      // query records
+  static constexpr int TS = 2 * QC;   // W_Q table slots
+  static constexpr int SLOTS = SLOTS_, WL = WL_, WH = WH_, WC = WC_, TPB = TPB_, MINB = MINB_;
+  static constexpr int WARPS = TPB / 32;
+  static constexpr int BUF = SLOTS > 8 * WL ? SLOTS : 8 * WL;  // bytes of the counters' array
+  static constexpr int KEEP = 2 * WC > 8 * WL ? 2 * WC : 8 * WL;  // bytes of the kept counters' array
+  static_assert(TPB >= QC && WL % 256 == 0 && WL < 0xFFFF, "a record per thread; 16-bit hit numbers");
+  static_assert((SLOTS <= 32768 || WC == 0) && WH <= 65536 && WC % 32 == 0,
+                "16 bits for a counter, with one value to spare, and for an entry");
+  static_assert(TS * 4 <= WL * 8, "W_Q's table lies over the hits");
+  static_assert(SLOTS / 8 + 4 * WL <= BUF, "the needed entries lie behind the counters' bits");
+  static_assert(WARPS * TS * 4 <= 8 * WL, "the warps' last hits per hash lie over the events");
+  static_assert(WH / 32 >= 2 * (WL / 32), "the event bits lie over the list starts");
+};
+using CtaNarrow = CtaShape<16384, 2048, 16384, 16384, 256, 4>;
+using CtaBroad = CtaShape<32768, 4096, 65536, 16384, 256, 3>;
+// One CTA per SM, the smaller one beside the serving kernel: 64 registers per
+// thread, so that both kernels' registers fit.
+using CtaDeep = CtaShape<65536, 12288, 65536, 0, 512, 2>;
+using CtaMid = CtaShape<65536, 8192, 65536, 0, 512, 2>;
 
 template <typename W>
-struct CtaSmemT : WindowSmemT<W> {
-  uint32_t map[64];
-  uint32_t sum[kCWarps], lists_of[kCWarps];
-  uint32_t most;
+struct CtaSmemT {
+  uint32_t table[W::BUF / 4];         // counters; a bit per counter and the needed entries; hits or events
+  // W_Q's hash table; the kept counters; then hits or events
+  unsigned long long hits[W::KEEP / 8];
+  uint2 lists[W::QC];                 // posting lists
+  uint32_t starts[W::WH / 32];        // bit e: a list starts at hit e; later event bits
+  uint32_t strands[W::TS / 16];       // W_Q's strands, two bits per table slot
+  uint32_t sum[4][W::WARPS];
+  uint32_t uncounted;                 // hits less counters
   int nhit;
   int64_t win;
 };
+
+// Sorts the n distinct keys v[0..n) by the whole CTA: a chunk per warp in
+// registers, then merged in pairs by rank, between v and w; returns where
+// they end up.  Both hold n rounded up to 256.
+template <typename W>
+__device__ unsigned long long* cta_sort_hits(unsigned long long* v, unsigned long long* w, int n) {
+  const int warp = threadIdx.x >> 5;
+  int chunk = 32;
+  while (chunk < 256 && chunk * W::WARPS < n) chunk <<= 1;
+  for (int from = warp * chunk; from < n; from += W::WARPS * chunk) {
+    const int len = min(chunk, n - from);
+    if (chunk == 32) warp_sort_hits<1>(v + from, len);
+    else if (chunk == 64) warp_sort_hits<2>(v + from, len);
+    else if (chunk == 128) warp_sort_hits<4>(v + from, len);
+    else warp_sort_hits<8>(v + from, len);
+  }
+  __syncthreads();
+  for (int width = chunk; width < n; width <<= 1) {
+    for (int x = threadIdx.x; x < n; x += W::TPB) {
+      const unsigned long long key = v[x];
+      const int other = (x & ~(width - 1)) ^ width;  // the chunk this one merges with
+      int lo = 0, hi = min(width, n - other);
+      while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        if (v[other + mid] < key) lo = mid + 1; else hi = mid;
+      }
+      w[(x & ~(2 * width - 1)) + (x & (width - 1)) + lo] = key;
+    }
+    __syncthreads();
+    unsigned long long* const t = v;
+    v = w;
+    w = t;
+  }
+  return v;
+}
+
+// strand_runs for both strands of a window by the whole CTA: each warp takes
+// an equal stretch of the hits (then of the events), whose places come from
+// the counts of the stretches before.  hits: n sorted hits; events: 8 n
+// bytes for enters and leaves; what follows lies over the hits.
+template <typename W>
+__device__ void cta_runs(const FArgs& a, WinInfo w, unsigned long long* hits, uint32_t* events, int n,
+                         CtaSmemT<W>& S) {
+  const int tid = threadIdx.x, lane = lane_id(), warp = tid >> 5;
+  const uint32_t lt = lanemask_lt();
+  const uint32_t span = (uint32_t)a.span;
+  uint32_t* bits0 = S.starts;                // per word of 32 hits or events
+  uint32_t* bits1 = S.starts + W::WL / 32;
+  auto mine = [&](int count, int* from, int* to) {
+    const int words = (count + 31) >> 5, per = (words + W::WARPS - 1) / W::WARPS;
+    *from = min(warp * per, words);
+    *to = min(*from + per, words);
+  };
+  // sum of row r before this warp, and in all
+  auto places = [&](int r, int* before, int* total) {
+    const uint32_t v = lane < W::WARPS ? S.sum[r][lane] : 0u;
+    *before = (int)__reduce_add_sync(0xffffffffu, lane < warp ? v : 0u);
+    *total = (int)__reduce_add_sync(0xffffffffu, v);
+  };
+  int w0, w1;
+  // ---- stretches: a hit joined to the previous one of its hash does not
+  // enter, and that one does not leave; first within this warp's hits
+  mine(n, &w0, &w1);
+  uint16_t* last = reinterpret_cast<uint16_t*>(events) + warp * (2 * W::TS);
+  for (int x = lane; x < W::TS; x += 32) reinterpret_cast<uint32_t*>(last)[x] = 0xFFFFFFFFu;
+  __syncwarp();
+  auto join = [&](int p, int x, uint32_t t) {
+    if (t - hit_pos(hits[p]) > span + 1u) return;
+    atomicOr(reinterpret_cast<unsigned int*>(hits + x) + 1, (unsigned int)(kHitNoEnter >> 32));
+    atomicOr(reinterpret_cast<unsigned int*>(hits + p) + 1, (unsigned int)(kHitNoLeave >> 32));
+  };
+  // strand and hash of a hit
+  auto key_of = [](unsigned long long h) { return ((uint32_t)h & 0xFFFFFu) | ((uint32_t)(h >> 63) * W::TS); };
+  for (int wd = w0; wd < w1; ++wd) {
+    const int x = wd * 32 + lane;
+    const bool ok = x < n;
+    const unsigned long long h = ok ? hits[x] : 0ull;
+    const uint32_t key = key_of(h);
+    const unsigned peers = __match_any_sync(0xffffffffu, ok ? key : (0x80000000u | (uint32_t)lane));
+    const unsigned lower = peers & lt;
+    int p = -1;
+    if (ok) {
+      if (lower) p = wd * 32 + 31 - __clz(lower);
+      else if (last[key] != 0xFFFFu) p = last[key];
+    }
+    const unsigned alone = __ballot_sync(0xffffffffu, ok && p < 0);
+    if (lane == 0) bits0[wd] = alone;
+    __syncwarp();
+    if (p >= 0) join(p, x, hit_pos(h));
+    if (ok && (peers >> lane) == 1u) last[key] = (uint16_t)x;
+    __syncwarp();
+  }
+  __syncthreads();
+  // then with the hits of the warps before
+  if (warp > 0) {
+    for (int wd = w0; wd < w1; ++wd) {
+      if (!((bits0[wd] >> lane) & 1u)) continue;
+      const int x = wd * 32 + lane;
+      const unsigned long long h = hits[x];
+      const uint16_t* l = last + key_of(h);
+      for (int q = warp - 1; q >= 0; --q) {
+        l -= 2 * W::TS;
+        if (*l == 0xFFFFu) continue;
+        join(*l, x, hit_pos(h));
+        break;
+      }
+    }
+  }
+  __syncthreads();
+  // ---- enters and leaves, strand 0's and then strand 1's
+  {
+    int ne = 0, nl = 0, ne0 = 0, nl0 = 0;
+    for (int wd = w0; wd < w1; ++wd) {
+      const int x = wd * 32 + lane;
+      const unsigned long long h = x < n ? hits[x] : (kHitNoEnter | kHitNoLeave);
+      const unsigned be = __ballot_sync(0xffffffffu, !(h & kHitNoEnter));
+      const unsigned bl = __ballot_sync(0xffffffffu, !(h & kHitNoLeave));
+      const unsigned b0 = __ballot_sync(0xffffffffu, !(h >> 63));
+      ne += __popc(be);
+      nl += __popc(bl);
+      ne0 += __popc(be & b0);
+      nl0 += __popc(bl & b0);
+    }
+    if (lane == 0) {
+      S.sum[0][warp] = ne;
+      S.sum[1][warp] = nl;
+      S.sum[2][warp] = ne0;
+      S.sum[3][warp] = nl0;
+    }
+  }
+  __syncthreads();
+  uint32_t* enter = events;
+  uint32_t* leave = events + n;
+  int ne, nl, ne0, nl0;
+  {
+    int e, l, skip;
+    places(0, &e, &ne);
+    places(1, &l, &nl);
+    places(2, &skip, &ne0);
+    places(3, &skip, &nl0);
+    for (int wd = w0; wd < w1; ++wd) {
+      const int x = wd * 32 + lane;
+      const unsigned long long h = x < n ? hits[x] : (kHitNoEnter | kHitNoLeave);
+      const uint32_t t = hit_pos(h);
+      const unsigned be = __ballot_sync(0xffffffffu, !(h & kHitNoEnter));
+      const unsigned bl = __ballot_sync(0xffffffffu, !(h & kHitNoLeave));
+      if (!(h & kHitNoEnter)) enter[e + __popc(be & lt)] = t;
+      // t + 1 + span, short of wrapping (no window starts that far)
+      if (!(h & kHitNoLeave))
+        leave[l + __popc(bl & lt)] = t < 0xFFFFFFFFu - span - 1u ? t + span + 1u : 0xFFFFFFFFu;
+      e += __popc(be);
+      l += __popc(bl);
+    }
+  }
+  __syncthreads();
+  // ---- shared counts: where runs start and end
+  uint16_t* val = reinterpret_cast<uint16_t*>(hits);  // shared count at each enter
+  uint16_t* first = val + n;                          // per run: the enter that starts it
+  uint32_t* end = reinterpret_cast<uint32_t*>(hits) + n;  // per run: its last j + span
+  const int m = w.m;
+  int e0, e1, l0, l1;
+  mine(ne, &e0, &e1);
+  mine(nl, &l0, &l1);
+  {
+    int c = 0;
+    for (int wd = e0; wd < e1; ++wd) {
+      const int x = wd * 32 + lane;
+      bool start = false;
+      if (x < ne) {
+        const int o = x >= ne0;
+        const int xe = x - (o ? ne0 : 0), lb = o ? nl0 : 0, ln = o ? nl - nl0 : nl0;
+        const uint32_t j = enter[x];
+        const int before = lb_u32(leave + lb, ln, j);  // leaves before j
+        const int upto = before + (before < ln && leave[lb + before] == j ? 1 : 0);
+        const int v = xe + 1 - upto;
+        val[x] = (uint16_t)v;
+        start = v >= m && xe - before < m;
+      }
+      const unsigned b = __ballot_sync(0xffffffffu, start);
+      if (lane == 0) bits0[wd] = b;
+      c += __popc(b);
+    }
+    int d = 0;
+    for (int wd = l0; wd < l1; ++wd) {
+      const int x = wd * 32 + lane;
+      bool stop = false;
+      if (x < nl) {
+        const int o = x >= nl0;
+        const int xl = x - (o ? nl0 : 0), eb = o ? ne0 : 0, en = o ? ne - ne0 : ne0;
+        const uint32_t j = leave[x];
+        const int before = lb_u32(enter + eb, en, j);
+        const int upto = before + (before < en && enter[eb + before] == j ? 1 : 0);
+        stop = upto - (xl + 1) < m && before - xl >= m;
+      }
+      const unsigned b = __ballot_sync(0xffffffffu, stop);
+      if (lane == 0) bits1[wd] = b;
+      d += __popc(b);
+    }
+    if (lane == 0) {
+      S.sum[0][warp] = c;
+      S.sum[1][warp] = d;
+    }
+  }
+  __syncthreads();
+  int nr, at, to, skip;
+  places(0, &at, &nr);
+  places(1, &to, &skip);
+  if (nr == 0) return;
+  for (int wd = e0; wd < e1; ++wd) {
+    const unsigned b = bits0[wd];
+    if ((b >> lane) & 1u) first[at + __popc(b & lt)] = (uint16_t)(wd * 32 + lane);
+    at += __popc(b);
+  }
+  for (int wd = l0; wd < l1; ++wd) {
+    const unsigned b = bits1[wd];
+    if ((b >> lane) & 1u) end[to + __popc(b & lt)] = leave[wd * 32 + lane] - 1u;
+    to += __popc(b);
+  }
+  __syncthreads();
+  // ---- every run starts and ends once, in order; many runs: one per lane;
+  // few: a warp each, which shares their enters out
+  const bool by_lane = nr >= 4 * W::WARPS;
+  for (int r = by_lane ? lane * W::WARPS + warp : warp; r < nr; r += by_lane ? W::TPB : W::WARPS) {
+    const int o = first[r] >= ne0;
+    w.o = o;
+    emit_valid(a, w, enter + (o ? ne0 : 0), val + (o ? ne0 : 0), o ? ne - ne0 : ne0,
+               leave + (o ? nl0 : 0), o ? nl - nl0 : nl0, enter[first[r]], end[r], by_lane);
+  }
+}
+
+// For the 16 counters of four words of the table (one word: two bins, both
+// strands): whether a counter and that of the same strand in the bin before
+// or after reach m.  before, after: the words on either side.
+__device__ __forceinline__ uint32_t pass_bits(uint32_t before, uint4 c, uint32_t after, uint32_t m) {
+  const uint32_t word[6] = {before, c.x, c.y, c.z, c.w, after};
+  const uint32_t reach = (0x8000u - m) * 0x10001u;  // a 16-bit field plus this: top bit set from m on
+  uint32_t out = 0;
+#pragma unroll
+  for (int x = 1; x <= 4; ++x) {
+#pragma unroll
+    for (int o = 0; o < 2; ++o) {
+      // 16-bit fields: the word's two bins; the bin before and the bin after
+      const uint32_t own = __byte_perm(word[x], 0u, o ? 0x4341 : 0x4240);
+      const uint32_t side = __byte_perm(word[x - 1], word[x + 1], o ? 0x0503 : 0x0402) & 0x00FF00FFu;
+      const uint32_t pair = own + __byte_perm(own, 0u, 0x1032);
+      const uint32_t hit = ((pair + reach) | (own + side + reach)) & 0x80008000u;
+      // bits 15 and 31 to counters o and 2 + o
+      out |= ((hit >> 15) & 1u) << (4 * (x - 1) + o) | (hit >> 31) << (4 * (x - 1) + 2 + o);
+    }
+  }
+  return out;
+}
 
 // One query window by the whole CTA; a window the shape cannot hold goes to
 // io.out_list, or for its posting entries to io.wide_list.  The caller
@@ -1465,7 +1766,7 @@ struct CtaSmemT : WindowSmemT<W> {
 template <typename W>
 __device__ void cta_window(const FArgs& a, const TierIO& io, CtaSmemT<W>& S, int64_t wdx) {
   const int tid = threadIdx.x, lane = lane_id(), warp = tid >> 5;
-  const uint32_t lt = lanemask_lt();
+  const uint32_t lt = lanemask_lt(), le = lt | (1u << lane);
   const uint32_t i = __ldcg(a.win_i + wdx), qa = __ldcg(a.win_qa + wdx);
   const int c = (int)(__ldcg(a.win_qb + wdx) - qa);
   if (c == 0) return;
@@ -1475,13 +1776,13 @@ __device__ void cta_window(const FArgs& a, const TierIO& io, CtaSmemT<W>& S, int
     else io.out_list[atomicAdd(io.out_count, 1u)] = (uint32_t)wdx;
   };
   if (c > W::QC) return hand_over(false);
-  if (tid < 64) S.map[tid] = 0u;
+  uint32_t* tab = reinterpret_cast<uint32_t*>(S.hits);  // W_Q
+  if (tid < W::TS / 4) reinterpret_cast<uint4*>(tab)[tid] = make_uint4(0, 0, 0, 0);
   if (tid < W::TS / 16) S.strands[tid] = 0u;
   if (tid == 0) {
-    S.most = 0;
+    S.uncounted = 0;
     S.nhit = 0;
   }
-  __syncthreads();
   // ---- this thread's record: hash and strand, posting range
   uint32_t key = 0, st = 0, len = 0;
   bool kept = false;
@@ -1503,115 +1804,38 @@ __device__ void cta_window(const FArgs& a, const TierIO& io, CtaSmemT<W>& S, int
         posting_window(a.tsorted, a.tsamp, &st, &len, a.tseq[sq], a.tseq[sq + 1]);
       }
     }
-    if (kept) {
-      const uint32_t g = (h * 0x9E3779B1u) >> 21;
-      atomicOr(&S.map[g >> 5], 1u << (g & 31));
-    } else {
-      len = 0;
-    }
+    if (!kept) len = 0;
   }
   // ---- posting lists with an entry, one after another
   const uint32_t v = min(len, 1u << 20);  // no sum can wrap
   const uint32_t inc = warp_inclusive_sum(v);
   const unsigned some = __ballot_sync(0xffffffffu, len > 0);
-  if (lane == 31) S.sum[warp] = inc;
-  if (lane == 0) S.lists_of[warp] = __popc(some);
+  if (lane == 31) S.sum[0][warp] = inc;
+  if (lane == 0) S.sum[1][warp] = __popc(some);
   __syncthreads();
   uint32_t at = inc - v, lid = __popc(some & lt), H = 0;
 #pragma unroll
-  for (int x = 0; x < kCWarps; ++x) {
-    const uint32_t y = S.sum[x];
+  for (int x = 0; x < W::QC / 32; ++x) {
+    const uint32_t y = S.sum[0][x];
     if (x < warp) {
       at += y;
-      lid += S.lists_of[x];
+      lid += S.sum[1][x];
     }
     H += y;
   }
-  const int s_least = (int)__reduce_add_sync(0xffffffffu, __popc(S.map[lane]) + __popc(S.map[lane + 32]));
-  if (s_least == 0 || H == 0) return;
+  if (H == 0) return;
   if (H > io.hlim || H > (uint32_t)W::WH) return hand_over(true);
   const int nchunk = (int)(H + 31) >> 5;
   uint32_t nslots = 1024;
   while (nslots < 4u * H && nslots < (uint32_t)W::SLOTS) nslots <<= 1;
   const uint32_t smask = nslots - 1;
-  for (int x = tid; x < nchunk; x += kCThreads) S.starts[x] = 0u;
-  for (int x = tid; x < (int)nslots / 16; x += kCThreads)
+  for (int x = tid; x < nchunk; x += W::TPB) S.starts[x] = 0u;
+  for (int x = tid; x < (int)nslots / 16; x += W::TPB)
     reinterpret_cast<uint4*>(S.table)[x] = make_uint4(0, 0, 0, 0);
-  __syncthreads();
-  if (len > 0) {
-    S.lists[lid] = make_uint2(st - at, key & 1u);
-    atomicOr(&S.starts[at >> 5], 1u << (at & 31));
-  }
-  __syncthreads();
-  // this warp's chunks of 32 hits, and the lists that start before them
-  const int per = (nchunk + kCWarps - 1) / kCWarps;
-  const int c0 = min(warp * per, nchunk), c1 = min(c0 + per, nchunk);
-  int first_list = 0;
-  for (int x = lane; x < c0; x += 32) first_list += __popc(S.starts[x]);
-  first_list = (int)__reduce_add_sync(0xffffffffu, first_list) - 1;
-  const uint32_t tlo = first_useful(a, i);
-  auto each_hit = [&](auto f) {
-    constexpr int kAhead = 4;  // chunks in flight
-    int lists_before = first_list;
-    for (int ch = c0; ch < c1; ch += kAhead) {
-      uint64_t r[kAhead];
-      uint32_t y[kAhead];
-#pragma unroll
-      for (int q = 0; q < kAhead; ++q) {
-        const uint32_t e = (uint32_t)(ch + q) * 32 + lane;
-        r[q] = 0;
-        y[q] = 0;
-        if (ch + q < c1) {
-          const unsigned sb = S.starts[ch + q];
-          const int li = lists_before + __popc(sb & (lt | (1u << lane)));
-          lists_before += __popc(sb);
-          if (e < H) {
-            const uint2 list = S.lists[li];
-            y[q] = list.y;
-            r[q] = __ldg(a.tsorted + (list.x + e));
-          }
-        }
-      }
-#pragma unroll
-      for (int q = 0; q < kAhead; ++q) {
-        if (ch + q >= c1) break;
-        const uint32_t t = rec_pos(r[q]);
-        const bool on = (uint32_t)(ch + q) * 32 + lane < H && !useless_hit(a, t, i, tlo);
-        f(on, t, (y[q] ^ rec_strand(r[q])) & 1u, y[q]);
-      }
-    }
-  };
-  {
-    uint32_t most = 0;
-    each_hit([&](bool on, uint32_t t, uint32_t o, uint32_t) {
-      if (!on) return;
-      const uint32_t sl = slot_of(t, o, smask), sh = (sl & 3u) * 8u;
-      most = max(most, ((atomicAdd(&S.table[sl >> 2], 1u << sh) >> sh) & 0xFFu) + 1u);
-    });
-    most = __reduce_max_sync(0xffffffffu, most);
-    if (lane == 0) atomicMax(&S.most, most);
-  }
-  __syncthreads();
-  const uint32_t most = S.most;
-  if (most > 255u) return hand_over(false);  // a counter ran into its neighbour
-  {
-    const uint32_t m = (uint32_t)a.mtab[s_least];
-    bool pass = false;
-    if (2u * most >= m) {
-      const int nw = (int)nslots / 4;
-      for (int x = tid; x < nw; x += kCThreads) pass |= word_passes(S.table, x, nw, m);
-    }
-    if (!__syncthreads_or(pass)) {
-      if (io.stats && tid == 0) atomicAdd(a.stats + 0, (unsigned long long)H);
-      return;
-    }
-  }
   // ---- W_Q: a hash's id is its slot; a record whose hash and strand are in
   // already adds nothing
-  uint32_t* tab = reinterpret_cast<uint32_t*>(S.hits);
-  for (int x = tid; x < W::TS / 4; x += kCThreads) reinterpret_cast<uint4*>(tab)[x] = make_uint4(0, 0, 0, 0);
-  __syncthreads();
   bool fresh = false;
+  uint32_t how = 0;
   if (kept) {
     const uint32_t h = key >> 1;
     static_assert(W::TS == 512, "nine bits of the hash pick a slot");
@@ -1624,70 +1848,190 @@ __device__ void cta_window(const FArgs& a, const TierIO& io, CtaSmemT<W>& S, int
     }
     const uint32_t bit = 1u << ((slot & 15) * 2 + (key & 1u));
     const bool twice = (atomicOr(&S.strands[slot >> 4], bit) & bit) != 0u;
-    if (len > 0) S.lists[lid].y = (key & 1u) | (twice ? 2u : 0u) | (slot << 2);
+    how = (key & 1u) | (twice ? 2u : 0u) | (slot << 2);
   }
   const int s = __syncthreads_count(fresh);
   const int m = a.mtab[s];
-  each_hit([&](bool on, uint32_t t, uint32_t o, uint32_t y) {
-    bool need = false;
-    if (on && !(y & 2u)) {
-      const uint32_t b = t >> kBinShift;
-      auto cnt = [&](uint32_t bin) {
-        const uint32_t sl = ((bin << 1) | o) & smask;
-        return (S.table[sl >> 2] >> ((sl & 3u) * 8u)) & 0xFFu;
-      };
-      const uint32_t n0 = cnt(b);
-      need = n0 + cnt(b + 1) >= (uint32_t)m || (b > 0 && n0 + cnt(b - 1) >= (uint32_t)m);
+  if (len > 0) {
+    S.lists[lid] = make_uint2(st - at, how);
+    atomicOr(&S.starts[at >> 5], 1u << (at & 31));
+  }
+  __syncthreads();
+  // this warp's chunks of 32 hits, and the lists that start before them
+  const int per = (nchunk + W::WARPS - 1) / W::WARPS;
+  const int c0 = min(warp * per, nchunk), c1 = min(c0 + per, nchunk);
+  int first_list = 0;
+  for (int x = lane; x < c0; x += 32) first_list += __popc(S.starts[x]);
+  first_list = (int)__reduce_add_sync(0xffffffffu, first_list) - 1;
+  const uint32_t tlo = first_useful(a, i);
+  constexpr int kAhead = 4;  // chunks in flight
+  // calls f(ch, sl) for kAhead chunks from ch on, from chunk c on: each hit's
+  // counter, kNoSlot for none
+  constexpr uint32_t kNoSlot = 0xFFFFFFFFu;  // its low 16 bits are no counter either
+  auto each_hits = [&](int c, int lists_before, auto f) {
+    for (int ch = c; ch < c1; ch += kAhead) {
+      uint64_t r[kAhead];
+      uint32_t y[kAhead], sl[kAhead];
+#pragma unroll
+      for (int q = 0; q < kAhead; ++q) {
+        const uint32_t e = (uint32_t)(ch + q) * 32 + lane;
+        r[q] = 0;
+        y[q] = 2u;
+        if (ch + q < c1) {
+          const unsigned sb = S.starts[ch + q];
+          const int li = lists_before + __popc(sb & le);
+          lists_before += __popc(sb);
+          if (e < H) {
+            const uint2 list = S.lists[li];
+            y[q] = list.y;
+            r[q] = __ldg(a.tsorted + (list.x + e));
+          }
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < kAhead; ++q) {
+        const uint32_t t = rec_pos(r[q]);
+        const bool on = !(y[q] & 2u) && !useless_hit(a, t, i, tlo);
+        sl[q] = on ? slot_of(t, (y[q] ^ rec_strand(r[q])) & 1u, smask) : kNoSlot;
+      }
+      f(ch, sl);
     }
-    const unsigned bn = __ballot_sync(0xffffffffu, need);
-    if (bn) {
-      int to = 0;
-      if (lane == 0) to = atomicAdd(&S.nhit, __popc(bn));
-      to = __shfl_sync(0xffffffffu, to, 0) + __popc(bn & lt);
-      if (need && to < W::WL)
-        S.hits[to] = ((unsigned long long)o << 63) | ((unsigned long long)t << 20) | (y >> 2);
+  };
+  uint16_t* kept_sl = reinterpret_cast<uint16_t*>(S.hits);
+  {
+    uint32_t n_on = 0;
+    each_hits(c0, first_list, [&](int ch, const auto& sl) {
+#pragma unroll
+      for (int q = 0; q < kAhead; ++q) {
+        if (ch + q < c1 && ch + q < W::WC / 32) kept_sl[(ch + q) * 32 + lane] = (uint16_t)sl[q];
+        if (sl[q] == kNoSlot) continue;
+        atomicAdd(&S.table[sl[q] >> 2], 1u << ((sl[q] & 3u) * 8u));
+        ++n_on;
+      }
+    });
+    n_on = __reduce_add_sync(0xffffffffu, n_on);
+    if (lane == 0) atomicAdd(&S.uncounted, n_on);
+  }
+  __syncthreads();
+  // ---- a bit per counter: its bin and the one before or after reach m.  A
+  // counter that ran into its neighbour makes the bytes' sum less than the
+  // hits counted.
+  {
+    constexpr int kPer = (W::SLOTS / 16 + W::TPB - 1) / W::TPB;  // four words at a time
+    const int nw = (int)nslots / 4;
+    uint32_t bits[(kPer + 1) / 2] = {};
+    uint32_t counted = 0;
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) {
+      const int x = (q * W::TPB + tid) * 4;
+      if (x >= nw) break;
+      const uint4 c4 = *reinterpret_cast<const uint4*>(S.table + x);
+      bits[q / 2] |= pass_bits(S.table[(x - 1) & (nw - 1)], c4, S.table[(x + 4) & (nw - 1)],
+                               (uint32_t)m) << (16 * (q & 1));
+      counted = __dp4a(c4.x, 0x01010101u, __dp4a(c4.y, 0x01010101u,
+                __dp4a(c4.z, 0x01010101u, __dp4a(c4.w, 0x01010101u, counted))));
     }
-  });
+    uint32_t any = 0;
+#pragma unroll
+    for (int q = 0; q < (kPer + 1) / 2; ++q) any |= bits[q];
+    counted = __reduce_add_sync(0xffffffffu, counted);
+    if (lane == 0) atomicSub(&S.uncounted, counted);
+    any = __syncthreads_or(any != 0u);
+    if (S.uncounted != 0u) return hand_over(false);
+    if (!any) {
+      if (io.stats && tid == 0) atomicAdd(a.stats + 0, (unsigned long long)H);
+      return;
+    }
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) {
+      const int x = q * W::TPB + tid;
+      if (x * 4 >= nw) break;
+      reinterpret_cast<uint16_t*>(S.table)[x] = (uint16_t)(bits[q / 2] >> (16 * (q & 1)));
+    }
+  }
+  __syncthreads();
+  // ---- the entries whose counter's bit is set, with their lists; then their
+  // records again
+  uint32_t* needed = S.table + W::SLOTS / 32;  // list << 16 | entry
+  auto bit_of = [&](uint32_t sl) {
+    return sl != kNoSlot && ((S.table[(sl >> 5) & (W::SLOTS / 32 - 1)] >> (sl & 31u)) & 1u) != 0u;
+  };
+  // N chunks from ch on
+  int lists_before = first_list;
+  auto take = [&](int ch, const auto& sl) {
+    constexpr int N = sizeof(sl) / 4;
+    unsigned b[N];
+    int n = 0;
+#pragma unroll
+    for (int q = 0; q < N; ++q) {
+      b[q] = __ballot_sync(0xffffffffu, bit_of(sl[q]));
+      n += __popc(b[q]);
+    }
+    int to = 0;
+    if (n && lane == 0) to = atomicAdd(&S.nhit, n);
+    to = __shfl_sync(0xffffffffu, to, 0);
+#pragma unroll
+    for (int q = 0; q < N; ++q) {
+      const unsigned sb = ch + q < c1 ? S.starts[ch + q] : 0u;
+      const int k = to + __popc(b[q] & lt);
+      if (((b[q] >> lane) & 1u) && k < W::WL)
+        needed[k] = (uint32_t)(lists_before + __popc(sb & le)) << 16 | (uint32_t)((ch + q) * 32 + lane);
+      to += __popc(b[q]);
+      lists_before += __popc(sb);
+    }
+  };
+  int ch = c0;
+  constexpr int kKept = 4;
+  for (; ch < c1 && (W::WC >= W::WH || ch + kKept <= W::WC / 32); ch += kKept) {
+    uint32_t sl[kKept];
+#pragma unroll
+    for (int q = 0; q < kKept; ++q) {
+      const uint32_t v = ch + q < c1 ? kept_sl[(ch + q) * 32 + lane] : 0xFFFFu;
+      sl[q] = v == 0xFFFFu ? kNoSlot : v;
+    }
+    take(ch, sl);
+  }
+  if (W::WC < W::WH) each_hits(ch, lists_before, take);
   __syncthreads();
   const int L = S.nhit;
   if (L > W::WL) return hand_over(false);
+  for (int x = tid; x < L; x += kAhead * W::TPB) {
+    uint64_t r[kAhead];
+    uint32_t y[kAhead];
+#pragma unroll
+    for (int q = 0; q < kAhead; ++q) {
+      if (x + q * W::TPB >= L) break;
+      const uint32_t z = needed[x + q * W::TPB];
+      const uint2 list = S.lists[z >> 16];
+      y[q] = list.y;
+      r[q] = __ldg(a.tsorted + (list.x + (z & 0xFFFFu)));
+    }
+#pragma unroll
+    for (int q = 0; q < kAhead; ++q) {
+      if (x + q * W::TPB >= L) break;
+      S.hits[x + q * W::TPB] = ((unsigned long long)((y[q] ^ rec_strand(r[q])) & 1u) << 63) |
+                               ((unsigned long long)rec_pos(r[q]) << 20) | (y[q] >> 2);
+    }
+  }
+  __syncthreads();
   if (io.stats && tid == 0) {
     atomicAdd(a.stats + 0, (unsigned long long)H);
     atomicAdd(a.stats + 1, (unsigned long long)L);
   }
   if (L < m) return;
-  if (L <= 256) {
-    if (warp == 0) {
-      if (L <= 128) warp_sort_hits<4>(S.hits, L);
-      else warp_sort_hits<8>(S.hits, L);
-    }
-  } else {
-    const int np = next_pow2(L);
-    for (int x = L + tid; x < np; x += kCThreads) S.hits[x] = ~0ull;
-    __syncthreads();
-    block_sort(S.hits, np);
-  }
-  __syncthreads();
-  if (warp >= 2) return;
-  int split = 0;  // first hit with o = 1
-  for (int base = 0; base < L; base += 32)
-    split += __popc(__ballot_sync(0xffffffffu, base + lane < L && (S.hits[base + lane] >> 63) == 0));
-  const int n = warp ? L - split : split;
-  if (n < m) return;
+  unsigned long long* const other = reinterpret_cast<unsigned long long*>(S.table);
+  unsigned long long* const sorted = cta_sort_hits<W>(S.hits, other, L);
   WinInfo w;
   w.i = i;
   w.qseq = __ldcg(a.win_seq + wdx);
   w.s = s;
   w.m = m;
-  w.o = warp;
-  static_assert(W::TS * 4 <= W::QC * 8, "both strands' per-hash places lie over the lists");
-  strand_runs(a, w, S.hits + (warp ? split : 0), n,
-              event_mem(S.table + (warp ? 4 * split : 0), n,
-                        reinterpret_cast<uint16_t*>(S.lists) + warp * W::TS, W::TS));
+  w.o = 0;
+  cta_runs<W>(a, w, sorted, reinterpret_cast<uint32_t*>(sorted == other ? S.hits : other), L, S);
 }
 
 template <typename W>
-__global__ void __launch_bounds__(kCThreads, W::MINB) k_filter_cta(FArgs a, TierIO io) {
+__global__ void __launch_bounds__(W::TPB, W::MINB) k_filter_cta(FArgs a, TierIO io) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   CtaSmemT<W>& S = *reinterpret_cast<CtaSmemT<W>*>(smem_raw);
   const int64_t count = (int64_t)*io.in_count;
@@ -1709,15 +2053,14 @@ template <typename W>
 int launch_cta_tier(sedef_ctx* ctx, const FArgs& a, const TierIO& io, int64_t max_windows,
                     const char* name) {
   const size_t sm = sizeof(CtaSmemT<W>);
-  static_assert(sizeof(CtaSmemT<W>) <= kTierSmemFloor, "the CTA tiers always run");
   SEDEF_TRY(ensure_smem_attr((const void*)k_filter_cta<W>, sm));
   int per_sm = 0;
-  SEDEF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_filter_cta<W>, kCThreads, sm));
+  SEDEF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_filter_cta<W>, W::TPB, sm));
   if (per_sm < 1) per_sm = 1;
   int64_t grid = (int64_t)ctx_sm_count(ctx) * per_sm;
   if (grid > max_windows) grid = max_windows;
   if (grid < 1) grid = 1;
-  SEDEF_KERNEL(ctx, name, k_filter_cta<W><<<(int)grid, kCThreads, sm, ctx_stream(ctx)>>>(a, io));
+  SEDEF_KERNEL(ctx, name, k_filter_cta<W><<<(int)grid, W::TPB, sm, ctx_stream(ctx)>>>(a, io));
   return SEDEF_OK;
 }
 
@@ -1828,8 +2171,7 @@ __global__ void __launch_bounds__(kSThreads) k_slow_emit(FArgs a, int64_t v0, in
   }
 }
 
-// Dense groups of the overflow windows [v0, v1): one warp per window and
-// strand writes one task (window, strand, Jlo, Jhi) per group.
+// A dense group of an overflow window: one task of the sweep.
 struct SlowTask {
   uint32_t v;   // overflow-list index
   uint32_t o;
@@ -1846,38 +2188,98 @@ __device__ __forceinline__ void slow_segment(const uint64_t* keys, int64_t lo, i
   *split = l;
 }
 
+// Writes a task for each lane that has one.  The whole warp calls.
+__device__ __forceinline__ void slow_task(SlowTask* tasks, unsigned long long* ntask, int64_t task_cap,
+                                          bool has, uint32_t v, uint32_t o, int64_t jlo, int64_t jhi) {
+  const unsigned b = __ballot_sync(0xffffffffu, has);
+  if (b == 0) return;
+  unsigned long long at = 0;
+  if (lane_id() == 0) at = atomicAdd(ntask, (unsigned long long)__popc(b));
+  at = __shfl_sync(0xffffffffu, at, 0) + __popc(b & lanemask_lt());
+  if (has && (int64_t)at < task_cap) {
+    SlowTask t;
+    t.v = v;
+    t.o = o;
+    t.jlo = jlo < 0 ? 0 : jlo;
+    t.jhi = jhi;
+    tasks[at] = t;
+  }
+}
+
+// kGroupHits hits of a strand per warp: it takes the groups that start among
+// them, to their ends.  Whether a dense hit starts a group depends on the
+// nearest dense hit before it alone, at most span + 1 back.  (One warp per
+// window, through both strands: 0.48 ms for a window of 22 k hits, 0.05 this
+// way.)
+constexpr int kGroupHits = 512;
+
 __global__ void k_slow_groups(FArgs a, int64_t v0, int64_t v1, const unsigned long long* base,
                               const int32_t* s_of, const uint64_t* keys, SlowTask* tasks,
                               unsigned long long* ntask, int64_t task_cap, const uint32_t* dnov,
                               int64_t hcap) {
-  const int64_t nw = (int64_t)gridDim.x * (blockDim.x >> 5);
+  const int lane = lane_id();
+  const unsigned lt = lanemask_lt();
+  const int64_t parts = (int64_t)gridDim.y * (blockDim.x >> 5);
+  const int64_t part = (int64_t)blockIdx.y * (blockDim.x >> 5) + (threadIdx.x >> 5);
   v1 = live_n(v1, dnov);
-  for (int64_t v = v0 + (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); v < v1;
-       v += nw) {
+  for (int64_t v = v0 + blockIdx.x; v < v1; v += gridDim.x) {
     const int s = s_of[v];
     if (s == 0 || base[v + 1] < base[v] || (int64_t)(base[v + 1] - base[v0]) > hcap) continue;
     const int m = a.mtab[s];
     const int64_t lo = (int64_t)(base[v] - base[v0]), hi = (int64_t)(base[v + 1] - base[v0]);
+    if (lo + part * kGroupHits >= hi) continue;
     int64_t split;
     slow_segment(keys, lo, hi, &split);
     for (int o = 0; o < 2; ++o) {
-      const int64_t b = o ? split : lo, e = o ? hi : split;
-      find_groups([&](int64_t x) { return make_uint2((uint32_t)keys[b + x], 0u); }, e - b, m,
-                  a.span, [&](bool mine, int64_t jlo, int64_t jhi) {
-                    const unsigned bm = __ballot_sync(0xffffffffu, mine);
-                    if (bm == 0) return;
-                    unsigned long long at = 0;
-                    if (lane_id() == 0) at = atomicAdd(ntask, (unsigned long long)__popc(bm));
-                    at = __shfl_sync(0xffffffffu, at, 0) + __popc(bm & lanemask_lt());
-                    if (mine && (int64_t)at < task_cap) {
-                      SlowTask t;
-                      t.v = (uint32_t)v;
-                      t.o = (uint32_t)o;
-                      t.jlo = jlo < 0 ? 0 : jlo;
-                      t.jhi = jhi;
-                      tasks[at] = t;
-                    }
-                  });
+      const uint64_t* k = keys + (o ? split : lo);
+      const int64_t n = o ? hi - split : split - lo;  // hits of the strand
+      const int64_t nd = n - m + 1;                   // the first of m hits lies before this one
+      auto dense = [&](int64_t x, int64_t* jlo, int64_t* jhi) {
+        if (x < 0 || x >= nd) return false;
+        const int64_t ta = (uint32_t)k[x], tb = (uint32_t)k[x + m - 1];
+        *jlo = tb - a.span;
+        *jhi = ta;
+        return tb - ta <= a.span;
+      };
+      for (int64_t x0 = part * kGroupHits; x0 < nd; x0 += parts * kGroupHits) {
+        const int64_t x1 = min(x0 + kGroupHits, nd);
+        int64_t carry_hi = INT64_MIN, cur_lo = 0;  // jhi of the nearest dense hit before; the open group
+        bool open = false;
+        const int64_t reach = (int64_t)(uint32_t)k[x0] - a.span - 1;
+        for (int64_t y = x0 - 32; y > -32; y -= 32) {
+          int64_t jlo, jhi = 0;
+          const unsigned dm = __ballot_sync(0xffffffffu, dense(y + lane, &jlo, &jhi));
+          if (dm) {
+            carry_hi = __shfl_sync(0xffffffffu, jhi, 31 - __clz(dm));
+            break;
+          }
+          if (y <= 0 || (int64_t)(uint32_t)k[y] < reach) break;
+        }
+        for (int64_t y = x0; y < x1 || (open && y < nd); y += 32) {
+          const int64_t x = y + lane;
+          int64_t jlo = 0, jhi = INT64_MIN;
+          const bool is = dense(x, &jlo, &jhi);
+          const unsigned dm = __ballot_sync(0xffffffffu, is);
+          const int64_t near = __shfl_sync(0xffffffffu, jhi, dm & lt ? 31 - __clz(dm & lt) : lane);
+          const int64_t before = dm & lt ? near : carry_hi;
+          const bool start = is && (before == INT64_MIN || jlo > before + 1);
+          const unsigned starts = __ballot_sync(0xffffffffu, start);
+          const int64_t lo_near = __shfl_sync(0xffffffffu, jlo, starts & lt ? 31 - __clz(starts & lt) : lane);
+          // a start closes the group before it, when that one is this warp's
+          const int own = (int)min(max(x1 - y, (int64_t)0), (int64_t)32);
+          const unsigned mine = own >= 32 ? 0xffffffffu : (1u << own) - 1u;
+          const bool closes = start && (starts & lt ? (((starts & lt & mine) >> (31 - __clz(starts & lt))) & 1u) != 0u : open);
+          slow_task(tasks, ntask, task_cap, closes, (uint32_t)v, (uint32_t)o,
+                    starts & lt ? lo_near : cur_lo, before);
+          if (starts) {
+            const int l = 31 - __clz(starts);
+            cur_lo = __shfl_sync(0xffffffffu, jlo, l);
+            open = ((mine >> l) & 1u) != 0u;
+          }
+          if (dm) carry_hi = __shfl_sync(0xffffffffu, jhi, 31 - __clz(dm));
+        }
+        slow_task(tasks, ntask, task_cap, open && lane == 0, (uint32_t)v, (uint32_t)o, cur_lo, carry_hi);
+      }
     }
   }
 }
@@ -2867,7 +3269,8 @@ const FastLaunch kTier2[] = {launch_fast<256, 8192, 2048>, launch_fast<256, 4096
                              launch_fast<512, 8192, 2048>};
 constexpr int kNumTier2 = 3;
 // Second wide tier: windows with more collected hits than the CTA tiers keep
-// (regions with many homologous copies), before the global path.  32,768
+// (regions with many homologous copies) or with a counter past 255, before
+// the global path.  32,768
 // (bin, o) slots and 16,384 collected hits.
 constexpr int kWideSlots = 32768;
 const FastLaunch kTierWide2 = launch_fast<512, 16384, 1024, kWideSlots>;
@@ -2879,6 +3282,10 @@ using WideMidSmem = FastSmemT<512, 8192, 1024, kWideSlots>;
 static_assert(sizeof(FastSmemT<512, 8192, 2048, 2048>) <= kTierSmemFloor &&
                   sizeof(WindowSmemT<WarpDense>) * kWWarps <= kTierSmemFloor,
               "a tier that always runs needs more shared memory than a tier cap may be");
+static_assert(sizeof(CtaSmemT<CtaNarrow>) <= kTierSmemFloor && sizeof(CtaSmemT<CtaBroad>) <= kTierSmemFloor &&
+                  sizeof(CtaSmemT<CtaMid>) <= sizeof(WideMidSmem) &&
+                  sizeof(CtaSmemT<CtaDeep>) <= sizeof(FastSmemT<512, 16384, 1024, kWideSlots>),
+              "a CTA tier runs where its neighbour in the chain does");
 // variant = (warp tier off) * 12 + t1 * kNumTier2 + t2
 constexpr int kNumShapes = kNumTier1 * kNumTier2;
 constexpr int kNumVariants = 2 * kNumShapes;
@@ -2941,8 +3348,7 @@ int global_path_eager(sedef_ctx* ctx, const FArgs& a, int64_t nov, unsigned long
       SlowTask* tasks = (SlowTask*)ctx_alloc(ctx, (size_t)nh * sizeof(SlowTask));
       if (!tasks) return SEDEF_ERR_OOM;
       SEDEF_CUDA(cudaMemsetAsync(counters + 6, 0, 8, st));
-      const int64_t gw = (nb + 7) / 8;
-      int g2 = (int)(gw < (int64_t)ctx_sm_count(ctx) * 8 ? gw : (int64_t)ctx_sm_count(ctx) * 8);
+      const dim3 g2((unsigned)(nb < (int64_t)ctx_sm_count(ctx) * 2 ? nb : (int64_t)ctx_sm_count(ctx) * 2), 4);
       SEDEF_KERNEL(ctx, "k_slow_groups",
                    k_slow_groups<<<g2, 256, 0, st>>>(a, v0, v1, d_base, os, skeys, tasks,
                                                      counters + 6, (int64_t)nh, nullptr,
@@ -3130,7 +3536,8 @@ int run_filter(sedef_ctx* ctx, const uint64_t* qrec, int64_t nq, const int64_t* 
   // [8] tier-2 work, [9] windows tier 1 handed to tier 2, [10] sample size,
   // [11] global-path hits (planned pass), [12]/[13] warp-tier hand-overs and
   // work, [14] windows for the broad CTA tier, [15] its work, [16]/[17] the
-  // same for the second wide tier, [18]/[19] for the narrow CTA tier
+  // same for the deep CTA tier, [20] its work counter, [21] what it handed to
+  // the second wide tier, [18]/[19] for the narrow CTA tier
   unsigned long long* counters = (unsigned long long*)ctx_alloc(ctx, 256);
   sedef_run_t* raw = (sedef_run_t*)ctx_alloc(ctx, (size_t)(cap > 0 ? cap : 1) * sizeof(sedef_run_t));
   if (!wi || !wqa || !wqb || !wseq || !ovl || !ovl1 || !counters || !raw) return SEDEF_ERR_OOM;
@@ -3276,7 +3683,7 @@ int run_filter(sedef_ctx* ctx, const uint64_t* qrec, int64_t nq, const int64_t* 
       float best_rep = 1e30f;
       for (int rep = 0; rep < 3; ++rep) {  // the first repetition warms up
         SEDEF_CUDA(cudaMemsetAsync(counters, 0, 80, st));
-        SEDEF_CUDA(cudaMemsetAsync(counters + 12, 0, 64, st));
+        SEDEF_CUDA(cudaMemsetAsync(counters + 12, 0, 80, st));
         TierIO io0{d_sample, (const unsigned int*)(counters + 10), ovlx,
                    (unsigned int*)(counters + 18), (unsigned int*)(counters + 13), 0};
         TierIO io{d_sample, (const unsigned int*)(counters + 10), ovl1,
@@ -3289,7 +3696,9 @@ int run_filter(sedef_ctx* ctx, const uint64_t* qrec, int64_t nq, const int64_t* 
                    (unsigned int*)(counters + 19), 0};
         TierIO iow{ovlw, (const unsigned int*)(counters + 14), ovlw2,
                    (unsigned int*)(counters + 16), (unsigned int*)(counters + 15), 0};
-        TierIO iow2{ovlw2, (const unsigned int*)(counters + 16), ovl,
+        TierIO iod{ovlw2, (const unsigned int*)(counters + 16), ovl1,
+                   (unsigned int*)(counters + 21), (unsigned int*)(counters + 20), 0};
+        TierIO iow2{ovl1, (const unsigned int*)(counters + 21), ovl,
                     (unsigned int*)(counters + 1), (unsigned int*)(counters + 17), 0};
         SEDEF_CUDA(cudaEventRecord(e0, st));
         if (warp_tier) {
@@ -3300,6 +3709,7 @@ int run_filter(sedef_ctx* ctx, const uint64_t* qrec, int64_t nq, const int64_t* 
         }
         SEDEF_TRY(launch_cta_tier<CtaNarrow>(ctx, a, iox, ns, "k_filter_tune"));
         SEDEF_TRY(launch_cta_tier<CtaBroad>(ctx, a, iow, ns, "k_filter_tune"));
+        SEDEF_TRY(launch_cta_tier<CtaDeep>(ctx, a, iod, ns, "k_filter_tune"));
         SEDEF_TRY(kTierWide2(ctx, a, iow2, ns, "k_filter_tune"));
         SEDEF_CUDA(cudaEventRecord(e1, st));
         SEDEF_CUDA(cudaEventSynchronize(e1));
@@ -3345,7 +3755,8 @@ int run_filter(sedef_ctx* ctx, const uint64_t* qrec, int64_t nq, const int64_t* 
     TierIO iox{ovlx, (const unsigned int*)(counters + 18), ovlw, (unsigned int*)(counters + 14),
                (unsigned int*)(counters + 19), 1};
     SEDEF_TRY(launch_cta_tier<CtaNarrow>(ctx, a, iox, nwin, "k_filter_cta"));
-    // where the second wide tier's CTA would pass the context's cap, its
+    // where the deep and the second wide tier's CTA would pass the context's
+    // cap, their
     // 8,192-hit form takes its place, or, where that would pass it too, the
     // wide tier hands its leftovers straight to the global path
     const size_t scap = ctx_tier_smem_cap(ctx);
@@ -3355,10 +3766,17 @@ int run_filter(sedef_ctx* ctx, const uint64_t* qrec, int64_t nq, const int64_t* 
     TierIO iow{ovlw, (const unsigned int*)(counters + 14), second ? ovlw2 : ovl,
                (unsigned int*)(counters + (second ? 16 : 1)), (unsigned int*)(counters + 15), 1};
     SEDEF_TRY(launch_cta_tier<CtaBroad>(ctx, a, iow, nwin, "k_filter_wide"));
-    TierIO iow2{ovlw2, (const unsigned int*)(counters + 16), ovl, (unsigned int*)(counters + 1),
+    TierIO iod{ovlw2, (const unsigned int*)(counters + 16), ovl1, (unsigned int*)(counters + 21),
+               (unsigned int*)(counters + 20), 1};
+    TierIO iow2{ovl1, (const unsigned int*)(counters + 21), ovl, (unsigned int*)(counters + 1),
                 (unsigned int*)(counters + 17), 1};
-    if (wide2) SEDEF_TRY(kTierWide2(ctx, a, iow2, nwin, "k_filter_wide2"));
-    if (mid) SEDEF_TRY(kTierWideMid(ctx, a, iow2, nwin, "k_filter_widemid"));
+    if (wide2) {
+      SEDEF_TRY(launch_cta_tier<CtaDeep>(ctx, a, iod, nwin, "k_filter_deep"));
+      SEDEF_TRY(kTierWide2(ctx, a, iow2, nwin, "k_filter_wide2"));
+    } else if (mid) {
+      SEDEF_TRY(launch_cta_tier<CtaMid>(ctx, a, iod, nwin, "k_filter_deep"));
+      SEDEF_TRY(kTierWideMid(ctx, a, iow2, nwin, "k_filter_widemid"));
+    }
   }
 
   unsigned long long* h_cnt = nullptr;
@@ -3397,8 +3815,7 @@ int run_filter(sedef_ctx* ctx, const uint64_t* qrec, int64_t nq, const int64_t* 
     while ((int64_t(1) << wbits) < nwin) ++wbits;
     SEDEF_TRY(radix_sort_u64(ctx, keys, vals, skeys, svals, H, 0, 33 + wbits, dhits));
     SEDEF_CUDA(cudaMemsetAsync(counters + 6, 0, 8, st));
-    const int64_t gw = (nwin + 7) / 8;
-    const int g2 = (int)(gw < (int64_t)ctx_sm_count(ctx) * 8 ? gw : (int64_t)ctx_sm_count(ctx) * 8);
+    const dim3 g2((unsigned)(nwin < (int64_t)ctx_sm_count(ctx) * 2 ? nwin : (int64_t)ctx_sm_count(ctx) * 2), 4);
     SEDEF_KERNEL(ctx, "k_slow_groups",
                  k_slow_groups<<<g2, 256, 0, st>>>(a, 0, nwin, d_base, os, skeys, tasks,
                                                    counters + 6, H, dnov, H));
@@ -3476,11 +3893,11 @@ namespace sedef {
 namespace {
 
 constexpr int kServeMaxSlots = 64;
-// One CTA per SM of 256 threads (16 K registers) and ~30 KB of shared
+// One CTA per SM of 256 threads (16 K registers) and ~53 KB of shared
 // memory: the rest of every SM stays free for the admission and finishing
 // kernels (the radix sort's scatter alone takes ~39 K registers per CTA),
 // which would otherwise wait for the persistent kernel to leave.
-constexpr int kServeTPB = kCThreads;
+constexpr int kServeTPB = CtaNarrow::TPB;
 using ServeSmem = CtaSmemT<CtaNarrow>;
 // Windows with more posting entries than the shape keeps go to the slot's
 // wide list before they are read; the finishing call runs the broad CTA tier
@@ -3852,7 +4269,7 @@ int sedef_server_create(sedef_ctx* ctx, const uint64_t* d_trec, const uint64_t* 
   // An SM splits its unified L1 / shared memory when a CTA arrives on an
   // idle SM and keeps the split while any CTA stays.  The persistent kernel
   // stays, so it asks for the largest shared-memory split: the other
-  // streams' kernels then find 228 - 30 KB per SM (the large refine kernel
+  // streams' kernels then find 228 - 53 KB per SM (the large refine kernel
   // takes 125 KB) instead of waiting for the persistent kernel to leave.
   if (cudaFuncSetAttribute(k_serve, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)sizeof(ServeSmem)) != cudaSuccess ||
@@ -4096,13 +4513,17 @@ int sedef_server_finish(sedef_server* srv, int32_t slot, sedef_cand_t* h_cands, 
     {
       // the windows k_serve handed on for their many hits: the broad tier,
       // as an ordinary launch beside k_serve; what it cannot hold, and what
-      // k_serve could not hold, goes through the 8,192-hit wide tier, and
-      // what that cannot hold joins the slot's overflow list
+      // k_serve could not hold, goes through the 8,192-hit deep and second
+      // wide tiers, and what those cannot hold joins the slot's overflow list
       StageScope stage(c, "filter");
       TierIO iow{L.wl, (const unsigned int*)(L.counters + 14), L.ml,
                  (unsigned int*)(L.counters + 16), (unsigned int*)(L.counters + 15), 1};
       int wst = launch_cta_tier<CtaBroad>(c, L.a, iow, L.nwin, "k_filter_wide");
-      TierIO iom{L.ml, (const unsigned int*)(L.counters + 16), L.ov,
+      // the broad tier is through with the slot's wide list
+      TierIO iod{L.ml, (const unsigned int*)(L.counters + 16), L.wl,
+                 (unsigned int*)(L.counters + 21), (unsigned int*)(L.counters + 20), 1};
+      if (wst == SEDEF_OK) wst = launch_cta_tier<CtaMid>(c, L.a, iod, L.nwin, "k_filter_deep");
+      TierIO iom{L.wl, (const unsigned int*)(L.counters + 21), L.ov,
                  (unsigned int*)(L.counters + 1), (unsigned int*)(L.counters + 17), 1};
       if (wst == SEDEF_OK) wst = kTierWideMid(c, L.a, iom, L.nwin, "k_filter_widemid");
       if (wst != SEDEF_OK) return release(wst);

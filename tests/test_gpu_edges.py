@@ -337,3 +337,34 @@ def test_posting_ranges_parted(ctx):
     for k, s in enumerate(parts):
         alone, m = ctx.sedef_selfsearch(to_dev(s), [0, len(s)], binding.params(w=5))
         assert np.array_equal(binding.struct_view(alone, binding.CAND_DTYPE), rows[k]), k
+
+
+@pytest.mark.parametrize("copies", [16, 24, 35, 70, 105, 150, 640])
+@pytest.mark.parametrize("gap", [0, 1200])
+def test_filter_many_copies(ctx, copies, gap):
+    """Windows whose collected hits come around what each shape of the CTA tier, the tier after it
+    and the global path hold, in one dense group on each strand and in one per copy; with the
+    shared memory of every tier, of the ones beside a serving kernel, and of the smallest ones."""
+    rng = np.random.default_rng(copies + gap)
+    unit = synth.random_bases(rng, 1_500, 0.45)
+    parts = []
+    for k in range(copies):
+        pc = synth.mutate(rng, unit, 0.98)
+        parts += [synth.reverse_complement(pc) if k % 5 == 4 else pc,
+                  synth.random_bases(rng, gap + int(rng.integers(0, 40)), 0.45)]
+    target = synth.genome_from_parts([np.concatenate(parts), synth.random_bases(rng, 5_000, 0.45)])
+    query = synth.genome_from_parts([np.concatenate([synth.random_bases(rng, 600, 0.45), unit,
+                                                     synth.random_bases(rng, 500, 0.45)])])
+    d = oracle.params(self_mode=0)
+    qrec, trec = (oracle.sketch(g.seq, g.offsets, d) for g in (query, target))
+    want = oracle.filter_runs(qrec, query.offsets, trec, target.offsets, d, threads=16)
+    assert len(want) >= 4
+    p = binding.params_from_dict(d)
+    dq, dt = (ctx.sedef_sketch(*ctx.sedef_pack(to_dev(g.seq)), g.offsets, p).clone() for g in (query, target))
+    srt, off = ctx.sedef_index(dt, p)
+    c = binding.Context(0)
+    for nbytes in (-1, 180_000, 100 * 1024):
+        c.sedef_set_tier_smem_limit(nbytes)
+        runs, _ = c.sedef_filter(dq, query.offsets, dt, srt, off, target.offsets, p)
+        assert_rows_equal(run_rows(runs), want, f"runs with {nbytes} bytes of shared memory")
+    c.close()
