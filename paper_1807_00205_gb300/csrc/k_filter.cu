@@ -868,8 +868,8 @@ __global__ void __launch_bounds__(TPB) k_filter_fast(FArgs a, TierIO io) {
 
 // ------------------------------------------------------------- warp tier --
 //
-// Small windows (at most kWH posting entries and 256 collected hits) by one
-// warp each, no block barriers:
+// Small windows (at most 2,048 posting entries and 128 collected hits, or 256
+// in the form for many records) by one warp each, no block barriers:
 //   1. every posting of every query record is counted into 8-bit (bin, o)
 //      counters, without building W_Q first: a hash that occurs twice in the
 //      window only counts too much.  The number of distinct hashes is bounded
@@ -890,13 +890,17 @@ __global__ void __launch_bounds__(TPB) k_filter_fast(FArgs a, TierIO io) {
 // Bound by instruction issue and, as a window's path is long and the warps
 // of an SM are all at different places of it, by the instruction cache: sorts
 // unrolled in place, or four chunks of postings in flight, made it slower
-// (13.5 -> 18.8 ms on the batch below), and a separate small kernel for step
-// 1 gained 5% there and lost 16% on an assembly.  The form that built W_Q for
+// (13.5 -> 18.8 ms on the batch below; one to three in flight in a loop of one
+// copy 8.2 -> 8.4 to 8.9), and a separate small kernel for step 1 gained 5%
+// there and lost 16% on an assembly.  The form that built W_Q for
 // every window, looked at the hits before the window too, searched the
 // posting lists per hit and swept groups with one lane took about 4,600
-// instructions a window: 4.7 M windows of a 200-genome batch 21.7 -> 8.2 ms
-// (tier 1 over the windows handed on 3.9 -> 0.5 ms), a 240 Mbp assembly 10.8
-// -> 3.5 ms.
+// instructions a window: 4.7 M windows of a 200-genome batch 21.7 -> 7.0 ms
+// (tier 1 over the windows handed on 3.9 -> 0.2 ms), a 240 Mbp assembly 10.8
+// -> 3.0 ms.  Of that the sort by the number of hits (32, 64, 128) gave 0.5 ms
+// on the batch, and room for 128 collected hits instead of 256, which makes
+// 32 warps per SM of 28, 0.7 more; 2,048 counters and 36 warps gave 0.4 more
+// there and cost 0.5 on the assembly (more windows look as if they passed).
 
 constexpr int kWWarps = 4;
 
@@ -910,7 +914,7 @@ struct WindowShape {
   static_assert(TS * 4 <= WL * 8, "W_Q's table lies over the hits");
   static_assert(WL * 16 <= SLOTS, "the strands' events lie over the counters");
 };
-using WarpSparse = WindowShape<128, 4096, 256, 2048, 7>;
+using WarpSparse = WindowShape<128, 4096, 128, 2048, 8>;
 using WarpDense = WindowShape<256, 4096, 256, 2048, 5>;
 
 template <typename W>
@@ -1380,7 +1384,9 @@ __global__ void __launch_bounds__(32 * kWWarps, W::MINB) k_filter_warp(FArgs a, 
       n_hits += H;
       n_collected += L;
       if (L < m) continue;
-      if (L <= 128) warp_sort_hits<4>(S.hits, L);
+      if (L <= 32) warp_sort_hits<1>(S.hits, L);
+      else if (L <= 64) warp_sort_hits<2>(S.hits, L);
+      else if (kWL <= 128 || L <= 128) warp_sort_hits<4>(S.hits, L);
       else warp_sort_hits<8>(S.hits, L);
       int split = 0;  // first hit with o = 1
       for (int base = 0; base < L; base += 32)
