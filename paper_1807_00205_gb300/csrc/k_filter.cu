@@ -2853,11 +2853,11 @@ __global__ void __launch_bounds__(32 * (kLean ? kRWarps : kRWarpsBig)) k_refine(
 // events fit there; a lane reads its two event streams 16 bytes at a time,
 // one load ahead.  Measured against the form that sorted a merged domain per
 // run into shared-memory slots and took 32 runs per warp whatever their
-// number: 1.26 M runs of a 200-genome batch 17.4 -> 5.4 ms, 2.5 M runs of a
-// 240 Mbp assembly 19.7 -> 6.6 ms, 299 runs of a 2 Mbp genome 1.75 -> 0.08 ms.
+// number: 1.26 M runs of a 200-genome batch 17.4 -> 4.1 ms, 2.5 M runs of a
+// 240 Mbp assembly 19.7 -> 5.0 ms, 299 runs of a 2 Mbp genome 1.75 -> 0.08 ms.
 // Runs beyond the lean limits (more than 256 query records,
-// 512 span records, a span of 65,536 bases or more W_Q hashes than the
-// launch's counters) go to the large kernel.
+// 512 span records, a span of 65,536 bases, more W_Q hashes than the launch's
+// counters or a count past 255) go to the large kernel.
 
 constexpr int kBWarps = 4;
 constexpr int kBQC = 256, kBRC = 512;
@@ -2871,23 +2871,27 @@ constexpr uint32_t kEvNoLeave = 1u << 26;  // its hash stays in the window
 constexpr int kBTabMax = 1024;
 constexpr int kBTabWords = kBTabMax + kBTabMax / 2;
 
-// Shared words of a warp for rolls with at most scap W_Q hashes: 16-bit
+// Shared words of a warp for rolls with at most scap W_Q hashes: 8-bit
 // counts and shared bits for 32 lanes, each lane in its own bank (the setup's
-// hash table lies over them).
+// hash table lies over them).  A count past 255 sends its run to the large
+// kernel.  32 warps fit on an SM at w = 16; with counts of 16 bits and room
+// for 256 W_Q hashes there were 16, and 2.5 M runs of a 240 Mbp assembly took
+// 6.6 ms instead of 5.0, 1.26 M of a 200-genome batch 5.4 instead of 4.1.
 __host__ __device__ constexpr int roll_words(int scap) {
-  return (scap / 2 + scap / 32) * 32 > kBTabWords ? (scap / 2 + scap / 32) * 32 : kBTabWords;
+  return (scap / 4 + scap / 32) * 32 > kBTabWords ? (scap / 4 + scap / 32) * 32 : kBTabWords;
 }
 __host__ __device__ constexpr size_t refine_warp_bytes(int scap) {
-  return (size_t)kBQC * 4 + kBQC + (size_t)roll_words(scap) * 4;
+  return (size_t)scap * 5 + (size_t)roll_words(scap) * 4;
 }
 
 // Rolls one run (single lane) over target starts j_a + [0, jend].  cnt and sb
 // are the lane's zeroed counters and shared bits (one 32-bit word per 32).
-__device__ void roll_run(const uint32_t* __restrict__ ev, int nrel, int s, int mx, int jend, int span,
+// False: a count ran over.
+__device__ bool roll_run(const uint32_t* __restrict__ ev, int nrel, int s, int mx, int jend, int span,
                          uint32_t* cnt, uint32_t* sb, int* best_out, int* jstar_out) {
   const uint4* ev4 = reinterpret_cast<const uint4*>(ev);
-  auto count = [&](int q) -> uint16_t& {
-    return reinterpret_cast<uint16_t*>(cnt + ((q >> 1) << 5))[q & 1];
+  auto count = [&](int q) -> uint8_t& {
+    return reinterpret_cast<uint8_t*>(cnt + ((q >> 2) << 5))[q & 3];
   };
   auto shared_bit = [&](int r) { return (int)((sb[(r >> 5) << 5] >> (r & 31)) & 1u); };
   uint4 eb = ev4[0], en = ev4[1], lb = eb, ln = en;  // next events of either stream
@@ -2922,7 +2926,7 @@ __device__ void roll_run(const uint32_t* __restrict__ ev, int nrel, int s, int m
         sb[(q >> 5) << 5] |= 1u << (q & 31);
         if (q < R) ++est;
       } else {
-        ++count(q);
+        if (++count(q) == 0) return false;
         if (q < R && R + ++B > s) {
           --R;
           B -= count(R);
@@ -2959,6 +2963,7 @@ __device__ void roll_run(const uint32_t* __restrict__ ev, int nrel, int s, int m
   }
   *best_out = best;
   *jstar_out = jstar;
+  return true;
 }
 
 // Sorts 32 * NR keys held by a warp (key of index lane * NR + x in v[x]).
@@ -3019,7 +3024,7 @@ __global__ void __launch_bounds__(32 * kBWarps) k_refine_batch(RefineArgs a) {
   unsigned char* base_s = smem_raw + (size_t)warp * refine_warp_bytes(scap);
   uint32_t* scratch = reinterpret_cast<uint32_t*>(base_s);
   uint32_t* wq_h = scratch + roll_words(scap);
-  uint8_t* wq_m = reinterpret_cast<uint8_t*>(wq_h + kBQC);
+  uint8_t* wq_m = reinterpret_cast<uint8_t*>(wq_h + scap);
   const int64_t nwarps = (int64_t)gridDim.x * kBWarps;
   uint32_t* ev_base = a.events + ((int64_t)blockIdx.x * kBWarps + warp) * (a.ev_words + kEvPad);
   // few runs: spread them over the warps (one warp took 32 runs one after
@@ -3035,21 +3040,24 @@ __global__ void __launch_bounds__(32 * kBWarps) k_refine_batch(RefineArgs a) {
 
   auto flush = [&]() {
     __syncwarp();
-    const int nw = (scap / 2) * 32;  // counters, then shared bits
+    const int nw = (scap / 4) * 32;  // counters, then shared bits
     uint4* z4 = reinterpret_cast<uint4*>(scratch);
-    for (int x = lane; x < (smax + 1) / 2 * 8; x += 32) z4[x] = make_uint4(0, 0, 0, 0);
+    for (int x = lane; x < (smax + 3) / 4 * 8; x += 32) z4[x] = make_uint4(0, 0, 0, 0);
     for (int x = lane; x < (smax + 31) / 32 * 8; x += 32) z4[nw / 4 + x] = make_uint4(0, 0, 0, 0);
     __syncwarp();
     if (lane < nslots) {
       const sedef_run_t run = a.runs[my_run];
       int best, jstar;
-      roll_run(ev_base + my_off, my_nrel, my_s, run.max_shared, (int)(run.j_b - run.j_a), a.span,
-               scratch + lane, scratch + nw + lane, &best, &jstar);
-      sedef_run_t& out = a.runs[my_run];
-      out.est = (uint16_t)(best < 0 ? 0 : best);
-      out.den = (uint16_t)my_s;
-      out.j_star = run.j_a + (uint32_t)jstar;
-      out.keep = (best >= a.mtab[my_s]) ? 1 : 0;
+      if (roll_run(ev_base + my_off, my_nrel, my_s, run.max_shared, (int)(run.j_b - run.j_a), a.span,
+                   scratch + lane, scratch + nw + lane, &best, &jstar)) {
+        sedef_run_t& out = a.runs[my_run];
+        out.est = (uint16_t)(best < 0 ? 0 : best);
+        out.den = (uint16_t)my_s;
+        out.j_star = run.j_a + (uint32_t)jstar;
+        out.keep = (best >= a.mtab[my_s]) ? 1 : 0;
+      } else {
+        a.big[atomicAdd(a.nbig, 1u)] = (uint32_t)my_run;
+      }
     }
     __syncwarp();
     nslots = 0;
@@ -3098,8 +3106,10 @@ __global__ void __launch_bounds__(32 * kBWarps) k_refine_batch(RefineArgs a) {
           const unsigned bal = __ballot_sync(0xffffffffu, first);
           if (first) {
             const int d = s + __popc(bal & lanemask_lt());
-            wq_h[d] = h;
-            wq_m[d] = (uint8_t)mask;
+            if (d < scap) {
+              wq_h[d] = h;
+              wq_m[d] = (uint8_t)mask;
+            }
           }
           s += __popc(bal);
         }

@@ -368,3 +368,27 @@ def test_filter_many_copies(ctx, copies, gap):
         runs, _ = c.sedef_filter(dq, query.offsets, dt, srt, off, target.offsets, p)
         assert_rows_equal(run_rows(runs), want, f"runs with {nbytes} bytes of shared memory")
     c.close()
+
+
+def test_refine_crowded_rank(ctx):
+    """More than 255 hashes of a target window between two neighbours of W_Q (here all below the
+    first): past the batched kernel's counters, so its runs go to the large one."""
+    d = oracle.params(self_mode=0, w=5, n=1000)  # windows of 989 starts
+    rng = np.random.default_rng(5)
+    unit = np.frombuffer(b"GATTCTG", dtype=np.uint8)
+    q = np.full(1_600, ord("N"), dtype=np.uint8)
+    q[700:900] = np.tile(unit, 29)[:200]
+    t = np.concatenate([synth.random_bases(rng, 100, 0.45), np.tile(unit, 7)[:45],
+                        synth.random_bases(rng, 1_500, 0.45)])
+    query, target = synth.genome_from_parts([q]), synth.genome_from_parts([t])
+    qrec, trec = (oracle.sketch(g.seq, g.offsets, d) for g in (query, target))
+    wq, inside = np.unique(qrec[:, 0]), trec[trec[:, 1] < 989][:, 0]
+    assert np.bincount(np.searchsorted(wq, np.setdiff1d(inside, wq)))[0] > 255
+    want = oracle.filter_runs(qrec, query.offsets, trec, target.offsets, d)
+    assert len(want) == 3
+    p = binding.params_from_dict(d)
+    dq, dt = (ctx.sedef_sketch(*ctx.sedef_pack(to_dev(g.seq)), g.offsets, p).clone() for g in (query, target))
+    srt, off = ctx.sedef_index(dt, p)
+    runs, _ = ctx.sedef_filter(dq, query.offsets, dt, srt, off, target.offsets, p)
+    assert_rows_equal(run_rows(runs), want, "runs")
+    assert ctx.sedef_filter_stats()["big_refine"] == len(want)
