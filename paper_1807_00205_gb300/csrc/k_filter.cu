@@ -628,7 +628,7 @@ struct TierIO {
   unsigned int* next;             // work counter of this tier
   int stats;                      // count hits in the filter statistics
   // windows with more than hlim hits are handed over before their hits are
-  // enumerated: to wide_list when set (the wide tier), else to out_list
+  // enumerated: to wide_list when set (the next larger shape), else to out_list
   uint32_t hlim = 0xFFFFFFFFu;
   uint32_t* wide_list = nullptr;
   unsigned int* wide_count = nullptr;
@@ -1459,7 +1459,7 @@ int launch_warp_tier(sedef_ctx* ctx, const FArgs& a, const TierIO& io, int64_t m
 //   6. the runs come from the strands' events as in the warp tier, with every
 //      step shared out to all warps.
 //
-// Bound by instruction issue (about half of the slots) and by latency: some
+// Bound by instruction issue (two thirds of the slots) and by latency: some
 // 4,000 cycles until a window's posting ranges are known, then steps that a
 // barrier ends.  A window of 10 k entries and 800 collected hits against a
 // 3.1 Gbp index takes 86 k cycles with four CTAs on an SM: postings 25 k,
@@ -2875,7 +2875,7 @@ constexpr int kBTabWords = kBTabMax + kBTabMax / 2;
 // counts and shared bits for 32 lanes, each lane in its own bank (the setup's
 // hash table lies over them).  A count past 255 sends its run to the large
 // kernel.  32 warps fit on an SM at w = 16; with counts of 16 bits and room
-// for 256 W_Q hashes there were 16, and 2.5 M runs of a 240 Mbp assembly took
+// for 256 W_Q hashes there were 20, and 2.5 M runs of a 240 Mbp assembly took
 // 6.6 ms instead of 5.0, 1.26 M of a 200-genome batch 5.4 instead of 4.1.
 __host__ __device__ constexpr int roll_words(int scap) {
   return (scap / 4 + scap / 32) * 32 > kBTabWords ? (scap / 4 + scap / 32) * 32 : kBTabWords;
