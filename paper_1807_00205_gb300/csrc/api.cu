@@ -21,8 +21,7 @@ struct sedef_ctx {
   sedef::Pool io;  // buffers of sedef_selfsearch_host, kept across calls
   void* pinned = nullptr;
   size_t pinned_cap = 0;
-  int* wait_flag = nullptr;    // mapped host word (ctx_wait_flag)
-  int* d_wait_flag = nullptr;  // its device view
+  unsigned int sort_polls = sedef::kSortPolls;  // reads of a status before a sort tile counts for itself
   // tracing: one (name, start, stop) per traced launch since the last report
   bool trace = false;
   struct Mark {
@@ -185,13 +184,8 @@ void ctx_set_anchor_total(sedef_ctx* ctx, int64_t a) { ctx->filter_stats[7] = a;
 int ctx_device(sedef_ctx* ctx) { return ctx->device; }
 int ctx_sm_count(sedef_ctx* ctx) { return ctx->sm_count; }
 
-int* ctx_wait_flag(sedef_ctx* ctx) { return ctx->d_wait_flag; }
-
-int ctx_check_waits(sedef_ctx* ctx) {
-  if (__atomic_load_n(ctx->wait_flag, __ATOMIC_ACQUIRE) == 0) return SEDEF_OK;
-  __atomic_store_n(ctx->wait_flag, 0, __ATOMIC_RELEASE);
-  return fail(SEDEF_ERR_TIMEOUT, "a sort tile's wait for the tiles before it gave up");
-}
+unsigned int ctx_sort_polls(sedef_ctx* ctx) { return ctx->sort_polls; }
+void ctx_set_sort_polls(sedef_ctx* ctx, unsigned int polls) { ctx->sort_polls = polls; }
 
 void* host_buf(sedef_ctx* ctx, Planned* pl, size_t bytes) {
   if (!pl) return ctx_host(ctx, bytes);
@@ -361,14 +355,6 @@ int sedef_create(int device, void* stream, sedef_ctx** out) {
   c->pool.limit = c->io.limit = &c->scratch_limit;
   c->pool.held = c->io.held = &c->scratch_held;
   cudaDeviceGetAttribute(&c->sm_count, cudaDevAttrMultiProcessorCount, device);
-  if (cudaHostAlloc((void**)&c->wait_flag, 64, cudaHostAllocMapped) != cudaSuccess ||
-      cudaHostGetDevicePointer((void**)&c->d_wait_flag, c->wait_flag, 0) != cudaSuccess) {
-    cudaGetLastError();
-    if (c->wait_flag) cudaFreeHost(c->wait_flag);
-    delete c;
-    return fail(SEDEF_ERR_OOM, "sedef_create: mapped host allocation failed");
-  }
-  *c->wait_flag = 0;
   *out = c;
   return SEDEF_OK;
 }
@@ -385,7 +371,6 @@ int sedef_destroy(sedef_ctx* ctx) {
   ctx->pool.release();
   ctx->io.release();
   if (ctx->pinned) cudaFreeHost(ctx->pinned);
-  cudaFreeHost(ctx->wait_flag);
   delete ctx;
   return SEDEF_OK;
 }
@@ -410,6 +395,15 @@ int sedef_set_tier_smem_limit(sedef_ctx* ctx, int64_t bytes) {
                 "sedef_set_tier_smem_limit: the filter tiers other than the second wide tier "
                 "need up to 100 KB per CTA");
   ctx->tier_smem_cap = bytes < 0 ? SIZE_MAX : (size_t)bytes;
+  return SEDEF_OK;
+}
+
+// Not part of the interface (sedef.h does not declare it): the tests' way to a
+// sort whose waits run out.  polls < 0: the default; a captured pass keeps the
+// value its context had.
+int sedef_debug_sort_polls(sedef_ctx* ctx, int32_t polls) {
+  if (!ctx) return fail(SEDEF_ERR_INVALID, "ctx is NULL");
+  ctx->sort_polls = polls < 0 ? kSortPolls : (unsigned int)polls;
   return SEDEF_OK;
 }
 

@@ -394,11 +394,11 @@ int64_t ctx_scratch_limit(sedef_ctx* ctx);  // sedef_set_scratch_limit's cap (-1
 void ctx_pool_restore(sedef_ctx* ctx, const std::vector<char>& used_before);
 void* ctx_host(sedef_ctx* ctx, size_t bytes);  // pinned host scratch
 int ctx_device(sedef_ctx* ctx);
-// The word (device view) that a kernel sets when one of its bounded waits
-// gives up, and the check that reports it (SEDEF_ERR_TIMEOUT) once the
-// context's stream has been synchronized.
-int* ctx_wait_flag(sedef_ctx* ctx);
-int ctx_check_waits(sedef_ctx* ctx);
+// Reads of one unpublished status word before a sort tile's wait ends (the
+// default: about a second).
+constexpr unsigned int kSortPolls = 1u << 20;
+unsigned int ctx_sort_polls(sedef_ctx* ctx);
+void ctx_set_sort_polls(sedef_ctx* ctx, unsigned int polls);
 int ctx_sm_count(sedef_ctx* ctx);
 void ctx_set_stats(sedef_ctx* ctx, const int64_t* v, int n);  // last sedef_filter call
 void ctx_set_anchor_total(sedef_ctx* ctx, int64_t a);         // last sedef_chain call

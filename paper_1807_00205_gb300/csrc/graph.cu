@@ -120,6 +120,7 @@ int sedef_graph_create(sedef_ctx* ctx, const uint8_t* d_seq, const int64_t* h_of
   int rc = sedef_create(ctx_device(ctx), g->stream, &g->ctx);
   if (rc != SEDEF_OK) return bail(rc);
   ctx_set_filter_variant(g->ctx, ctx_filter_variant(ctx));
+  ctx_set_sort_polls(g->ctx, ctx_sort_polls(ctx));
   // the graph's scratch counts against the caller's cap
   if ((rc = sedef_set_scratch_limit(g->ctx, ctx_scratch_limit(ctx))) != SEDEF_OK) return bail(rc);
   auto at_least_1 = [](int64_t v) { return v < 1 ? (int64_t)1 : v; };
@@ -194,7 +195,6 @@ int sedef_graph_wait(sedef_graph* g, int64_t* h_need) {
   if (!g) return fail(SEDEF_ERR_INVALID, "sedef_graph_wait: no graph");
   SEDEF_CUDA(cudaSetDevice(ctx_device(g->ctx)));
   SEDEF_CUDA(cudaStreamSynchronize(g->last ? g->last : g->stream));
-  SEDEF_TRY(ctx_check_waits(g->ctx));
   uint32_t flags = 0;
   std::memcpy(&flags, g->h_block, 4);
   unsigned long long need[8];

@@ -636,7 +636,6 @@ int run_chain2(sedef_ctx* ctx, const uint32_t* packed, const uint32_t* nbits, in
     ctx_pool_restore(ctx, used_before);
     r0 = r1;
   }
-  SEDEF_TRY(ctx_check_waits(ctx));  // the last batch's copies have synchronized
   *nout = (int64_t)all.size();
   if ((int64_t)all.size() > cap) return fail(SEDEF_ERR_CAPACITY, "sedef_chain2: output buffer too small");
   if (!all.empty())

@@ -3878,7 +3878,7 @@ int run_filter(sedef_ctx* ctx, const uint64_t* qrec, int64_t nq, const int64_t* 
                               (int64_t)(h_cnt[3] & 0xFFFFFFFFull), slow_hits_total};
     ctx_set_stats(ctx, stats, 7);
   }
-  return ctx_check_waits(ctx);
+  return SEDEF_OK;
 }
 
 }  // namespace sedef

@@ -7,7 +7,8 @@
 // in one read of the keys; then each pass is one kernel: a CTA takes tiles of
 // 4,096 keys in ticket order, every warp ranks its keys by votes, the CTA
 // finds where each digit of its tile goes by a decoupled look-back over the
-// tiles before it, stages the tile in shared memory in digit order, and
+// tiles before it (or, should they not publish in time, by counting their keys
+// itself), stages the tile in shared memory in digit order, and
 // consecutive threads write consecutive output addresses (coalesced runs per
 // digit).  Up to 4,096 keys are sorted by one CTA in one launch, all passes
 // in shared memory.
@@ -111,9 +112,8 @@ struct RsScratch {
   unsigned int* ticket;        // per pass
   uint32_t* hist;              // [pass][256] keys of each digit
   unsigned long long* status;  // [tile][256]
-  int* err;                    // set when a look-back wait gives up
+  unsigned int polls;          // reads of one unpublished status before the wait ends
 };
-constexpr unsigned int kRsSpins = 1u << 20;  // polls of one tile before giving up
 
 // Digit counts of every pass.
 __global__ void __launch_bounds__(kRsThreads) k_rs_hist(const uint64_t* __restrict__ keys, int64_t n,
@@ -170,6 +170,19 @@ __device__ __forceinline__ void rank_round(uint32_t* wcnt, uint32_t d, uint32_t 
   if (d < 256 && rank == 0) wcnt[d] = before + __popc(peers);
   __syncwarp();
   loc = before + rank;
+}
+
+// This thread's digit among the first `end` keys, counted by the whole CTA.
+// For a tile whose wait ran out: what it would have read from the tiles before
+// it, so every key goes to its place whatever the other CTAs do.  Out of line:
+// the pass has no registers to spare.
+__device__ __noinline__ uint32_t count_before(const uint64_t* kin, int64_t end, int shift, uint32_t dmask,
+                                              uint32_t* cnt) {
+  cnt[threadIdx.x] = 0;
+  __syncthreads();
+  for (int64_t x = threadIdx.x; x < end; x += kRsThreads) atomicAdd(cnt + digit_of(kin[x], shift, dmask), 1u);
+  __syncthreads();
+  return cnt[threadIdx.x];
 }
 
 // One pass.  Bound by shared-memory and issue work per key (votes, staging)
@@ -248,6 +261,7 @@ __global__ void __launch_bounds__(kRsThreads, kVals ? 3 : 4) k_rs_pass(
     // keys of this digit in the tiles before: a tile's predecessors were all
     // taken before it by CTAs that publish their counts before they wait
     uint32_t before = 0;
+    bool ran_out = false;
     if (tile > 0) {
       int64_t j = tile - 1;
       unsigned int spins = 0;
@@ -261,10 +275,7 @@ __global__ void __launch_bounds__(kRsThreads, kVals ? 3 : 4) k_rs_pass(
 #pragma unroll
         for (int x = 0; x < kWide; ++x) {
           if (v[x] < kAgg) {  // not yet: read again from this tile
-            if (++spins > kRsSpins) {
-              atomicExch(sc.err, 1);
-              done = true;
-            }
+            if (++spins > sc.polls) ran_out = done = true;
             break;
           }
           spins = 0;
@@ -277,10 +288,15 @@ __global__ void __launch_bounds__(kRsThreads, kVals ? 3 : 4) k_rs_pass(
         }
       }
     }
-    st_relaxed_gpu(mine, kPrefix | (before + count));
+    if (!ran_out) st_relaxed_gpu(mine, kPrefix | (before + count));
     S.gofs[d] = S.base[d] + before - start;
     if (threadIdx.x == 0) S.tile = (long long)atomicAdd(sc.ticket + pass, 1u);
-    __syncthreads();
+    if (__syncthreads_or(ran_out)) {
+      before = count_before(kin, tile * kRsTile, shift, dmask, S.wcnt[0]);
+      if (ran_out) st_relaxed_gpu(mine, kPrefix | (before + count));
+      S.gofs[d] = S.base[d] + before - start;
+      __syncthreads();
+    }
 #pragma unroll 4
     for (int x = threadIdx.x; x < cnt; x += kRsThreads) {
       const uint64_t kk = S.keys[x];
@@ -480,8 +496,7 @@ int radix_sort_u64(sedef_ctx* ctx, const uint64_t* keys_in, const uint32_t* vals
   if (!scratch || (passes > 1 && (!ktmp || (vals_out && !vtmp)))) return SEDEF_ERR_OOM;
   RsScratch sc;
   sc.ticket = (unsigned int*)scratch;
-  sc.err = ctx_wait_flag(ctx);
-  if (!sc.err) return SEDEF_ERR_OOM;
+  sc.polls = ctx_sort_polls(ctx);
   sc.hist = (uint32_t*)(scratch + 64);
   sc.status = (unsigned long long*)(scratch + head);
   SEDEF_CUDA(cudaMemsetAsync(scratch, 0, head + (size_t)ntiles * 256 * 8, st));
