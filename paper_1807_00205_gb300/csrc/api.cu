@@ -556,6 +556,9 @@ int sedef_filter_autotune(sedef_ctx* ctx, const uint64_t* d_qrec, int64_t nq, co
   SEDEF_TRY(derive(p, &D));
   SEDEF_TRY(check_offsets(h_qoff, nqseq, "query"));
   SEDEF_TRY(check_offsets(h_toff, ntseq, "target"));
+  // a batch's query sequence k is searched in target sequence k
+  if (D.self_mode == 2 && nqseq > ntseq)
+    return fail(SEDEF_ERR_INVALID, "self mode 2 needs a target sequence for every query sequence");
   if (nq < 0 || nt < 0 || (nq > 0 && !d_qrec) || (nt > 0 && (!d_trec || !d_tsorted)) || !d_toff)
     return fail(SEDEF_ERR_INVALID, "bad record arrays");
   SEDEF_CUDA(cudaSetDevice(ctx->device));

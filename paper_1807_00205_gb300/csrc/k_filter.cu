@@ -3605,15 +3605,17 @@ int run_filter(sedef_ctx* ctx, const uint64_t* qrec, int64_t nq, const int64_t* 
   a.after_own = D.overlap <= D.n ? 1 : 0;
   if (D.self_mode == 2 || (D.self_mode == 1 && a.after_own)) {
     // self-search: every query record's useful posting range, once (the warp
-    // tier reads them by record offset).  An eager pass walks the index (the
-    // query records are its records, with the same sequence offsets); a
+    // tier reads them by record offset).  An eager pass walks the index when
+    // the query records are its records, with the same sequence offsets; a
     // planned pass, whose counts live on the device, searches per record.
     // With target starts at i + n - overlap or later and overlap <= n, only
     // the entries after the record's own one can be hits.
     const std::vector<char> used_before = ctx_pool_snapshot(ctx);
     uint2* qp = (uint2*)ctx_alloc(ctx, (size_t)nq * sizeof(uint2));
     const int64_t nw = (a.ttotal + 31) >> 5;
-    const bool walk = !pl && nqseq == ntseq &&
+    // The walk ranks target positions among the query's, so both have to be
+    // one array (the autotuner may be given others).
+    const bool walk = !pl && qrec == trec && nq == nt && nqseq == ntseq &&
                       std::memcmp(h_qoff, h_toff, (size_t)(ntseq + 1) * sizeof(int64_t)) == 0;
     uint32_t* pbits = walk ? (uint32_t*)ctx_alloc(ctx, (size_t)(nw + 1) * 4) : nullptr;
     uint32_t* pcnt = walk ? (uint32_t*)ctx_alloc(ctx, (size_t)(nw + 1) * 4) : nullptr;
