@@ -42,6 +42,7 @@ struct sedef_ctx {
   const char* stage = "";  // label of traced launches (sedef::StageScope)
   size_t scratch_limit = SIZE_MAX;  // device bytes both pools may hold
   size_t scratch_held = 0;
+  bool extras = true;  // ctx_extras
 };
 
 namespace sedef {
@@ -156,6 +157,12 @@ TraceScope::~TraceScope() {
 
 cudaStream_t ctx_stream(sedef_ctx* ctx) { return ctx->stream; }
 void ctx_pool_reset(sedef_ctx* ctx) { ctx->pool.reset(); }
+void ctx_pool_release(sedef_ctx* ctx) {
+  cudaStreamSynchronize(ctx->stream);
+  ctx->pool.release();
+}
+bool ctx_extras(sedef_ctx* ctx) { return ctx->extras; }
+void ctx_set_extras(sedef_ctx* ctx, bool on) { ctx->extras = on; }
 int ctx_use_stream_ordered_alloc(sedef_ctx* ctx) {
   ctx->pool.ordered = ctx->io.ordered = &ctx->stream;
   if (!ctx_host(ctx, 1 << 20)) return SEDEF_ERR_OOM;
@@ -499,9 +506,10 @@ int sedef_sketch(sedef_ctx* ctx, const uint32_t* d_packed, const uint32_t* d_mas
   if (!d_packed || !d_mask || !d_nbits) return fail(SEDEF_ERR_INVALID, "NULL input buffer");
   if (rec_cap > 0 && !d_rec) return fail(SEDEF_ERR_INVALID, "NULL output buffer");
   SEDEF_CUDA(cudaSetDevice(ctx->device));
-  ctx->pool.reset();
   StageScope stage(ctx, "sketch");
-  return run_sketch(ctx, d_packed, d_mask, d_nbits, h_seq_off, nseq, D, d_rec, rec_cap, h_nrec);
+  return with_room(ctx, [&] {
+    return run_sketch(ctx, d_packed, d_mask, d_nbits, h_seq_off, nseq, D, d_rec, rec_cap, h_nrec);
+  });
 }
 
 int sedef_index(sedef_ctx* ctx, const uint64_t* d_rec, int64_t nrec, const sedef_params* p,
@@ -513,10 +521,11 @@ int sedef_index(sedef_ctx* ctx, const uint64_t* d_rec, int64_t nrec, const sedef
   if (!d_off || (nrec > 0 && (!d_rec || !d_sorted))) return fail(SEDEF_ERR_INVALID, "NULL buffer");
   if (nrec > 0 && d_rec == d_sorted) return fail(SEDEF_ERR_INVALID, "d_rec and d_sorted overlap");
   SEDEF_CUDA(cudaSetDevice(ctx->device));
-  ctx->pool.reset();
   StageScope stage(ctx, "index");
   if (nrec > 0)
-    SEDEF_TRY(radix_sort_u64(ctx, d_rec, nullptr, d_sorted, nullptr, nrec, 33, 33 + 2 * D.k));
+    SEDEF_TRY(with_room(ctx, [&] {
+      return radix_sort_u64(ctx, d_rec, nullptr, d_sorted, nullptr, nrec, 33, 33 + 2 * D.k);
+    }));
   return build_offsets(ctx, d_sorted, nrec, D.k, d_off);
 }
 
@@ -538,13 +547,14 @@ int sedef_filter(sedef_ctx* ctx, const uint64_t* d_qrec, int64_t nq, const int64
     return fail(SEDEF_ERR_INVALID, "bad record arrays");
   if (run_cap > 0 && !d_runs) return fail(SEDEF_ERR_INVALID, "NULL output buffer");
   SEDEF_CUDA(cudaSetDevice(ctx->device));
-  ctx->pool.reset();
   std::vector<int32_t> mt(kMaxWindowRecs + 1);
   mtable(p, mt.data(), kMaxWindowRecs, nullptr);
   *h_nruns = 0;
   StageScope stage(ctx, "filter");
-  return run_filter(ctx, d_qrec, nq, h_qoff, nqseq, d_trec, d_tsorted, d_toff, nt, h_toff, ntseq,
-                    D, mt.data(), d_runs, run_cap, h_nruns, 0);
+  return with_room(ctx, [&] {
+    return run_filter(ctx, d_qrec, nq, h_qoff, nqseq, d_trec, d_tsorted, d_toff, nt, h_toff, ntseq,
+                      D, mt.data(), d_runs, run_cap, h_nruns, 0);
+  });
 }
 
 int sedef_filter_autotune(sedef_ctx* ctx, const uint64_t* d_qrec, int64_t nq, const int64_t* h_qoff,
@@ -562,15 +572,16 @@ int sedef_filter_autotune(sedef_ctx* ctx, const uint64_t* d_qrec, int64_t nq, co
   if (nq < 0 || nt < 0 || (nq > 0 && !d_qrec) || (nt > 0 && (!d_trec || !d_tsorted)) || !d_toff)
     return fail(SEDEF_ERR_INVALID, "bad record arrays");
   SEDEF_CUDA(cudaSetDevice(ctx->device));
-  ctx->pool.reset();
   std::vector<int32_t> mt(kMaxWindowRecs + 1);
   mtable(p, mt.data(), kMaxWindowRecs, nullptr);
   int64_t chosen = 0;
-  // runs from the timing passes are discarded (capacity 1)
-  sedef_run_t* scratch = (sedef_run_t*)ctx_alloc(ctx, sizeof(sedef_run_t));
-  if (!scratch) return SEDEF_ERR_OOM;
-  SEDEF_TRY(run_filter(ctx, d_qrec, nq, h_qoff, nqseq, d_trec, d_tsorted, d_toff, nt, h_toff, ntseq,
-                       D, mt.data(), scratch, 1, &chosen, 1));
+  SEDEF_TRY(with_room(ctx, [&] {
+    // runs from the timing passes are discarded (capacity 1)
+    sedef_run_t* scratch = (sedef_run_t*)ctx_alloc(ctx, sizeof(sedef_run_t));
+    if (!scratch) return (int)SEDEF_ERR_OOM;
+    return run_filter(ctx, d_qrec, nq, h_qoff, nqseq, d_trec, d_tsorted, d_toff, nt, h_toff, ntseq,
+                      D, mt.data(), scratch, 1, &chosen, 1);
+  }));
   SEDEF_CUDA(cudaStreamSynchronize(ctx->stream));
   if (variant_out) *variant_out = (int32_t)ctx->filter_variant;
   return SEDEF_OK;
@@ -597,7 +608,6 @@ int sedef_chain(sedef_ctx* ctx, const sedef_run_t* d_runs, int64_t nruns, const 
   if (nruns < 0 || (nruns > 0 && !d_runs)) return fail(SEDEF_ERR_INVALID, "bad runs");
   if (cap > 0 && !d_chains) return fail(SEDEF_ERR_INVALID, "NULL output buffer");
   SEDEF_CUDA(cudaSetDevice(ctx->device));
-  ctx->pool.reset();
   std::vector<int32_t> mt(kMaxWindowRecs + 1);
   mtable(p, mt.data(), kMaxWindowRecs, nullptr);
   *h_nchains = 0;
@@ -605,8 +615,10 @@ int sedef_chain(sedef_ctx* ctx, const sedef_run_t* d_runs, int64_t nruns, const 
   if ((nq > 0 && !d_qrec) || (nt > 0 && !d_tsorted) || !d_toff)
     return fail(SEDEF_ERR_INVALID, "bad record arrays");
   StageScope stage(ctx, "chain");
-  return run_chain(ctx, d_runs, nruns, d_qrec, nq, h_qoff, nqseq, d_tsorted, nt, d_toff, h_toff,
-                   ntseq, D, mt.data(), d_chains, cap, h_nchains);
+  return with_room(ctx, [&] {
+    return run_chain(ctx, d_runs, nruns, d_qrec, nq, h_qoff, nqseq, d_tsorted, nt, d_toff, h_toff,
+                     ntseq, D, mt.data(), d_chains, cap, h_nchains);
+  });
 }
 
 int sedef_extend(sedef_ctx* ctx, const sedef_run_t* d_runs, int64_t nruns, const uint64_t* d_qext,
@@ -630,10 +642,11 @@ int sedef_extend(sedef_ctx* ctx, const sedef_run_t* d_runs, int64_t nruns, const
   if (cap > 0 && !d_regions) return fail(SEDEF_ERR_INVALID, "NULL output buffer");
   if (nruns == 0) return SEDEF_OK;
   SEDEF_CUDA(cudaSetDevice(ctx->device));
-  ctx->pool.reset();
   StageScope stage(ctx, "extend");
-  return run_extend(ctx, d_runs, nruns, d_qext, nq, h_qoff, nqseq, d_text, nt, h_toff, ntseq, D,
-                    p, max_len, d_regions, cap, h_nregions);
+  return with_room(ctx, [&] {
+    return run_extend(ctx, d_runs, nruns, d_qext, nq, h_qoff, nqseq, d_text, nt, h_toff, ntseq, D,
+                      p, max_len, d_regions, cap, h_nregions);
+  });
 }
 
 int sedef_chain2(sedef_ctx* ctx, const uint32_t* d_packed, const uint32_t* d_nbits, int64_t nbases,
@@ -649,9 +662,10 @@ int sedef_chain2(sedef_ctx* ctx, const uint32_t* d_packed, const uint32_t* d_nbi
   if (cap > 0 && !d_out) return fail(SEDEF_ERR_INVALID, "NULL output buffer");
   if (nregions == 0) return SEDEF_OK;
   SEDEF_CUDA(cudaSetDevice(ctx->device));
-  ctx->pool.reset();
   StageScope stage(ctx, "chain2");
-  return run_chain2(ctx, d_packed, d_nbits, nbases, d_regions, nregions, D, d_out, cap, h_nout);
+  return with_room(ctx, [&] {
+    return run_chain2(ctx, d_packed, d_nbits, nbases, d_regions, nregions, D, d_out, cap, h_nout);
+  });
 }
 
 int sedef_merge(sedef_ctx* ctx, const sedef_chain_t* d_chains, int64_t nchains,
@@ -665,11 +679,12 @@ int sedef_merge(sedef_ctx* ctx, const sedef_chain_t* d_chains, int64_t nchains,
   if (nchains < 0 || (nchains > 0 && !d_chains)) return fail(SEDEF_ERR_INVALID, "bad chains");
   if (cap > 0 && !d_cands) return fail(SEDEF_ERR_INVALID, "NULL output buffer");
   SEDEF_CUDA(cudaSetDevice(ctx->device));
-  ctx->pool.reset();
   *h_ncands = 0;
   if (nchains == 0) return SEDEF_OK;
   StageScope stage(ctx, "merge");
-  return run_merge(ctx, d_chains, nchains, h_qoff, nqseq, h_toff, ntseq, D, d_cands, cap, h_ncands);
+  return with_room(ctx, [&] {
+    return run_merge(ctx, d_chains, nchains, h_qoff, nqseq, h_toff, ntseq, D, d_cands, cap, h_ncands);
+  });
 }
 
 }  // extern "C"
@@ -696,6 +711,10 @@ int selfsearch_device(sedef_ctx* ctx, const uint8_t* seq, const int64_t* h_seq_o
 #define DALLOC(ptr, bytes)                                                 \
   do {                                                                     \
     ptr = (decltype(ptr))ctx->io.alloc((bytes) ? (bytes) : 256);           \
+    if (!ptr) { /* the scratch of the stages before is free by now */      \
+      ctx_pool_release(ctx);                                               \
+      ptr = (decltype(ptr))ctx->io.alloc((bytes) ? (bytes) : 256);         \
+    }                                                                      \
     if (!ptr) return fail(SEDEF_ERR_OOM, "selfsearch: device allocation failed"); \
   } while (0)
   DALLOC(packed, nwords16 * 4);

@@ -386,6 +386,24 @@ cudaStream_t ctx_stream(sedef_ctx* ctx);
 void* ctx_alloc(sedef_ctx* ctx, size_t bytes);
 std::vector<char> ctx_pool_snapshot(sedef_ctx* ctx);
 void ctx_pool_reset(sedef_ctx* ctx);  // every pool block free for the next call
+void ctx_pool_release(sedef_ctx* ctx);  // every pool block given back (drains the stream)
+// Whether a call may take buffers that it can do without (the posting ranges
+// of a self-search, the batched refine's events).  A call that finds no room
+// runs once more without them and with nothing held over from earlier calls,
+// so a cap that holds what a call needs is enough for it.
+bool ctx_extras(sedef_ctx* ctx);
+void ctx_set_extras(sedef_ctx* ctx, bool on);
+template <typename F>
+int with_room(sedef_ctx* ctx, F call) {
+  ctx_pool_reset(ctx);
+  const int status = call();
+  if (status != SEDEF_ERR_OOM) return status;
+  ctx_pool_release(ctx);
+  ctx_set_extras(ctx, false);
+  const int again = call();
+  ctx_set_extras(ctx, true);
+  return again;
+}
 // The context allocates its scratch in stream order and keeps a 1 MB pinned
 // buffer, so that its calls never synchronize with other streams' kernels
 // (a persistent kernel on another stream would hold them up).

@@ -147,21 +147,32 @@ int sedef_graph_create(sedef_ctx* ctx, const uint8_t* d_seq, const int64_t* h_of
   g->runs = d_runs;
   g->chains = d_chains;
   g->cands = d_cands;
-  g->d_block = (unsigned char*)ctx_alloc(c, kBlockBytes);
   g->h_block = (unsigned char*)host_buf(c, &g->pl, kBlockBytes);
-  if (!g->d_block || !g->h_block) return bail(SEDEF_ERR_OOM);
+  if (!g->h_block) return bail(SEDEF_ERR_OOM);
   std::memset(g->h_block, 0, kBlockBytes);
-  g->pl.flags = (uint32_t*)g->d_block;
-  g->pl.need = (unsigned long long*)(g->d_block + 32);
   std::vector<int32_t> mt(kMaxWindowRecs + 1);
   mtable(p, mt.data(), kMaxWindowRecs, nullptr);
 
-  if (cudaStreamBeginCapture(g->stream, cudaStreamCaptureModeRelaxed) != cudaSuccess)
-    return bail(cuda_fail(cudaGetLastError(), "sedef_graph_create: begin capture"));
-  rc = record_pass(g, d_seq, h_off, nseq, D, mt.data());
+  // where the cap has no room a second recording does without the buffers
+  // that a pass can do without
   cudaGraph_t graph = nullptr;
-  const cudaError_t ec = cudaStreamEndCapture(g->stream, &graph);
-  g->graph = graph;
+  cudaError_t ec = cudaSuccess;
+  for (int again = 0; again < 2; ++again) {
+    g->d_block = (unsigned char*)ctx_alloc(c, kBlockBytes);
+    if (!g->d_block) return bail(SEDEF_ERR_OOM);
+    g->pl.flags = (uint32_t*)g->d_block;
+    g->pl.need = (unsigned long long*)(g->d_block + 32);
+    if (cudaStreamBeginCapture(g->stream, cudaStreamCaptureModeRelaxed) != cudaSuccess)
+      return bail(cuda_fail(cudaGetLastError(), "sedef_graph_create: begin capture"));
+    rc = record_pass(g, d_seq, h_off, nseq, D, mt.data());
+    ec = cudaStreamEndCapture(g->stream, &graph);
+    g->graph = graph;
+    if (rc != SEDEF_ERR_OOM || again) break;
+    if (graph) cudaGraphDestroy(graph);
+    g->graph = graph = nullptr;
+    ctx_pool_release(c);
+    ctx_set_extras(c, false);
+  }
   if (rc != SEDEF_OK) return bail(rc);
   if (ec != cudaSuccess || !graph) return bail(cuda_fail(ec, "sedef_graph_create: end capture"));
   const cudaError_t ei = cudaGraphInstantiate(&g->exec, graph, 0);

@@ -3380,6 +3380,70 @@ int global_path_eager(sedef_ctx* ctx, const FArgs& a, int64_t nov, unsigned long
   return SEDEF_OK;
 }
 
+// Every query record's useful posting range of a self-search, once (the tiers
+// read them by record offset).  An eager pass walks the index when the query
+// records are its records, with the same sequence offsets (walk); a planned
+// pass, whose counts live on the device, searches per record.  With target
+// starts at i + n - overlap or later and overlap <= n, only the entries after
+// the record's own one can be hits.  SEDEF_ERR_OOM: no room for them (kernels
+// that are queued by then only touch this function's own blocks).
+int posting_ranges(sedef_ctx* ctx, const FArgs& a, int64_t nq, int64_t nt, const uint32_t* dnq, bool walk,
+                   uint2** out) {
+  cudaStream_t st = ctx_stream(ctx);
+  uint2* qp = (uint2*)ctx_alloc(ctx, (size_t)nq * sizeof(uint2));
+  if (!qp) return SEDEF_ERR_OOM;
+  *out = qp;
+  int64_t g = (nq + 255) / 256;
+  if (g > (int64_t)ctx_sm_count(ctx) * 16) g = (int64_t)ctx_sm_count(ctx) * 16;
+  if (g < 1) g = 1;
+  if (!walk) {
+    SEDEF_KERNEL(ctx, "k_qpost", k_qpost<<<(int)g, 256, 0, st>>>(a, nq, dnq, qp));
+    return SEDEF_OK;
+  }
+  const int64_t nw = (a.ttotal + 31) >> 5;
+  uint32_t* pbits = (uint32_t*)ctx_alloc(ctx, (size_t)(nw + 1) * 4);
+  uint32_t* pcnt = (uint32_t*)ctx_alloc(ctx, (size_t)(nw + 1) * 4);
+  uint32_t* pbef = (uint32_t*)ctx_alloc(ctx, (size_t)(nw + 1) * 4);
+  RankWord* rw = (RankWord*)ctx_alloc(ctx, (size_t)(nw + 1) * sizeof(RankWord));
+  const int64_t sblocks = ((a.ttotal - 1) >> kSeqShift) + 1;
+  int32_t* stab = (int32_t*)ctx_alloc(ctx, (size_t)sblocks * 4);
+  if (!pbits || !pcnt || !pbef || !rw || !stab) return SEDEF_ERR_OOM;
+  int64_t gw = (nw + 255) / 256;
+  if (gw > (int64_t)ctx_sm_count(ctx) * 16) gw = (int64_t)ctx_sm_count(ctx) * 16;
+  if (gw < 1) gw = 1;
+  SEDEF_CUDA(cudaMemsetAsync(pbits, 0, (size_t)(nw + 1) * 4, st));
+  SEDEF_KERNEL(ctx, "k_pos_bits", k_pos_bits<<<(int)g, 256, 0, st>>>(a.qrec, nq, pbits));
+  SEDEF_KERNEL(ctx, "k_pos_popc", k_pos_popc<<<(int)gw, 256, 0, st>>>(pbits, nw, pcnt));
+  SEDEF_TRY(scan_exclusive_u32(ctx, pcnt, pbef, nw, pbef + nw));
+  SEDEF_KERNEL(ctx, "k_rank_words", k_rank_words<<<(int)gw, 256, 0, st>>>(pbits, pbef, nw, rw));
+  SEDEF_KERNEL(ctx, "k_seq_table",
+               k_seq_table<<<(int)((sblocks + 255) / 256), 256, 0, st>>>(a.tseq, a.ntseq, sblocks, stab));
+  int64_t gq = (nt + 1023) / 1024;
+  if (gq > (int64_t)ctx_sm_count(ctx) * 8) gq = (int64_t)ctx_sm_count(ctx) * 8;
+  uint64_t *pk = nullptr, *pks = nullptr;
+  uint32_t *pv = nullptr, *pvs = nullptr;
+  const std::vector<char> no_parts = ctx_pool_snapshot(ctx);
+  if (nt >= kPartRecords) {
+    pk = (uint64_t*)ctx_alloc(ctx, (size_t)nt * 8);
+    pks = pk ? (uint64_t*)ctx_alloc(ctx, (size_t)nt * 8) : nullptr;
+    pv = pks ? (uint32_t*)ctx_alloc(ctx, (size_t)nt * 4) : nullptr;
+    pvs = pv ? (uint32_t*)ctx_alloc(ctx, (size_t)nt * 4) : nullptr;
+    if (!pvs) pk = nullptr;  // no room under the context's cap
+  }
+  SEDEF_KERNEL(ctx, "k_qpost", k_qpost_index<<<(int)gq, 256, 0, st>>>(a, nt, rw, stab, qp, pk, pv));
+  if (pk) {
+    const int pb = bits_below(a.ttotal);
+    // two CTAs per SM: the CTAs drift apart, and with more of them the
+    // stretch of records being written no longer stays in L2 (119 M
+    // records: 0.9 ms; four CTAs per SM 1.7, eight 4.4)
+    const int64_t gp = (int64_t)ctx_sm_count(ctx) * 2;
+    SEDEF_TRY(radix_sort_u64(ctx, pk, pv, pks, pvs, nt, 32 + (pb > 8 ? pb - 8 : 0), 32 + pb));
+    SEDEF_KERNEL(ctx, "k_qpost_place", k_qpost_place<<<(int)gp, 256, 0, st>>>(pks, pvs, nt, rw, qp));
+  }
+  ctx_pool_restore(ctx, no_parts);
+  return SEDEF_OK;
+}
+
 // Orders the `total` raw runs by (window, o, j_a) into `runs` and refines
 // them (the winnowed MinHash estimate at every breakpoint of each run).
 // druns / dnt: live counts of a planned pass (nullptr when eager).
@@ -3475,7 +3539,8 @@ int order_and_refine(sedef_ctx* ctx, const FArgs& a, const Derived& D, int nqseq
   // context's scratch fewer warps, and where not even one CTA's fit the large
   // kernel takes every run
   ra.scap = scap;
-  while (true) {
+  const std::vector<char> used_before = ctx_pool_snapshot(ctx);
+  while (ctx_extras(ctx)) {
     const int64_t per_warp = (total + rgrid * kBWarps - 1) / (rgrid * kBWarps);
     ra.ev_words = per_warp * (kBRC + 8) < kEvWords ? (int)per_warp * (kBRC + 8) : kEvWords;
     ra.events = (uint32_t*)ctx_alloc(ctx, (size_t)(rgrid * kBWarps) * (ra.ev_words + kEvPad) * 4);
@@ -3491,6 +3556,7 @@ int order_and_refine(sedef_ctx* ctx, const FArgs& a, const Derived& D, int nqseq
   SEDEF_KERNEL(ctx, "k_refine_big",
                k_refine<kMaxWindowRecs, 1024, false><<<ctx_sm_count(ctx), 32 * kRWarpsBig, big_sm,
                                                        st>>>(ra));
+  ctx_pool_restore(ctx, used_before);  // the events
   return SEDEF_OK;
 }
 
@@ -3603,72 +3669,20 @@ int run_filter(sedef_ctx* ctx, const uint64_t* qrec, int64_t nq, const int64_t* 
     a.tsamp = samp;
   }
   a.after_own = D.overlap <= D.n ? 1 : 0;
-  if (D.self_mode == 2 || (D.self_mode == 1 && a.after_own)) {
-    // self-search: every query record's useful posting range, once (the warp
-    // tier reads them by record offset).  An eager pass walks the index when
-    // the query records are its records, with the same sequence offsets; a
-    // planned pass, whose counts live on the device, searches per record.
-    // With target starts at i + n - overlap or later and overlap <= n, only
-    // the entries after the record's own one can be hits.
-    const std::vector<char> used_before = ctx_pool_snapshot(ctx);
-    uint2* qp = (uint2*)ctx_alloc(ctx, (size_t)nq * sizeof(uint2));
-    const int64_t nw = (a.ttotal + 31) >> 5;
+  const std::vector<char> used_before = ctx_pool_snapshot(ctx);
+  if (ctx_extras(ctx) && (D.self_mode == 2 || (D.self_mode == 1 && a.after_own))) {
     // The walk ranks target positions among the query's, so both have to be
     // one array (the autotuner may be given others).
     const bool walk = !pl && qrec == trec && nq == nt && nqseq == ntseq &&
                       std::memcmp(h_qoff, h_toff, (size_t)(ntseq + 1) * sizeof(int64_t)) == 0;
-    uint32_t* pbits = walk ? (uint32_t*)ctx_alloc(ctx, (size_t)(nw + 1) * 4) : nullptr;
-    uint32_t* pcnt = walk ? (uint32_t*)ctx_alloc(ctx, (size_t)(nw + 1) * 4) : nullptr;
-    uint32_t* pbef = walk ? (uint32_t*)ctx_alloc(ctx, (size_t)(nw + 1) * 4) : nullptr;
-    RankWord* rw = walk ? (RankWord*)ctx_alloc(ctx, (size_t)(nw + 1) * sizeof(RankWord)) : nullptr;
-    const int64_t sblocks = ((a.ttotal - 1) >> kSeqShift) + 1;
-    int32_t* stab = walk ? (int32_t*)ctx_alloc(ctx, (size_t)sblocks * 4) : nullptr;
-    if (!qp || (walk && (!pbits || !pcnt || !pbef || !rw || !stab))) {
+    uint2* qp = nullptr;
+    const int got = posting_ranges(ctx, a, nq, nt, dnq, walk, &qp);
+    if (got == SEDEF_ERR_OOM) {
       // no room under the context's cap: the tiers look postings up themselves
-      if (D.self_mode == 2) return SEDEF_ERR_OOM;
       ctx_pool_restore(ctx, used_before);
       qp = nullptr;
     } else {
-      int64_t g = (nq + 255) / 256;
-      if (g > (int64_t)ctx_sm_count(ctx) * 16) g = (int64_t)ctx_sm_count(ctx) * 16;
-      if (g < 1) g = 1;
-      if (!walk) {
-        SEDEF_KERNEL(ctx, "k_qpost", k_qpost<<<(int)g, 256, 0, st>>>(a, nq, dnq, qp));
-      } else {
-        int64_t gw = (nw + 255) / 256;
-        if (gw > (int64_t)ctx_sm_count(ctx) * 16) gw = (int64_t)ctx_sm_count(ctx) * 16;
-        if (gw < 1) gw = 1;
-        SEDEF_CUDA(cudaMemsetAsync(pbits, 0, (size_t)(nw + 1) * 4, st));
-        SEDEF_KERNEL(ctx, "k_pos_bits", k_pos_bits<<<(int)g, 256, 0, st>>>(qrec, nq, pbits));
-        SEDEF_KERNEL(ctx, "k_pos_popc", k_pos_popc<<<(int)gw, 256, 0, st>>>(pbits, nw, pcnt));
-        SEDEF_TRY(scan_exclusive_u32(ctx, pcnt, pbef, nw, pbef + nw));
-        SEDEF_KERNEL(ctx, "k_rank_words", k_rank_words<<<(int)gw, 256, 0, st>>>(pbits, pbef, nw, rw));
-        SEDEF_KERNEL(ctx, "k_seq_table",
-                     k_seq_table<<<(int)((sblocks + 255) / 256), 256, 0, st>>>(a.tseq, ntseq, sblocks, stab));
-        int64_t gq = (nt + 1023) / 1024;
-        if (gq > (int64_t)ctx_sm_count(ctx) * 8) gq = (int64_t)ctx_sm_count(ctx) * 8;
-        uint64_t *pk = nullptr, *pks = nullptr;
-        uint32_t *pv = nullptr, *pvs = nullptr;
-        const std::vector<char> no_parts = ctx_pool_snapshot(ctx);
-        if (nt >= kPartRecords) {
-          pk = (uint64_t*)ctx_alloc(ctx, (size_t)nt * 8);
-          pks = pk ? (uint64_t*)ctx_alloc(ctx, (size_t)nt * 8) : nullptr;
-          pv = pks ? (uint32_t*)ctx_alloc(ctx, (size_t)nt * 4) : nullptr;
-          pvs = pv ? (uint32_t*)ctx_alloc(ctx, (size_t)nt * 4) : nullptr;
-          if (!pvs) pk = nullptr;  // no room under the context's cap
-        }
-        SEDEF_KERNEL(ctx, "k_qpost", k_qpost_index<<<(int)gq, 256, 0, st>>>(a, nt, rw, stab, qp, pk, pv));
-        if (pk) {
-          const int pb = bits_below(a.ttotal);
-          // two CTAs per SM: the CTAs drift apart, and with more of them the
-          // stretch of records being written no longer stays in L2 (119 M
-          // records: 0.9 ms; four CTAs per SM 1.7, eight 4.4)
-          const int64_t gp = (int64_t)ctx_sm_count(ctx) * 2;
-          SEDEF_TRY(radix_sort_u64(ctx, pk, pv, pks, pvs, nt, 32 + (pb > 8 ? pb - 8 : 0), 32 + pb));
-          SEDEF_KERNEL(ctx, "k_qpost_place", k_qpost_place<<<(int)gp, 256, 0, st>>>(pks, pvs, nt, rw, qp));
-        }
-        ctx_pool_restore(ctx, no_parts);
-      }
+      SEDEF_TRY(got);
     }
     a.qpost = qp;
   }
@@ -3796,6 +3810,9 @@ int run_filter(sedef_ctx* ctx, const uint64_t* qrec, int64_t nq, const int64_t* 
       SEDEF_TRY(kTierWideMid(ctx, a, iow2, nwin, "k_filter_widemid"));
     }
   }
+  // only the tiers read the posting ranges: what follows may use their memory
+  ctx_pool_restore(ctx, used_before);
+  a.qpost = nullptr;
 
   unsigned long long* h_cnt = nullptr;
   int64_t nov = 0, slow_hits_total = 0;
@@ -4561,63 +4578,64 @@ int sedef_server_finish(sedef_server* srv, int32_t slot, sedef_cand_t* h_cands, 
       status = fail(SEDEF_ERR_CUDA, "sedef_server_finish: counter copy failed");
     if (status != SEDEF_OK) return release(status);
     const int64_t total = (int64_t)h_cnt[0];
-    sedef_run_t* runs = nullptr;
-    if (total > L.run_cap) {
-      // more runs than the slot holds: the whole filter again, sized exactly
-      runs = (sedef_run_t*)ctx_alloc(c, (size_t)total * sizeof(sedef_run_t));
-      if (!runs) return release(SEDEF_ERR_OOM);
-      int64_t got = 0;
-      status = run_filter(c, L.qrec, L.nrec, qoff, 1, s->trec, s->tsorted, s->toff, s->nt,
-                          s->h_toff.data(), (int)s->h_toff.size() - 1, s->D, s->mtab.data(), runs,
-                          total, &got, 0);
-      if (status != SEDEF_OK) return release(status);
-    } else if (total > 0) {
-      runs = (sedef_run_t*)ctx_alloc(c, (size_t)total * sizeof(sedef_run_t));
-      if (!runs) return release(SEDEF_ERR_OOM);
-      {
+    sedef_cand_t* cands = nullptr;
+    auto candidates = [&]() -> int {  // of the raw runs, into cands and nc
+      sedef_run_t* runs = (sedef_run_t*)ctx_alloc(c, (size_t)total * sizeof(sedef_run_t));
+      if (!runs) return SEDEF_ERR_OOM;
+      if (total > L.run_cap) {
+        // more runs than the slot holds: the whole filter again, sized exactly
+        int64_t got = 0;
+        SEDEF_TRY(run_filter(c, L.qrec, L.nrec, qoff, 1, s->trec, s->tsorted, s->toff, s->nt,
+                             s->h_toff.data(), (int)s->h_toff.size() - 1, s->D, s->mtab.data(), runs,
+                             total, &got, 0));
+      } else {
         StageScope stage(c, "runsort");
-        status = order_and_refine(c, L.a, s->D, 1, (const int64_t*)L.d_up + 2, L.nwin, L.wqa, L.wqb,
-                                  L.qrec, L.nrec, s->trec, s->nt, s->toff, L.counters, L.raw, total,
-                                  runs, nullptr, nullptr);
+        SEDEF_TRY(order_and_refine(c, L.a, s->D, 1, (const int64_t*)L.d_up + 2, L.nwin, L.wqa, L.wqb,
+                                   L.qrec, L.nrec, s->trec, s->nt, s->toff, L.counters, L.raw, total,
+                                   runs, nullptr, nullptr));
       }
-      if (status != SEDEF_OK) return release(status);
-    }
-    if (total > 0) {
       sedef_chain_t* chains = (sedef_chain_t*)ctx_alloc(c, (size_t)total * sizeof(sedef_chain_t));
-      if (!chains) return release(SEDEF_ERR_OOM);
+      if (!chains) return SEDEF_ERR_OOM;
       int64_t nch = 0;
       {
         StageScope stage(c, "chain");
-        status = run_chain(c, runs, total, L.qrec, L.nrec, qoff, 1, s->tsorted, s->nt, s->toff,
-                           s->h_toff.data(), (int)s->h_toff.size() - 1, s->D, s->mtab.data(),
-                           chains, total, &nch);
+        SEDEF_TRY(run_chain(c, runs, total, L.qrec, L.nrec, qoff, 1, s->tsorted, s->nt, s->toff,
+                            s->h_toff.data(), (int)s->h_toff.size() - 1, s->D, s->mtab.data(),
+                            chains, total, &nch));
+      }
+      if (nch == 0) return SEDEF_OK;
+      cands = (sedef_cand_t*)ctx_alloc(c, (size_t)nch * sizeof(sedef_cand_t));
+      if (!cands) return SEDEF_ERR_OOM;
+      StageScope stage(c, "merge");
+      return run_merge(c, chains, nch, qoff, 1, s->h_toff.data(), (int)s->h_toff.size() - 1, s->D, cands,
+                       nch, &nc);
+    };
+    if (total > 0) {
+      status = candidates();
+      if (status == SEDEF_ERR_OOM) {
+        // once more without the buffers a call can do without
+        ctx_pool_release(c);
+        ctx_set_extras(c, false);
+        // the runs handed to the large refine kernel are counted anew
+        if (cudaMemsetAsync(L.counters + 3, 0, 8, st) == cudaSuccess) status = candidates();
+        ctx_set_extras(c, true);
       }
       if (status != SEDEF_OK) return release(status);
-      if (nch > 0) {
-        sedef_cand_t* cands = (sedef_cand_t*)ctx_alloc(c, (size_t)nch * sizeof(sedef_cand_t));
-        if (!cands) return release(SEDEF_ERR_OOM);
-        {
-          StageScope stage(c, "merge");
-          status = run_merge(c, chains, nch, qoff, 1, s->h_toff.data(),
-                             (int)s->h_toff.size() - 1, s->D, cands, nch, &nc);
-        }
-        if (status != SEDEF_OK) return release(status);
-        if (nc > cap) {  // keep them for the next call; the slot stays handed out
-          L.fin.resize((size_t)nc);
-          if (cudaMemcpyAsync(L.fin.data(), cands, (size_t)nc * sizeof(sedef_cand_t),
-                              cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-              cudaStreamSynchronize(st) != cudaSuccess)
-            return release(fail(SEDEF_ERR_CUDA, "sedef_server_finish: copy failed"));
-          L.fin_ready = true;
-          *h_ncands = nc;
-          return fail(SEDEF_ERR_CAPACITY, "sedef_server_finish: candidate buffer too small");
-        }
-        if (nc > 0 &&
-            cudaMemcpyAsync(h_cands, cands, (size_t)nc * sizeof(sedef_cand_t),
-                            cudaMemcpyDeviceToHost, st) != cudaSuccess)
-          return release(fail(SEDEF_ERR_CUDA, "sedef_server_finish: copy failed"));
-      }
     }
+    if (nc > cap) {  // keep them for the next call; the slot stays handed out
+      L.fin.resize((size_t)nc);
+      if (cudaMemcpyAsync(L.fin.data(), cands, (size_t)nc * sizeof(sedef_cand_t),
+                          cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+          cudaStreamSynchronize(st) != cudaSuccess)
+        return release(fail(SEDEF_ERR_CUDA, "sedef_server_finish: copy failed"));
+      L.fin_ready = true;
+      *h_ncands = nc;
+      return fail(SEDEF_ERR_CAPACITY, "sedef_server_finish: candidate buffer too small");
+    }
+    if (nc > 0 &&
+        cudaMemcpyAsync(h_cands, cands, (size_t)nc * sizeof(sedef_cand_t), cudaMemcpyDeviceToHost, st) !=
+            cudaSuccess)
+      return release(fail(SEDEF_ERR_CUDA, "sedef_server_finish: copy failed"));
   }
   if (cudaStreamSynchronize(st) != cudaSuccess)
     return release(fail(SEDEF_ERR_CUDA, "sedef_server_finish: stream failed"));

@@ -135,6 +135,7 @@ extern "C" int sedef_qgram(sedef_ctx* ctx, const uint32_t* d_packed, const uint3
   A.need = (int)need;
   A.shared = d_shared;
   A.pass = d_pass;
+  ctx_pool_reset(ctx);
   unsigned long long* cnt = (unsigned long long*)ctx_alloc(ctx, 8);
   if (!cnt) return SEDEF_ERR_OOM;
   SEDEF_CUDA(cudaMemsetAsync(cnt, 0, 8, st));

@@ -1,0 +1,150 @@
+"""Scratch caps: a cap that suffices keeps sufficing when it is raised, and buffers that a call can
+do without (posting ranges, refine events) are not what it fails for."""
+import numpy as np
+import pytest
+
+from paper_1807_00205_gb300 import binding, synth
+from tests.gpu_helpers import need_gpu
+
+pytestmark = pytest.mark.gpu
+
+
+def to_dev(a):
+    return need_gpu().from_numpy(np.ascontiguousarray(a)).to("cuda:0")
+
+
+def genome(mode):
+    return synth.small_case(5, lengths=(600_000, 300_000) if mode == 1 else (300_000,) * 3, n_sd=40,
+                            sd_lo=2000, sd_hi=9000, mask_frac=0.25)
+
+
+def accepted(ctx, caps, call):
+    """Which caps `call` passes under; any other outcome than success and OOM is an error."""
+    ok = np.zeros(len(caps), dtype=bool)
+    for k, cap in enumerate(caps):
+        ctx.sedef_set_scratch_limit(0)
+        ctx.sedef_set_scratch_limit(int(cap))
+        try:
+            call()
+            ok[k] = True
+        except binding.SedefError as e:
+            assert e.status == -2, e  # SEDEF_ERR_OOM
+    return ok
+
+
+@pytest.mark.parametrize("pd", [dict(), dict(k=13), dict(w=3, n=300, query_step=100), dict(self_mode=2),
+                                dict(self_mode=2, k=14)])
+def test_filter_caps(pd):
+    ctx = binding.Context(0)
+    g = genome(pd.get("self_mode", 1))
+    p = binding.params(**pd)
+    rec = ctx.sedef_sketch(*ctx.sedef_pack(to_dev(g.seq)), g.offsets, p)
+    srt, off = ctx.sedef_index(rec, p)
+    want, n = ctx.sedef_filter(rec, g.offsets, rec, srt, off, g.offsets, p)
+    want = want.cpu()
+    # the records' ranges alone are 8 bytes each; the caps reach well below that
+    caps = np.geomspace(4 * rec.numel(), 64 << 20, 120).astype(np.int64)
+    ctx.sedef_trace_enable(True)
+    with_ranges = []
+
+    def call():
+        ctx.sedef_trace_report(reset=True)
+        runs, m = ctx.sedef_filter(rec, g.offsets, rec, srt, off, g.offsets, p, cap=n + 1)
+        assert m == n and bool((runs.cpu() == want).all())
+        with_ranges.append(any(x.endswith("k_pos_bits") for x in ctx.sedef_trace_report(reset=True)))
+
+    ok = accepted(ctx, caps, call)
+    first = int(np.argmax(ok))
+    assert ok[first:].all(), caps[first:][~ok[first:]]
+    assert caps[first] < 8 * rec.numel()
+    assert not with_ranges[0] and with_ranges[-1]
+    ctx.close()
+
+
+def test_stage_after_stage_caps():
+    """One context through the whole search: what the filter could do without is there for the
+    calls after it."""
+    ctx = binding.Context(0)
+    g = genome(1)
+    p = binding.params()
+    d = to_dev(g.seq)
+    want = binding.struct_view(ctx.sedef_selfsearch(d, g.offsets, p)[0], binding.CAND_DTYPE)
+    out = ctx.selfsearch(d, g.offsets, p)
+
+    def call():
+        runs, n = ctx.sedef_filter(out["rec"], g.offsets, out["rec"], out["sorted"], out["off"], g.offsets, p,
+                                   cap=out["nruns"] + 1)
+        chains, m = ctx.sedef_chain(runs, n, out["rec"], g.offsets, out["sorted"], out["off"], g.offsets, p)
+        cands, _ = ctx.sedef_merge(chains, m, g.offsets, g.offsets, p)
+        assert np.array_equal(binding.struct_view(cands, binding.CAND_DTYPE), want)
+
+    caps = np.geomspace(100 << 10, 64 << 20, 120).astype(np.int64)
+    ok = accepted(ctx, caps, call)
+    first = int(np.argmax(ok))
+    assert 0 < first and ok[first:].all(), caps[first:][~ok[first:]]
+
+    def whole():
+        assert np.array_equal(binding.struct_view(ctx.sedef_selfsearch(d, g.offsets, p)[0],
+                                                  binding.CAND_DTYPE), want)
+
+    caps = np.linspace(64 << 20, 84 << 20, 160).astype(np.int64)  # the offset table alone: 64 MB and 4 bytes
+    ok = accepted(ctx, caps, whole)
+    first = int(np.argmax(ok))
+    assert 0 < first and ok[first:].all(), caps[first:][~ok[first:]]
+    ctx.close()
+
+
+@pytest.mark.parametrize("mode", [1, 2])
+def test_graph_caps(mode):
+    """A captured pass is recorded without the ranges and events where the cap has no room for them."""
+    ctx = binding.Context(0)
+    g = genome(mode)
+    p = binding.params(self_mode=mode)
+    d = to_dev(g.seq)
+    want = ctx.selfsearch(d, g.offsets, p)
+    rows = binding.struct_view(want["cands"], binding.CAND_DTYPE)
+    need = dict(records=want["rec"].numel(), slow_hits=1000, runs=want["nruns"],
+                anchors=40 * want["nruns"] + 1000, chains=want["nchains"], cands=want["ncands"])
+    nodes = []
+
+    def call():
+        gr = binding.Graph(ctx, d, g.offsets, p, need)
+        gr.launch()
+        gr.wait()
+        assert np.array_equal(binding.struct_view(gr.outputs()["cands"], binding.CAND_DTYPE), rows)
+        nodes.append(gr.nodes)
+        gr.close()
+
+    caps = np.geomspace(1 << 20, 32 << 20, 250).astype(np.int64)
+    ok = accepted(ctx, caps, call)
+    first = int(np.argmax(ok))
+    assert 0 < first and ok[first:].all(), caps[first:][~ok[first:]]
+    assert nodes[0] < nodes[-1]
+    ctx.close()
+
+
+def test_server_caps():
+    """A served request under the caps of the server's context."""
+    ctx = binding.Context(0)
+    g = synth.small_case(8, lengths=(400_000,), n_sd=20, sd_lo=2000, sd_hi=9000)
+    p = binding.params(self_mode=0)
+    rec = ctx.sedef_sketch(*ctx.sedef_pack(to_dev(g.seq)), g.offsets, p)
+    srt, off = ctx.sedef_index(rec, p)
+    query = g.seq[50_000:230_000]
+    rows = []
+
+    def call():
+        srv = binding.DeviceServer(ctx, rec, srt, off, g.offsets, p, slots=1, slot_bases=200_000)
+        try:
+            slot = srv.submit(query)
+            assert srv.poll(5.0) == slot
+            rows.append(srv.finish(slot))
+        finally:
+            srv.close()
+
+    caps = np.geomspace(64 << 10, 16 << 20, 60).astype(np.int64)
+    ok = accepted(ctx, caps, call)
+    first = int(np.argmax(ok))
+    assert 0 < first and ok[first:].all(), caps[first:][~ok[first:]]
+    assert len(rows[0]) > 0 and all(np.array_equal(r, rows[-1]) for r in rows)
+    ctx.close()
