@@ -3437,8 +3437,15 @@ int posting_ranges(sedef_ctx* ctx, const FArgs& a, int64_t nq, int64_t nt, const
     // stretch of records being written no longer stays in L2 (119 M
     // records: 0.9 ms; four CTAs per SM 1.7, eight 4.4)
     const int64_t gp = (int64_t)ctx_sm_count(ctx) * 2;
-    SEDEF_TRY(radix_sort_u64(ctx, pk, pv, pks, pvs, nt, 32 + (pb > 8 ? pb - 8 : 0), 32 + pb));
-    SEDEF_KERNEL(ctx, "k_qpost_place", k_qpost_place<<<(int)gp, 256, 0, st>>>(pks, pvs, nt, rw, qp));
+    const int sorted = radix_sort_u64(ctx, pk, pv, pks, pvs, nt, 32 + (pb > 8 ? pb - 8 : 0), 32 + pb);
+    if (sorted == SEDEF_ERR_OOM) {
+      // no room for the sort's own scratch: straight to their records after all
+      SEDEF_KERNEL(ctx, "k_qpost",
+                   k_qpost_index<<<(int)gq, 256, 0, st>>>(a, nt, rw, stab, qp, nullptr, nullptr));
+    } else {
+      SEDEF_TRY(sorted);
+      SEDEF_KERNEL(ctx, "k_qpost_place", k_qpost_place<<<(int)gp, 256, 0, st>>>(pks, pvs, nt, rw, qp));
+    }
   }
   ctx_pool_restore(ctx, no_parts);
   return SEDEF_OK;

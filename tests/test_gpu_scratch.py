@@ -148,3 +148,46 @@ def test_server_caps():
     assert 0 < first and ok[first:].all(), caps[first:][~ok[first:]]
     assert len(rows[0]) > 0 and all(np.array_equal(r, rows[-1]) for r in rows)
     ctx.close()
+
+
+def test_parted_ranges_caps():
+    """More records than the ranges are parted from (16 M), with room for the parts and not for the
+    sort's own scratch: the ranges go straight to their records, so the hits looked at are as many
+    as without a cap (without ranges they would be about twice as many)."""
+    torch = need_gpu()
+    ctx = binding.Context(0)
+    rng = np.random.default_rng(2)
+    s = np.empty(17_400_000, dtype=np.uint8)
+    synth.random_bases_chunked(rng, s, 0.5)
+    for at in range(0, 200_000, 10_000):
+        s[9_000_000 + at:9_004_000 + at] = s[at:at + 4_000]
+    g = synth.genome_from_parts([s])
+    p = binding.params(w=1, n=100, query_step=5_000)
+    rec = ctx.sedef_sketch(*ctx.sedef_pack(to_dev(s)), g.offsets, p, cap=len(s))
+    assert rec.numel() > 16 << 20
+    srt, off = ctx.sedef_index(rec, p)
+    ctx.sedef_trace_enable(True)
+
+    def run(cap):
+        ctx.sedef_set_scratch_limit(0)
+        ctx.sedef_set_scratch_limit(int(cap))
+        ctx.sedef_trace_report(reset=True)
+        runs, n = ctx.sedef_filter(rec, g.offsets, rec, srt, off, g.offsets, p, cap=1 << 20)
+        placed = any(x.endswith("k_qpost_place") for x in ctx.sedef_trace_report(reset=True))
+        return runs.cpu(), ctx.sedef_filter_stats()["hits"], placed
+
+    want, hits, placed = run(4 << 30)
+    assert placed and len(want) > 0
+    lo, hi = 256 << 20, 4 << 30  # the smallest cap under which the parts are placed
+    while hi - lo > 64 << 10:
+        mid = (lo + hi) // 2
+        if run(mid)[2]:
+            hi = mid
+        else:
+            lo = mid
+    # the sort's scratch is half a byte a record
+    for cap in (lo, lo - rec.numel() // 4, lo - rec.numel() // 2 + (64 << 10), lo - rec.numel()):
+        runs, n, placed = run(cap)
+        assert not placed and n == hits, cap
+        assert torch.equal(runs, want), cap
+    ctx.close()
