@@ -905,15 +905,18 @@ int run_merge(sedef_ctx* ctx, const sedef_chain_t* chains, int64_t n, const int6
   const uint32_t* dn = pl ? pl->n_chains : nullptr;
   int64_t *dq = nullptr, *dt = nullptr;
   SEDEF_TRY(upload_offsets(ctx, pl, h_qoff, nqseq, h_toff, ntseq, &dq, &dt));
-  uint64_t* key = (uint64_t*)ctx_alloc(ctx, (size_t)n * 8);
+  // 56 bytes a chain: the flags and their sums take the sort keys' place, the
+  // components' boxes that of the chains'
+  uint64_t* key = (uint64_t*)ctx_alloc(ctx, (size_t)(n + 1) * 8);
   uint64_t* skey = (uint64_t*)ctx_alloc(ctx, (size_t)n * 8);
   uint32_t* perm = (uint32_t*)ctx_alloc(ctx, (size_t)n * 4);
   int32_t* parent = (int32_t*)ctx_alloc(ctx, (size_t)n * 4);
-  Agg* agg = (Agg*)ctx_alloc(ctx, (size_t)n * sizeof(Agg));
-  uint32_t* flag = (uint32_t*)ctx_alloc(ctx, (size_t)(n + 1) * 4);
-  uint32_t* pos = (uint32_t*)ctx_alloc(ctx, (size_t)(n + 1) * 4);
   LinkBox* boxes = (LinkBox*)ctx_alloc(ctx, (size_t)n * sizeof(LinkBox));
-  if (!key || !skey || !perm || !parent || !agg || !flag || !pos || !boxes) return SEDEF_ERR_OOM;
+  if (!key || !skey || !perm || !parent || !boxes) return SEDEF_ERR_OOM;
+  uint32_t* flag = (uint32_t*)key;
+  uint32_t* pos = flag + (n + 1);
+  static_assert(sizeof(Agg) <= sizeof(LinkBox), "a component's box fits in a chain's place");
+  Agg* agg = (Agg*)boxes;
   const int g = grid_of(n, 256);
   // sort keys of only as many bits as the positions have
   const int qbits = bits_below(h_qoff[nqseq] + 1), tbits = bits_below(h_toff[ntseq] + 1);
@@ -955,7 +958,7 @@ int run_merge(sedef_ctx* ctx, const sedef_chain_t* chains, int64_t n, const int6
   }
   if (nc == 0) return SEDEF_OK;
   sedef_cand_t* tmp = (sedef_cand_t*)ctx_alloc(ctx, (size_t)nc * sizeof(sedef_cand_t));
-  uint64_t* ckey = (uint64_t*)ctx_alloc(ctx, (size_t)nc * 8);
+  uint64_t* ckey = nc <= n ? skey : (uint64_t*)ctx_alloc(ctx, (size_t)nc * 8);
   uint64_t* cskey = (uint64_t*)ctx_alloc(ctx, (size_t)nc * 8);
   uint32_t* cperm = (uint32_t*)ctx_alloc(ctx, (size_t)nc * 4);
   if (!tmp || !ckey || !cskey || !cperm) return SEDEF_ERR_OOM;

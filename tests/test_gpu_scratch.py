@@ -191,3 +191,24 @@ def test_parted_ranges_caps():
         assert not placed and n == hits, cap
         assert torch.equal(runs, want), cap
     ctx.close()
+
+
+def test_merge_caps():
+    """Scratch of the merge: 56 bytes a chain and its sort's 12.5, 52 a candidate."""
+    ctx = binding.Context(0)
+    g = synth.small_case(6, lengths=(700_000, 500_000), n_sd=60, sd_lo=2000, sd_hi=9000, mask_frac=0.25)
+    p = binding.params(self_mode=0, query_step=100)
+    rec = ctx.sedef_sketch(*ctx.sedef_pack(to_dev(g.seq)), g.offsets, p)
+    srt, off = ctx.sedef_index(rec, p)
+    runs, n = ctx.sedef_filter(rec, g.offsets, rec, srt, off, g.offsets, p)
+    chains, m = ctx.sedef_chain(runs, n, rec, g.offsets, srt, off, g.offsets, p)
+    cands, nc = ctx.sedef_merge(chains, m, g.offsets, g.offsets, p)
+    assert m > 4096
+    small = 24 << 10  # offsets, the sorts' heads, each array rounded up to 256 bytes
+
+    def merge():
+        got, k = ctx.sedef_merge(chains, m, g.offsets, g.offsets, p)
+        assert k == nc and np.array_equal(got.cpu(), cands.cpu())
+
+    assert accepted(ctx, [68.5 * m + 52 * nc + (12.5 * nc if nc > 4096 else 0) + small], merge).all()
+    ctx.close()
