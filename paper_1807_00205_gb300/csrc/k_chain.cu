@@ -807,7 +807,9 @@ int run_chain(sedef_ctx* ctx, const sedef_run_t* runs, int64_t nruns, const uint
   uint32_t* cnt = (uint32_t*)ctx_alloc(ctx, (size_t)(nruns + 1) * 4);
   a.big = (uint32_t*)ctx_alloc(ctx, (size_t)nruns * 4);
   sedef_chain_t* tmp = (sedef_chain_t*)ctx_alloc(ctx, (size_t)nruns * sizeof(sedef_chain_t));
-  if (!sums || !cnt || !a.big || !tmp) return SEDEF_ERR_OOM;
+  // the big seeds' anchor offsets, then the chains' places
+  uint32_t* pos = (uint32_t*)ctx_alloc(ctx, (size_t)(nruns + 1) * 4);
+  if (!sums || !cnt || !a.big || !tmp || !pos) return SEDEF_ERR_OOM;
   SEDEF_CUDA(cudaMemsetAsync(sums, 0, 24, st));
   a.atotal = sums;
   a.nbig = (uint32_t*)(sums + 1);
@@ -834,8 +836,7 @@ int run_chain(sedef_ctx* ctx, const sedef_run_t* runs, int64_t nruns, const uint
   if (nbig > 0) {
     // the seeds past the shared-memory sizes (a planned pass does not know
     // whether there are any)
-    uint32_t* aoff = (uint32_t*)ctx_alloc(ctx, (size_t)(nbig + 1) * 4);
-    if (!aoff) return SEDEF_ERR_OOM;
+    uint32_t* aoff = pos;
     const int wb = grid_of(nbig * 32 < most * 256 ? nbig * 32 : most * 256, 256);
     if (pl) SEDEF_CUDA(cudaMemsetAsync(cnt, 0, (size_t)(nbig + 1) * 4, st));
     SEDEF_KERNEL(ctx, "k_anchor_count", k_anchor_count<<<wb, 256, 0, st>>>(a, cnt));
@@ -870,8 +871,6 @@ int run_chain(sedef_ctx* ctx, const sedef_run_t* runs, int64_t nruns, const uint
     SEDEF_KERNEL(ctx, "k_chain_dp", k_chain_dp<<<wb, 256, 0, st>>>(a, aoff, anchors, f, pred, tmp));
   }
   uint32_t* flag = cnt;  // reuse
-  uint32_t* pos = (uint32_t*)ctx_alloc(ctx, (size_t)(nruns + 1) * 4);
-  if (!pos) return SEDEF_ERR_OOM;
   const uint32_t* dn = pl ? pl->n_runs : nullptr;
   SEDEF_KERNEL(ctx, "k_chain_flags",
                k_chain_flags<<<grid_of(nruns, 256), 256, 0, st>>>(tmp, nruns, flag, dn));

@@ -489,7 +489,7 @@ int radix_sort_u64(sedef_ctx* ctx, const uint64_t* keys_in, const uint32_t* vals
     return SEDEF_OK;
   }
   const int64_t ntiles = (n + kRsTile - 1) / kRsTile;
-  const size_t head = 64 + (size_t)kRsPasses * 256 * 4;
+  const size_t head = 64 + (size_t)passes * 256 * 4;
   char* scratch = (char*)ctx_alloc(ctx, head + (size_t)ntiles * 256 * 8);
   uint64_t* ktmp = passes > 1 ? (uint64_t*)ctx_alloc(ctx, (size_t)n * 8) : nullptr;
   uint32_t* vtmp = vals_out && passes > 1 ? (uint32_t*)ctx_alloc(ctx, (size_t)n * 4) : nullptr;

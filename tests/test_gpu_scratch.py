@@ -212,3 +212,34 @@ def test_merge_caps():
 
     assert accepted(ctx, [68.5 * m + 52 * nc + (12.5 * nc if nc > 4096 else 0) + small], merge).all()
     ctx.close()
+
+
+@pytest.mark.parametrize("pd", [dict(self_mode=0, query_step=100), dict(w=1, n=500, query_step=500)])
+def test_chain_caps(pd):
+    """Scratch of the chain: 52 bytes a run, 16 an anchor of the seeds past what one warp holds (in a
+    self-search 256 query records: a window of 500 bases has 489 of them at w = 1)."""
+    ctx = binding.Context(0)
+    g = synth.small_case(6, lengths=(700_000, 500_000), n_sd=60, sd_lo=2000, sd_hi=9000)
+    p = binding.params(**pd)
+    rec = ctx.sedef_sketch(*ctx.sedef_pack(to_dev(g.seq)), g.offsets, p, cap=g.length)
+    srt, off = ctx.sedef_index(rec, p)
+    runs, n = ctx.sedef_filter(rec, g.offsets, rec, srt, off, g.offsets, p)
+    # many of the same seeds, so that the bytes a run count
+    runs = runs.reshape(n, -1).repeat(128, 1).reshape(-1)
+    n *= 128
+    args = (runs, n, rec, g.offsets, srt, off, g.offsets, p)
+    ctx.sedef_trace_enable(True)
+    chains, m = ctx.sedef_chain(*args)
+    big = any(x.endswith("k_anchor_fill") for x in ctx.sedef_trace_report(reset=True))
+    assert big == (p.w == 1)
+    anchors = ctx.sedef_filter_stats()["anchors"] if big else 0
+    keep = int(binding.struct_view(runs, binding.RUN_DTYPE)["keep"].sum())
+    assert 4 * keep > 64 << 10  # so that four bytes a kept run more would show
+    small = 24 << 10  # offsets, table, each array rounded up to 256 bytes, the scan's sums
+
+    def chain():
+        got, k = ctx.sedef_chain(*args)
+        assert k == m and np.array_equal(got.cpu(), chains.cpu())
+
+    assert accepted(ctx, [52 * n + 16 * anchors + small], chain).all()
+    ctx.close()
