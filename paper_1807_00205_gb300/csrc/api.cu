@@ -596,10 +596,12 @@ int sedef_filter_variant(sedef_ctx* ctx, int32_t set, int32_t* current, int32_t*
   return SEDEF_OK;
 }
 
-int sedef_chain(sedef_ctx* ctx, const sedef_run_t* d_runs, int64_t nruns, const uint64_t* d_qrec,
-                int64_t nq, const int64_t* h_qoff, int32_t nqseq, const uint64_t* d_tsorted,
-                const uint32_t* d_toff, int64_t nt, const int64_t* h_toff, int32_t ntseq,
-                const sedef_params* p, sedef_chain_t* d_chains, int64_t cap, int64_t* h_nchains) {
+// one_sketch: the index is known to be that of the query records.
+static int chain_call(sedef_ctx* ctx, const sedef_run_t* d_runs, int64_t nruns, const uint64_t* d_qrec,
+                      int64_t nq, const int64_t* h_qoff, int32_t nqseq, const uint64_t* d_tsorted,
+                      const uint32_t* d_toff, int64_t nt, const int64_t* h_toff, int32_t ntseq,
+                      const sedef_params* p, sedef_chain_t* d_chains, int64_t cap,
+                      int64_t* h_nchains, bool one_sketch) {
   if (!ctx || !h_nchains) return fail(SEDEF_ERR_INVALID, "NULL argument");
   Derived D;
   SEDEF_TRY(derive(p, &D));
@@ -617,8 +619,16 @@ int sedef_chain(sedef_ctx* ctx, const sedef_run_t* d_runs, int64_t nruns, const 
   StageScope stage(ctx, "chain");
   return with_room(ctx, [&] {
     return run_chain(ctx, d_runs, nruns, d_qrec, nq, h_qoff, nqseq, d_tsorted, nt, d_toff, h_toff,
-                     ntseq, D, mt.data(), d_chains, cap, h_nchains);
+                     ntseq, D, mt.data(), d_chains, cap, h_nchains, nullptr, one_sketch);
   });
+}
+
+int sedef_chain(sedef_ctx* ctx, const sedef_run_t* d_runs, int64_t nruns, const uint64_t* d_qrec,
+                int64_t nq, const int64_t* h_qoff, int32_t nqseq, const uint64_t* d_tsorted,
+                const uint32_t* d_toff, int64_t nt, const int64_t* h_toff, int32_t ntseq,
+                const sedef_params* p, sedef_chain_t* d_chains, int64_t cap, int64_t* h_nchains) {
+  return chain_call(ctx, d_runs, nruns, d_qrec, nq, h_qoff, nqseq, d_tsorted, d_toff, nt, h_toff, ntseq, p,
+                    d_chains, cap, h_nchains, false);
 }
 
 int sedef_extend(sedef_ctx* ctx, const sedef_run_t* d_runs, int64_t nruns, const uint64_t* d_qext,
@@ -749,8 +759,8 @@ int selfsearch_device(sedef_ctx* ctx, const uint8_t* seq, const int64_t* h_seq_o
   SEDEF_TRY(status);
   ctx->last_runs = nruns;
   DALLOC(chains, (size_t)(nruns ? nruns : 1) * sizeof(sedef_chain_t));
-  SEDEF_TRY(sedef_chain(ctx, runs, nruns, rec, nrec, h_seq_off, nseq, sorted, off, nrec, h_seq_off,
-                        nseq, p, chains, nruns, &nch));
+  SEDEF_TRY(chain_call(ctx, runs, nruns, rec, nrec, h_seq_off, nseq, sorted, off, nrec, h_seq_off,
+                       nseq, p, chains, nruns, &nch, true));
   DALLOC(cands, (size_t)(nch ? nch : 1) * sizeof(sedef_cand_t));
   SEDEF_TRY(sedef_merge(ctx, chains, nch, h_seq_off, nseq, h_seq_off, nseq, p, cands, nch, &nc));
 #undef DALLOC

@@ -357,7 +357,7 @@ int run_chain(sedef_ctx* ctx, const sedef_run_t* runs, int64_t nruns, const uint
               const int64_t* h_qoff, int nqseq, const uint64_t* tsorted, int64_t nt,
               const uint32_t* toff, const int64_t* h_toff, int ntseq, const Derived& D,
               const int32_t* h_mtab, sedef_chain_t* chains, int64_t cap, int64_t* nchains,
-              Planned* pl = nullptr);
+              Planned* pl = nullptr, bool one_sketch = false);  // tsorted: the index of qrec
 int run_merge(sedef_ctx* ctx, const sedef_chain_t* chains, int64_t nchains, const int64_t* h_qoff,
               int nqseq, const int64_t* h_toff, int ntseq, const Derived& D, sedef_cand_t* cands,
               int64_t cap, int64_t* ncands, Planned* pl = nullptr);

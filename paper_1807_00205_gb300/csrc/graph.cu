@@ -58,7 +58,8 @@ int record_pass(sedef_graph* g, const uint8_t* d_seq, const int64_t* h_off, int 
   SEDEF_TRY(run_filter(c, g->rec, cp.records, h_off, nseq, g->rec, g->srt, g->off, cp.records,
                        h_off, nseq, D, mt, g->runs, cp.runs, &nruns, 0, &g->pl));
   SEDEF_TRY(run_chain(c, g->runs, cp.runs, g->rec, cp.records, h_off, nseq, g->srt, cp.records,
-                      g->off, h_off, nseq, D, mt, g->chains, cp.chains, &nch, &g->pl));
+                      g->off, h_off, nseq, D, mt, g->chains, cp.chains, &nch, &g->pl,
+                      D.self_mode != 0));
   SEDEF_TRY(run_merge(c, g->chains, cp.chains, h_off, nseq, h_off, nseq, D, g->cands, cp.cands,
                       &nc, &g->pl));
   SEDEF_CUDA(cudaMemcpyAsync(g->h_block, g->d_block, kBlockBytes, cudaMemcpyDeviceToHost, st));

@@ -2,8 +2,9 @@
 // merge of chains into SD candidates.
 //
 // Chain: one warp per kept run finds its anchors, runs the DP over them in
-// shared memory and writes the chain (k_chain_seeds).  In a self-search the
-// target records by position are the query records, so the anchors are a join
+// shared memory and writes the chain (k_chain_seeds).  In a self-search whose
+// target records are the query records (a caller's index is compared with them
+// first) the anchors are a join
 // of two contiguous stretches: the window's records go into a hash table and
 // the target span's records probe it.  Otherwise each query minimizer searches
 // its posting list for the target span (an interpolated search, then a short
@@ -51,6 +52,9 @@ struct ChainArgs {
   // seeds past k_chain_seeds' sizes: run indices and their number
   uint32_t* big = nullptr;
   uint32_t* nbig = nullptr;
+  // query records less target records, summed (k_same_records): zero when they
+  // are the same; nullptr: known to be
+  const unsigned long long* differ = nullptr;
 };
 
 // The chain DP is quadratic in a seed's anchors; a seed inside an unmasked
@@ -110,6 +114,38 @@ __device__ __forceinline__ void window_range(const ChainArgs& a, int64_t i, int6
   *qb = lower_bound_by(a.qrec, *qa, a.nq, (uint64_t)(i + a.span + 1), pos_of);
 }
 
+// The finalizer of SplitMix64 (Steele, Lea, Flood: Fast Splittable
+// Pseudorandom Number Generators, 2014).
+__device__ __forceinline__ unsigned long long mix64(unsigned long long z) {
+  z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
+  z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
+  return z ^ (z >> 31);
+}
+
+// Adds to differ[0..2) two mixes of every query record and takes those of the
+// index's away.  Both sums are zero when the arrays hold the same records in
+// any order, and otherwise with a chance of 2^-128: the join may take the
+// target's records by position from the query's.  Bound by reading both
+// arrays once (16 bytes a record).
+__global__ void __launch_bounds__(256) k_same_records(const uint64_t* __restrict__ q,
+                                                      const uint64_t* __restrict__ t, int64_t n,
+                                                      unsigned long long* differ) {
+  unsigned long long a = 0, b = 0;
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+#pragma unroll 4
+  for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < n; x += stride) {
+    const unsigned long long u = q[x], v = t[x];
+    a += mix64(u) - mix64(v);
+    b += mix64(~u) - mix64(~v);
+  }
+  a = warp_sum(a);
+  b = warp_sum(b);
+  if (lane_id() == 0 && (a | b)) {
+    atomicAdd(differ, a);
+    atomicAdd(differ + 1, b);
+  }
+}
+
 // What k_chain_seeds keeps of a seed in shared memory.
 constexpr int kSeedWarps = 8;
 constexpr int kSeedQ = 256;            // query records
@@ -133,6 +169,8 @@ struct alignas(16) SeedSmem {
 // 1.2 ms.
 template <bool kJoin>
 __global__ void __launch_bounds__(32 * kSeedWarps) k_chain_seeds(ChainArgs a, sedef_chain_t* out) {
+  // of the two forms the one for the records at hand
+  if (a.differ && ((a.differ[0] | a.differ[1]) != 0ull) == kJoin) return;
   resolve(a);
   __shared__ SeedSmem smem[kSeedWarps];
   SeedSmem& S = smem[threadIdx.x >> 5];
@@ -760,7 +798,7 @@ int run_chain(sedef_ctx* ctx, const sedef_run_t* runs, int64_t nruns, const uint
               const int64_t* h_qoff, int nqseq, const uint64_t* tsorted, int64_t nt,
               const uint32_t* toff, const int64_t* h_toff, int ntseq, const Derived& D,
               const int32_t* h_mtab, sedef_chain_t* chains, int64_t cap, int64_t* nchains,
-              Planned* pl) {
+              Planned* pl, bool one_sketch) {
   cudaStream_t st = ctx_stream(ctx);
   int64_t *dq = nullptr, *dt = nullptr;
   SEDEF_TRY(upload_offsets(ctx, pl, h_qoff, nqseq, h_toff, ntseq, &dq, &dt));
@@ -802,26 +840,35 @@ int run_chain(sedef_ctx* ctx, const sedef_run_t* runs, int64_t nruns, const uint
     a.flags = pl->flags;
   }
   // [0] anchors of every seed, [1] seeds for the device-memory path, [2] the
-  // most anchors one of them has
-  unsigned long long* sums = (unsigned long long*)ctx_alloc(ctx, 24);
+  // most anchors one of them has, [3] and [4] k_same_records' sums
+  unsigned long long* sums = (unsigned long long*)ctx_alloc(ctx, 40);
   uint32_t* cnt = (uint32_t*)ctx_alloc(ctx, (size_t)(nruns + 1) * 4);
   a.big = (uint32_t*)ctx_alloc(ctx, (size_t)nruns * 4);
   sedef_chain_t* tmp = (sedef_chain_t*)ctx_alloc(ctx, (size_t)nruns * sizeof(sedef_chain_t));
   // the big seeds' anchor offsets, then the chains' places
   uint32_t* pos = (uint32_t*)ctx_alloc(ctx, (size_t)(nruns + 1) * 4);
   if (!sums || !cnt || !a.big || !tmp || !pos) return SEDEF_ERR_OOM;
-  SEDEF_CUDA(cudaMemsetAsync(sums, 0, 24, st));
+  SEDEF_CUDA(cudaMemsetAsync(sums, 0, 40, st));
   a.atotal = sums;
   a.nbig = (uint32_t*)(sums + 1);
   uint32_t* amax = (uint32_t*)(sums + 2);
-  // a self-search's query records are its target records by position
-  const bool join = D.self_mode != 0 && nq == nt && nqseq == ntseq &&
-                    std::memcmp(h_qoff, h_toff, (size_t)(ntseq + 1) * sizeof(int64_t)) == 0;
+  // a self-search's query records are its target records by position: where
+  // the caller gave an index that may be another's, both forms are launched
+  // and the one that the records call for runs
+  const bool join = one_sketch || (D.self_mode != 0 && nq == nt && nqseq == ntseq &&
+                    std::memcmp(h_qoff, h_toff, (size_t)(ntseq + 1) * sizeof(int64_t)) == 0);
   const int64_t most = (int64_t)ctx_sm_count(ctx) * 5;
   const int sg = (int)((nruns + kSeedWarps - 1) / kSeedWarps < most ? (nruns + kSeedWarps - 1) / kSeedWarps : most);
+  if (join && !one_sketch) {
+    a.differ = sums + 3;
+    const int64_t cg = (nq + 1023) / 1024;
+    SEDEF_KERNEL(ctx, "k_same_records",
+                 k_same_records<<<(int)(cg < most ? (cg > 0 ? cg : 1) : most), 256, 0, st>>>(
+                     qrec, tsorted, nq, sums + 3));
+  }
   if (join)
     SEDEF_KERNEL(ctx, "k_chain_seeds", k_chain_seeds<true><<<sg, 32 * kSeedWarps, 0, st>>>(a, tmp));
-  else
+  if (!one_sketch)
     SEDEF_KERNEL(ctx, "k_chain_seeds", k_chain_seeds<false><<<sg, 32 * kSeedWarps, 0, st>>>(a, tmp));
   int64_t nbig = nruns, A = 0;
   unsigned long long* h_sums = nullptr;
