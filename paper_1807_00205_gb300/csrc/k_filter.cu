@@ -2212,12 +2212,16 @@ __device__ __forceinline__ void slow_task(SlowTask* tasks, unsigned long long* n
   }
 }
 
-// kGroupHits hits of a strand per warp: it takes the groups that start among
-// them, to their ends.  Whether a dense hit starts a group depends on the
-// nearest dense hit before it alone, at most span + 1 back.  (One warp per
-// window, through both strands: 0.48 ms for a window of 22 k hits, 0.05 this
-// way.)
+// A window's hits are shared out to `parts` warps, kGroupHits of a strand at a
+// time: a warp takes the groups that start among them, to their ends.  Whether
+// a dense hit starts a group depends on the nearest dense hit before it alone,
+// at most span + 1 back.  As many parts as the grid has warps to spare for the
+// windows at hand; one part takes a strand in one go.  (One warp for a window
+// of 22 k hits, through both strands: 0.48 ms, 0.05 in 32 parts; 32 parts for
+// each of 40 k windows of 500 or 1,800 hits: 1.56 and 4.9 ms, 0.18 and 0.48 with
+// a warp each.)
 constexpr int kGroupHits = 512;
+constexpr int kGroupParts = 32;
 
 __global__ void k_slow_groups(FArgs a, int64_t v0, int64_t v1, const unsigned long long* base,
                               const int32_t* s_of, const uint64_t* keys, SlowTask* tasks,
@@ -2225,15 +2229,20 @@ __global__ void k_slow_groups(FArgs a, int64_t v0, int64_t v1, const unsigned lo
                               int64_t hcap) {
   const int lane = lane_id();
   const unsigned lt = lanemask_lt();
-  const int64_t parts = (int64_t)gridDim.y * (blockDim.x >> 5);
-  const int64_t part = (int64_t)blockIdx.y * (blockDim.x >> 5) + (threadIdx.x >> 5);
   v1 = live_n(v1, dnov);
-  for (int64_t v = v0 + blockIdx.x; v < v1; v += gridDim.x) {
+  if (v1 <= v0) return;
+  const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
+  int parts = 1;  // a power of two: the grid's warps are a multiple of kGroupParts
+  while (parts < kGroupParts && 2 * parts * (v1 - v0) <= warps) parts <<= 1;
+  const int64_t chunk = parts > 1 ? kGroupHits : INT64_MAX / 2;
+  const int64_t w = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  const int64_t part = w & (parts - 1);
+  for (int64_t v = v0 + w / parts; v < v1; v += warps / parts) {
     const int s = s_of[v];
     if (s == 0 || base[v + 1] < base[v] || (int64_t)(base[v + 1] - base[v0]) > hcap) continue;
     const int m = a.mtab[s];
     const int64_t lo = (int64_t)(base[v] - base[v0]), hi = (int64_t)(base[v + 1] - base[v0]);
-    if (lo + part * kGroupHits >= hi) continue;
+    if (part > 0 && lo + part * chunk >= hi) continue;
     int64_t split;
     slow_segment(keys, lo, hi, &split);
     for (int o = 0; o < 2; ++o) {
@@ -2247,8 +2256,8 @@ __global__ void k_slow_groups(FArgs a, int64_t v0, int64_t v1, const unsigned lo
         *jhi = ta;
         return tb - ta <= a.span;
       };
-      for (int64_t x0 = part * kGroupHits; x0 < nd; x0 += parts * kGroupHits) {
-        const int64_t x1 = min(x0 + kGroupHits, nd);
+      for (int64_t x0 = part ? part * chunk : 0; x0 < nd; x0 += parts * chunk) {
+        const int64_t x1 = min(x0 + chunk, nd);
         int64_t carry_hi = INT64_MIN, cur_lo = 0;  // jhi of the nearest dense hit before; the open group
         bool open = false;
         const int64_t reach = (int64_t)(uint32_t)k[x0] - a.span - 1;
@@ -3364,7 +3373,9 @@ int global_path_eager(sedef_ctx* ctx, const FArgs& a, int64_t nov, unsigned long
       SlowTask* tasks = (SlowTask*)ctx_alloc(ctx, (size_t)nh * sizeof(SlowTask));
       if (!tasks) return SEDEF_ERR_OOM;
       SEDEF_CUDA(cudaMemsetAsync(counters + 6, 0, 8, st));
-      const dim3 g2((unsigned)(nb < (int64_t)ctx_sm_count(ctx) * 2 ? nb : (int64_t)ctx_sm_count(ctx) * 2), 4);
+      // a warp per part of a window, up to eight CTAs per SM
+      const int64_t gw = (nb * kGroupParts + 7) / 8, g8 = (int64_t)ctx_sm_count(ctx) * 8;
+      const int g2 = (int)(gw < g8 ? gw : g8);
       SEDEF_KERNEL(ctx, "k_slow_groups",
                    k_slow_groups<<<g2, 256, 0, st>>>(a, v0, v1, d_base, os, skeys, tasks,
                                                      counters + 6, (int64_t)nh, nullptr,
@@ -3857,7 +3868,8 @@ int run_filter(sedef_ctx* ctx, const uint64_t* qrec, int64_t nq, const int64_t* 
     while ((int64_t(1) << wbits) < nwin) ++wbits;
     SEDEF_TRY(radix_sort_u64(ctx, keys, vals, skeys, svals, H, 0, 33 + wbits, dhits));
     SEDEF_CUDA(cudaMemsetAsync(counters + 6, 0, 8, st));
-    const dim3 g2((unsigned)(nwin < (int64_t)ctx_sm_count(ctx) * 2 ? nwin : (int64_t)ctx_sm_count(ctx) * 2), 4);
+    const int64_t gw = (nwin * kGroupParts + 7) / 8, g8 = (int64_t)ctx_sm_count(ctx) * 8;
+    const int g2 = (int)(gw < g8 ? gw : g8);
     SEDEF_KERNEL(ctx, "k_slow_groups",
                  k_slow_groups<<<g2, 256, 0, st>>>(a, 0, nwin, d_base, os, skeys, tasks,
                                                    counters + 6, H, dnov, H));
