@@ -1185,20 +1185,28 @@ __global__ void __launch_bounds__(32 * kWWarps, W::MINB) k_filter_warp(FArgs a, 
       l_qa = a.win_qa[l_w];
       l_qb = a.win_qb[l_w];
     }
+    {
+      // windows of too many records go on together: side by side in the list
+      // they share records and postings in the tiers after this one
+      const bool over = l_qb - l_qa > (uint32_t)QC;
+      const unsigned bo = __ballot_sync(0xffffffffu, over);
+      if (bo) {
+        unsigned int to = 0;
+        if (lane == 0) to = atomicAdd(io.out_count, (unsigned int)__popc(bo));
+        to = __shfl_sync(0xffffffffu, to, 0);
+        if (over) io.out_list[to + __popc(bo & lt)] = l_w;
+      }
+    }
     for (int kk = 0; kk < nk; ++kk) {
       const uint32_t wdx = __shfl_sync(0xffffffffu, l_w, kk), i = __shfl_sync(0xffffffffu, l_i, kk);
       const uint32_t qa = __shfl_sync(0xffffffffu, l_qa, kk);
       const int c = (int)(__shfl_sync(0xffffffffu, l_qb, kk) - qa);
-      if (c == 0) continue;
+      if (c == 0 || c > QC) continue;
       auto hand_over = [&](bool wide) {
         if (lane != 0) return;
         if (wide && io.wide_list) io.wide_list[atomicAdd(io.wide_count, 1u)] = wdx;
         else io.out_list[atomicAdd(io.out_count, 1u)] = wdx;
       };
-      if (c > QC) {
-        hand_over(false);
-        continue;
-      }
       __syncwarp();  // the previous window's shared memory is free
       S.starts[lane] = 0u;
       S.starts[lane + 32] = 0u;
