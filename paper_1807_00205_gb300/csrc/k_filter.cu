@@ -3399,6 +3399,26 @@ int global_path_eager(sedef_ctx* ctx, const FArgs& a, int64_t nov, unsigned long
   return SEDEF_OK;
 }
 
+// Whether the ranges pay.  They cost a walk over all records whatever the
+// windows; they save a window's records a look into the offset table, the hits
+// before the window (half of the mean posting list) and, in a batch, the search
+// for the genome's part of the list.  Measured with and without them (w = 16,
+// n = 750: 87 records a window), the walk takes 36 ps a record and seven
+// launches, the search of a planned pass 52; a window gains 0.75 ns at 10 Mbp,
+// 2 to 3 at 100 Mbp, 11 at 1 Gbp, 6 to 13 in batches of 100 and 200 Mbp.
+// Filter of 1 Gbp with windows every 250 bases 80.9 ms with, 123 without;
+// every 3,000 equal; every 1 Mbp 3.8 and 0.23; of 10 Mbp 0.37 and 0.35; of 200
+// genomes of 1 Mbp 1.7 and 7.0, every 5,000 bases 1.0 and 0.59.  Windows past
+// the tiers' 256 records do not read them.
+bool ranges_pay(const Derived& D, int64_t nwin, int64_t nt, bool planned) {
+  const double records = 2.0 * (D.span + 1) / (D.w + 1);
+  if (records > kQCap) return false;
+  const double list = (double)nt / (double)(int64_t(1) << (2 * D.k));
+  const double gain_ns = (double)nwin * records * ((D.self_mode == 2 ? 0.057 : 0.023) + 0.015 * list);
+  const double cost_ns = planned ? 5e3 + 0.052 * (double)nt : 60e3 + 0.036 * (double)nt;
+  return gain_ns > cost_ns;
+}
+
 // Every query record's useful posting range of a self-search, once (the tiers
 // read them by record offset).  An eager pass walks the index when the query
 // records are its records, with the same sequence offsets (walk); a planned
@@ -3696,7 +3716,8 @@ int run_filter(sedef_ctx* ctx, const uint64_t* qrec, int64_t nq, const int64_t* 
   }
   a.after_own = D.overlap <= D.n ? 1 : 0;
   const std::vector<char> used_before = ctx_pool_snapshot(ctx);
-  if (ctx_extras(ctx) && (D.self_mode == 2 || (D.self_mode == 1 && a.after_own))) {
+  if (ctx_extras(ctx) && (D.self_mode == 2 || (D.self_mode == 1 && a.after_own)) &&
+      ranges_pay(D, nwin, nt, pl != nullptr)) {
     // The walk ranks target positions among the query's, so both have to be
     // one array (the autotuner may be given others).
     const bool walk = !pl && qrec == trec && nq == nt && nqseq == ntseq &&

@@ -18,6 +18,7 @@ def test_autotune_on_other_records(mode, which):
     ctx = binding.Context(0)
     g = synth.small_case(31, lengths=(120_000, 60_000), n_sd=8, sd_lo=1500, sd_hi=6000, mask_frac=0.1)
     d = oracle.params(self_mode=mode)
+    d["step"] = 3  # many windows: the ranges pay
     p = binding.params_from_dict(d)
     rec = ctx.sedef_sketch(*ctx.sedef_pack(torch.from_numpy(g.seq).to("cuda:0")), g.offsets, p)
     srt, off = ctx.sedef_index(rec, p)
@@ -30,7 +31,8 @@ def test_autotune_on_other_records(mode, which):
     assert any(x.endswith("k_qpost") for x in names) and not any(x.endswith("k_pos_bits") for x in names)
     recs = oracle.sketch(g.seq, g.offsets, d)
     runs, _ = ctx.sedef_filter(rec, g.offsets, rec, srt, off, g.offsets, p)
-    assert_rows_equal(run_rows(runs), oracle.filter_runs(recs, g.offsets, recs, g.offsets, d), "runs")
+    assert_rows_equal(run_rows(runs), oracle.filter_runs(recs, g.offsets, recs, g.offsets, d, threads=16),
+                      "runs")
     assert any(x.endswith("k_pos_bits") for x in ctx.sedef_trace_report(reset=True))
     with pytest.raises(binding.SedefError) as e:  # no target sequence for the third one
         ctx.sedef_filter_autotune(query, [0, 60_000, 120_000, g.length], rec, srt, off, g.offsets,

@@ -32,8 +32,9 @@ def accepted(ctx, caps, call):
     return ok
 
 
-@pytest.mark.parametrize("pd", [dict(), dict(k=13), dict(w=3, n=300, query_step=100), dict(self_mode=2),
-                                dict(self_mode=2, k=14)])
+# windows every few bases, so that the ranges pay
+@pytest.mark.parametrize("pd", [dict(query_step=20), dict(k=13, query_step=20), dict(w=3, n=300, query_step=10),
+                                dict(self_mode=2, query_step=40), dict(self_mode=2, k=14, query_step=40)])
 def test_filter_caps(pd):
     ctx = binding.Context(0)
     g = genome(pd.get("self_mode", 1))
@@ -42,8 +43,11 @@ def test_filter_caps(pd):
     srt, off = ctx.sedef_index(rec, p)
     want, n = ctx.sedef_filter(rec, g.offsets, rec, srt, off, g.offsets, p)
     want = want.cpu()
-    # the records' ranges alone are 8 bytes each; the caps reach well below that
-    caps = np.geomspace(4 * rec.numel(), 64 << 20, 120).astype(np.int64)
+    # the records' ranges alone are 8 bytes each, what a window and a run need less than 64 and 128;
+    # the caps reach below that
+    windows = ctx.sedef_filter_stats()["windows"]
+    with_per_window = 64 * windows + 128 * n
+    caps = np.geomspace(16 * windows, 128 << 20, 120).astype(np.int64)
     ctx.sedef_trace_enable(True)
     with_ranges = []
 
@@ -56,7 +60,7 @@ def test_filter_caps(pd):
     ok = accepted(ctx, caps, call)
     first = int(np.argmax(ok))
     assert ok[first:].all(), caps[first:][~ok[first:]]
-    assert caps[first] < 8 * rec.numel()
+    assert caps[first] < with_per_window + 8 * rec.numel()
     assert not with_ranges[0] and with_ranges[-1]
     ctx.close()
 
@@ -66,7 +70,7 @@ def test_stage_after_stage_caps():
     calls after it."""
     ctx = binding.Context(0)
     g = genome(1)
-    p = binding.params()
+    p = binding.params(query_step=20)
     d = to_dev(g.seq)
     want = binding.struct_view(ctx.sedef_selfsearch(d, g.offsets, p)[0], binding.CAND_DTYPE)
     out = ctx.selfsearch(d, g.offsets, p)
@@ -99,7 +103,7 @@ def test_graph_caps(mode):
     """A captured pass is recorded without the ranges and events where the cap has no room for them."""
     ctx = binding.Context(0)
     g = genome(mode)
-    p = binding.params(self_mode=mode)
+    p = binding.params(self_mode=mode, query_step=100)
     d = to_dev(g.seq)
     want = ctx.selfsearch(d, g.offsets, p)
     rows = binding.struct_view(want["cands"], binding.CAND_DTYPE)
@@ -162,7 +166,7 @@ def test_parted_ranges_caps():
     for at in range(0, 200_000, 10_000):
         s[9_000_000 + at:9_004_000 + at] = s[at:at + 4_000]
     g = synth.genome_from_parts([s])
-    p = binding.params(w=1, n=100, query_step=5_000)
+    p = binding.params(w=1, n=100, query_step=60)
     rec = ctx.sedef_sketch(*ctx.sedef_pack(to_dev(s)), g.offsets, p, cap=len(s))
     assert rec.numel() > 16 << 20
     srt, off = ctx.sedef_index(rec, p)
