@@ -49,7 +49,8 @@ struct ChainArgs {
   int64_t acap = 0;
   uint32_t* flags = nullptr;
   unsigned long long* atotal = nullptr;  // exact anchor total
-  // seeds past k_chain_seeds' sizes: run indices and their number
+  // seeds past k_chain_seeds' sizes: run indices and their number (big
+  // nullptr: every run)
   uint32_t* big = nullptr;
   uint32_t* nbig = nullptr;
   // query records less target records, summed (k_same_records): zero when they
@@ -374,14 +375,26 @@ __global__ void __launch_bounds__(32 * kSeedWarps) k_chain_seeds(ChainArgs a, se
   if (lane == 0 && anchors) atomicAdd(a.atotal, anchors);
 }
 
-// Anchors of the seeds k_chain_seeds left (big[0..nbig)).
+// The seeds of the device-memory path: those k_chain_seeds left, or every run.
+__device__ __forceinline__ int64_t seed_count(const ChainArgs& a) {
+  return a.big ? (int64_t)*a.nbig : a.nruns;
+}
+__device__ __forceinline__ int64_t seed_run(const ChainArgs& a, int64_t r) {
+  return a.big ? (int64_t)a.big[r] : r;
+}
+
+// Their anchors.
 __global__ void k_anchor_count(ChainArgs a, uint32_t* count) {
   resolve(a);
   const int lane = lane_id();
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < (int64_t)*a.nbig;
+  for (int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < seed_count(a);
        r += nw) {
-    const sedef_run_t run = a.runs[a.big[r]];
+    const sedef_run_t run = a.runs[seed_run(a, r)];
+    if (!run.keep) {
+      if (lane == 0) count[r] = 0;
+      continue;
+    }
     int total = 0;
     int64_t qa = 0, qb = 0;
     if (lane == 0) window_range(a, run.i, &qa, &qb);
@@ -406,11 +419,11 @@ __global__ void k_anchor_fill(ChainArgs a, const uint32_t* aoff, uint64_t* ancho
   resolve(a);
   const int lane = lane_id();
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < (int64_t)*a.nbig;
+  for (int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < seed_count(a);
        r += nw) {
-    const sedef_run_t run = a.runs[a.big[r]];
+    const sedef_run_t run = a.runs[seed_run(a, r)];
     // 32-bit offsets: a range that wraps or ends past the capacity is skipped
-    if (aoff[r + 1] < aoff[r] || (int64_t)aoff[r + 1] > a.acap ||
+    if (aoff[r + 1] == aoff[r] || aoff[r + 1] < aoff[r] || (int64_t)aoff[r + 1] > a.acap ||
         aoff[r + 1] - aoff[r] > (uint32_t)kMaxChainAnchors)
       continue;
     int64_t qa = 0, qb = 0;
@@ -446,7 +459,7 @@ __global__ void k_anchor_fill(ChainArgs a, const uint32_t* aoff, uint64_t* ancho
 __device__ void chain_one(const ChainArgs& a, int64_t r, const uint32_t* aoff, const uint64_t* anchors,
                           int32_t* f, int32_t* pred, sedef_chain_t* out) {
   const int lane = lane_id();
-  const sedef_run_t run = a.runs[a.big[r]];
+  const sedef_run_t run = a.runs[seed_run(a, r)];
   sedef_chain_t c;
   c.i = run.i;
   c.o = run.o;
@@ -462,7 +475,7 @@ __device__ void chain_one(const ChainArgs& a, int64_t r, const uint32_t* aoff, c
   if (A == 0 || over || big) {
     if (lane == 0) {
       c.qseq = c.q0 = c.q1 = c.tseq = c.t0 = c.t1 = 0;
-      out[a.big[r]] = c;
+      out[seed_run(a, r)] = c;
     }
     return;
   }
@@ -532,14 +545,14 @@ __device__ void chain_one(const ChainArgs& a, int64_t r, const uint32_t* aoff, c
   c.t0 = t0;
   c.t1 = t1;
   c.score = (score >= a.mtab[run.s]) ? (uint16_t)score : 0;
-  out[a.big[r]] = c;
+  out[seed_run(a, r)] = c;
 }
 
 __global__ void k_chain_dp(ChainArgs a, const uint32_t* aoff, const uint64_t* anchors, int32_t* f,
                            int32_t* pred, sedef_chain_t* out) {
   resolve(a);
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < (int64_t)*a.nbig; r += nw)
+  for (int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < seed_count(a); r += nw)
     chain_one(a, r, aoff, anchors, f, pred, out);
 }
 
@@ -839,42 +852,51 @@ int run_chain(sedef_ctx* ctx, const sedef_run_t* runs, int64_t nruns, const uint
     a.dnt = pl->n_rec;
     a.flags = pl->flags;
   }
-  // [0] anchors of every seed, [1] seeds for the device-memory path, [2] the
-  // most anchors one of them has, [3] and [4] k_same_records' sums
-  unsigned long long* sums = (unsigned long long*)ctx_alloc(ctx, 40);
-  uint32_t* cnt = (uint32_t*)ctx_alloc(ctx, (size_t)(nruns + 1) * 4);
-  a.big = (uint32_t*)ctx_alloc(ctx, (size_t)nruns * 4);
-  sedef_chain_t* tmp = (sedef_chain_t*)ctx_alloc(ctx, (size_t)nruns * sizeof(sedef_chain_t));
-  // the big seeds' anchor offsets, then the chains' places
-  uint32_t* pos = (uint32_t*)ctx_alloc(ctx, (size_t)(nruns + 1) * 4);
-  if (!sums || !cnt || !a.big || !tmp || !pos) return SEDEF_ERR_OOM;
-  SEDEF_CUDA(cudaMemsetAsync(sums, 0, 40, st));
-  a.atotal = sums;
-  a.nbig = (uint32_t*)(sums + 1);
-  uint32_t* amax = (uint32_t*)(sums + 2);
   // a self-search's query records are its target records by position: where
   // the caller gave an index that may be another's, both forms are launched
   // and the one that the records call for runs
   const bool join = one_sketch || (D.self_mode != 0 && nq == nt && nqseq == ntseq &&
                     std::memcmp(h_qoff, h_toff, (size_t)(ntseq + 1) * sizeof(int64_t)) == 0);
+  // Windows of more records than k_chain_seeds keeps, on average (the join
+  // takes kSeedQ records, the search kSeedA anchors): its try came on top of
+  // what the device-memory path costs.  Chains of 10 Mbp, before there were
+  // two paths, with every seed tried, and now: joined w = 5 0.38, 0.47, 0.38 ms
+  // (w = 6 0.34 -> 0.20 tried), searched w = 4 4.9, 6.2, 5.0 (w = 5 3.8 -> 1.9
+  // tried).
+  const bool dense = 2 * (D.span + 1) > (join ? kSeedQ * 9 / 10 : kSeedA) * (D.w + 1);
+  // [0] anchors of every seed, [1] seeds for the device-memory path, [2] the
+  // most anchors one of them has, [3] and [4] k_same_records' sums
+  unsigned long long* sums = (unsigned long long*)ctx_alloc(ctx, 40);
+  uint32_t* cnt = (uint32_t*)ctx_alloc(ctx, (size_t)(nruns + 1) * 4);
+  a.big = dense ? nullptr : (uint32_t*)ctx_alloc(ctx, (size_t)nruns * 4);
+  sedef_chain_t* tmp = (sedef_chain_t*)ctx_alloc(ctx, (size_t)nruns * sizeof(sedef_chain_t));
+  // the big seeds' anchor offsets, then the chains' places
+  uint32_t* pos = (uint32_t*)ctx_alloc(ctx, (size_t)(nruns + 1) * 4);
+  if (!sums || !cnt || (!dense && !a.big) || !tmp || !pos) return SEDEF_ERR_OOM;
+  SEDEF_CUDA(cudaMemsetAsync(sums, 0, 40, st));
+  a.atotal = sums;
+  a.nbig = (uint32_t*)(sums + 1);
+  uint32_t* amax = (uint32_t*)(sums + 2);
   const int64_t most = (int64_t)ctx_sm_count(ctx) * 5;
   const int sg = (int)((nruns + kSeedWarps - 1) / kSeedWarps < most ? (nruns + kSeedWarps - 1) / kSeedWarps : most);
-  if (join && !one_sketch) {
+  if (join && !one_sketch && !dense) {
     a.differ = sums + 3;
     const int64_t cg = (nq + 1023) / 1024;
     SEDEF_KERNEL(ctx, "k_same_records",
                  k_same_records<<<(int)(cg < most ? (cg > 0 ? cg : 1) : most), 256, 0, st>>>(
                      qrec, tsorted, nq, sums + 3));
   }
-  if (join)
+  if (join && !dense)
     SEDEF_KERNEL(ctx, "k_chain_seeds", k_chain_seeds<true><<<sg, 32 * kSeedWarps, 0, st>>>(a, tmp));
-  if (!one_sketch)
+  if (!one_sketch && !dense)
     SEDEF_KERNEL(ctx, "k_chain_seeds", k_chain_seeds<false><<<sg, 32 * kSeedWarps, 0, st>>>(a, tmp));
   int64_t nbig = nruns, A = 0;
   unsigned long long* h_sums = nullptr;
   if (!pl) {
     h_sums = (unsigned long long*)ctx_host(ctx, 24);
     if (!h_sums) return SEDEF_ERR_OOM;
+  }
+  if (!pl && !dense) {
     SEDEF_CUDA(cudaMemcpyAsync(h_sums, sums, 24, cudaMemcpyDeviceToHost, st));
     SEDEF_CUDA(cudaStreamSynchronize(st));
     nbig = (int64_t)(h_sums[1] & 0xFFFFFFFFull);
@@ -884,7 +906,8 @@ int run_chain(sedef_ctx* ctx, const sedef_run_t* runs, int64_t nruns, const uint
     // the seeds past the shared-memory sizes (a planned pass does not know
     // whether there are any)
     uint32_t* aoff = pos;
-    const int wb = grid_of(nbig * 32 < most * 256 ? nbig * 32 : most * 256, 256);
+    // a warp per seed; a pass that mostly has none of them starts fewer
+    const int wb = grid_of(!pl || dense || nbig * 32 < most * 256 ? nbig * 32 : most * 256, 256);
     if (pl) SEDEF_CUDA(cudaMemsetAsync(cnt, 0, (size_t)(nbig + 1) * 4, st));
     SEDEF_KERNEL(ctx, "k_anchor_count", k_anchor_count<<<wb, 256, 0, st>>>(a, cnt));
     SEDEF_KERNEL(ctx, "k_max_u32",
