@@ -49,7 +49,9 @@ __device__ __forceinline__ uint32_t codes4(uint32_t v, uint32_t& code) {
 
 // A thread classifies its 16 bytes four at a time (one at a time, 17
 // instructions a base, was bound by their issue: 3.1 Gbp in 2.78 ms; now 1.00
-// ms, 4.65 TB/s read and written); 16 bytes with a letter other than ACGT among them go one at a time.
+// ms, 4.65 TB/s read and written).  16 bytes with another one among them are
+// gone over once more, four at a time too (one at a time, 200 Mbp with an N in
+// every 16 took 0.237 ms, 0.133 this way).
 template <bool kAligned>
 __global__ void __launch_bounds__(256) k_pack(const uint8_t* __restrict__ seq, int64_t n,
                                               uint32_t* __restrict__ packed,
@@ -79,12 +81,14 @@ __global__ void __launch_bounds__(256) k_pack(const uint8_t* __restrict__ seq, i
         if (other) {
           word = m16 = 0;
 #pragma unroll
-          for (int x = 0; x < 16; ++x) {
-            uint32_t code, ms, isn;
-            classify((v[x >> 2] >> (8 * (x & 3))) & 0xFFu, code, ms, isn);
-            word |= code << (2 * x);
-            m16 |= ms << x;
-            n16 |= isn << x;
+          for (int x = 0; x < 4; ++x) {
+            uint32_t code;
+            // a one in each byte that is no base, and in each lowercase letter
+            const uint32_t no = __vcmpgtu4(codes4(v[x], code), 0u) & 0x01010101u;
+            const uint32_t low = __vcmpgeu4(v[x], 0x61616161u) & __vcmpleu4(v[x], 0x7A7A7A7Au) & 0x01010101u;
+            word |= (((code & ~(no * 3u)) * 0x01041040u) >> 24) << (8 * x);
+            m16 |= ((low * 0x01020408u) >> 24) << (4 * x);
+            n16 |= ((no * 0x01020408u) >> 24) << (4 * x);
           }
         }
       } else {
