@@ -328,9 +328,10 @@ int sedef_filter(sedef_ctx* ctx, const uint64_t* d_qrec, int64_t nq, const int64
                  const sedef_params* p, sedef_run_t* d_runs, int64_t run_cap, int64_t* h_nruns);
 
 /*
- * Autotuner of the filter's first shared-memory tier: times each compiled
- * shape (threads per query window; hits and dense groups a window may keep
- * in shared memory) on a uniform sample of the query windows (at least
+ * Autotuner of the filter's first shared-memory tier: times the warp tier
+ * (shape 0; the shapes below half of their number are the same) and each
+ * compiled shape that can take its place (threads per query window; hits and
+ * dense groups a window may keep in shared memory) on a uniform sample of the query windows (at least
  * 65,536 or one in sixteen; best of two timed runs each) with the same
  * arguments as sedef_filter, and keeps the fastest for later
  * sedef_filter calls on this context; *variant_out receives its number.

@@ -3738,9 +3738,10 @@ int run_filter(sedef_ctx* ctx, const uint64_t* qrec, int64_t nq, const int64_t* 
                    qrec, nq, a.qseq, nqseq, (const int64_t*)(d_up + ow), nwin, D.step, D.span, wi,
                    wqa, wqb, wseq, dnq));
   if (tune) {
-    // time every first-tier shape on a uniform sample of windows (at least
-    // 65,536 or a sixteenth of them, so that a run lasts long enough to
-    // time); keep the fastest
+    // time the warp tier (the variants with it launch the same kernels: it
+    // stands for them as variant 0) and every shape that takes its place, on a
+    // uniform sample of windows (at least 65,536 or a sixteenth of them, so
+    // that a run lasts long enough to time); keep the fastest
     const int64_t want = nwin / 16 > 65536 ? nwin / 16 : 65536;
     const int64_t stride = nwin > want ? nwin / want : 1;
     std::vector<uint32_t> sample;
@@ -3755,7 +3756,7 @@ int run_filter(sedef_ctx* ctx, const uint64_t* qrec, int64_t nq, const int64_t* 
     SEDEF_CUDA(cudaEventCreate(&e1));
     int best_v = 0;
     float best_ms = 1e30f;
-    for (int v = 0; v < kNumVariants; ++v) {
+    for (int v = 0; v < kNumVariants; v = v == 0 ? kNumShapes : v + 1) {
       float ms = 0.f;
       const int sh = v % kNumShapes;
       const bool warp_tier = v < kNumShapes;

@@ -39,3 +39,21 @@ def test_autotune_on_other_records(mode, which):
                                   binding.params(self_mode=2))
     assert e.value.status == -1
     ctx.close()
+
+
+def test_each_shape_is_timed_once():
+    """The shapes with the warp tier are one and the same: timed once, reported as shape 0."""
+    torch = need_gpu()
+    ctx = binding.Context(0)
+    g = synth.small_case(32, lengths=(90_000,), n_sd=4)
+    p = binding.params()
+    rec = ctx.sedef_sketch(*ctx.sedef_pack(torch.from_numpy(g.seq).to("cuda:0")), g.offsets, p)
+    srt, off = ctx.sedef_index(rec, p)
+    count = ctx.sedef_filter_variant()[1]
+    ctx.sedef_trace_enable(True)
+    v = ctx.sedef_filter_autotune(rec, g.offsets, rec, srt, off, g.offsets, p)
+    assert v == 0 or count // 2 <= v < count
+    timed = [n for k, (n, _) in ctx.sedef_trace_report(reset=True).items() if k.endswith("k_filter_tune")]
+    # three times each: the warp tier and four after it, tier 1 and 2 and the four
+    assert timed == [3 * (5 + count // 2 * 6)]
+    ctx.close()
