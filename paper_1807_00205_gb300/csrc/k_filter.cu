@@ -78,7 +78,6 @@ struct FArgs {
   int64_t run_cap;
   uint32_t* ov_list;
   unsigned int* nov;
-  unsigned int* next_window;
   unsigned long long* stats;  // [0] hits enumerated, [1] hits collected (fast path)
 };
 
@@ -2407,16 +2406,15 @@ __global__ void k_gather_runs(const sedef_run_t* in, const uint32_t* perm, int64
 
 // ----------------------------------------------------------------- refine --
 //
-// Two kernels: a lean one (k_refine_batch: at most 256 query records and 512
-// span records per run) and a large one (any run, in pieces of at most 1024
-// span records) for the runs the lean one hands over.
+// Two kernels: k_refine_batch (at most 256 query records and 512 span records
+// per run) and k_refine (any run, in pieces of at most 1024 span records) for
+// the runs that k_refine_batch hands over.
 //
 // The estimate at j never exceeds the number of W_Q hashes shared with the
 // window (the filter's shared_o(j)), so it is evaluated only where that
 // count exceeds the best estimate so far, and the run is finished as soon
 // as the best estimate reaches the run's max_shared.
 
-constexpr int kRWarps = 8;     // lean kernel: warps per CTA
 constexpr int kRWarpsBig = 4;  // large kernel
 
 template <int QC, int RC>
@@ -2518,14 +2516,14 @@ struct RefineArgs {
   unsigned int* nbig;
   const uint4* ranges;  // per run: query records [x, y), span records [z, w)
   unsigned long long* next;  // chunk counters of the two kernels
-  // lean kernel: event words (ev_words + kEvPad per warp), W_Q hashes per roll
+  // k_refine_batch: event words (ev_words + kEvPad per warp), W_Q hashes per roll
   uint32_t* events = nullptr;
   int ev_words = 0;
   int scap = 0;
 };
 
-template <int QC, int RC, bool kLean>
-__global__ void __launch_bounds__(32 * (kLean ? kRWarps : kRWarpsBig)) k_refine(RefineArgs a) {
+template <int QC, int RC>
+__global__ void __launch_bounds__(32 * kRWarpsBig) k_refine(RefineArgs a) {
   a.nruns = live_n(a.nruns, a.dnruns);
   a.nt = live_n(a.nt, a.dnt);
   using RW = RefineWarpT<QC, RC>;
@@ -2534,7 +2532,7 @@ __global__ void __launch_bounds__(32 * (kLean ? kRWarps : kRWarpsBig)) k_refine(
   const int warp = threadIdx.x >> 5, lane = lane_id();
   RW& R = reinterpret_cast<RW*>(smem_raw)[warp];
   auto pos_of = [](uint64_t r) { return (uint64_t)((r >> 1) & 0xFFFFFFFFull); };
-  const int64_t count = kLean ? a.nruns : (int64_t)*a.nbig;
+  const int64_t count = (int64_t)*a.nbig;
   // contiguous chunks of runs per warp (runs of one window are adjacent, so
   // W_Q is built once per window and chunk), handed out dynamically
   constexpr int kChunk = 16;
@@ -2542,26 +2540,19 @@ __global__ void __launch_bounds__(32 * (kLean ? kRWarps : kRWarpsBig)) k_refine(
   int s = 0;
   while (true) {
     int64_t c0 = 0;
-    if (lane == 0) c0 = (int64_t)atomicAdd(kLean ? a.next : a.next + 1, (unsigned long long)kChunk);
+    if (lane == 0) c0 = (int64_t)atomicAdd(a.next + 1, (unsigned long long)kChunk);
     c0 = __shfl_sync(0xffffffffu, c0, 0);
     if (c0 >= count) break;
     const int64_t c1 = min(count, c0 + kChunk);
   for (int64_t t = c0; t < c1; ++t) {
-    const int64_t ri = kLean ? t : (int64_t)a.big[t];
+    const int64_t ri = (int64_t)a.big[t];
     const sedef_run_t run = a.runs[ri];
     const int64_t i = run.i, ja = run.j_a, jb = run.j_b;
     const int o = run.o;
-    const uint4 rg = a.ranges[ri];  // query records [qa, qb), span records [rlo, rend)
+    const uint4 rg = a.ranges[ri];  // query records [qa, qb), span records from rlo on
     const int64_t qa = rg.x, qb = rg.y;
     int64_t rlo = rg.z;
-    const int64_t rend = rg.w;
     const int c = (int)(qb - qa);
-    if (kLean) {
-      if (c > QC || rend - rlo > RC) {
-        if (lane == 0) a.big[atomicAdd(a.nbig, 1u)] = (uint32_t)ri;
-        continue;
-      }
-    }
     if (qa != prev_qa || qb != prev_qb) {
     prev_qa = qa;
     prev_qb = qb;
@@ -2842,7 +2833,7 @@ __global__ void __launch_bounds__(32 * (kLean ? kRWarps : kRWarpsBig)) k_refine(
   }
 }
 
-// ------------------------------------------------- batched lean refine ----
+// ------------------------------------------------- batched refine ----
 //
 // A warp sets up runs one at a time (cooperatively), writing each run's
 // events to its own stretch of device memory, then every lane rolls one run,
@@ -2872,7 +2863,7 @@ __global__ void __launch_bounds__(32 * (kLean ? kRWarps : kRWarpsBig)) k_refine(
 // run into shared-memory slots and took 32 runs per warp whatever their
 // number: 1.26 M runs of a 200-genome batch 17.4 -> 4.1 ms, 2.5 M runs of a
 // 240 Mbp assembly 19.7 -> 5.0 ms, 299 runs of a 2 Mbp genome 1.75 -> 0.08 ms.
-// Runs beyond the lean limits (more than 256 query records,
+// Runs beyond its limits (more than 256 query records,
 // 512 span records, a span of 65,536 bases, more W_Q hashes than the launch's
 // counters or a count past 255) go to the large kernel.
 
@@ -3503,9 +3494,9 @@ int order_and_refine(sedef_ctx* ctx, const FArgs& a, const Derived& D, int nqseq
   // (2 / (w + 1) of its starts): the sizes between runs differ by a few
   int scap = ((int)(1.35 * 2.0 * (D.span + 1) / (D.w + 1)) + 31) / 32 * 32;
   scap = scap < 64 ? 64 : (scap > kBQC ? kBQC : scap);
-  const size_t lean_sm = refine_warp_bytes(scap) * kBWarps;
-  SEDEF_TRY(ensure_smem_attr((const void*)k_refine_batch, lean_sm));
-  SEDEF_TRY(ensure_smem_attr((const void*)k_refine<kMaxWindowRecs, 1024, false>,
+  const size_t batch_sm = refine_warp_bytes(scap) * kBWarps;
+  SEDEF_TRY(ensure_smem_attr((const void*)k_refine_batch, batch_sm));
+  SEDEF_TRY(ensure_smem_attr((const void*)k_refine<kMaxWindowRecs, 1024>,
                              sizeof(RefineWarpT<kMaxWindowRecs, 1024>) * kRWarpsBig));
   // order runs by (i, o); the sweep emits each window's runs in j order
   ctx_set_stage(ctx, "runsort");
@@ -3543,7 +3534,7 @@ int order_and_refine(sedef_ctx* ctx, const FArgs& a, const Derived& D, int nqseq
   }
   SEDEF_KERNEL(ctx, "k_gather_runs",
                k_gather_runs<<<tb, 256, 0, st>>>(raw, perm, total, runs, druns));
-  // refine: lean kernel over all runs, then the large kernel over the runs
+  // refine: k_refine_batch over all runs, then the large kernel over the runs
   // it handed over (their count stays on the device)
   ctx_set_stage(ctx, "refine");
   uint32_t* big = (uint32_t*)ctx_alloc(ctx, (size_t)total * 4);
@@ -3576,7 +3567,7 @@ int order_and_refine(sedef_ctx* ctx, const FArgs& a, const Derived& D, int nqseq
   const size_t big_sm = sizeof(Big) * kRWarpsBig;
   int rper = 0;
   SEDEF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&rper, k_refine_batch, 32 * kBWarps,
-                                                           lean_sm));
+                                                           batch_sm));
   if (rper < 1) rper = 1;
   int64_t rgrid = (total + kBWarps - 1) / kBWarps;
   if (rgrid > (int64_t)ctx_sm_count(ctx) * rper) rgrid = (int64_t)ctx_sm_count(ctx) * rper;
@@ -3595,12 +3586,12 @@ int order_and_refine(sedef_ctx* ctx, const FArgs& a, const Derived& D, int nqseq
   }
   if (ra.events) {
     SEDEF_KERNEL(ctx, "k_refine",
-                 k_refine_batch<<<(int)rgrid, 32 * kBWarps, lean_sm, st>>>(ra));
+                 k_refine_batch<<<(int)rgrid, 32 * kBWarps, batch_sm, st>>>(ra));
   } else {
     SEDEF_KERNEL(ctx, "k_refine_all", k_refine_all<<<tb, 256, 0, st>>>(ra));
   }
   SEDEF_KERNEL(ctx, "k_refine_big",
-               k_refine<kMaxWindowRecs, 1024, false><<<ctx_sm_count(ctx), 32 * kRWarpsBig, big_sm,
+               k_refine<kMaxWindowRecs, 1024><<<ctx_sm_count(ctx), 32 * kRWarpsBig, big_sm,
                                                        st>>>(ra));
   ctx_pool_restore(ctx, used_before);  // the events
   return SEDEF_OK;
@@ -3699,7 +3690,6 @@ int run_filter(sedef_ctx* ctx, const uint64_t* qrec, int64_t nq, const int64_t* 
   a.run_cap = cap;
   a.ov_list = ovl;
   a.nov = (unsigned int*)(counters + 1);
-  a.next_window = (unsigned int*)(counters + 2);
   a.stats = counters + 4;
 
   a.qpost = nullptr;
@@ -4445,7 +4435,6 @@ int sedef_server_create(sedef_ctx* ctx, const uint64_t* d_trec, const uint64_t* 
     a.run_cap = L.run_cap;
     a.ov_list = L.ov;
     a.nov = (unsigned int*)(L.counters + 1);
-    a.next_window = (unsigned int*)(L.counters + 2);
     a.stats = L.counters + 4;
     sdev[k].a = a;
     sdev[k].done = L.done;
