@@ -232,6 +232,7 @@ __device__ void sweep_group(const FArgs& a, const WinInfo& w, Get get, int64_t L
 // global path of a 950 kbp region against a 3.1 Gbp index).
 template <typename Get, typename Emit>
 __device__ void find_groups(Get get, int64_t L, int m, int span, Emit emit) {
+  m = max(m, 1);  // a threshold of 0 (a tiny tau) asks no more of the hits than 1
   const int lane = lane_id();
   const unsigned lt = lanemask_lt();
   int64_t carry_hi = INT64_MIN;  // largest jhi of the dense hits seen so far
@@ -2247,7 +2248,7 @@ __global__ void k_slow_groups(FArgs a, int64_t v0, int64_t v1, const unsigned lo
   for (int64_t v = v0 + w / parts; v < v1; v += warps / parts) {
     const int s = s_of[v];
     if (s == 0 || base[v + 1] < base[v] || (int64_t)(base[v + 1] - base[v0]) > hcap) continue;
-    const int m = a.mtab[s];
+    const int m = max(a.mtab[s], 1);
     const int64_t lo = (int64_t)(base[v] - base[v0]), hi = (int64_t)(base[v + 1] - base[v0]);
     if (part > 0 && lo + part * chunk >= hi) continue;
     int64_t split;

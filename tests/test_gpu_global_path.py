@@ -69,3 +69,21 @@ def test_groups_of_many_windows_are_cheap(ctx):
         ms = {k.split(":")[1]: v[1] for k, v in ctx.sedef_trace_report(reset=True).items() if k.startswith("filter")}
     ctx.sedef_trace_enable(False)
     assert ms["k_slow_groups"] < 0.5 * ms["k_rs_pass"], ms
+
+
+@pytest.mark.parametrize("w", [1, 16])
+def test_threshold_of_zero(ctx, w):
+    """tau so small that m(s) = 0: a dense group is one hit, and none before the first is read."""
+    g = copies(30_000)
+    p = binding.params(self_mode=0, w=w, n=400, k=14, query_step=300, delta_m=2.0)
+    m = np.ones(400, dtype=np.int32)
+    assert ctx.lib.sedef_threshold_table(binding.ctypes.byref(p), m.ctypes.data, 399, None) == 0 and not m.any()
+    rec = ctx.sedef_sketch(*ctx.sedef_pack(to_dev(g.seq)), g.offsets, p, cap=g.length)
+    srt, off = ctx.sedef_index(rec, p)
+    for v in (0, 12):
+        ctx.sedef_filter_variant(v)
+        runs, n = ctx.sedef_filter(rec, g.offsets, rec, srt, off, g.offsets, p)
+        rows = binding.struct_view(runs, binding.RUN_DTYPE)
+        assert n == len(rows) and (w == 16 or n > 0)
+        assert (rows["j_a"] <= rows["j_b"]).all() and (rows["j_b"].astype(np.int64) + 400 <= g.length).all()
+    ctx.sedef_filter_variant(0)
