@@ -193,8 +193,10 @@ int sedef_set_stream(sedef_ctx* ctx, void* stream);
 /*
  * Caps the device scratch memory the context may hold (its pool and the
  * buffers of sedef_selfsearch*) at `bytes` (< 0: no cap, the default).  A
- * call whose scratch would pass the cap fails with SEDEF_ERR_OOM as if
- * cudaMalloc had failed, and the context stays usable.  Lowering the cap
+ * call whose scratch would pass the cap runs once more from an empty pool and
+ * without the buffers that only make it faster; when that does not fit either
+ * it fails with SEDEF_ERR_OOM as if cudaMalloc had failed, and the context
+ * stays usable.  Lowering the cap
  * below what the context holds gives its blocks back first.  Synchronizes.
  */
 int sedef_set_scratch_limit(sedef_ctx* ctx, int64_t bytes);
@@ -234,8 +236,10 @@ uint64_t sedef_launch_count(void);
 
 /*
  * Counters of the context's last sedef_filter call, out[0..n): query
- * windows, windows sent to the global-memory path, hits enumerated and hits
- * collected by the shared-memory path, runs, runs refined by the large
+ * windows, windows sent to the global-memory path, hits enumerated (posting
+ * entries looked at: in a self-search that resolves its records' posting
+ * ranges first, only those after a record's own) and hits collected by the
+ * shared-memory path, runs, runs refined by the large
  * refine kernel, hits of the global-memory path; out[7] = anchors of the
  * context's last sedef_chain call (at most 8 values).  out[6] and out[7]
  * are the totals a captured pass needs as capacities.

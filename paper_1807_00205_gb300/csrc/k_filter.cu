@@ -1443,7 +1443,7 @@ int launch_warp_tier_as(sedef_ctx* ctx, const FArgs& a, const TierIO& io, int64_
 
 // w: winnowing window.  A query window holds 2 / (w + 1) of its starts as
 // records on average; the shape for 256 records has five CTAs per SM where
-// the one for 128 has seven, so it is taken only where 128 would not do.
+// the one for 128 has eight, so it is taken only where 128 would not do.
 int launch_warp_tier(sedef_ctx* ctx, const FArgs& a, const TierIO& io, int64_t max_windows, int w,
                      const char* name) {
   if (1.35 * 2.0 * (a.span + 1) / (w + 1) <= 128.0)
@@ -3264,9 +3264,10 @@ int launch_fast(sedef_ctx* ctx, const FArgs& a, const TierIO& io_in, int64_t max
   SEDEF_TRY(ensure_smem_attr((const void*)k_filter_fast<TPB, LCAP, GCAP, SLOTS>, sm));
   // a table of 2,048 counters separates about as many hits: a window with
   // more passes nearly all of them on to its sort, and is better off in the
-  // wide tier (a 100 Mbp chromosome's tiers took 17.6 ms with the line at
-  // twice as many hits and 10.2 ms with it here; half as many: the wide
-  // tier's fixed cost per window, a 240 Mbp assembly 57.0 -> 65.7 ms)
+  // CTA tier (measured when these shapes came after the warp tier on every
+  // pass: a 100 Mbp chromosome's tiers 17.6 ms with the line at twice as many
+  // hits and 10.2 ms with it here; half as many: the next tier's fixed cost per
+  // window, a 240 Mbp assembly's pass 57.0 -> 65.7 ms)
   TierIO io = io_in;
   io.hlim = (uint32_t)(SLOTS == kSlots ? SLOTS : 2 * SLOTS);
   int per_sm = 0;
@@ -3970,8 +3971,9 @@ namespace {
 constexpr int kServeMaxSlots = 64;
 // One CTA per SM of 256 threads (16 K registers) and ~53 KB of shared
 // memory: the rest of every SM stays free for the admission and finishing
-// kernels (the radix sort's scatter alone takes ~39 K registers per CTA),
-// which would otherwise wait for the persistent kernel to leave.
+// kernels (a CTA of the deep and second wide tiers takes 32 K registers, a sort
+// pass 16 to 20 K), which would otherwise wait for the persistent kernel to
+// leave.
 constexpr int kServeTPB = CtaNarrow::TPB;
 using ServeSmem = CtaSmemT<CtaNarrow>;
 // Windows with more posting entries than the shape keeps go to the slot's

@@ -316,9 +316,11 @@ __device__ __forceinline__ uint32_t reverse_pairs(uint32_t v) {
 // kMode 0: count the records of each CTA tile; 1: write them at the tile
 // offsets given; 2: one pass, offsets by look-back.
 //
-// Bound by the integer pipes: little over one warp instruction per base at
-// k = 12, w = 16 (the form that hashed into shared memory and took van Herk
-// minima from it ran 8.1).  A lane holds as many positions as its registers
+// Bound by the integer pipe and the tile's barriers: two warp instructions a
+// base at k = 12, w = 16 (the form that hashed into shared memory and took van
+// Herk minima from it ran 8.1); on 240 Mbp the pipe is busy 73% of the time,
+// and what the warps wait for otherwise is warp 0's look-back between the two
+// barriers of a tile (7 of 13 stalled warps).  A lane holds as many positions as its registers
 // allow (16 keys and their shifted copies in 64 registers, four CTAs per SM);
 // the lanes without windows, two of 32 at w = 16, are the waste.  3.1 Gbp:
 // 33.7 -> 9.8 ms, 240 Mbp: 2.6 -> 0.78 ms.  Of that the look-back was most:
@@ -577,8 +579,8 @@ int run_sketch(sedef_ctx* ctx, const uint32_t* packed, const uint32_t* mask, con
     if (*nrec > cap) return fail(SEDEF_ERR_CAPACITY, "sedef_sketch: record buffer too small");
     return SEDEF_OK;
   }
-  // planned pass (one CUDA graph, no waits between CTAs): count, scan and
-  // write; the write pass stores the records below the capacity and the
+  // planned pass (one CUDA graph): count, scan and write, without waits
+  // between CTAs; the write pass stores the records below the capacity and the
   // exact total stays on the device
   uint32_t* cnt = (uint32_t*)ctx_alloc(ctx, (size_t)(a.ntiles + 1) * 4);
   uint32_t* toff = (uint32_t*)ctx_alloc(ctx, (size_t)(a.ntiles + 1) * 4);

@@ -185,10 +185,12 @@ __device__ __noinline__ uint32_t count_before(const uint64_t* kin, int64_t end, 
   return cnt[threadIdx.x];
 }
 
-// One pass.  Bound by shared-memory and issue work per key (votes, staging)
-// and, between CTAs, by the look-back: a thread per digit reads eight tiles'
-// status at once.  365 M records over 24 bits: 8.0 -> 5.2 ms with the count
-// (three kernels a pass, 147 registers and one CTA of 256 threads per SM).
+// One pass.  Bound by the integer pipe: six to seven warp instructions a key,
+// most of them the votes (73% of the pipe and 60% of the issue slots busy in a
+// sort of 14.3 M records, waits for the keys' loads next).  Between CTAs a
+// thread per digit reads eight tiles' status at once.  194 M records over 24
+// bits: 8.0 -> 5.2 ms with the count, 2.1 TB/s or 31% of the copy rate (before:
+// three kernels a pass, 147 registers and one CTA of 256 threads per SM).
 template <bool kVals>
 __global__ void __launch_bounds__(kRsThreads, kVals ? 3 : 4) k_rs_pass(
     const uint64_t* __restrict__ kin, const uint32_t* __restrict__ vin, uint64_t* __restrict__ kout,
