@@ -172,16 +172,20 @@ __device__ __forceinline__ void rank_round(uint32_t* wcnt, uint32_t d, uint32_t 
   loc = before + rank;
 }
 
-// This thread's digit among the first `end` keys, counted by the whole CTA.
-// For a tile whose wait ran out: what it would have read from the tiles before
-// it, so every key goes to its place whatever the other CTAs do.  Out of line:
-// the pass has no registers to spare.
+// This thread's digit among the first `end` keys, counted by its warp: what a
+// tile whose wait ran out would have read from the tiles before it, so every
+// key goes to its place whatever the other CTAs do.  cnt: the warp's row, which
+// only its own staging reads.  Out of line: the pass has no registers to spare.
 __device__ __noinline__ uint32_t count_before(const uint64_t* kin, int64_t end, int shift, uint32_t dmask,
                                               uint32_t* cnt) {
+  __syncwarp();
   cnt[threadIdx.x] = 0;
-  __syncthreads();
-  for (int64_t x = threadIdx.x; x < end; x += kRsThreads) atomicAdd(cnt + digit_of(kin[x], shift, dmask), 1u);
-  __syncthreads();
+  __syncwarp();
+  for (int64_t x = threadIdx.x & 31; x < end; x += 32) {
+    const uint32_t d = digit_of(kin[x], shift, dmask);
+    if ((d >> 5) == (threadIdx.x >> 5)) atomicAdd(cnt + d, 1u);
+  }
+  __syncwarp();
   return cnt[threadIdx.x];
 }
 
@@ -290,15 +294,12 @@ __global__ void __launch_bounds__(kRsThreads, kVals ? 3 : 4) k_rs_pass(
         }
       }
     }
-    if (!ran_out) st_relaxed_gpu(mine, kPrefix | (before + count));
+    if (__any_sync(0xffffffffu, ran_out))
+      before = count_before(kin, tile * kRsTile, shift, dmask, S.wcnt[warp]);
+    st_relaxed_gpu(mine, kPrefix | (before + count));
     S.gofs[d] = S.base[d] + before - start;
     if (threadIdx.x == 0) S.tile = (long long)atomicAdd(sc.ticket + pass, 1u);
-    if (__syncthreads_or(ran_out)) {
-      before = count_before(kin, tile * kRsTile, shift, dmask, S.wcnt[0]);
-      if (ran_out) st_relaxed_gpu(mine, kPrefix | (before + count));
-      S.gofs[d] = S.base[d] + before - start;
-      __syncthreads();
-    }
+    __syncthreads();
 #pragma unroll 4
     for (int x = threadIdx.x; x < cnt; x += kRsThreads) {
       const uint64_t kk = S.keys[x];
