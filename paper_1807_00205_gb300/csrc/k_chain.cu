@@ -170,8 +170,7 @@ struct alignas(16) SeedSmem {
 // 1.2 ms.
 template <bool kJoin>
 __global__ void __launch_bounds__(32 * kSeedWarps) k_chain_seeds(ChainArgs a, sedef_chain_t* out) {
-  // of the two forms the one for the records at hand
-  if (a.differ && ((a.differ[0] | a.differ[1]) != 0ull) == kJoin) return;
+  if (kJoin && a.differ && (a.differ[0] | a.differ[1]) != 0ull) return;  // other records
   resolve(a);
   __shared__ SeedSmem smem[kSeedWarps];
   SeedSmem& S = smem[threadIdx.x >> 5];
@@ -853,8 +852,8 @@ int run_chain(sedef_ctx* ctx, const sedef_run_t* runs, int64_t nruns, const uint
     a.flags = pl->flags;
   }
   // a self-search's query records are its target records by position: where
-  // the caller gave an index that may be another's, both forms are launched
-  // and the one that the records call for runs
+  // the caller gave an index that may be another's, the join returns at once
+  // when it is, and the search is launched after the counts are read
   const bool join = one_sketch || (D.self_mode != 0 && nq == nt && nqseq == ntseq &&
                     std::memcmp(h_qoff, h_toff, (size_t)(ntseq + 1) * sizeof(int64_t)) == 0);
   // Windows of more records than k_chain_seeds keeps, on average (the join
@@ -888,17 +887,22 @@ int run_chain(sedef_ctx* ctx, const sedef_run_t* runs, int64_t nruns, const uint
   }
   if (join && !dense)
     SEDEF_KERNEL(ctx, "k_chain_seeds", k_chain_seeds<true><<<sg, 32 * kSeedWarps, 0, st>>>(a, tmp));
-  if (!one_sketch && !dense)
+  if (!join && !dense)
     SEDEF_KERNEL(ctx, "k_chain_seeds", k_chain_seeds<false><<<sg, 32 * kSeedWarps, 0, st>>>(a, tmp));
   int64_t nbig = nruns, A = 0;
   unsigned long long* h_sums = nullptr;
   if (!pl) {
-    h_sums = (unsigned long long*)ctx_host(ctx, 24);
+    h_sums = (unsigned long long*)ctx_host(ctx, 40);
     if (!h_sums) return SEDEF_ERR_OOM;
   }
   if (!pl && !dense) {
-    SEDEF_CUDA(cudaMemcpyAsync(h_sums, sums, 24, cudaMemcpyDeviceToHost, st));
+    SEDEF_CUDA(cudaMemcpyAsync(h_sums, sums, 40, cudaMemcpyDeviceToHost, st));
     SEDEF_CUDA(cudaStreamSynchronize(st));
+    if (a.differ && (h_sums[3] | h_sums[4]) != 0ull) {
+      SEDEF_KERNEL(ctx, "k_chain_seeds", k_chain_seeds<false><<<sg, 32 * kSeedWarps, 0, st>>>(a, tmp));
+      SEDEF_CUDA(cudaMemcpyAsync(h_sums, sums, 24, cudaMemcpyDeviceToHost, st));
+      SEDEF_CUDA(cudaStreamSynchronize(st));
+    }
     nbig = (int64_t)(h_sums[1] & 0xFFFFFFFFull);
     ctx_set_anchor_total(ctx, (int64_t)h_sums[0]);
   }
